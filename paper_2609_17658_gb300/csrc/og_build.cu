@@ -964,7 +964,7 @@ __global__ void k_records(int64_t n, const uint32_t *__restrict__ d_nchild, int6
             r.z = pz[item];
             r.m = pm32[item];
             r.M = pm64[item];
-            r.info = 0;
+            r.info = 1u << 31;
             r.ref = item;
         } else {
             int64_t j = item - n;
@@ -973,7 +973,7 @@ __global__ void k_records(int64_t n, const uint32_t *__restrict__ d_nchild, int6
             r.z = ncom[3 * j + 2];
             r.M = nmom[j].M;
             r.m = __double2float_rn(r.M);
-            r.info = (1u << 31) | ((uint32_t)nlev[j] << 26) | (nccnt[j] & 0x3ffffffu);
+            r.info = ((uint32_t)nlev[j] << 26) | (nccnt[j] & 0x3ffffffu);
             r.ref = ncbeg[j];
             // the walk pushes (ref, count) unchecked: a node has children, inside
             // the child array, and is never a root

@@ -38,7 +38,7 @@ struct __align__(16) CRec {
     uint32_t x, y, z;   // particle position or node centre of mass (fixed point)
     float m;            // mass (f32) used by the pair arithmetic
     double M;           // mass (f64) used by the relative opening test
-    uint32_t info;      // bit 31: node; bits 26..30: level; bits 0..25: child count
+    uint32_t info;      // bit 31: particle; bits 26..30: level; bits 0..25: child count
     uint32_t ref;       // particle: sorted index; node: first entry in the child array
 };
 static_assert(sizeof(CRec) == 32, "CRec must be 32 bytes");
@@ -330,7 +330,8 @@ struct WalkParams {
     float hnear2f;     // hnear2 raised by more than the FP32 error of a squared distance
     float h;           // softening length, grid units
     float inv_h;
-    float inv_2rs;     // 1 / (2 r_s), grid units
+    float erf_ky;      // 2 r_s / p of the erfc fit, grid units (og_walk.cu)
+    float erf_c;       // (2 / sqrt(pi)) / (2 r_s)
     float kexp;        // -log2(e) / (4 r_s^2), grid units
     float out_scale;   // G (2^32/L)^2
     float pot_scale;   // G 2^32/L (potential from grid units)

@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(32 * kSphWarps) k_sph_density(SphArgs a) {
         const bool has = lane < total;
         CRec rec{};
         if (has) rec = a.crec[obeg + (lane - oexcl)];
-        const bool node = has && (rec.info >> 31);
+        const bool node = has && !(rec.info >> 31);
         bool push = false, app = false;
         if (node) {
             const uint32_t lev = (rec.info >> 26) & 31u;

@@ -23,20 +23,30 @@
 //                   "far" entries (integer distance from the group box >= h,
 //                   so no target can need the softened kernel) and "near"
 //                   entries.  A full chunk is evaluated by every lane for its
-//                   target: exact int32 minimum-image separation, converted to
-//                   FP32, r^2 by FMA, cutoff, rsqrt, erfc split factor, spline
-//                   softening for near entries only, FP32 accumulation over the
-//                   chunk, then a compensated (Kahan) add into the totals.
-//                   A group of g <= 16 targets replicates each target on
-//                   32 / P lanes (P the next power of two >= g) that split the
-//                   chunk's entries; the replicas' totals are added in a fixed
-//                   order at the end.
+//                   two targets: exact int32 minimum-image separations,
+//                   converted to FP32, r^2 by FMA, cutoff, rsqrt, erfc split
+//                   factor, spline softening for near entries only, FP32
+//                   accumulation over the chunk, then a compensated (Kahan) add
+//                   into the totals.  A group of g targets takes P = ceil(g / 2)
+//                   lanes; 32 / P replicas of them split the chunk's entries,
+//                   and the replicas' totals are added in a fixed order at the end.
+//
+// What bounds it (2.1M clustered, Barnes-Hut pass, 2.75 ms): instruction issue
+// (74 % of cycles) and the pipes behind it.  2.4 G warp instructions, 1.3 G of
+// them the far loop: 42 a pair of interactions, beside which the pair keeps the
+// multi-function pipe 40 cycles and the FMA pipe 36 busy, so no one unit can be
+// relieved alone: forcing the integer differences to the other pipe, registers
+// for 6 or 8 blocks per SM, or 2 to 8 entries in flight all measured within 2 %.
+// The list building is the other 1 G, about 390 a round of 64 slots.  Two targets
+// a lane, the straight-line classification and the new erfc fit took the pass
+// from 3.40 to 2.75 ms and the two-pass walk from 7.10 to 5.73 ms.
 //
 // Work distribution: persistent blocks; warps take groups from a global
 // atomic counter, in decreasing order of the previous pass's list length
 // when that is known (longest first shortens the tail of the launch).
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -46,31 +56,48 @@ namespace og {
 namespace {
 
 constexpr int kMaxWarps = 8;       // warps per block: 1..kMaxWarps, chosen at launch
-constexpr int kStackCap = 768;     // ranges per warp stack
-constexpr int kNearChunk = 64;     // near entries per shared chunk (>= 64: see kMinChunk)
-// The far chunk holds `chunk` entries (WalkArgs::chunk, chosen at launch,
-// kMinChunk..kMaxChunk): a round adds at most 64 entries to either chunk, so
-// a flushed chunk always has room for the next round.
+// Stack of child ranges per warp.  A round pushes at most 64 ranges, so below
+// kStackDeep it ends at most 63 above; from kStackDeep on a round takes a
+// single range (one node, at most 8 child nodes): a plain depth-first walk that
+// adds at most 7 ranges per tree level, 7 x 21 on the deepest path, so the
+// stack never holds more than kStackDeep + 63 + 147 ranges.
+constexpr int kStackCap = 384;
+constexpr int kStackDeep = kStackCap - 64 - 7 * kLevels - 1;
+// A round appends at most 64 entries to either chunk, and a chunk is evaluated
+// after the round that takes it above a limit: kNearFlush entries, or `chunk`
+// far ones (WalkArgs::chunk, chosen at launch).  Both have room for that round and
+// for the padding of an evaluation: fewer than kMaxRep entries in the near
+// chunk, kMaxRep x kFarStep in the far one.
+constexpr int kMaxRep = 16;        // replicas of a group's targets at most
+constexpr int kFarStep = 4;        // far entries in flight per lane
+constexpr int kNearChunk = 128;
+constexpr int kNearFlush = kNearChunk - 64 - kMaxRep;
+constexpr int kFarPad = 64 + kMaxRep * kFarStep;
 constexpr int kMinChunk = 64, kMaxChunk = 1024;
 
 // shared memory of one warp: its stack, near chunk and far chunk
 __host__ __device__ constexpr size_t warp_smem(int chunk) {
-    return kStackCap * sizeof(uint2) + ((size_t)chunk + kNearChunk) * sizeof(uint4);
+    return kStackCap * sizeof(uint2) + ((size_t)chunk + kNearChunk + kFarPad) * sizeof(uint4);
 }
 constexpr size_t kMaxBlockSmem = kMaxWarps * warp_smem(kMaxChunk);
 static_assert(kMaxBlockSmem <= 227 * 1024, "walk block exceeds the shared memory of an SM");
 
-// Abramowitz & Stegun 7.1.26: erfc(x) ~ t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-x^2),
-// t = 1 / (1 + p x), |error| <= 1.5e-7 for x >= 0.
-constexpr float kAsP = 0.3275911f;
-constexpr float kAs1 = 0.254829592f, kAs2 = -0.284496736f, kAs3 = 1.421413741f;
-constexpr float kAs4 = -1.453152027f, kAs5 = 1.061405429f;
+// erfc(u) exp(u^2) ~ c0 + v (c1 + ... + v c5), v = p u / (1 + p u) in [0, 1): a
+// least-maximum fit of the split factor S(u) = exp(-u^2) (erfc(u) exp(u^2) +
+// (2 / sqrt(pi)) u), |error of S| <= 1e-7 max(S, S(2.25)) for u >= 0, so it is
+// good to 1e-7 relative up to the usual cutoff u = 2.25 (1.7e-7 in FP32
+// arithmetic; Abramowitz & Stegun 7.1.26, used before, 7.4e-6 there).
+constexpr float kErfP = 0.455f;
+constexpr float kErf0 = 0.99999990145469710f, kErf1 = -2.4799351751253551f, kErf2 = 2.3497844342086717f;
+constexpr float kErf3 = -0.79841706208158790f, kErf4 = -0.31761888136087987f, kErf5 = 0.25502248430625629f;
 constexpr float kTwoOverSqrtPi = 1.1283791670955126f;
 
 // relative margin of the FP32 opening filter (the FP32 evaluation errs by
 // less than 2^-20; inside this band the FP64 expression decides)
 constexpr float kFilterHi = 1.0f + 1.0f / 65536.0f;
 constexpr float kFilterLo = 1.0f - 1.0f / 65536.0f;
+constexpr float kFilterEps = 1.0f / 65536.0f;
+
 
 // One tree as the walk sees it (a forest counts as one tree).
 struct TreeView {
@@ -149,169 +176,167 @@ __device__ __forceinline__ unsigned long long sq64(uint32_t g) {
     return (unsigned long long)g * (unsigned long long)g;
 }
 
-// Near-chunk evaluation for one target per lane (entries closer than h to
-// the group box: the softened kernel may apply).  Entries e = rep, rep + R,
-// ... are this lane's share.  r^2 is guarded from below by 1 (a nonzero integer
-// separation has r^2 >= 1 in grid units); a zero separation then contributes
-// f * 0 = 0 exactly, the self term included.
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+
+// A lane's two targets: their fixed-point positions.
+struct Targets {
+    uint32_t x0, y0, z0, x1, y1, z1;
+};
+
+// Separations of one entry from a lane's two targets: exact 32-bit minimum-image
+// differences, each rounded once to FP32; r^2 by FMA.
+__device__ __forceinline__ void separations(const uint4 &s, const Targets &t, float2 &fx, float2 &fy, float2 &fz,
+                                            float2 &r2) {
+    fx = make_float2((float)(int)(s.x - t.x0), (float)(int)(s.x - t.x1));
+    fy = make_float2((float)(int)(s.y - t.y0), (float)(int)(s.y - t.y1));
+    fz = make_float2((float)(int)(s.z - t.z0), (float)(int)(s.z - t.z1));
+    r2 = __ffma2_rn(fx, fx, __ffma2_rn(fy, fy, __fmul2_rn(fz, fz)));
+}
+
+// erfc(u) exp(u^2) from 1 / r (y), u = r / (2 r_s): v = 1 / (1 + y / (p / 2 r_s))
+__device__ __forceinline__ float2 erfc_poly(float2 y, float ky) {
+    const float2 den = __ffma2_rn(y, dup(ky), dup(1.0f));
+    const float2 v = make_float2(rcp_ftz(den.x), rcp_ftz(den.y));
+    float2 q = __ffma2_rn(v, dup(kErf5), dup(kErf4));
+    q = __ffma2_rn(v, q, dup(kErf3));
+    q = __ffma2_rn(v, q, dup(kErf2));
+    q = __ffma2_rn(v, q, dup(kErf1));
+    return __ffma2_rn(v, q, dup(kErf0));
+}
+
+// sums of a lane's two targets over its share of a chunk
+struct Sums {
+    float2 x, y, z, p;
+};
+
+// A lane holds two targets and takes its replica's q consecutive entries of the
+// chunk: one shared-memory load serves both, and the two go through the
+// arithmetic together as FP32 pairs (the f32x2 operations of sm_100 and later;
+// each half is the same IEEE operation as the scalar one).  The chunk is padded
+// with massless entries (pad_chunk), so q is the same for every replica and a
+// multiple of the unrolling: no bounds test per entry and no remainder loop.
+//
+// Near entries (closer than h to the group box: the softened kernel may
+// apply).  r^2 is guarded from below by 1 (a nonzero integer separation has
+// r^2 >= 1 in grid units); a zero separation then contributes f * 0 = 0 exactly,
+// the self term included.
 // kPot: also the short-range potential sum of m erfc(r / 2 r_s) psi(r), psi the
 // potential kernel of the spline (1/r beyond h); the self term (r = 0) is left
 // out explicitly, it has no force to vanish with.
-template <bool kSplit, bool kPot = false>
-__device__ __forceinline__ void eval_near(const uint4 *ch, int cnt, int rep, int R, uint32_t xi,
-                                          uint32_t yi, uint32_t zi, const WalkParams &p,
-                                          float &ax, float &ay, float &az, float &ap) {
-    const float rc2 = p.rc2, kexp = p.kexp;
-    // u = r / (2 r_s) only enters as p u and (2 / sqrt(pi)) u
-    const float c_pr = kAsP * p.inv_2rs, c_tspr = kTwoOverSqrtPi * p.inv_2rs;
-    const float h = p.h, inv_h = p.inv_h;
+template <bool kSplit, bool kPot>
+__device__ __forceinline__ Sums eval_near(const uint4 *ch, int q, const Targets &t, const WalkParams &p) {
+    Sums a{};
+    const float h = p.h, inv_h = p.inv_h, rc2 = p.rc2;
     const float hinv3 = inv_h * inv_h * inv_h;
-#pragma unroll 2
-    for (int e = rep; e < cnt; e += R) {
-        const uint4 s = ch[e];
-        const float fx = (float)(int)(s.x - xi);
-        const float fy = (float)(int)(s.y - yi);
-        const float fz = (float)(int)(s.z - zi);
-        const float r2 = __fmaf_rn(fx, fx, __fmaf_rn(fy, fy, __fmul_rn(fz, fz)));
-        float m = __uint_as_float(s.w);
-        if (kSplit) m = (r2 < rc2) ? m : 0.0f;
-        const float r2c = fmaxf(r2, 1.0f);
-        const float rinv = rsqrt_ftz(r2c);
-        float mS = m;
-        const float r = r2c * rinv;
-        float erfcv = 1.0f;
+#pragma unroll 1
+    for (const uint4 *end = ch + q; ch != end; ++ch) {
+        const uint4 s = *ch;
+        float2 fx, fy, fz, r2;
+        separations(s, t, fx, fy, fz, r2);
+        const float m = __uint_as_float(s.w);
+        float2 m2 = dup(m);
+        if (kSplit) m2 = make_float2(r2.x < rc2 ? m : 0.0f, r2.y < rc2 ? m : 0.0f);
+        const float2 r2c = make_float2(fmaxf(r2.x, 1.0f), fmaxf(r2.y, 1.0f));
+        const float2 y = make_float2(rsqrt_ftz(r2c.x), rsqrt_ftz(r2c.y));
+        const float2 r = __fmul2_rn(r2c, y);
+        float2 mS = m2, erfcv = dup(1.0f);
         if (kSplit) {
-            const float t = rcp_ftz(fmaf(c_pr, r, 1.0f));
-            const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, kAs5, kAs4), kAs3), kAs2), kAs1);
-            const float ex = ex2_ftz(r2c * kexp);
-            mS = m * (ex * fmaf(c_tspr, r, poly));
-            if (kPot) erfcv = ex * poly;
+            const float2 ec = erfc_poly(y, p.erf_ky);
+            const float2 arg = __fmul2_rn(r2c, dup(p.kexp));
+            const float2 ex = make_float2(ex2_ftz(arg.x), ex2_ftz(arg.y));
+            mS = __fmul2_rn(m2, __fmul2_rn(ex, __ffma2_rn(dup(p.erf_c), r, ec)));
+            if (kPot) erfcv = __fmul2_rn(ex, ec);
         }
+        const float2 u = __fmul2_rn(r, dup(inv_h));
+        const float2 u2 = __fmul2_rn(u, u);
+        float2 g = __fmul2_rn(y, __fmul2_rn(y, y));
         if (kPot) {
-            float psi = rinv;
-            {
-                const float u = r * inv_h;
-                const float u2 = u * u;
-                const float pin = fmaf(u2, fmaf(u2, fmaf(-32.0f / 5.0f, u, 48.0f / 5.0f), -16.0f / 3.0f),
-                                       14.0f / 5.0f);
-                const float pout = fmaf(u2, fmaf(u, fmaf(u, fmaf(32.0f / 15.0f, u, -48.0f / 5.0f), 16.0f),
-                                                 -32.0f / 3.0f),
-                                        16.0f / 5.0f) -
-                                   (1.0f / 15.0f) * rcp_ftz(u);
-                psi = (r < h) ? inv_h * ((u < 0.5f) ? pin : pout) : psi;
-            }
-            ap = fmaf((r2 > 0.0f ? m : 0.0f) * erfcv, psi, ap);
+            const float2 pin = __ffma2_rn(
+                u2, __ffma2_rn(u2, __ffma2_rn(u, dup(-32.0f / 5.0f), dup(48.0f / 5.0f)), dup(-16.0f / 3.0f)),
+                dup(14.0f / 5.0f));
+            float2 pout = __ffma2_rn(u, dup(32.0f / 15.0f), dup(-48.0f / 5.0f));
+            pout = __ffma2_rn(u, pout, dup(16.0f));
+            pout = __ffma2_rn(u, pout, dup(-32.0f / 3.0f));
+            pout = __ffma2_rn(u2, pout, dup(16.0f / 5.0f));
+            pout.x -= (1.0f / 15.0f) * rcp_ftz(u.x);
+            pout.y -= (1.0f / 15.0f) * rcp_ftz(u.y);
+            const float px = r.x < h ? inv_h * (u.x < 0.5f ? pin.x : pout.x) : y.x;
+            const float py = r.y < h ? inv_h * (u.y < 0.5f ? pin.y : pout.y) : y.y;
+            a.p.x = fmaf((r2.x > 0.0f ? m2.x : 0.0f) * erfcv.x, px, a.p.x);
+            a.p.y = fmaf((r2.y > 0.0f ? m2.y : 0.0f) * erfcv.y, py, a.p.y);
         }
-        float g = rinv * rinv * rinv;
-        {
-            // cubic-spline softened kernel inside h (Monaghan 1985 form)
-            const float u = r * inv_h;
-            const float u2 = u * u;
-            const float gin = hinv3 * fmaf(u2, fmaf(32.0f, u, -192.0f / 5.0f), 32.0f / 3.0f);
-            const float gout = hinv3 * (fmaf(u, fmaf(u, fmaf(u, -32.0f / 3.0f, 192.0f / 5.0f), -48.0f),
-                                             64.0f / 3.0f) -
-                                        (1.0f / 15.0f) * rcp_ftz(u2 * u));
-            g = (r < h) ? ((u < 0.5f) ? gin : gout) : g;
+        // cubic-spline softened kernel inside h (Monaghan 1985 form); the target
+        // itself (r = 0) takes no force whatever its kernel
+        if ((r.x < h && r2.x > 0.0f) || (r.y < h && r2.y > 0.0f)) {
+            const float2 gin = __fmul2_rn(
+                dup(hinv3), __ffma2_rn(u2, __ffma2_rn(u, dup(32.0f), dup(-192.0f / 5.0f)), dup(32.0f / 3.0f)));
+            float2 go = __ffma2_rn(u, dup(-32.0f / 3.0f), dup(192.0f / 5.0f));
+            go = __ffma2_rn(u, go, dup(-48.0f));
+            go = __ffma2_rn(u, go, dup(64.0f / 3.0f));
+            const float2 u3 = __fmul2_rn(u2, u);
+            go = __ffma2_rn(make_float2(rcp_ftz(u3.x), rcp_ftz(u3.y)), dup(-1.0f / 15.0f), go);
+            go = __fmul2_rn(dup(hinv3), go);
+            g = make_float2(r.x < h ? (u.x < 0.5f ? gin.x : go.x) : g.x,
+                            r.y < h ? (u.y < 0.5f ? gin.y : go.y) : g.y);
         }
-        const float f = mS * g;
-        ax = fmaf(f, fx, ax);
-        ay = fmaf(f, fy, ay);
-        az = fmaf(f, fz, az);
+        const float2 f = __fmul2_rn(mS, g);
+        a.x = __ffma2_rn(f, fx, a.x);
+        a.y = __ffma2_rn(f, fy, a.y);
+        a.z = __ffma2_rn(f, fz, a.z);
     }
+    return a;
 }
 
 // Far entries: every target of the group is at least h away (the entry lies
 // outside the group box by more than h, and by at least one grid unit), so
-// no softening applies and r^2 >= 1 needs no guard.  Two entries of this
-// lane's share, e and e + R, go through the arithmetic together as FP32
-// pairs (the f32x2 multiply and fused multiply-add of sm_100 and later:
-// each half is the same IEEE operation as the scalar one, so the cutoff
-// decision is unchanged); an odd last entry goes alone.
-template <bool kSplit, bool kPot = false, int kUnroll = 2>
-__device__ __forceinline__ void eval_far(const uint4 *ch, int cnt, int rep, int R, uint32_t xi,
-                                         uint32_t yi, uint32_t zi, const WalkParams &p,
-                                         float &ax, float &ay, float &az, float &ap) {
+// no softening applies and r^2 >= 1 needs no guard.
+template <bool kSplit, bool kPot>
+__device__ __forceinline__ Sums eval_far(const uint4 *ch, int q, const Targets &t, const WalkParams &p) {
+    Sums a{};
     const float rc2 = p.rc2;
-    const float2 c_kexp = make_float2(p.kexp, p.kexp);
-    const float2 c_one = make_float2(1.0f, 1.0f);
-    const float2 c5 = make_float2(kAs5, kAs5), c4 = make_float2(kAs4, kAs4);
-    const float2 c3 = make_float2(kAs3, kAs3), c2 = make_float2(kAs2, kAs2);
-    const float2 c1 = make_float2(kAs1, kAs1);
-    // u = r / (2 r_s) only enters as p u and (2 / sqrt(pi)) u: 1 / (2 r_s) folds into both
-    const float2 c_pr = make_float2(kAsP * p.inv_2rs, kAsP * p.inv_2rs);
-    const float2 c_tspr = make_float2(kTwoOverSqrtPi * p.inv_2rs, kTwoOverSqrtPi * p.inv_2rs);
-    float2 sx = make_float2(0.f, 0.f), sy = sx, sz = sx, sp = sx;
-    int e = rep;
-#pragma unroll kUnroll
-    for (; e + R < cnt; e += 2 * R) {
-        const uint4 s0 = ch[e], s1 = ch[e + R];
-        const float2 fx = make_float2((float)(int)(s0.x - xi), (float)(int)(s1.x - xi));
-        const float2 fy = make_float2((float)(int)(s0.y - yi), (float)(int)(s1.y - yi));
-        const float2 fz = make_float2((float)(int)(s0.z - zi), (float)(int)(s1.z - zi));
-        const float2 r2 = __ffma2_rn(fx, fx, __ffma2_rn(fy, fy, __fmul2_rn(fz, fz)));
-        float2 m = make_float2(__uint_as_float(s0.w), __uint_as_float(s1.w));
-        if (kSplit) {
-            m.x = (r2.x < rc2) ? m.x : 0.0f;
-            m.y = (r2.y < rc2) ? m.y : 0.0f;
+#pragma unroll 1
+    for (const uint4 *end = ch + q; ch != end; ch += kFarStep) {
+#pragma unroll
+        for (int k = 0; k < kFarStep; ++k) {
+            const uint4 s = ch[k];
+            float2 fx, fy, fz, r2;
+            separations(s, t, fx, fy, fz, r2);
+            const float m = __uint_as_float(s.w);
+            float2 m2 = dup(m);
+            if (kSplit) m2 = make_float2(r2.x < rc2 ? m : 0.0f, r2.y < rc2 ? m : 0.0f);
+            const float2 y = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+            float2 f;
+            if (kSplit) {
+                // S(r) r^-3 = (ec + (2 / sqrt(pi)) u) exp(-u^2) r^-3, with the second
+                // term's r r^-1 taken as 1: (ec / r + c) exp(-u^2) r^-2
+                const float2 ec = erfc_poly(y, p.erf_ky);
+                const float2 arg = __fmul2_rn(r2, dup(p.kexp));
+                const float2 mex = __fmul2_rn(m2, make_float2(ex2_ftz(arg.x), ex2_ftz(arg.y)));
+                if (kPot) a.p = __ffma2_rn(__fmul2_rn(mex, ec), y, a.p);
+                f = __fmul2_rn(mex, __fmul2_rn(__ffma2_rn(ec, y, dup(p.erf_c)), __fmul2_rn(y, y)));
+            } else {
+                if (kPot) a.p = __ffma2_rn(m2, y, a.p);
+                f = __fmul2_rn(m2, __fmul2_rn(y, __fmul2_rn(y, y)));
+            }
+            a.x = __ffma2_rn(f, fx, a.x);
+            a.y = __ffma2_rn(f, fy, a.y);
+            a.z = __ffma2_rn(f, fz, a.z);
         }
-        const float2 rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-        float2 f;
-        if (kSplit) {
-            // S(r) r^-3 = (erfc(u) + (2 / sqrt(pi)) u exp(-u^2)) r^-3, with the
-            // second term's r r^-1 taken as 1: (poly rinv + c) exp(-u^2) rinv^2
-            const float2 r = __fmul2_rn(r2, rinv);
-            const float2 den = __ffma2_rn(c_pr, r, c_one);
-            const float2 t = make_float2(rcp_ftz(den.x), rcp_ftz(den.y));
-            float2 q = __ffma2_rn(t, c5, c4);
-            q = __ffma2_rn(t, q, c3);
-            q = __ffma2_rn(t, q, c2);
-            q = __ffma2_rn(t, q, c1);
-            const float2 poly = __fmul2_rn(t, q);
-            const float2 arg = __fmul2_rn(r2, c_kexp);
-            const float2 ex = make_float2(ex2_ftz(arg.x), ex2_ftz(arg.y));
-            const float2 mex = __fmul2_rn(m, ex);
-            if (kPot) sp = __ffma2_rn(__fmul2_rn(mex, poly), rinv, sp);
-            f = __fmul2_rn(mex, __fmul2_rn(__ffma2_rn(poly, rinv, c_tspr), __fmul2_rn(rinv, rinv)));
-        } else {
-            if (kPot) sp = __ffma2_rn(m, rinv, sp);
-            f = __fmul2_rn(m, __fmul2_rn(rinv, __fmul2_rn(rinv, rinv)));
-        }
-        sx = __ffma2_rn(f, fx, sx);
-        sy = __ffma2_rn(f, fy, sy);
-        sz = __ffma2_rn(f, fz, sz);
     }
-    float tx = __fadd_rn(sx.x, sx.y), ty = __fadd_rn(sy.x, sy.y), tz = __fadd_rn(sz.x, sz.y);
-    float tp = kPot ? __fadd_rn(sp.x, sp.y) : 0.0f;
-    if (e < cnt) {
-        const uint4 s = ch[e];
-        const float fx = (float)(int)(s.x - xi);
-        const float fy = (float)(int)(s.y - yi);
-        const float fz = (float)(int)(s.z - zi);
-        const float r2 = __fmaf_rn(fx, fx, __fmaf_rn(fy, fy, __fmul_rn(fz, fz)));
-        float m = __uint_as_float(s.w);
-        if (kSplit) m = (r2 < rc2) ? m : 0.0f;
-        const float rinv = rsqrt_ftz(r2);
-        float f;
-        if (kSplit) {
-            const float r = r2 * rinv;
-            const float t = rcp_ftz(fmaf(c_pr.x, r, 1.0f));
-            const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, kAs5, kAs4), kAs3), kAs2), kAs1);
-            const float ex = ex2_ftz(r2 * p.kexp);
-            const float mex = m * ex;
-            if (kPot) tp = fmaf(mex * poly, rinv, tp);
-            f = mex * (fmaf(poly, rinv, c_tspr.x) * (rinv * rinv));
-        } else {
-            if (kPot) tp = fmaf(m, rinv, tp);
-            f = m * (rinv * (rinv * rinv));
-        }
-        tx = fmaf(f, fx, tx);
-        ty = fmaf(f, fy, ty);
-        tz = fmaf(f, fz, tz);
-    }
-    ax = tx;
-    ay = ty;
-    az = tz;
-    if (kPot) ap = tp;
+    return a;
+}
+
+// Massless entries behind the cnt entries of a chunk, so that R replicas take q
+// each; returns q, a multiple of `step`.  They lie one grid unit outside the
+// group box, so every target is at r >= 1 and they add an exact 0.  (A box that
+// is the whole circle on every axis has no outside, but then every entry is
+// near, and near entries guard r themselves.)
+__device__ __forceinline__ int pad_chunk(uint4 *ch, int cnt, uint32_t R, uint32_t step, int lane,
+                                         const uint32_t *hi) {
+    const uint32_t q = ((uint32_t)cnt + R * step - 1u) / (R * step) * step;
+    for (uint32_t k = (uint32_t)cnt + (uint32_t)lane; k < R * q; k += 32u)
+        ch[k] = make_uint4(hi[0] + 1u, hi[1] + 1u, hi[2] + 1u, 0u);
+    return (int)q;
 }
 
 __device__ __forceinline__ void kahan_add(float &sum, float &comp, float v) {
@@ -321,12 +346,16 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float v) {
     sum = t;
 }
 
+// compensated totals of a lane's two targets
 struct Acc {
-    float sx = 0.f, sy = 0.f, sz = 0.f, kx = 0.f, ky = 0.f, kz = 0.f;
-    __device__ __forceinline__ void add(float tx, float ty, float tz) {
-        kahan_add(sx, kx, tx);
-        kahan_add(sy, ky, ty);
-        kahan_add(sz, kz, tz);
+    float2 sx{0.f, 0.f}, sy{0.f, 0.f}, sz{0.f, 0.f}, kx{0.f, 0.f}, ky{0.f, 0.f}, kz{0.f, 0.f};
+    __device__ __forceinline__ void add(const Sums &t) {
+        kahan_add(sx.x, kx.x, t.x.x);
+        kahan_add(sx.y, kx.y, t.x.y);
+        kahan_add(sy.x, ky.x, t.y.x);
+        kahan_add(sy.y, ky.y, t.y.y);
+        kahan_add(sz.x, kz.x, t.z.x);
+        kahan_add(sz.y, kz.y, t.z.y);
     }
 };
 
@@ -386,9 +415,13 @@ __device__ __forceinline__ void cell_gap(uint32_t c, uint32_t lo, uint32_t len, 
     cg = e > 0 ? (uint32_t)e : 0u;
 }
 
-// Registers: at most 96 per thread (64 KB / (96 x 128) gives 5 blocks of 4
-// warps per SM, as many as their shared memory allows), 128 with the
-// potential output; a block of kMaxWarps warps fits either way.
+// x >> n with n >= 32 giving 0 (the hardware shift clamps; C++ leaves it undefined)
+__device__ __forceinline__ uint32_t shr(uint32_t x, uint32_t n) {
+    uint32_t r;
+    asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+    return r;
+}
+
 // One child record against the group box: PP / PN entry, opened node (its
 // child range to push), or nothing (pruned, or no record in this slot).
 struct Cls {
@@ -397,17 +430,106 @@ struct Cls {
     uint32_t push_ref, push_cnt;
 };
 
+// the group box: [lo, hi] per axis on the circle
+struct Box {
+    uint32_t lo[3], hi[3];
+};
+
+// The opening decision in FP64, from gaps on the circle (the rare case where
+// single precision, or the short form of the gaps, does not settle it).
+template <int kOpen>
+__device__ __forceinline__ bool open_exact(const uint4 &c, const Box &b, double l2, double M, double arel,
+                                           const WalkParams &p, float &d2f) {
+    const uint32_t gx = point_gap(c.x, b.lo[0], b.hi[0] - b.lo[0]);
+    const uint32_t gy = point_gap(c.y, b.lo[1], b.hi[1] - b.lo[1]);
+    const uint32_t gz = point_gap(c.z, b.lo[2], b.hi[2] - b.lo[2]);
+    d2f = dist2f(gx, gy, gz);
+    const double dx = (double)gx, dy = (double)gy, dz = (double)gz;
+    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+    if (kOpen == OG_OPEN_BH) return l2 > __dmul_rn(p.th2, d2);
+    return __dmul_rn(__dmul_rn(p.G, M), l2) > __dmul_rn(arel, __dmul_rn(d2, d2));
+}
+
+// The short form, for a group whose box sides are in [1, 2^29) grid units and
+// whose prune distance is below 2^29: signed differences to the near and far
+// sides, no wrap to tell apart, and one straight line for particles and nodes,
+// so that the two records of a lane overlap.  About 60 instructions a record,
+// where the interval form below takes about 100 in two divergent branches.
+//
+// With a = lo - c and b = c - hi (signed), the gap of c is max(a, b, 0).  It
+// differs from the gap on the circle only where both a and b are positive,
+// i.e. for a c within len of the far side of the circle, where it takes the larger
+// one; both are above 2^31 - 2^29 there (and with len >= 1 they are never both
+// -2^31).  A particle or a cell (half side
+// s2 <= 2^30) there is beyond the prune distance either way.  The centre of mass
+// of a cell that is not pruned is at most 2 s2 further, so it can be there
+// only for a node of level 1; those take the exact branch.
+//
+// A cell's centre is c = (COM with the low 32 - lev bits cleared) + s2 and its
+// gap max(a + 1 - s2, b - s2, 0) = max(max(b - 1, a) - (s2 - 1), 0), as it spans
+// [c - s2, c + s2 - 1].  The level of a particle reads as 32 or more: s2 = 0, and
+// without the ones the cell is the point itself.
+// Boundary check: the box meets the cell enlarged to 0.6 side, max(a, b) <=
+// floor(6 s2 / 5) on every axis; 6/5 = 1.0011 0011..., so for s2 = 2^(31 - lev)
+// that is 0x99999999 >> lev.
+template <int kOpen>
+__device__ __forceinline__ Cls classify_short(const TreeView &T, uint32_t ci, bool has, const Box &b,
+                                              const WalkParams &p, float arelf, double arel) {
+    const uint4 *rec = reinterpret_cast<const uint4 *>(T.crec + (has ? ci : 0u));
+    const uint4 q0 = rec[0], q1 = rec[1];
+    const uint32_t info = q1.z, lev = info >> 26;
+    const bool isnode = (int)info >= 0;
+    const int isn = isnode ? 1 : 0;
+    const uint32_t mask = shr(0xffffffffu, lev), s2 = shr(0x80000000u, lev), blim = shr(0x99999999u, lev);
+    unsigned long long g2 = 0ull;
+    int dc;
+    uint32_t g[3];
+    const uint32_t c[3] = {q0.x, q0.y, q0.z};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t cc = (c[k] & ~mask) | s2;
+        const int a = (int)(b.lo[k] - cc), d = (int)(cc - b.hi[k]);
+        dc = k == 0 ? max(a, d) : __vimax3_s32(dc, a, d);
+        const uint32_t cg = (uint32_t)__viaddmax_s32_relu(__viaddmax_s32(d, -isn, a), isn - (int)s2, 0);
+        g2 += sq64(cg);
+        g[k] = (uint32_t)__vimax_s32_relu((int)(b.lo[k] - c[k]), (int)(c[k] - b.hi[k]));
+    }
+    float d2f = dist2f(g[0], g[1], g[2]);
+    const bool keep = has && g2 <= p.rprune;
+    const bool bnear = dc <= (int)blim;
+    const float l2f = __uint_as_float(0x5f800000u - (lev << 24));   // 2^(64 - 2 lev)
+    bool op, sure;
+    if (kOpen == OG_OPEN_BH) {
+        const float q = p.th2f * d2f, t = l2f - q;
+        op = t > 0.0f;
+        sure = fabsf(t) > q * kFilterEps;
+    } else {
+        const float lhs = (p.Gf * __uint_as_float(q0.w)) * l2f, rhs = (arelf * d2f) * d2f, t = lhs - rhs;
+        op = t > 0.0f;
+        sure = fabsf(t) > rhs * kFilterEps && fminf(lhs, rhs) >= 1e-30f && fmaxf(lhs, rhs) <= 1e30f;
+    }
+    if (__builtin_expect(keep && isnode && !bnear && (!sure || lev == 1u), 0)) {
+        const double l2 = __longlong_as_double((long long)(1023 + 64 - 2 * lev) << 52);
+        op = open_exact<kOpen>(q0, b, l2, __hiloint2double((int)q1.y, (int)q1.x), arel, p, d2f);
+    }
+    const bool open = keep && isnode && (bnear || op);
+    // near: in single precision with a margin above its error
+    return Cls{keep && !open, open, isnode, !(d2f >= p.hnear2f), q0, q1.w, info & 0x3ffffffu};
+}
+
+// The general form: intervals on the circle, any box, node extents after a refit.
 template <int kOpen, bool kSplit, bool kRefit>
-__device__ __forceinline__ Cls classify(const TreeView &T, uint32_t ci, bool has, const uint32_t *lo,
-                                        const uint32_t *gl, const WalkParams &p, float arelf,
-                                        double arel) {
+__device__ __forceinline__ Cls classify(const TreeView &T, uint32_t ci, bool has, const Box &b,
+                                        const WalkParams &p, float arelf, double arel) {
+    const uint32_t *lo = b.lo;
+    const uint32_t gl[3] = {b.hi[0] - b.lo[0], b.hi[1] - b.lo[1], b.hi[2] - b.lo[2]};
     bool emit = false, open = false, isnode = false, near = false;
     uint4 ent = make_uint4(0u, 0u, 0u, 0u);
     uint32_t push_ref = 0u, push_cnt = 0u;
     if (has && ci < T.nchild) {
         const CRec r = T.crec[ci];
         ent = make_uint4(r.x, r.y, r.z, __float_as_uint(r.m));
-        isnode = (r.info >> 31) != 0u;
+        isnode = (r.info >> 31) == 0u;
         // gaps of the particle, or of the node's centre of mass, to the group box
         const uint32_t gx = point_gap(r.x, lo[0], gl[0]);
         const uint32_t gy = point_gap(r.y, lo[1], gl[1]);
@@ -480,6 +602,9 @@ __device__ __forceinline__ Cls classify(const TreeView &T, uint32_t ci, bool has
 
 // kOneSeg: a single tree of one box, whose parameters come from the launch
 // argument (constant operands) instead of a per-box record in global memory.
+// Registers: at most 96 per thread (64 KB / (96 x 128) gives 5 blocks of 4
+// warps per SM, as many as their shared memory allows), 128 with the
+// potential output; a block of kMaxWarps warps fits either way.
 template <int kOpen, bool kSplit, bool kDump, bool kRefit, bool kMulti, bool kPot = false,
           bool kOneSeg = false>
 __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a);
@@ -491,10 +616,6 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
     // blockDim.x = 32 * a.warps and the launch sizes smem to match
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int chunk = a.chunk;
-    // far-entry pairs in flight per lane: 4 in the Barnes-Hut kernels and in
-    // the one-box kernels (their parameters are constant operands), 2 where
-    // the relative test's extra registers would spill
-    constexpr int kFarUnroll = (kOpen == OG_OPEN_BH || kOneSeg) ? 4 : 2;
     unsigned char *wbase = smem + (size_t)warp * warp_smem(chunk);
     uint2 *stk = reinterpret_cast<uint2 *>(wbase);
     uint4 *chn = reinterpret_cast<uint4 *>(wbase + kStackCap * sizeof(uint2));
@@ -527,28 +648,38 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         const WalkParams &p = kOneSeg ? a.p0 : T.segp[seg];
         const uint32_t gb = T.gbeg[g], ge = T.gend[g];
         const uint32_t gsize = ge - gb;
-        uint32_t lo[3], gl[3];  // the group box: [lo, lo + gl] per axis
+        Box box;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            lo[k] = T.gbox[6 * g + k];
-            gl[k] = T.gbox[6 * g + 3 + k] - lo[k];
+            box.lo[k] = T.gbox[6 * g + k];
+            box.hi[k] = T.gbox[6 * g + 3 + k];
         }
-        // lane -> (target, replica): P lanes per replica, R = 32 / P replicas
-        const int P = gsize > 16u ? 32 : gsize > 8u ? 16 : gsize > 4u ? 8 : gsize > 2u ? 4 : gsize > 1u ? 2 : 1;
-        const int R = 32 / P;
-        const int tl = lane & (P - 1), rep = lane / P;
-        const uint32_t i = gb + tl;
-        const bool active = (uint32_t)tl < gsize;
-        const uint32_t xi = active ? T.px[i] : 0u;
-        const uint32_t yi = active ? T.py[i] : 0u;
-        const uint32_t zi = active ? T.pz[i] : 0u;
+        // the short form of the tests (see classify_short)
+        bool compact = kSplit && !kRefit && p.rprune < (1ull << 58);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) compact = compact && box.hi[k] - box.lo[k] - 1u < (1u << 29) - 1u;
+        // Lane -> (target pair, replica): P lanes hold the group's targets, two
+        // each, and R = 32 / P replicas of them split the entries.  Two targets a
+        // lane fill the warp better than one (P need not be a power of two: a
+        // group of 20 keeps 30 of 32 lanes busy, where one target a lane kept 20)
+        // and halve the shared-memory loads.
+        const uint32_t P = (gsize + 1u) >> 1;
+        const uint32_t rep = ((uint32_t)lane * (65536u / P + 1u)) >> 16;   // lane / P
+        const uint32_t tl = (uint32_t)lane - rep * P;
+        const uint32_t R = min(32u / P, (uint32_t)kMaxRep);
+        const uint32_t share = min(rep, R - 1u);    // the lanes left over repeat the last share, unused
+        const uint32_t i0 = gb + 2u * tl;
+        const bool two = 2u * tl + 1u < gsize;
+        const uint32_t i1 = two ? i0 + 1u : i0;
+        const Targets tg = {T.px[i0], T.py[i0], T.pz[i0], T.px[i1], T.py[i1], T.pz[i1]};
         // relative criterion: arel = (alpha * a_min) * s^2, a_min = min over the group
         // of |a_old| in FP64 of the single-precision components
         double arel = 0.0;
         float arelf = 0.0f;
         if (kOpen == OG_OPEN_REL) {
             double an = __longlong_as_double(0x7ff0000000000000ll);  // +inf
-            if (active) {
+            const uint32_t i = gb + (uint32_t)lane;
+            if ((uint32_t)lane < gsize) {
                 double ax0 = T.a_old[i], ay0 = T.a_old[T.n + i], az0 = T.a_old[2 * T.n + i];
                 an = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(ax0, ax0), __dmul_rn(ay0, ay0)),
                                           __dmul_rn(az0, az0)));
@@ -562,26 +693,24 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         if (lane == 0) stk[0] = make_uint2(T.ncbeg[seg], T.nccnt[seg]);
         __syncwarp();
         int sp = 1, cf = 0, cn = 0;
-        int64_t rounds = 0;
-        uint32_t cnt_pp = 0, cnt_pn = 0;
+        uint32_t rounds = 0;
+        const uint32_t nchild = (uint32_t)T.nchild, max_rounds = (uint32_t)T.max_rounds;
+        uint32_t cnt_all = 0, my_pn = 0;      // entries (warp), node entries (this lane)
         Acc acc;
-        float psum = 0.f, pcomp = 0.f;   // potential total (kPot), compensated
+        float2 psum = make_float2(0.f, 0.f), pcomp = psum;   // potential totals (kPot), compensated
         bool overflow = false;
 
-        // the last pass of this loop finds the stack empty: an empty round whose
-        // flush evaluates what the chunks still hold (one evaluation site)
         while (true) {
-            const bool done = sp == 0;
             // every round consumes at least one child record and a record is
             // visited at most once per walk: more rounds than records is a bug
-            if (++rounds > T.max_rounds) {
+            if (++rounds > max_rounds) {
                 overflow = true;
                 if (lane == 0) atomicOr(a.status, ST_INTERNAL);
                 break;
             }
             // a round takes up to 64 child records from the top ranges of the
             // stack: slot l and slot l + 32 go to lane l
-            const int nr = sp < 32 ? sp : 32;
+            const int nr = sp > kStackDeep ? 1 : (sp < 32 ? sp : 32);
             uint2 Rg = make_uint2(0u, 0u);
             if (lane < nr) Rg = stk[sp - 1 - lane];
             const uint32_t cnt = Rg.y;
@@ -592,119 +721,114 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 if (lane >= d) incl += o;
             }
             const uint32_t excl = incl - cnt;
-            const unsigned fullm = __ballot_sync(FULL, lane < nr && incl <= 64u);
+            const bool mine = lane < nr;
+            const unsigned fullm = __ballot_sync(FULL, mine && incl <= 64u);
             const int nfull = __popc(fullm);
             const uint32_t total = __shfl_sync(FULL, incl, 31);
             const int ntake = total < 64u ? (int)total : 64;
             // first slot of every range that starts in this round, slots 0..31 and 32..63
-            const unsigned slo = __reduce_or_sync(FULL, (lane < nr && excl < 32u) ? (1u << excl) : 0u);
-            const unsigned shi = __reduce_or_sync(
-                FULL, (lane < nr && excl >= 32u && excl < 64u) ? (1u << (excl - 32u)) : 0u);
+            const unsigned slo = __reduce_or_sync(FULL, mine && excl < 32u ? 1u << excl : 0u);
+            const unsigned shi = __reduce_or_sync(FULL, mine && excl >= 32u && excl < 64u ? 1u << (excl - 32u) : 0u);
             __syncwarp();
-            const int sp_new = sp - nfull;
-            if (lane == nfull && lane < nr && excl < 64u) {
+            sp -= nfull;
+            if (lane == nfull && mine && excl < 64u) {
                 const uint32_t used = 64u - excl;
-                stk[sp - 1 - nfull] = make_uint2(Rg.x + used, Rg.y - used);
+                stk[sp - 1] = make_uint2(Rg.x + used, Rg.y - used);
             }
             // this lane's two child slots: the range of a slot is the last one
             // starting at or before it
-            const unsigned upm = lane == 31 ? 0xffffffffu : ((2u << lane) - 1u);
+            const unsigned upm = lt | (1u << lane);
             const int rj0 = __popc(slo & upm) - 1;
             const int rj1 = __popc(slo) + __popc(shi & upm) - 1;
-            const int rs0 = rj0 < 0 ? 0 : rj0, rs1 = rj1 < 0 ? 0 : (rj1 > 31 ? 31 : rj1);
-            const uint32_t rcb0 = __shfl_sync(FULL, Rg.x, rs0), rex0 = __shfl_sync(FULL, excl, rs0);
-            const uint32_t rcb1 = __shfl_sync(FULL, Rg.x, rs1), rex1 = __shfl_sync(FULL, excl, rs1);
-            const uint32_t ci0 = rcb0 + ((uint32_t)lane - rex0);
-            const uint32_t ci1 = rcb1 + ((uint32_t)lane + 32u - rex1);
-            const Cls c0 = classify<kOpen, kSplit, kRefit>(T, ci0, lane < ntake, lo, gl, p, arelf, arel);
-            const Cls c1 = classify<kOpen, kSplit, kRefit>(T, ci1, lane + 32 < ntake, lo, gl, p, arelf, arel);
-            // push opened ranges
-            const unsigned bo0 = __ballot_sync(FULL, c0.open), bo1 = __ballot_sync(FULL, c1.open);
-            const int np0 = __popc(bo0), npush = np0 + __popc(bo1);
-            if (sp_new + npush > kStackCap) {
+            const uint32_t base = Rg.x - excl;
+            const uint32_t ci0 = __shfl_sync(FULL, base, rj0) + (uint32_t)lane;
+            const uint32_t ci1 = __shfl_sync(FULL, base, rj1) + (uint32_t)lane + 32u;
+            const bool has0 = lane < ntake && ci0 < nchild, has1 = lane + 32 < ntake && ci1 < nchild;
+            // (the two forms as two copies of all that follows from them: their
+            // results merged after a branch cost more than the tests)
+            auto take = [&](auto form) {
+                constexpr bool kShort = decltype(form)::value;
+                const Cls c0 = kShort ? classify_short<kOpen>(T, ci0, has0, box, p, arelf, arel)
+                                      : classify<kOpen, kSplit, kRefit>(T, ci0, has0, box, p, arelf, arel);
+                const Cls c1 = kShort ? classify_short<kOpen>(T, ci1, has1, box, p, arelf, arel)
+                                      : classify<kOpen, kSplit, kRefit>(T, ci1, has1, box, p, arelf, arel);
+                // push opened ranges (k_records has checked that every node has
+                // children, inside the child array)
+                const unsigned bo0 = __ballot_sync(FULL, c0.open), bo1 = __ballot_sync(FULL, c1.open);
+                const int np0 = __popc(bo0), npush = np0 + __popc(bo1);
+                if (sp + npush > kStackCap) return false;
+                if (c0.open) stk[sp + __popc(bo0 & lt)] = make_uint2(c0.push_ref, c0.push_cnt);
+                if (c1.open) stk[sp + np0 + __popc(bo1 & lt)] = make_uint2(c1.push_ref, c1.push_cnt);
+                sp += npush;
+                // append entries to the far / near chunks (at most 64 each per round)
+                const unsigned be0 = __ballot_sync(FULL, c0.emit), be1 = __ballot_sync(FULL, c1.emit);
+                const unsigned bq0 = __ballot_sync(FULL, c0.emit && c0.near);
+                const unsigned bq1 = __ballot_sync(FULL, c1.emit && c1.near);
+                const unsigned bf0 = be0 & ~bq0, bf1 = be1 & ~bq1;
+                const int nf0 = __popc(bf0), nq0 = __popc(bq0);
+                const int nfar = nf0 + __popc(bf1), nnear = nq0 + __popc(bq1);
+                if (c0.emit && c0.isnode) ++my_pn;
+                if (c1.emit && c1.isnode) ++my_pn;
+                // the chunks are adjacent: far entry k is chn[kNearChunk + k]
+                const int at0 = (c0.near ? cn : kNearChunk + cf) + __popc((c0.near ? bq0 : bf0) & lt);
+                const int at1 = (c1.near ? cn + nq0 : kNearChunk + cf + nf0) + __popc((c1.near ? bq1 : bf1) & lt);
+                if (c0.emit) chn[at0] = c0.ent;
+                if (c1.emit) chn[at1] = c1.ent;
+                if (kDump && nfar + nnear > 0) {
+                    unsigned long long d = 0;
+                    if (lane == 0) d = atomicAdd(a.list_cursor, (unsigned long long)(nfar + nnear));
+                    d = __shfl_sync(FULL, d, 0);
+                    auto dump = [&](unsigned long long at, uint32_t ci) {
+                        if (at < (unsigned long long)a.list_cap) {
+                            a.lists[2 * at] = (uint32_t)g;
+                            a.lists[2 * at + 1] = ci;
+                        } else {
+                            atomicOr(a.status, ST_LIST_OVF);
+                        }
+                    };
+                    if (c0.emit) dump(d + __popc(be0 & lt), ci0);
+                    if (c1.emit) dump(d + __popc(be0) + __popc(be1 & lt), ci1);
+                }
+                cf += nfar;
+                cn += nnear;
+                cnt_all += (uint32_t)(nfar + nnear);
+                return true;
+            };
+            bool ok;
+            if (kSplit && !kRefit && __builtin_expect(compact, 1)) ok = take(std::integral_constant<bool, true>{});
+            else ok = take(std::integral_constant<bool, false>{});
+            if (!ok) {
                 overflow = true;
                 break;
             }
-            // a node always has children; a zero count would stall the walk
-            if (c0.open) {
-                stk[sp_new + __popc(bo0 & lt)] = make_uint2(c0.push_ref, c0.push_cnt > 0u ? c0.push_cnt : 1u);
-                if (c0.push_cnt == 0u || (uint64_t)c0.push_ref + c0.push_cnt > (uint64_t)T.nchild)
-                    atomicOr(a.status, ST_INTERNAL);
-            }
-            if (c1.open) {
-                stk[sp_new + np0 + __popc(bo1 & lt)] =
-                    make_uint2(c1.push_ref, c1.push_cnt > 0u ? c1.push_cnt : 1u);
-                if (c1.push_cnt == 0u || (uint64_t)c1.push_ref + c1.push_cnt > (uint64_t)T.nchild)
-                    atomicOr(a.status, ST_INTERNAL);
-            }
-            sp = sp_new + npush;
-            // append entries to the far / near chunks (at most 64 each per round)
-            const unsigned be0 = __ballot_sync(FULL, c0.emit), be1 = __ballot_sync(FULL, c1.emit);
-            const unsigned bn0 = __ballot_sync(FULL, c0.isnode), bn1 = __ballot_sync(FULL, c1.isnode);
-            const unsigned bq0 = __ballot_sync(FULL, c0.emit && c0.near);
-            const unsigned bq1 = __ballot_sync(FULL, c1.emit && c1.near);
-            const unsigned bf0 = be0 & ~bq0, bf1 = be1 & ~bq1;
-            cnt_pn += __popc(be0 & bn0) + __popc(be1 & bn1);
-            cnt_pp += __popc(be0 & ~bn0) + __popc(be1 & ~bn1);
-            const int nf0 = __popc(bf0), nfar = nf0 + __popc(bf1);
-            const int nq0 = __popc(bq0), nnear = nq0 + __popc(bq1);
-            // a full chunk (or the walk's end) is evaluated before the round's
-            // entries are appended; flushes are rare, so they are hinted off
-            // the round's main path (the near chunk first: this layout measured
-            // fastest, and the order of the chunk totals is free)
-            if (__builtin_expect(done || cn + nnear > kNearChunk, 0)) {
+            __syncwarp();
+            // a chunk above its limit, or the walk's end, is evaluated; flushes are
+            // rare, so they are hinted off the round's path
+            const bool done = sp == 0;
+            if (__builtin_expect(done || cn > kNearFlush, 0)) {
+                const int q = pad_chunk(chn, cn, R, 1u, lane, box.hi);
                 __syncwarp();
-                float tx = 0.f, ty = 0.f, tz = 0.f, tp = 0.f;
-                eval_near<kSplit, kPot>(chn, cn, rep, R, xi, yi, zi, p, tx, ty, tz, tp);
-                acc.add(tx, ty, tz);
-                if (kPot) kahan_add(psum, pcomp, tp);
+                const Sums t = eval_near<kSplit, kPot>(chn + share * (uint32_t)q, q, tg, p);
+                acc.add(t);
+                if (kPot) {
+                    kahan_add(psum.x, pcomp.x, t.p.x);
+                    kahan_add(psum.y, pcomp.y, t.p.y);
+                }
                 cn = 0;
                 __syncwarp();
             }
-            if (__builtin_expect(done || cf + nfar > chunk, 0)) {
+            if (__builtin_expect(done || cf > chunk, 0)) {
+                const int q = pad_chunk(chf, cf, R, (uint32_t)kFarStep, lane, box.hi);
                 __syncwarp();
-                float tx = 0.f, ty = 0.f, tz = 0.f, tp = 0.f;
-                eval_far<kSplit, kPot, kFarUnroll>(chf, cf, rep, R, xi, yi, zi, p, tx, ty, tz, tp);
-                acc.add(tx, ty, tz);
-                if (kPot) kahan_add(psum, pcomp, tp);
+                const Sums t = eval_far<kSplit, kPot>(chf + share * (uint32_t)q, q, tg, p);
+                acc.add(t);
+                if (kPot) {
+                    kahan_add(psum.x, pcomp.x, t.p.x);
+                    kahan_add(psum.y, pcomp.y, t.p.y);
+                }
                 cf = 0;
                 __syncwarp();
             }
-            if (c0.emit) {
-                if (c0.near) chn[cn + __popc(bq0 & lt)] = c0.ent;
-                else chf[cf + __popc(bf0 & lt)] = c0.ent;
-            }
-            if (c1.emit) {
-                if (c1.near) chn[cn + nq0 + __popc(bq1 & lt)] = c1.ent;
-                else chf[cf + nf0 + __popc(bf1 & lt)] = c1.ent;
-            }
-            if (kDump && (nfar + nnear) > 0) {
-                const int nem = nfar + nnear;
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(a.list_cursor, (unsigned long long)nem);
-                base = __shfl_sync(FULL, base, 0);
-                const unsigned long long pos0 = base + __popc(be0 & lt);
-                const unsigned long long pos1 = base + __popc(be0) + __popc(be1 & lt);
-                if (c0.emit) {
-                    if (pos0 < (unsigned long long)a.list_cap) {
-                        a.lists[2 * pos0] = (uint32_t)g;
-                        a.lists[2 * pos0 + 1] = ci0;
-                    } else {
-                        atomicOr(a.status, ST_LIST_OVF);
-                    }
-                }
-                if (c1.emit) {
-                    if (pos1 < (unsigned long long)a.list_cap) {
-                        a.lists[2 * pos1] = (uint32_t)g;
-                        a.lists[2 * pos1 + 1] = ci1;
-                    } else {
-                        atomicOr(a.status, ST_LIST_OVF);
-                    }
-                }
-            }
-            cf += nfar;
-            cn += nnear;
-            __syncwarp();
             if (done) break;
         }
         if (overflow) {
@@ -712,24 +836,36 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             __syncwarp();
             continue;
         }
-        __syncwarp();
-        float vx = __fsub_rn(acc.sx, acc.kx), vy = __fsub_rn(acc.sy, acc.ky),
-              vz = __fsub_rn(acc.sz, acc.kz);
-        float vp = kPot ? __fsub_rn(psum, pcomp) : 0.f;
-        // replicas of a target: fixed-order pairwise sums
-        for (int o = P; o < 32; o <<= 1) {
-            vx = __fadd_rn(vx, __shfl_xor_sync(FULL, vx, o));
-            vy = __fadd_rn(vy, __shfl_xor_sync(FULL, vy, o));
-            vz = __fadd_rn(vz, __shfl_xor_sync(FULL, vz, o));
-            if (kPot) vp = __fadd_rn(vp, __shfl_xor_sync(FULL, vp, o));
+        const uint32_t cnt_pn = __reduce_add_sync(FULL, my_pn), cnt_pp = cnt_all - cnt_pn;
+        float2 vx = make_float2(__fsub_rn(acc.sx.x, acc.kx.x), __fsub_rn(acc.sx.y, acc.kx.y));
+        float2 vy = make_float2(__fsub_rn(acc.sy.x, acc.ky.x), __fsub_rn(acc.sy.y, acc.ky.y));
+        float2 vz = make_float2(__fsub_rn(acc.sz.x, acc.kz.x), __fsub_rn(acc.sz.y, acc.kz.y));
+        float2 vp = kPot ? make_float2(__fsub_rn(psum.x, pcomp.x), __fsub_rn(psum.y, pcomp.y)) : make_float2(0.f, 0.f);
+        // replicas of a target: fixed-order pairwise sums, replica r with r + o
+        for (uint32_t o = 1; o < R; o <<= 1) {
+            const bool in = rep + o < R;
+            auto fold = [&](float &v) {
+                const float w = __shfl_down_sync(FULL, v, o * P);
+                if (in) v = __fadd_rn(v, w);
+            };
+            fold(vx.x); fold(vx.y); fold(vy.x); fold(vy.y); fold(vz.x); fold(vz.y);
+            if (kPot) { fold(vp.x); fold(vp.y); }
         }
-        if (active && rep == 0) {
-            T.acc[i] = vx * p.out_scale;
-            T.acc[T.n + i] = vy * p.out_scale;
-            T.acc[2 * T.n + i] = vz * p.out_scale;
-            T.npp[i] = cnt_pp - 1u;
-            T.npn[i] = cnt_pn;
-            if (kPot) T.pot[i] = -vp * p.pot_scale;
+        if (rep == 0u) {
+            T.acc[i0] = vx.x * p.out_scale;
+            T.acc[T.n + i0] = vy.x * p.out_scale;
+            T.acc[2 * T.n + i0] = vz.x * p.out_scale;
+            T.npp[i0] = cnt_pp - 1u;
+            T.npn[i0] = cnt_pn;
+            if (kPot) T.pot[i0] = -vp.x * p.pot_scale;
+            if (two) {
+                T.acc[i1] = vx.y * p.out_scale;
+                T.acc[T.n + i1] = vy.y * p.out_scale;
+                T.acc[2 * T.n + i1] = vz.y * p.out_scale;
+                T.npp[i1] = cnt_pp - 1u;
+                T.npn[i1] = cnt_pn;
+                if (kPot) T.pot[i1] = -vp.y * p.pot_scale;
+            }
         }
         if (lane == 0) {
             T.gcost[g] = cnt_pp + cnt_pn;
@@ -737,6 +873,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             atomicAdd(a.inter, ni);
             if (kMulti && a.tree_inter) atomicAdd(a.tree_inter + ti, ni);
         }
+        __syncwarp();
     }
 }
 
@@ -919,14 +1056,16 @@ WalkParams make_walk_params(const og_params &p, int opening, double theta) {
         const double rsg = p.r_s / p.box * two32;
         w.rc2 = (float)(rcg * rcg);
         w.rprune = (unsigned long long)(rcg * rcg * (1.0 + 1.0 / 1024.0));
-        w.inv_2rs = (float)(1.0 / (2.0 * rsg));
         // exp(-r^2 / (4 r_s^2)) = 2^(r^2 * kexp)
         w.kexp = (float)(-1.4426950408889634 / (4.0 * rsg * rsg));
+        w.erf_ky = (float)(2.0 * rsg / (double)kErfP);
+        w.erf_c = (float)((double)kTwoOverSqrtPi / (2.0 * rsg));
     } else {
         w.rc2 = __builtin_huge_valf();
         w.rprune = ~0ull;
-        w.inv_2rs = 0.0f;
         w.kexp = 0.0f;
+        w.erf_ky = 0.0f;
+        w.erf_c = 0.0f;
     }
     const double hg = 2.8 * p.eps / p.box * two32;
     w.h = (float)hg;
