@@ -335,6 +335,7 @@ struct WalkParams {
     float kexp;        // -log2(e) / (4 r_s^2), grid units
     float out_scale;   // G (2^32/L)^2
     float pot_scale;   // G 2^32/L (potential from grid units)
+    int split_long;    // long walks are split into parts (og_walk.cu)
 };
 // One walk launch over all groups of all boxes.  first_pass: the Barnes-Hut
 // pass that supplies a_old for the relative criterion (each box's

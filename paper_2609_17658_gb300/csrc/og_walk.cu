@@ -43,7 +43,8 @@
 //
 // Work distribution: persistent blocks; warps take groups from a global
 // atomic counter, in decreasing order of the previous pass's list length
-// when that is known (longest first shortens the tail of the launch).
+// when that is known (longest first shortens the tail of the launch), and in
+// parts where a list is much longer than the others (kQuota).
 #include <map>
 #include <mutex>
 #include <type_traits>
@@ -73,7 +74,24 @@ constexpr int kFarStep = 4;        // far entries in flight per lane
 constexpr int kNearChunk = 128;
 constexpr int kNearFlush = kNearChunk - 64 - kMaxRep;
 constexpr int kFarPad = 64 + kMaxRep * kFarStep;
-constexpr int kMinChunk = 64, kMaxChunk = 1024;
+constexpr int kMaxChunk = 1024;
+
+// Long walks in parts.  The relative criterion gives a few groups (large boxes,
+// small accelerations) lists 15 times the mean, and one warp needs 0.3-0.5 ms for
+// such a list, however idle the rest of the GPU is.  A walk that is not done
+// after kQuota rounds leaves what its stack then holds to kParts - 1 further parts,
+// which a second launch walks.  This depends on nothing but the group's own
+// walk, so a group's sums are the same whatever else is in the launch.
+// Only for boxes of 2049 to 196608 particles: below, no walk gets that far; above,
+// the other groups fill the time and the parts cost more than they save.
+// Clustered, accelerations given: 32k 197 -> 154 us, 100k 356 -> 262, 131k 433 ->
+// 309, 262k 499 -> 522 (not split); both passes: 65k 901 -> 554, 131k 785 -> 658,
+// 2.1M 5.71 -> 6.08 ms (not split).  A quota of 32, 40 or 64 rounds, or 16 and 32
+// parts: 262-302 us at 100k.  The Barnes-Hut lists are even enough that splitting
+// them gained nothing at any size (131k 258 -> 265-280 us).
+constexpr uint32_t kQuota = 48, kParts = 8;
+constexpr int kSpill = kStackCap;      // ranges a walk can leave
+constexpr int64_t kSplitMin = 2048, kSplitMax = 196608;
 
 // shared memory of one warp: its stack, near chunk and far chunk
 __host__ __device__ constexpr size_t warp_smem(int chunk) {
@@ -117,6 +135,12 @@ struct TreeView {
     float *pot;                   // [n] sorted, out (potential launches only)
     uint32_t *npp, *npn;          // [n] sorted, out
     int has_cost;                 // gcost holds the list lengths of a previous pass
+    // groups walked in parts (null: never); in scratch of the pass
+    uint2 *spill;                 // kSpill child ranges per group
+    uint32_t *nspill, *pdone;     // their number, and the further parts finished, per group
+    uint2 *pcnt;                  // [part][group] PP and PN entries
+    float *psum;                  // partial sums: [part][axis][particle]
+    int64_t nall;                 // groups of the tree (ngroups: those to walk)
 };
 
 struct WalkArgs {
@@ -130,6 +154,9 @@ struct WalkArgs {
     int64_t list_cap;
     unsigned long long *work;     // item counter
     int warps, chunk;             // launch shape: warps per block, far-chunk entries
+    uint2 *sitems;                // further parts of groups: (group, tree << 8 | part)
+    unsigned long long *nsplit;   // their number
+    int second;                   // the launch that walks them
     int one_seg;                  // a single tree of one box: its parameters are p0
     WalkParams p0;                // the box's parameters, in the launch's own argument space
     unsigned long long *inter;    // interactions evaluated
@@ -623,25 +650,41 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
     const unsigned FULL = 0xffffffffu;
     const unsigned lt = (1u << lane) - 1u;
 
-    while (true) {
-        unsigned long long gq = 0;
-        if (lane == 0) gq = atomicAdd(a.work, 1ull);
-        gq = __shfl_sync(FULL, gq, 0);
+    pdl_wait();
+    // Items: the groups, or in the second launch the further parts.  A warp's first
+    // item is its own number (neighbours on different SMs), the rest come from a
+    // counter: the first ones taken there too would queue every warp of the launch
+    // on one address.
+    const uint32_t nitems = a.second ? (uint32_t)*a.nsplit : (uint32_t)(kMulti ? a.nitems : a.tree0.ngroups);
+    uint32_t item = gridDim.x * (uint32_t)warp + blockIdx.x;
+    auto advance = [&] {
+        const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
+        if (nitems <= nwarps) return false;
+        uint32_t k = 0;
+        if (lane == 0) k = (uint32_t)atomicAdd(a.work + (a.second ? 4 : 0), 1ull);
+        item = nwarps + __shfl_sync(FULL, k, 0);
+        return true;
+    };
+    for (bool more = true; more && item < nitems; more = advance()) {
         int64_t g;
         int64_t ti = 0;
-        if (kMulti) {
-            if (gq >= (unsigned long long)a.nitems) break;
-            const uint64_t item = a.items ? a.items[gq] : gq;
+        uint32_t part = 0;
+        if (a.second) {
+            const uint2 it = a.sitems[item];
+            g = it.x;
+            part = it.y & 0xffu;
+            if (kMulti) ti = it.y >> 8;
+        } else if (kMulti) {
+            const uint64_t it = a.items ? a.items[item] : item;
             int64_t lo_t = 0, hi_t = a.ntrees;  // goff[lo_t] <= item < goff[hi_t]
             while (hi_t - lo_t > 1) {
                 const int64_t mid = (lo_t + hi_t) >> 1;
-                if (a.goff[mid] <= item) lo_t = mid; else hi_t = mid;
+                if (a.goff[mid] <= it) lo_t = mid; else hi_t = mid;
             }
             ti = lo_t;
-            g = (int64_t)(item - a.goff[ti]);
+            g = (int64_t)(it - a.goff[ti]);
         } else {
-            if (gq >= (unsigned long long)a.tree0.ngroups) break;
-            g = a.tree0.gorder ? (int64_t)a.tree0.gorder[gq] : (int64_t)gq;
+            g = a.tree0.gorder ? (int64_t)a.tree0.gorder[item] : (int64_t)item;
         }
         const TreeView &T = kMulti ? a.trees[ti] : a.tree0;
         const uint32_t seg = kOneSeg ? 0u : T.gseg[g];
@@ -690,9 +733,19 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             arelf = __double2float_rn(arel);
         }
 
-        if (lane == 0) stk[0] = make_uint2(T.ncbeg[seg], T.nccnt[seg]);
-        __syncwarp();
+        // the root's children, or this part's share of what the first part left
         int sp = 1, cf = 0, cn = 0;
+        if (part > 0u) {
+            const uint32_t left = T.nspill[g];
+            sp = left >= part ? (int)((left - part) / (kParts - 1u)) + 1 : 0;
+            for (int k = lane; k < sp; k += 32)
+                stk[k] = T.spill[(uint64_t)g * kSpill + part - 1u + (uint32_t)k * (kParts - 1u)];
+        } else if (lane == 0) {
+            stk[0] = make_uint2(T.ncbeg[seg], T.nccnt[seg]);
+        }
+        __syncwarp();
+        uint32_t quota = part > 0u || !p.split_long ? 0xffffffffu : kQuota;
+        bool leave = false;
         uint32_t rounds = 0;
         const uint32_t nchild = (uint32_t)T.nchild, max_rounds = (uint32_t)T.max_rounds;
         uint32_t cnt_all = 0, my_pn = 0;      // entries (warp), node entries (this lane)
@@ -804,7 +857,8 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             __syncwarp();
             // a chunk above its limit, or the walk's end, is evaluated; flushes are
             // rare, so they are hinted off the round's path
-            const bool done = sp == 0;
+            leave = rounds >= quota && sp > 0 && sp <= kSpill;
+            const bool done = sp == 0 || leave;
             if (__builtin_expect(done || cn > kNearFlush, 0)) {
                 const int q = pad_chunk(chn, cn, R, 1u, lane, box.hi);
                 __syncwarp();
@@ -836,7 +890,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             __syncwarp();
             continue;
         }
-        const uint32_t cnt_pn = __reduce_add_sync(FULL, my_pn), cnt_pp = cnt_all - cnt_pn;
+        uint32_t cnt_pn = __reduce_add_sync(FULL, my_pn), cnt_pp = cnt_all - cnt_pn;
         float2 vx = make_float2(__fsub_rn(acc.sx.x, acc.kx.x), __fsub_rn(acc.sx.y, acc.kx.y));
         float2 vy = make_float2(__fsub_rn(acc.sy.x, acc.ky.x), __fsub_rn(acc.sy.y, acc.ky.y));
         float2 vz = make_float2(__fsub_rn(acc.sz.x, acc.kz.x), __fsub_rn(acc.sz.y, acc.kz.y));
@@ -850,6 +904,58 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             };
             fold(vx.x); fold(vx.y); fold(vy.x); fold(vy.y); fold(vz.x); fold(vz.y);
             if (kPot) { fold(vp.x); fold(vp.y); }
+        }
+        // A group in parts: every part leaves its sums and counts, and the one that
+        // finishes last adds them up in the order of the parts.
+        if (leave || part > 0u) {
+            const uint64_t m = (uint64_t)T.n, ax = kPot ? 4u : 3u;
+            if (rep == 0u) {
+                float *w = T.psum + part * ax * m;
+                w[i0] = vx.x; w[m + i0] = vy.x; w[2 * m + i0] = vz.x;
+                if (kPot) w[3 * m + i0] = vp.x;
+                if (two) {
+                    w[i1] = vx.y; w[m + i1] = vy.y; w[2 * m + i1] = vz.y;
+                    if (kPot) w[3 * m + i1] = vp.y;
+                }
+            }
+            if (lane == 0) T.pcnt[(uint64_t)part * (uint64_t)T.nall + (uint64_t)g] = make_uint2(cnt_pp, cnt_pn);
+            if (part == 0u) {
+                // the further parts and the ranges they share (read by the second launch)
+                for (int k = lane; k < sp; k += 32) T.spill[(uint64_t)g * kSpill + k] = stk[k];
+                if (lane == 0) {
+                    T.nspill[g] = (uint32_t)sp;
+                    T.pdone[g] = 0u;
+                    const unsigned long long at = atomicAdd(a.nsplit, (unsigned long long)(kParts - 1u));
+                    for (uint32_t q = 1; q < kParts; ++q)
+                        a.sitems[at + q - 1u] = make_uint2((uint32_t)g, ((uint32_t)ti << 8) | q);
+                }
+                __syncwarp();
+                continue;
+            }
+            __threadfence();
+            __syncwarp();
+            uint32_t before = 0;
+            if (lane == 0) before = atomicAdd(&T.pdone[g], 1u);
+            before = __shfl_sync(FULL, before, 0);
+            if (before + 2u != kParts) continue;
+            __threadfence();
+            auto total = [&](uint64_t at) {
+                float v = __ldcg(T.psum + at);
+                for (uint32_t q = 1; q < kParts; ++q) v = __fadd_rn(v, __ldcg(T.psum + q * ax * m + at));
+                return v;
+            };
+            if (rep == 0u) {
+                vx = make_float2(total(i0), total(i1));
+                vy = make_float2(total(m + i0), total(m + i1));
+                vz = make_float2(total(2 * m + i0), total(2 * m + i1));
+                if (kPot) vp = make_float2(total(3 * m + i0), total(3 * m + i1));
+            }
+            cnt_pp = cnt_pn = 0u;
+            for (uint32_t q = 0; q < kParts; ++q) {
+                const uint2 c = __ldcg(&T.pcnt[(uint64_t)q * (uint64_t)T.nall + (uint64_t)g]);
+                cnt_pp += c.x;
+                cnt_pn += c.y;
+            }
         }
         if (rep == 0u) {
             T.acc[i0] = vx.x * p.out_scale;
@@ -902,7 +1008,15 @@ void launch_walk_t(const WalkArgs &a, int64_t nitems, cudaStream_t s, int sms) {
     int64_t grid = (int64_t)sms * per_sm;
     if (want < grid) grid = want;
     if (grid < 1) grid = 1;
-    kern<<<(unsigned)grid, a.warps * 32, smem, s>>>(a); note_launch();
+    launch_pdl(kern, (unsigned)grid, (unsigned)a.warps * 32u, smem, s, a);
+    if (a.nsplit) {
+        // the further parts: their number is known on the device only
+        WalkArgs b = a;
+        b.second = 1;
+        const int64_t most = nitems * (int64_t)(kParts - 1u), all = (int64_t)sms * per_sm;
+        grid = (most + a.warps - 1) / a.warps;
+        launch_pdl(kern, (unsigned)(grid < all ? grid : all), (unsigned)a.warps * 32u, smem, s, b);
+    }
 }
 
 template <int kOpen, bool kSplit>
@@ -978,10 +1092,32 @@ void launch(const WalkArgs &a, int opening, bool split, bool dump, bool refit, b
     else dispatch<OG_OPEN_REL>(a, split, dump, refit, multi, pot, nitems, s, sms);
 }
 
+// Scratch of one tree's pass: the partial results of groups walked in parts.
+struct PassScratch {
+    uint64_t n = 0, groups = 0, axes = 3;
+    bool used = false;
+    static uint64_t up(uint64_t b) { return (b + 255u) & ~(uint64_t)255u; }
+    uint64_t item_bytes() const { return used ? up(groups * (kParts - 1u) * sizeof(uint2)) : 0; }
+    uint64_t bytes() const {
+        if (!used) return 0;
+        return up(groups * kSpill * sizeof(uint2)) + 2 * up(groups * 4u) + up(groups * kParts * sizeof(uint2)) +
+               up(n * kParts * axes * 4u);
+    }
+    // hand out the arrays from q (bytes() long)
+    void place(char *q, TreeView &v) const {
+        if (!used) return;
+        v.spill = reinterpret_cast<uint2 *>(q); q += up(groups * kSpill * sizeof(uint2));
+        v.nspill = reinterpret_cast<uint32_t *>(q); q += up(groups * 4u);
+        v.pdone = reinterpret_cast<uint32_t *>(q); q += up(groups * 4u);
+        v.pcnt = reinterpret_cast<uint2 *>(q); q += up(groups * kParts * sizeof(uint2));
+        v.psum = reinterpret_cast<float *>(q);
+    }
+};
+
 // Per-box parameters of a pass (uploaded) and the tree's view.  The first
 // pass of the relative criterion is Barnes-Hut with theta_first_pass.
 og_status prepare_view(og_tree *t, int opening, bool first_pass, const float *a_old_sorted,
-                       float *acc_sorted, TreeView *v, WalkParams *wp0) {
+                       float *acc_sorted, bool pot, TreeView *v, WalkParams *wp0, PassScratch *sc) {
     cudaStream_t s = t->ctx->stream;
     const int64_t B = t->nseg;
     t->h_wp.resize((size_t)B);
@@ -991,7 +1127,13 @@ og_status prepare_view(og_tree *t, int opening, bool first_pass, const float *a_
         if (first_pass) t->h_wp[b].dump = false;
         // FP64 output: the last pass stores the unscaled sums, scaled in FP64 later
         if (!first_pass && t->unscaled_out) t->h_wp[b].out_scale = 1.0f;
+        const int64_t nb = (int64_t)t->h_seg_off[b + 1] - (int64_t)t->h_seg_off[b];
+        t->h_wp[b].split_long = opening == OG_OPEN_REL && nb > kSplitMin && nb <= kSplitMax;
+        if (t->h_wp[b].split_long) sc->used = true;
     }
+    sc->n = (uint64_t)t->n;
+    sc->groups = (uint64_t)t->ngroups;
+    sc->axes = pot ? 4u : 3u;
     *wp0 = t->h_wp[0];
     WalkParams *dp = t->segp + (first_pass ? 0 : B);
     cudaError_t err = cudaMemcpyAsync(dp, t->h_wp.data(), B * sizeof(WalkParams), cudaMemcpyHostToDevice, s);
@@ -1000,6 +1142,7 @@ og_status prepare_view(og_tree *t, int opening, bool first_pass, const float *a_
     w = TreeView{};
     w.n = t->n;
     w.ngroups = t->ngroups;
+    w.nall = t->ngroups;
     w.gbeg = t->gbeg;
     w.gend = t->gend;
     w.gbox = t->gbox;
@@ -1148,13 +1291,26 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
     cudaStream_t s = t->ctx->stream;
     WalkArgs a{};
     WalkParams wp;
-    og_status st = prepare_view(t, opening, first_pass, a_old_sorted, acc_sorted, &a.tree0, &wp);
+    PassScratch sc;
+    og_status st = prepare_view(t, opening, first_pass, a_old_sorted, acc_sorted, pot_sorted != nullptr, &a.tree0,
+                                &wp, &sc);
     if (st) return st;
     fill_common(a, t->ctx, t);
     a.one_seg = t->nseg == 1 ? 1 : 0;
     a.p0 = t->h_wp[0];
     cudaError_t err;
-    void *sort_tmp = nullptr;
+    void *sort_tmp = nullptr, *pass_tmp = nullptr;
+    if (sc.used) {
+        if ((err = dev_malloc_async(&pass_tmp, sc.item_bytes() + sc.bytes(), s)) != cudaSuccess)
+            return cuda_fail(err, "cudaMallocAsync (walk parts)");
+        a.sitems = static_cast<uint2 *>(pass_tmp);
+        a.nsplit = t->ctx->d_counters + 3;
+        sc.place(static_cast<char *>(pass_tmp) + sc.item_bytes(), a.tree0);
+    }
+    auto release = [&] {
+        if (pass_tmp) cudaFreeAsync(pass_tmp, s);
+        if (sort_tmp) cudaFreeAsync(sort_tmp, s);
+    };
     if (subset) {
         // only these groups, in this order (the walk takes them from gorder)
         a.tree0.gorder = subset;
@@ -1163,8 +1319,10 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
         // longest list first, from the costs of the previous pass on this tree
         const int64_t ng = t->ngroups;
         size_t bytes = (size_t)ng * 24 + radix_sort_scratch_bytes(ng) + 1024;
-        if ((err = dev_malloc_async(&sort_tmp, bytes, s)) != cudaSuccess)
+        if ((err = dev_malloc_async(&sort_tmp, bytes, s)) != cudaSuccess) {
+            release();
             return cuda_fail(err, "cudaMallocAsync (group order)");
+        }
         char *q = static_cast<char *>(sort_tmp);
         uint64_t *k0 = reinterpret_cast<uint64_t *>(q);
         uint64_t *k1 = k0 + ng;
@@ -1181,7 +1339,7 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
         // no host synchronisation: the counters go to a page-locked slot and
         // the times to events, both read by finish_deferred
         const int k = t->npend;
-        cudaMemsetAsync(t->ctx->d_counters, 0, 3 * sizeof(unsigned long long), s);
+        cudaMemsetAsync(t->ctx->d_counters, 0, 5 * sizeof(unsigned long long), s);
         cudaEventCreate(&t->pend_e0[k]);
         cudaEventCreate(&t->pend_e1[k]);
         cudaEventRecord(t->pend_e0[k], s);
@@ -1191,7 +1349,7 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
         cudaMemcpyAsync(pinned_counters(t->ctx, k), t->ctx->d_counters, 3 * sizeof(unsigned long long),
                         cudaMemcpyDeviceToHost, s);
         t->npend = k + 1;
-        if (sort_tmp) cudaFreeAsync(sort_tmp, s);
+        release();
         // the next pass may take this one's list lengths: stream order makes them ready
         t->have_cost = true;
         if (ms_out) *ms_out = 0.0f;
@@ -1199,7 +1357,7 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
     }
     unsigned long long h[3] = {0, 0, 0};
     for (int attempt = 0; attempt < 2; ++attempt) {
-        cudaMemsetAsync(t->ctx->d_counters, 0, 3 * sizeof(unsigned long long), s);
+        cudaMemsetAsync(t->ctx->d_counters, 0, 5 * sizeof(unsigned long long), s);
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
@@ -1218,7 +1376,7 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
         a.lists = t->lists;
         a.list_cap = t->list_cap;
     }
-    if (sort_tmp) cudaFreeAsync(sort_tmp, s);
+    release();
     if (st) return st;
     t->have_cost = true;
     t->interactions_last = (int64_t)h[1];
@@ -1234,12 +1392,13 @@ og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int openi
     if (ntrees < 1) return OG_OK;
     std::vector<TreeView> hv((size_t)ntrees);
     std::vector<uint64_t> hoff((size_t)ntrees + 1);
+    std::vector<PassScratch> sc((size_t)ntrees);
     bool split = false, refit = false;
     uint64_t total = 0;
     for (int64_t k = 0; k < ntrees; ++k) {
         WalkParams wp;
         og_status st = prepare_view(trees[k], opening, false, a_old_sorted ? a_old_sorted[k] : nullptr,
-                                    acc_sorted[k], &hv[k], &wp);
+                                    acc_sorted[k], false, &hv[k], &wp, &sc[k]);
         if (st) return st;
         if (k == 0) split = wp.split;
         else if (wp.split != split) {
@@ -1264,9 +1423,24 @@ og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int openi
     const int64_t nitems = (int64_t)total;
     size_t bytes = (size_t)ntrees * sizeof(TreeView) + (size_t)(ntrees + 1) * 8 + (size_t)nitems * 24 +
                    radix_sort_scratch_bytes(nitems) + (size_t)ntrees * 8 + 4096;
+    // the parts of long walks: their items, then every tree's scratch
+    const size_t parts_at = (bytes + 255) & ~(size_t)255;
+    size_t item_bytes = 0, pass_bytes = 0;
+    for (const PassScratch &x : sc) {
+        item_bytes += (size_t)x.item_bytes();
+        pass_bytes += (size_t)x.bytes();
+    }
+    bytes = parts_at + item_bytes + pass_bytes;
     void *tmp = nullptr;
     cudaError_t err;
     if ((err = dev_malloc_async(&tmp, bytes, s)) != cudaSuccess) return cuda_fail(err, "cudaMallocAsync (walk items)");
+    {
+        char *at = static_cast<char *>(tmp) + parts_at + item_bytes;
+        for (int64_t k = 0; k < ntrees; ++k) {
+            sc[k].place(at, hv[k]);
+            at += sc[k].bytes();
+        }
+    }
     char *q = static_cast<char *>(tmp);
     TreeView *dv = reinterpret_cast<TreeView *>(q);
     q += ((size_t)ntrees * sizeof(TreeView) + 255) & ~(size_t)255;
@@ -1291,9 +1465,13 @@ og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int openi
     a.items = alt ? v1 : v0;
     a.ntrees = ntrees;
     a.nitems = nitems;
+    if (item_bytes) {
+        a.sitems = reinterpret_cast<uint2 *>(static_cast<char *>(tmp) + parts_at);
+        a.nsplit = c->d_counters + 3;
+    }
     a.tree_inter = tint;
     cudaMemsetAsync(tint, 0, (size_t)ntrees * sizeof(unsigned long long), s);
-    cudaMemsetAsync(c->d_counters, 0, 3 * sizeof(unsigned long long), s);
+    cudaMemsetAsync(c->d_counters, 0, 5 * sizeof(unsigned long long), s);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
