@@ -29,7 +29,7 @@
 // deepest path: 31 + 147 < 200 entries above kSphDeep.  A push past the
 // capacity would still only set the stack-overflow status and drop the range.
 // The round count is bounded by the number of nodes plus the buckets' extra
-// rounds.
+// rounds.  Groups with very many candidates go to a block each (k_sph_long).
 #include <cmath>
 
 #include "og_internal.h"
@@ -53,6 +53,8 @@ struct SphArgs {
     const uint8_t *done;    // null, or per particle (key order): converged, skip
     const float *hg;        // smoothing length in grid units, sorted order
     int64_t ngroups;
+    uint32_t *longs;        // groups left to a block each: their number, then their ids
+    int limit;              // candidates above which a group is left to a block
     int64_t max_rounds;     // nodes + 2 + buckets' extra rounds (<= n / 32)
     double dens;            // 8 / pi * (2^32 / L)^3
     float *rho;             // caller order (key order without perm)
@@ -92,6 +94,205 @@ __global__ void k_sph_prep(int64_t n, const uint32_t *__restrict__ perm, const f
     hg[i] = __double2float_rn(v * to_grid);
 }
 
+// A group that finds more than `limit` candidates (SphArgs) is left to a block
+// (k_sph_long): a few groups of sparse particles beside a halo's core find tens of
+// thousands, and one warp took as long for one of them as the rest of the GPU
+// for all other groups (315 on average).  One warp searches 2048 in about 0.3 ms;
+// the fewer the groups, the sooner the rest is done and the lower the limit pays.
+// A call on clustered sets, start and with a limit of 512 / 1024 / 2048:
+// 10k particles 472 -> 188 / 248 / 370 us; 100k 1456 -> 538 / 446 / 554 us; 2.1M
+// 2.88 -> 2.55 (1024) / 2.28 (2048) / 2.33 ms (3072).
+inline int candidate_limit(int64_t ngroups) { return ngroups < 2000 ? 512 : ngroups < 20000 ? 1024 : 2048; }
+
+// the targets of a group, one per lane, and the search region
+struct SphTargets {
+    uint32_t me, xi, yi, zi;
+    bool active;
+    float hgi, h2i, inv_h;
+    unsigned long long hm2;
+    uint32_t lo[3], gl[3];
+};
+__device__ __forceinline__ SphTargets sph_targets(const SphArgs &a, int64_t g, unsigned lane) {
+    SphTargets t;
+    t.me = a.gbeg[g] + lane;
+    t.active = t.me < a.gend[g];
+    t.xi = t.active ? a.px[t.me] : 0u;
+    t.yi = t.active ? a.py[t.me] : 0u;
+    t.zi = t.active ? a.pz[t.me] : 0u;
+    t.hgi = t.active ? a.hg[t.me] : 0.0f;
+    t.h2i = __fmul_rn(t.hgi, t.hgi);
+    t.inv_h = t.active && t.hgi > 0.0f ? 1.0f / t.hgi : 0.0f;
+    // the group's search radius: the largest h, widened by a margin
+    const float hmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(t.hgi)));
+    const unsigned long long hm = (unsigned long long)(hmax * 1.0001f) + 2ull;
+    t.hm2 = hm * hm;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        t.lo[k] = a.gbox[6 * g + k];
+        t.gl[k] = a.gbox[6 * g + 3 + k] - t.lo[k];
+    }
+    return t;
+}
+
+// nc candidates for this lane's target
+__device__ __forceinline__ void sph_pairs(const uint4 *chunk, int nc, const SphTargets &g, float &sum, uint32_t &cnt) {
+    for (int t = 0; t < nc; ++t) {
+        const uint4 c = chunk[t];
+        const float fx = (float)(int32_t)(c.x - g.xi), fy = (float)(int32_t)(c.y - g.yi),
+                    fz = (float)(int32_t)(c.z - g.zi);
+        const float r2 = __fadd_rn(__fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy)), __fmul_rn(fz, fz));
+        if (r2 < g.h2i) {
+            ++cnt;
+            const float q = sqrtf(r2) * g.inv_h;
+            const float u = 1.0f - q;
+            const float w = q < 0.5f ? 1.0f - 6.0f * q * q * u : 2.0f * u * u * u;
+            sum = fmaf(__uint_as_float(c.w), w, sum);
+        }
+    }
+}
+
+// a child record: a node to open, a candidate, or neither
+__device__ __forceinline__ void sph_test(const CRec &rec, bool has, const SphTargets &t, bool &push, bool &app) {
+    const bool node = has && !(rec.info >> 31);
+    push = app = false;
+    if (node) {
+        const uint32_t lev = (rec.info >> 26) & 31u;
+        const uint32_t side = 1u << (32u - lev);    // lev >= 1 for a child node
+        const uint32_t msk = ~(side - 1u);
+        const unsigned long long g2 = sq(gap_boxes(t.lo[0], t.gl[0], rec.x & msk, side - 1u)) +
+                                      sq(gap_boxes(t.lo[1], t.gl[1], rec.y & msk, side - 1u)) +
+                                      sq(gap_boxes(t.lo[2], t.gl[2], rec.z & msk, side - 1u));
+        push = g2 <= t.hm2;
+    } else if (has) {
+        const unsigned long long g2 = sq(gap_point(rec.x, t.lo[0], t.gl[0])) +
+                                      sq(gap_point(rec.y, t.lo[1], t.gl[1])) +
+                                      sq(gap_point(rec.z, t.lo[2], t.gl[2]));
+        app = g2 <= t.hm2;
+    }
+}
+
+__device__ __forceinline__ void sph_store(const SphArgs &a, const SphTargets &t, float sum, uint32_t cnt) {
+    if (!t.active) return;
+    const uint32_t i = a.perm ? a.perm[t.me] : t.me;
+    const double hd = (double)t.hgi;
+    a.rho[i] = __double2float_rn(a.dens * (double)sum / (hd * hd * hd));
+    if (a.nngb) a.nngb[i] = cnt;
+}
+
+// A group by a block of kLongWarps warps: every round takes up to one record per
+// thread off one stack, and the chunk's candidates are shared out, warp w the w-th
+// part of them for all targets.  The rounds are ordered by block barriers and every
+// position by prefix sums, so the sums do not depend on the schedule.  Stack depth
+// as in k_sph_density: a round adds at most kLongThreads ranges, beyond kLongDeep
+// one range at a time.
+constexpr int kLongWarps = 16, kLongThreads = 32 * kLongWarps;
+constexpr int kLongStack = 2048, kLongDeep = kLongStack - kLongThreads - 200;
+constexpr int kLongChunk = 1024;
+
+// exclusive prefix over the block and its total; every thread calls it
+__device__ __forceinline__ uint32_t block_prefix(uint32_t v, uint32_t *tot, uint32_t &total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t inc = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += o;
+    }
+    __syncthreads();
+    if (lane == 31) tot[warp] = inc;
+    __syncthreads();
+    uint32_t before = 0u;
+    total = 0u;
+#pragma unroll
+    for (int k = 0; k < kLongWarps; ++k) {
+        const uint32_t x = tot[k];
+        if (k < warp) before += x;
+        total += x;
+    }
+    return before + inc - v;
+}
+
+__global__ void __launch_bounds__(kLongThreads) k_sph_long(SphArgs a) {
+    __shared__ unsigned long long stk[kLongStack];
+    __shared__ uint4 chunk[kLongChunk];
+    __shared__ uint32_t recs[kLongThreads], tot[kLongWarps];
+    __shared__ float psum[kLongWarps][32];
+    __shared__ uint32_t pcnt[kLongWarps][32];
+    const int warp = threadIdx.x >> 5, tid = threadIdx.x;
+    const unsigned lane = threadIdx.x & 31u;
+    const uint32_t nlong = a.longs[0];
+    for (uint32_t q = blockIdx.x; q < nlong; q += gridDim.x) {
+        const int64_t g = a.longs[1 + q];
+        const SphTargets t = sph_targets(a, g, lane);
+        if (a.done && __all_sync(0xffffffffu, !t.active || a.done[t.me] != 0)) continue;  // the whole block
+        float sum = 0.0f;
+        uint32_t cnt = 0;
+        int sp = 1, nc = 0;
+        __syncthreads();
+        if (tid == 0) stk[0] = (unsigned long long)a.ncbeg[0] | ((unsigned long long)a.nccnt[0] << 32);
+        __syncthreads();
+        for (int64_t round = 0; sp > 0 && round < a.max_rounds; ++round) {
+            // the top ranges of the stack, whole while they fit in the block; a first
+            // range that does not fit (a bucket) gives what does
+            const int top = sp > kLongDeep ? 1 : (sp < kLongThreads ? sp : kLongThreads);
+            const unsigned long long r = tid < top ? stk[sp - 1 - tid] : 0ull;
+            const uint32_t beg = (uint32_t)r, c = (uint32_t)(r >> 32);
+            uint32_t all;
+            const uint32_t cc = c <= (uint32_t)kLongThreads ? c : (uint32_t)kLongThreads + 1u;
+            const uint32_t excl = block_prefix(tid < top ? cc : 0u, tot, all);
+            const bool whole = tid < top && excl + cc <= (uint32_t)kLongThreads;
+            const bool bucket = tid == 0 && cc > (uint32_t)kLongThreads;
+            const int take = __syncthreads_count(whole);
+            if (whole)
+                for (uint32_t k = 0; k < c; ++k) recs[excl + k] = beg + k;
+            if (bucket) {
+                for (uint32_t k = 0; k < (uint32_t)kLongThreads; ++k) recs[k] = beg + k;
+                stk[sp - 1] = (unsigned long long)(beg + kLongThreads) | ((unsigned long long)(c - kLongThreads) << 32);
+            }
+            uint32_t total;
+            (void)block_prefix(whole ? c : bucket ? (uint32_t)kLongThreads : 0u, tot, total);
+            sp -= take;
+            CRec rec{};
+            const bool has = (uint32_t)tid < total;
+            if (has) rec = a.crec[recs[tid]];
+            bool push, app;
+            sph_test(rec, has, t, push, app);
+            // both counts in one prefix sum: pushes above, candidates below
+            uint32_t both;
+            const uint32_t at = block_prefix((push ? 1u << 16 : 0u) + (app ? 1u : 0u), tot, both);
+            if (push) {
+                const int pos = sp + (int)(at >> 16);
+                if (pos < kLongStack) stk[pos] = (unsigned long long)rec.ref | ((unsigned long long)(rec.info & 0x3ffffffu) << 32);
+                else atomicOr(a.status, ST_STACK_OVF);
+            }
+            if (app) chunk[nc + (int)(at & 0xffffu)] = make_uint4(rec.x, rec.y, rec.z, __float_as_uint(rec.m));
+            sp += (int)(both >> 16);
+            if (sp > kLongStack) sp = kLongStack;
+            nc += (int)(both & 0xffffu);
+            __syncthreads();
+            if (nc > kLongChunk - kLongThreads || sp == 0) {
+                const int b = nc * warp / kLongWarps, e = nc * (warp + 1) / kLongWarps;
+                sph_pairs(chunk + b, e - b, t, sum, cnt);
+                nc = 0;
+                __syncthreads();
+            }
+        }
+        if (sp > 0 && tid == 0) atomicOr(a.status, ST_INTERNAL);   // the round bound was reached
+        psum[warp][lane] = sum;
+        pcnt[warp][lane] = cnt;
+        __syncthreads();
+        if (warp == 0) {
+            float v = psum[0][lane];
+            uint32_t k = pcnt[0][lane];
+            for (int w = 1; w < kLongWarps; ++w) {
+                v = __fadd_rn(v, psum[w][lane]);
+                k += pcnt[w][lane];
+            }
+            sph_store(a, t, v, k);
+        }
+    }
+}
+
 __global__ void __launch_bounds__(32 * kSphWarps) k_sph_density(SphArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5;
@@ -103,46 +304,17 @@ __global__ void __launch_bounds__(32 * kSphWarps) k_sph_density(SphArgs a) {
     uint4 *chunk = reinterpret_cast<uint4 *>(smem_raw + (size_t)kSphWarps * kSphStack * 8) +
                    (size_t)warp * kSphChunk;
 
-    const uint32_t b = a.gbeg[g], e = a.gend[g];
-    const uint32_t me = b + lane;
-    const bool active = me < e;
-    const uint32_t xi = active ? a.px[me] : 0u, yi = active ? a.py[me] : 0u, zi = active ? a.pz[me] : 0u;
-    if (a.done && __all_sync(0xffffffffu, !active || a.done[me] != 0)) return;  // nothing to redo
-    const float hgi = active ? a.hg[me] : 0.0f;
-    const float h2i = __fmul_rn(hgi, hgi);
-    const float inv_h = active && hgi > 0.0f ? 1.0f / hgi : 0.0f;
-    // the group's search radius: the largest h, widened by a margin
-    const float hmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(hgi)));
-    const unsigned long long hm = (unsigned long long)(hmax * 1.0001f) + 2ull;
-    const unsigned long long hm2 = hm * hm;
-    uint32_t lo[3], gl[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        lo[k] = a.gbox[6 * g + k];
-        gl[k] = a.gbox[6 * g + 3 + k] - lo[k];
-    }
-
+    const SphTargets t = sph_targets(a, g, lane);
+    if (a.done && __all_sync(0xffffffffu, !t.active || a.done[t.me] != 0)) return;  // nothing to redo
     float sum = 0.0f;
     uint32_t cnt = 0;
     auto flush = [&](int nc) {
         __syncwarp();
-        for (int t = 0; t < nc; ++t) {
-            const uint4 c = chunk[t];
-            const float fx = (float)(int32_t)(c.x - xi), fy = (float)(int32_t)(c.y - yi),
-                        fz = (float)(int32_t)(c.z - zi);
-            const float r2 = __fadd_rn(__fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy)), __fmul_rn(fz, fz));
-            if (r2 < h2i) {
-                ++cnt;
-                const float q = sqrtf(r2) * inv_h;
-                const float u = 1.0f - q;
-                const float w = q < 0.5f ? 1.0f - 6.0f * q * q * u : 2.0f * u * u * u;
-                sum = fmaf(__uint_as_float(c.w), w, sum);
-            }
-        }
+        sph_pairs(chunk, nc, t, sum, cnt);
         __syncwarp();
     };
 
-    int sp = 0, nc = 0;
+    int sp = 0, nc = 0, found = 0;
     if (lane == 0) stk[0] = (unsigned long long)a.ncbeg[0] | ((unsigned long long)a.nccnt[0] << 32);
     sp = 1;
     __syncwarp();
@@ -184,22 +356,8 @@ __global__ void __launch_bounds__(32 * kSphWarps) k_sph_density(SphArgs a) {
         const bool has = lane < total;
         CRec rec{};
         if (has) rec = a.crec[obeg + (lane - oexcl)];
-        const bool node = has && !(rec.info >> 31);
-        bool push = false, app = false;
-        if (node) {
-            const uint32_t lev = (rec.info >> 26) & 31u;
-            const uint32_t side = 1u << (32u - lev);    // lev >= 1 for a child node
-            const uint32_t msk = ~(side - 1u);
-            const unsigned long long g2 = sq(gap_boxes(lo[0], gl[0], rec.x & msk, side - 1u)) +
-                                          sq(gap_boxes(lo[1], gl[1], rec.y & msk, side - 1u)) +
-                                          sq(gap_boxes(lo[2], gl[2], rec.z & msk, side - 1u));
-            push = g2 <= hm2;
-        } else if (has) {
-            const unsigned long long g2 = sq(gap_point(rec.x, lo[0], gl[0])) +
-                                          sq(gap_point(rec.y, lo[1], gl[1])) +
-                                          sq(gap_point(rec.z, lo[2], gl[2]));
-            app = g2 <= hm2;
-        }
+        bool push, app;
+        sph_test(rec, has, t, push, app);
         const unsigned bp = __ballot_sync(0xffffffffu, push);
         if (push) {
             const int pos = sp + __popc(bp & lt);
@@ -212,6 +370,11 @@ __global__ void __launch_bounds__(32 * kSphWarps) k_sph_density(SphArgs a) {
         if (app) chunk[nc + __popc(ba & lt)] = make_uint4(rec.x, rec.y, rec.z, __float_as_uint(rec.m));
         nc += __popc(ba);
         if (nc > kSphChunk - 32) {
+            found += nc;
+            if (found > a.limit) {
+                if (lane == 0) a.longs[1 + atomicAdd(&a.longs[0], 1u)] = (uint32_t)g;
+                return;
+            }
             flush(nc);
             nc = 0;
         }
@@ -219,12 +382,7 @@ __global__ void __launch_bounds__(32 * kSphWarps) k_sph_density(SphArgs a) {
     }
     if (sp > 0) atomicOr(a.status, ST_INTERNAL);   // the round bound was reached
     flush(nc);
-    if (active) {
-        const uint32_t i = a.perm ? a.perm[me] : me;
-        const double hd = (double)hgi;
-        a.rho[i] = __double2float_rn(a.dens * (double)sum / (hd * hd * hd));
-        if (a.nngb) a.nngb[i] = cnt;
-    }
+    sph_store(a, t, sum, cnt);
 }
 
 // One step of the smoothing-length iteration for every particle not yet
@@ -287,6 +445,20 @@ __global__ void k_sph_gather(int64_t n, const uint32_t *__restrict__ perm, const
 
 inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+// scratch of a search: the long groups' number and list
+inline size_t long_bytes(int64_t ng) { return (size_t)(ng + 1) * 4; }
+
+// the density of every group of the tree, at a.hg
+void search(SphArgs &a, char *scratch, cudaStream_t s) {
+    if (a.ngroups < 1) return;
+    a.longs = reinterpret_cast<uint32_t *>(scratch);
+    a.limit = candidate_limit(a.ngroups);
+    cudaMemsetAsync(a.longs, 0, 4, s);
+    k_sph_density<<<nblk(a.ngroups, kSphWarps), 32 * kSphWarps, kSphSmem, s>>>(a); note_launch();
+    const unsigned most = (unsigned)(a.ngroups < 456 ? a.ngroups : 456);   // 152 SMs x 3 blocks
+    k_sph_long<<<most, kLongThreads, 0, s>>>(a); note_launch();
+}
+
 }  // namespace
 }  // namespace og
 
@@ -312,7 +484,8 @@ extern "C" og_status og_tree_sph_density(og_tree *t, const float *h, float *rho,
     const size_t bh = (size_t)n * sizeof(float);
     // scratch: hg (sorted) [+ host staging: h in, rho and counts out]
     const size_t off_in = (bh + 255) & ~(size_t)255;
-    const size_t total = off_in + (dev ? 0 : 3 * off_in);
+    const size_t off_long = off_in + (dev ? 0 : 3 * off_in);
+    const size_t total = off_long + long_bytes(t->ngroups);
     char *buf = nullptr;
     cudaError_t e = dev_malloc_async(&buf, total, s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (sph)");
@@ -352,9 +525,7 @@ extern "C" og_status og_tree_sph_density(og_tree *t, const float *h, float *rho,
     a.rho = d_rho;
     a.nngb = d_cnt;
     a.status = c->d_status;
-    if (t->ngroups > 0) {
-        k_sph_density<<<nblk(t->ngroups, kSphWarps), 32 * kSphWarps, kSphSmem, s>>>(a); note_launch();
-    }
+    search(a, buf + off_long, s);
     cudaEventRecord(e1, s);
     if (!dev) {
         cudaMemcpyAsync(rho, d_rho, bh, cudaMemcpyDeviceToHost, s);
@@ -399,7 +570,8 @@ extern "C" og_status og_tree_sph_smoothing(og_tree *t, double n_target, double t
     // key-order state: h, lo, hi, grid h, rho, counts (4 B each), done (1 B); a
     // counter; host staging of h in/out, rho and counts out
     const size_t b4 = ((size_t)n * 4 + 255) & ~(size_t)255, b1 = ((size_t)n + 255) & ~(size_t)255;
-    const size_t total = 6 * b4 + b1 + 256 + (dev ? 0 : 3 * b4);
+    const size_t off_long = 6 * b4 + b1 + 256 + (dev ? 0 : 3 * b4);
+    const size_t total = off_long + long_bytes(t->ngroups);
     char *buf = nullptr;
     cudaError_t e = dev_malloc_async(&buf, total, s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (sph smoothing)");
@@ -450,7 +622,7 @@ extern "C" og_status og_tree_sph_smoothing(og_tree *t, double n_target, double t
     og_status st = OG_OK;
     while (it < max_iter) {
         k_sph_prep<<<nblk(n, 256), 256, 0, s>>>(n, nullptr, hs, to_grid, hg, c->d_status); note_launch();
-        k_sph_density<<<nblk(t->ngroups, kSphWarps), 32 * kSphWarps, kSphSmem, s>>>(a); note_launch();
+        search(a, buf + off_long, s);
         ++it;
         cudaMemsetAsync(left, 0, sizeof(unsigned long long), s);
         k_sph_update<<<nblk(n, 256), 256, 0, s>>>(n, n_target, tol, hcap, t->pm64, rs, hs, lo, hi, done, left);
@@ -465,7 +637,7 @@ extern "C" og_status og_tree_sph_smoothing(og_tree *t, double n_target, double t
         // last step needs them at its new h)
         a.done = nullptr;
         k_sph_prep<<<nblk(n, 256), 256, 0, s>>>(n, nullptr, hs, to_grid, hg, c->d_status); note_launch();
-        k_sph_density<<<nblk(t->ngroups, kSphWarps), 32 * kSphWarps, kSphSmem, s>>>(a); note_launch();
+        search(a, buf + off_long, s);
         k_sph_to_caller<<<nblk(n, 256), 256, 0, s>>>(n, t->perm, hs, rs, cs, d_h, d_rho, d_cnt); note_launch();
         cudaEventRecord(e1, s);
         if (!dev) {
