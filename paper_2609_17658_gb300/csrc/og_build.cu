@@ -118,25 +118,15 @@ __device__ __forceinline__ uint32_t quantize(double v, double box, double inv_bo
     return (uint32_t)floor(f * 4294967296.0);
 }
 
-// segment (box) of every particle of the concatenated input
-__global__ void k_fill_seg(int64_t n, int64_t B, const uint32_t *__restrict__ seg_off, uint32_t *pseg) {
-    pdl_wait();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int64_t lo = 0, hi = B;  // seg_off[lo] <= i < seg_off[hi]
-    while (hi - lo > 1) {
-        int64_t mid = (lo + hi) / 2;
-        if ((uint64_t)seg_off[mid] <= (uint64_t)i) lo = mid; else hi = mid;
-    }
-    pseg[i] = (uint32_t)lo;
-}
-
 // In a build (d_tot set) it also clears what later kernels accumulate into:
 // the device totals, the masses' set-bit span (empty: lowest 0x7f7f7f7f
 // above highest 0x80808080), the scans' look words and tile counters, and with
 // one box its sorted box indices (all 0).
-__global__ void k_quantize_keys(const double *__restrict__ pos, int64_t n, const uint32_t *__restrict__ pseg,
-                                const SegGeom *__restrict__ geom, uint4 *q4, uint64_t *key,
+// Several boxes (pseg set): it also finds and writes the box of every particle of
+// the caller's order, and reads the positions where the box has them (io).
+__global__ void k_quantize_keys(const double *__restrict__ pos, int64_t n, int64_t B,
+                                const uint32_t *__restrict__ seg_off, uint32_t *__restrict__ pseg,
+                                const BoxIO *__restrict__ io, const SegGeom *__restrict__ geom, uint4 *q4, uint64_t *key,
                                 uint64_t *key_copy, uint32_t *idx,
                                 uint32_t *sseg_zero, uint32_t *d_tot, int *mbits,
                                 unsigned long long *scan_look, int64_t nlook, uint32_t *status) {
@@ -151,12 +141,23 @@ __global__ void k_quantize_keys(const double *__restrict__ pos, int64_t n, const
     }
     if (i >= n) return;
     if (sseg_zero) sseg_zero[i] = 0u;
-    const SegGeom g = geom[pseg ? pseg[i] : 0];
+    uint32_t seg = 0;
+    const double *x3 = pos + 3 * i;
+    if (pseg) {
+        int64_t lo = 0, hi = B;  // seg_off[lo] <= i < seg_off[hi]
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) / 2;
+            if ((uint64_t)seg_off[mid] <= (uint64_t)i) lo = mid; else hi = mid;
+        }
+        pseg[i] = seg = (uint32_t)lo;
+        if (io) x3 = io[seg].pos + 3 * (i - (int64_t)seg_off[seg]);
+    }
+    const SegGeom g = geom[seg];
     const double box = g.box, inv_box = g.inv_box;
     const bool pow2 = g.pow2 != 0;
-    uint32_t x = quantize(pos[3 * i + 0], box, inv_box, pow2, g.shift, status);
-    uint32_t y = quantize(pos[3 * i + 1], box, inv_box, pow2, g.shift, status);
-    uint32_t z = quantize(pos[3 * i + 2], box, inv_box, pow2, g.shift, status);
+    uint32_t x = quantize(x3[0], box, inv_box, pow2, g.shift, status);
+    uint32_t y = quantize(x3[1], box, inv_box, pow2, g.shift, status);
+    uint32_t z = quantize(x3[2], box, inv_box, pow2, g.shift, status);
     q4[i] = make_uint4(x, y, z, 0u);   // one 16-byte record: the permute gathers it whole
     const uint64_t k = (spread21(x >> 11) << 2) | (spread21(y >> 11) << 1) | spread21(z >> 11);
     key[i] = k;
@@ -190,7 +191,8 @@ __global__ void k_gather_keys(int64_t n, const uint32_t *__restrict__ perm,
 // and highest exponents, merged by atomics only where they widen the span.
 __global__ void __launch_bounds__(kT) k_permute(int64_t n, const uint32_t *__restrict__ perm,
                                                 const uint4 *__restrict__ q4, const double *__restrict__ mass,
-                                                uint32_t *px, uint32_t *py, uint32_t *pz, float *pm32,
+                                                const BoxIO *__restrict__ io, const uint32_t *__restrict__ sseg,
+                                                const uint32_t *__restrict__ seg_off, uint32_t *px, uint32_t *py, uint32_t *pz, float *pm32,
                                                 double *pm64, uint32_t *inv, int *mbits, uint32_t *status) {
     pdl_wait();
     __shared__ int wlo[kT / 32], whi[kT / 32];
@@ -203,7 +205,13 @@ __global__ void __launch_bounds__(kT) k_permute(int64_t n, const uint32_t *__res
         px[i] = q.x;
         py[i] = q.y;
         pz[i] = q.z;
-        double m = mass[j];
+        double m;
+        if (io) {
+            const uint32_t b = sseg[i];
+            m = io[b].mass[j - seg_off[b]];
+        } else {
+            m = mass[j];
+        }
         if (!isfinite(m) || m < 0.0) atomicOr(status, ST_BAD_INPUT);
         pm64[i] = m;
         pm32[i] = __double2float_rn(m);
@@ -1178,10 +1186,8 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     cudaEventRecord(e0, s);
-    if (B > 1) {
-        launch_pdl(k_fill_seg, nblk(n), kT, 0, s, n, B, t->seg_off, pseg);
-    }
-    launch_pdl(k_quantize_keys, nblk(n), kT, 0, s, d_pos, n, B > 1 ? pseg : nullptr, t->geom, q4,
+    launch_pdl(k_quantize_keys, nblk(n), kT, 0, s, d_pos, n, B, t->seg_off, B > 1 ? pseg : nullptr,
+                                           (const BoxIO *)nullptr, t->geom, q4,
                                            keys, nullptr, idx, nullptr, nullptr, nullptr, nullptr, (int64_t)0,
                                            t->ctx->d_status);
     launch_pdl(k_repos, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, t->px, t->py, t->pz);
@@ -1336,9 +1342,6 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
     cudaEventRecord(e0, s);
 
     // a1, a2
-    if (B > 1) {
-        launch_pdl(k_fill_seg, nblk(n), kT, 0, s, n, B, t->seg_off, pseg);
-    }
     // the masses are checked where they are first read (k_permute), so that a
     // host copy of them can still be in flight here
     // one box: the keys and the permutation are sorted in place in the tree
@@ -1346,7 +1349,7 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
         keys = t->skey;
         idx = t->perm;
     }
-    launch_pdl(k_quantize_keys, nblk(n), kT, 0, s, d_pos, n, B > 1 ? pseg : nullptr, t->geom, q4,
+    launch_pdl(k_quantize_keys, nblk(n), kT, 0, s, d_pos, n, B, t->seg_off, B > 1 ? pseg : nullptr, t->io, t->geom, q4,
                                            keys, B > 1 ? key0 : nullptr, idx, B > 1 ? nullptr : t->sseg,
                                            d_tot, t->mbits, scan_look, nlook, status);
     // a3: by key, then (several boxes) stably by box
@@ -1371,7 +1374,7 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
         cudaMemcpyAsync(t->perm, idx_alt, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
     }
     if (t->mass_ready) cudaStreamWaitEvent(s, t->mass_ready, 0);
-    launch_pdl(k_permute, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, d_mass, t->px, t->py, t->pz, t->pm32,
+    launch_pdl(k_permute, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, d_mass, t->io, t->sseg, t->seg_off, t->px, t->py, t->pz, t->pm32,
                                      t->pm64, t->inv, t->mbits, status);
     // a4: nodes from splits.  The node count stays on the device (d_tot[0]
     // counts the first splits, m = B + that): the kernels up to the groups

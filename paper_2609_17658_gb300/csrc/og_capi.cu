@@ -93,6 +93,36 @@ __global__ void k_unpermute(int64_t n, const uint32_t *__restrict__ inv,
     if (npn) npn[j] = npn_s[i];
 }
 
+// k_unpermute into every box's own arrays
+__global__ void k_unpermute_boxes(int64_t n, const uint32_t *__restrict__ inv, const uint32_t *__restrict__ sseg,
+                                  const uint32_t *__restrict__ seg_off, const BoxIO *__restrict__ io,
+                                  const float *__restrict__ acc_sorted, const uint32_t *__restrict__ npp_s,
+                                  const uint32_t *__restrict__ npn_s) {
+    int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const uint32_t i = inv[j];
+    const uint32_t b = sseg[i];
+    const BoxIO x = io[b];
+    const uint64_t k = (uint64_t)j - seg_off[b];
+    x.acc[3 * k + 0] = acc_sorted[i];
+    x.acc[3 * k + 1] = acc_sorted[n + i];
+    x.acc[3 * k + 2] = acc_sorted[2 * n + i];
+    if (x.n_pp) x.n_pp[k] = npp_s[i];
+    if (x.n_pn) x.n_pn[k] = npn_s[i];
+}
+
+// k_gather_aold from every box's own array
+__global__ void k_gather_aold_boxes(int64_t n, const uint32_t *__restrict__ perm, const uint32_t *__restrict__ sseg,
+                                    const uint32_t *__restrict__ seg_off, const BoxIO *__restrict__ io, float *out) {
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t b = sseg[i];
+    const float *a = io[b].a_old + 3ull * (perm[i] - seg_off[b]);
+    out[i] = a[0];
+    out[n + i] = a[1];
+    out[2 * n + i] = a[2];
+}
+
 // FP64 output: the walk's unscaled FP32 sums times G (2^32 / L)^2 in FP64
 __global__ void k_unpermute_f64(int64_t n, const uint32_t *__restrict__ inv,
                                 const float *__restrict__ acc_sorted,
@@ -494,7 +524,10 @@ og_status force_sorted(og_tree *t, const float *d_aold, float *ms_walk_out, cons
     }
     const float *a_old_sorted = nullptr;
     if (t->prm.opening == OG_OPEN_REL) {
-        if (d_aold) {
+        if (t->io && t->io_aold) {
+            k_gather_aold_boxes<<<nblk(n), kT, 0, s>>>(n, t->perm, t->sseg, t->seg_off, t->io, t->a_old_sorted);
+            note_launch();
+        } else if (d_aold) {
             k_gather_aold<<<nblk(n), kT, 0, s>>>(n, t->perm, d_aold, t->a_old_sorted); note_launch();
         } else {
             // first pass: Barnes-Hut with theta_first_pass
@@ -812,8 +845,6 @@ og_status og_batch_force(og_ctx *c, int64_t nbox, const og_box *boxes, og_batch_
     cudaSetDevice(c->device);
     cudaStream_t s = c->stream;
     const bool dev = (p0.flags & OG_DEVICE_PTRS) != 0;
-    const cudaMemcpyKind in_kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    const cudaMemcpyKind out_kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -836,46 +867,74 @@ og_status og_batch_force(og_ctx *c, int64_t nbox, const og_box *boxes, og_batch_
         off += (uint32_t)boxes[b].n;
     }
     t->h_seg_off[nbox] = off;
-    // inputs, concatenated: positions, masses, previous accelerations
+    // inputs.  Device pointers: a table of the boxes' arrays, read and written by
+    // the kernels in place (512 boxes of 3 to 6 arrays each are as many copies of
+    // 2 to 4 us otherwise).  Host pointers: one buffer that holds them all.
     const bool have_aold = p0.opening == OG_OPEN_REL && boxes[0].a_old != nullptr;
-    size_t in_bytes = (size_t)total * 4 * sizeof(double) + (have_aold ? (size_t)total * 3 * sizeof(float) : 0) + 512;
+    const size_t table = ((size_t)nbox * sizeof(BoxIO) + 255) & ~(size_t)255;
+    size_t in_bytes = dev ? table
+                          : (size_t)total * 4 * sizeof(double) + (have_aold ? (size_t)total * 3 * sizeof(float) : 0) + 512;
     void *in = nullptr;
     cudaError_t e;
     if ((e = dev_malloc_async(&in, in_bytes, s)) != cudaSuccess) { delete t; return cuda_fail(e, "cudaMallocAsync (batch inputs)"); }
-    double *d_pos = static_cast<double *>(in);
-    double *d_mass = d_pos + 3 * total;
-    float *d_aold = have_aold ? reinterpret_cast<float *>(d_mass + total) : nullptr;
-    for (int64_t b = 0; b < nbox; ++b) {
-        const int64_t o = t->h_seg_off[b], nb = boxes[b].n;
-        cudaMemcpyAsync(d_pos + 3 * o, boxes[b].pos, (size_t)nb * 3 * sizeof(double), in_kind, s);
-        cudaMemcpyAsync(d_mass + o, boxes[b].mass, (size_t)nb * sizeof(double), in_kind, s);
-        if (have_aold) cudaMemcpyAsync(d_aold + 3 * o, boxes[b].a_old, (size_t)nb * 3 * sizeof(float), in_kind, s);
+    double *d_pos = nullptr, *d_mass = nullptr;
+    float *d_aold = nullptr;
+    std::vector<BoxIO> io;
+    if (dev) {
+        io.resize((size_t)nbox);
+        for (int64_t b = 0; b < nbox; ++b)
+            io[(size_t)b] = {boxes[b].pos, boxes[b].mass, boxes[b].a_old, boxes[b].acc, boxes[b].n_pp, boxes[b].n_pn};
+        cudaMemcpyAsync(in, io.data(), (size_t)nbox * sizeof(BoxIO), cudaMemcpyHostToDevice, s);
+        t->io = static_cast<const BoxIO *>(in);
+        t->io_aold = have_aold;
+        // one box takes the kernels' one-box path, which reads plain arrays
+        if (nbox == 1) {
+            d_pos = const_cast<double *>(boxes[0].pos);
+            d_mass = const_cast<double *>(boxes[0].mass);
+        }
+    } else {
+        d_pos = static_cast<double *>(in);
+        d_mass = d_pos + 3 * total;
+        d_aold = have_aold ? reinterpret_cast<float *>(d_mass + total) : nullptr;
+        for (int64_t b = 0; b < nbox; ++b) {
+            const int64_t o = t->h_seg_off[b], nb = boxes[b].n;
+            cudaMemcpyAsync(d_pos + 3 * o, boxes[b].pos, (size_t)nb * 3 * sizeof(double), cudaMemcpyHostToDevice, s);
+            cudaMemcpyAsync(d_mass + o, boxes[b].mass, (size_t)nb * sizeof(double), cudaMemcpyHostToDevice, s);
+            if (have_aold) cudaMemcpyAsync(d_aold + 3 * o, boxes[b].a_old, (size_t)nb * 3 * sizeof(float), cudaMemcpyHostToDevice, s);
+        }
     }
     og_status st = build_tree(t, d_pos, d_mass);
     if (st == OG_OK) st = check_status(c);
     float ms_walk = 0;
     if (st == OG_OK) st = force_sorted(t, d_aold, &ms_walk);
-    cudaFreeAsync(in, s);
     if (st != OG_OK) {
+        cudaFreeAsync(in, s);
         og_tree_free(t);
         return st;
     }
     // results back to every box in its own order
-    void *out = nullptr;
-    size_t out_bytes = (size_t)total * (3 * sizeof(float) + 2 * sizeof(uint32_t)) + 512;
-    if ((e = dev_malloc_async(&out, out_bytes, s)) != cudaSuccess) { og_tree_free(t); return cuda_fail(e, "cudaMallocAsync (batch outputs)"); }
-    float *o_acc = static_cast<float *>(out);
-    uint32_t *o_pp = reinterpret_cast<uint32_t *>(o_acc + 3 * total);
-    uint32_t *o_pn = o_pp + total;
-    k_unpermute<<<nblk(total), kT, 0, s>>>(total, t->inv, t->a_sorted, t->npp_sorted, t->npn_sorted,
-                                           o_acc, o_pp, o_pn); note_launch();
-    for (int64_t b = 0; b < nbox; ++b) {
-        const int64_t o = t->h_seg_off[b], nb = boxes[b].n;
-        cudaMemcpyAsync(boxes[b].acc, o_acc + 3 * o, (size_t)nb * 3 * sizeof(float), out_kind, s);
-        if (boxes[b].n_pp) cudaMemcpyAsync(boxes[b].n_pp, o_pp + o, (size_t)nb * sizeof(uint32_t), out_kind, s);
-        if (boxes[b].n_pn) cudaMemcpyAsync(boxes[b].n_pn, o_pn + o, (size_t)nb * sizeof(uint32_t), out_kind, s);
+    if (dev) {
+        k_unpermute_boxes<<<nblk(total), kT, 0, s>>>(total, t->inv, t->sseg, t->seg_off, t->io, t->a_sorted,
+                                                     t->npp_sorted, t->npn_sorted); note_launch();
+        cudaFreeAsync(in, s);
+    } else {
+        cudaFreeAsync(in, s);
+        void *out = nullptr;
+        size_t out_bytes = (size_t)total * (3 * sizeof(float) + 2 * sizeof(uint32_t)) + 512;
+        if ((e = dev_malloc_async(&out, out_bytes, s)) != cudaSuccess) { og_tree_free(t); return cuda_fail(e, "cudaMallocAsync (batch outputs)"); }
+        float *o_acc = static_cast<float *>(out);
+        uint32_t *o_pp = reinterpret_cast<uint32_t *>(o_acc + 3 * total);
+        uint32_t *o_pn = o_pp + total;
+        k_unpermute<<<nblk(total), kT, 0, s>>>(total, t->inv, t->a_sorted, t->npp_sorted, t->npn_sorted,
+                                               o_acc, o_pp, o_pn); note_launch();
+        for (int64_t b = 0; b < nbox; ++b) {
+            const int64_t o = t->h_seg_off[b], nb = boxes[b].n;
+            cudaMemcpyAsync(boxes[b].acc, o_acc + 3 * o, (size_t)nb * 3 * sizeof(float), cudaMemcpyDeviceToHost, s);
+            if (boxes[b].n_pp) cudaMemcpyAsync(boxes[b].n_pp, o_pp + o, (size_t)nb * sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+            if (boxes[b].n_pn) cudaMemcpyAsync(boxes[b].n_pn, o_pn + o, (size_t)nb * sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+        }
+        cudaFreeAsync(out, s);
     }
-    cudaFreeAsync(out, s);
     cudaEventRecord(e1, s);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) { og_tree_free(t); return cuda_fail(e, "batch"); }
     float ms = 0;

@@ -58,6 +58,15 @@ struct SegGeom {
     int shift;       // with pow2: x / box * 2^32 == x * 2^shift
 };
 
+// caller's device arrays of one box of a batch: the kernels that read inputs and
+// write results go through this table instead of concatenated copies
+struct BoxIO {
+    const double *pos, *mass;
+    const float *a_old;
+    float *acc;
+    uint32_t *n_pp, *n_pn;
+};
+
 // monopole moments of a node: one 32-byte record, so that a parent reading a
 // child node touches one sector
 struct __align__(32) NodeMom {
@@ -98,6 +107,9 @@ struct og_tree {
     std::vector<og::SegGeom> h_geom;  // geometry of each box (source of an async copy)
     uint32_t *seg_off = nullptr;      // device copy
     og::SegGeom *geom = nullptr;
+    const og::BoxIO *io = nullptr;    // device table of the boxes' own arrays (a batch of device pointers),
+                                      // or null: one array for all particles
+    bool io_aold = false;             // the table has previous accelerations
     og::WalkParams *segp = nullptr;   // per-box walk parameters of the current pass
     uint32_t *sseg = nullptr;         // box of each sorted particle
     uint32_t *gseg = nullptr;         // box of each group
