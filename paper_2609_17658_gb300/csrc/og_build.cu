@@ -26,8 +26,9 @@
 //                           sums over the sorted particles, one pass over the nodes
 //          k_level_hist .. k_level_scatter   node ids bucketed by tree level (a
 //                           refit's extents only, made on the first refit)
-//          k_extents_level  a refit's node extents, one launch per large level
-//          k_extents_run    a run of small levels in one block (a barrier per level)
+//          k_extents_ranges a refit's node extents from ranges of the sorted particles
+//          k_extents_level  the same level by level, for drifts above a quarter of the
+//          k_extents_run    box: a launch per large level, runs of small ones in a block
 //   a6     k_frontier       frontier node, unit and run start mark of every particle
 //          k_groupmark      group starts (then compacted into gbeg by a scan)
 //          k_group_fin      group ends, boxes and box index
@@ -937,16 +938,207 @@ __global__ void k_cell_ext(int64_t m, const uint8_t *__restrict__ nlev, const ui
     }
 }
 
-// refit: drifted fixed-point positions into sorted order (masses unchanged)
+// every third bit of a key, from bit 0
+__device__ __forceinline__ uint32_t gather21(uint64_t x) {
+    x &= 0x1249249249249249ull;
+    x = (x | (x >> 2)) & 0x10c30c30c30c30c3ull;
+    x = (x | (x >> 4)) & 0x100f00f00f00f00full;
+    x = (x | (x >> 8)) & 0x1f0000ff0000ffull;
+    x = (x | (x >> 16)) & 0x1f00000000ffffull;
+    x = (x | (x >> 32)) & 0x1fffffull;
+    return (uint32_t)x;
+}
+
+// A refit's node extents.  A node's extent is its cell joined with its members'
+// positions, as offsets from the cell origin, so it is a minimum and a maximum over
+// a range of the sorted particles.  They come from the particles at the ends of
+// the range and from tiles of 32 and 1024 particles in between, for all nodes at
+// once: joining the children instead takes one dependent launch per tree level
+// (16 us each at 200k particles, 210 us in all; this way 25).
+// A position counts from the key's cell the particle had in the build, X = origin
+// + signed drift, so it does not wrap where it leaves the box; a drift of a
+// quarter of the box or more is left to the level-by-level form.
+constexpr int kTile32 = 32, kTile1024 = 1024;
+struct Tile {
+    long long lo[3], hi[3];
+};
+
+__device__ __forceinline__ long long warp_min(long long v) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const long long o = __shfl_xor_sync(0xffffffffu, v, d);
+        v = o < v ? o : v;
+    }
+    return v;
+}
+__device__ __forceinline__ long long warp_max(long long v) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const long long o = __shfl_xor_sync(0xffffffffu, v, d);
+        v = o > v ? o : v;
+    }
+    return v;
+}
+constexpr long long kNoMin = 1ll << 62, kNoMax = -(1ll << 62);
+
+// refit: drifted fixed-point positions into sorted order (masses unchanged), and
+// the tiles of 32
 __global__ void k_repos(int64_t n, const uint32_t *__restrict__ perm, const uint4 *__restrict__ q4,
-                        uint32_t *px, uint32_t *py, uint32_t *pz) {
+                        const uint64_t *__restrict__ skey, uint32_t *px, uint32_t *py, uint32_t *pz,
+                        Tile *__restrict__ t32, uint32_t *far) {
     pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint4 q = q4[perm[i]];
-    px[i] = q.x;
-    py[i] = q.y;
-    pz[i] = q.z;
+    long long lo[3] = {kNoMin, kNoMin, kNoMin}, hi[3] = {kNoMax, kNoMax, kNoMax};
+    if (i < n) {
+        const uint4 q = q4[perm[i]];
+        px[i] = q.x;
+        py[i] = q.y;
+        pz[i] = q.z;
+        const uint64_t k = skey[i];
+        const uint32_t x[3] = {q.x, q.y, q.z};
+        bool wide = false;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const uint32_t o = gather21(k >> (2 - a)) << 11;
+            const int d = (int)(x[a] - o);
+            wide = wide || d >= (1 << 30) || d <= -(1 << 30);
+            lo[a] = hi[a] = (long long)o + d;
+        }
+        if (wide) atomicOr(far, 1u);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = warp_min(lo[a]);
+        hi[a] = warp_max(hi[a]);
+    }
+    if ((threadIdx.x & 31) == 0 && i < n) {
+        Tile t;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            t.lo[a] = lo[a];
+            t.hi[a] = hi[a];
+        }
+        t32[i >> 5] = t;
+    }
+}
+
+// tiles of 1024 from the tiles of 32, a warp each
+__global__ void k_tiles1024(int64_t n32, const Tile *__restrict__ t32, Tile *__restrict__ t1024) {
+    pdl_wait();
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (32 * w >= n32) return;
+    const int64_t k = 32 * w + lane;
+    Tile t;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        t.lo[a] = warp_min(k < n32 ? t32[k].lo[a] : kNoMin);
+        t.hi[a] = warp_max(k < n32 ? t32[k].hi[a] : kNoMax);
+    }
+    if (lane == 0) t1024[w] = t;
+}
+
+// extent [lo, hi] (offsets from the cell origin o) of a node, stored
+__device__ __forceinline__ void store_extent(uint32_t node, const uint32_t *o, const long long *lo, const long long *hi,
+                                             uint32_t *ext_s, uint32_t *ext_l) {
+    for (int a = 0; a < 3; ++a) {
+        if (hi[a] - lo[a] >= 0xffffffffll) {
+            ext_s[3 * node + a] = 0u;  // the whole circle
+            ext_l[3 * node + a] = 0xffffffffu;
+        } else {
+            ext_s[3 * node + a] = o[a] + (uint32_t)lo[a];
+            ext_l[3 * node + a] = (uint32_t)(hi[a] - lo[a]);
+        }
+    }
+}
+
+// extents of the nodes of level 2 and deeper: up to kThreadNode particles by one
+// thread, more by its warp
+constexpr uint32_t kThreadNode = 48;
+__global__ void __launch_bounds__(kT) k_extents_ranges(int64_t m, const uint8_t *__restrict__ nlev,
+                                                       const uint32_t *__restrict__ nbeg,
+                                                       const uint32_t *__restrict__ nend,
+                                                       const uint32_t *__restrict__ norg,
+                                                       const uint32_t *__restrict__ px,
+                                                       const uint32_t *__restrict__ py,
+                                                       const uint32_t *__restrict__ pz,
+                                                       const Tile *__restrict__ t32, const Tile *__restrict__ t1024,
+                                                       uint32_t *ext_s, uint32_t *ext_l) {
+    pdl_wait();
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int lev = j < m ? nlev[j] : 0;
+    const uint32_t b = lev >= 2 ? nbeg[j] : 0u, e = lev >= 2 ? nend[j] : 0u;
+    auto point = [&](uint32_t q, const uint32_t *o, long long *lo, long long *hi) {
+        const int d[3] = {(int)(px[q] - o[0]), (int)(py[q] - o[1]), (int)(pz[q] - o[2])};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = d[a] < lo[a] ? d[a] : lo[a];
+            hi[a] = d[a] > hi[a] ? d[a] : hi[a];
+        }
+    };
+    if (lev >= 2 && e - b <= kThreadNode) {
+        const uint32_t o[3] = {norg[3 * j], norg[3 * j + 1], norg[3 * j + 2]};
+        const long long side = 1ll << (32 - lev);
+        long long lo[3] = {0, 0, 0}, hi[3] = {side - 1, side - 1, side - 1};
+        for (uint32_t q = b; q < e; ++q) point(q, o, lo, hi);
+        store_extent((uint32_t)j, o, lo, hi, ext_s, ext_l);
+    }
+    for (unsigned todo = __ballot_sync(0xffffffffu, lev >= 2 && e - b > kThreadNode); todo; todo &= todo - 1u) {
+        const int src = __ffs((int)todo) - 1;
+        const uint32_t node = (uint32_t)(j - lane + src);
+        const uint32_t b0 = __shfl_sync(0xffffffffu, b, src), e0 = __shfl_sync(0xffffffffu, e, src);
+        const int L = __shfl_sync(0xffffffffu, lev, src);
+        const uint32_t o[3] = {norg[3 * node], norg[3 * node + 1], norg[3 * node + 2]};
+        const long long side = 1ll << (32 - L);
+        long long lo[3] = {0, 0, 0}, hi[3] = {side - 1, side - 1, side - 1};
+        // [b0, e0) = particles, tiles of 32 [p, q), tiles of 1024 [r, s) inside them
+        const uint32_t p = (b0 + 31u) / 32u, q = e0 / 32u;
+        auto tile = [&](const Tile &t) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const long long l = t.lo[a] - (long long)o[a], h = t.hi[a] - (long long)o[a];
+                lo[a] = l < lo[a] ? l : lo[a];
+                hi[a] = h > hi[a] ? h : hi[a];
+            }
+        };
+        if (b0 + lane < 32u * p) point(b0 + lane, o, lo, hi);
+        if (32u * q + lane < e0) point(32u * q + lane, o, lo, hi);
+        const uint32_t r = (p + 31u) / 32u, s = q / 32u;
+        if (r < s) {
+            if (p + lane < 32u * r) tile(t32[p + lane]);
+            if (32u * s + lane < q) tile(t32[32u * s + lane]);
+            for (uint32_t k = r + (uint32_t)lane; k < s; k += 32u) tile(t1024[k]);
+        } else {
+            for (uint32_t k = p + (uint32_t)lane; k < q; k += 32u) tile(t32[k]);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = warp_min(lo[a]);
+            hi[a] = warp_max(hi[a]);
+        }
+        if (lane == 0) store_extent(node, o, lo, hi, ext_s, ext_l);
+    }
+}
+
+// levels 1 and 0, where an offset may not fit 32 bits and takes the joined form:
+// a block per box, its nodes of level 1 and then the root
+__global__ void k_extents_top(int64_t n, const uint8_t *__restrict__ nlev, const uint32_t *__restrict__ nbeg,
+                              const uint32_t *__restrict__ nend, const uint32_t *__restrict__ ncbeg,
+                              const uint32_t *__restrict__ nccnt, const uint32_t *__restrict__ occ,
+                              const uint32_t *__restrict__ child, const uint32_t *__restrict__ px,
+                              const uint32_t *__restrict__ py, const uint32_t *__restrict__ pz, int64_t nchild,
+                              const uint32_t *__restrict__ norg, uint32_t *ext_s, uint32_t *ext_l) {
+    pdl_wait();
+    const uint32_t root = blockIdx.x;
+    const uint32_t slot = ncbeg[root] + threadIdx.x;
+    if (threadIdx.x < nccnt[root] && slot < (uint64_t)nchild && child[slot] >= n) {
+        const uint32_t j = (uint32_t)(child[slot] - n);
+        if (nlev[j] == 1) extent_node(n, nbeg, nend, ncbeg, occ, child, px, py, pz, nchild, norg, ext_s, ext_l, j, 1);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        extent_node(n, nbeg, nend, ncbeg, occ, child, px, py, pz, nchild, norg, ext_s, ext_l, root, 0);
 }
 
 // the walk's child records; the child count is *d_nchild (the build) or
@@ -1167,7 +1359,9 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
     }
     ensure_origins(t);   // from the build's positions, before k_repos moves them
     const size_t mom_bytes = moments_scratch_bytes(n);
-    size_t sb = (size_t)n * (16 + 8 + 4 + 4) + 4096 + mom_bytes + 4 * (kLevels + 3) * sizeof(uint32_t) + 256;
+    const int64_t n32 = (n + 31) / 32, n1024 = (n32 + 31) / 32;
+    size_t sb = (size_t)n * (16 + 8 + 4 + 4) + 4096 + mom_bytes + 4 * (kLevels + 3) * sizeof(uint32_t) + 256 +
+                (size_t)(n32 + n1024) * sizeof(Tile) + 1024;
     void *scratch = nullptr;
     if ((err = dev_malloc_async(&scratch, sb, s)) != cudaSuccess) return cuda_fail(err, "cudaMallocAsync (refit)");
     Bump W(scratch, sb);
@@ -1177,11 +1371,8 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
     uint32_t *pseg = W.take<uint32_t>(n);
     uint32_t *lcount = W.take<uint32_t>(4 * (kLevels + 3));
     void *mom_scratch = W.take<char>((int64_t)mom_bytes);
-    og_status st = level_lists(t, lcount);
-    if (st) {
-        cudaFreeAsync(scratch, s);
-        return st;
-    }
+    Tile *t32 = W.take<Tile>(n32), *t1024 = W.take<Tile>(n1024);
+    uint32_t *far = W.take<uint32_t>(1);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -1190,9 +1381,14 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
                                            (const BoxIO *)nullptr, t->geom, q4,
                                            keys, nullptr, idx, nullptr, nullptr, nullptr, nullptr, (int64_t)0,
                                            t->ctx->d_status);
-    launch_pdl(k_repos, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, t->px, t->py, t->pz);
+    cudaMemsetAsync(far, 0, sizeof(uint32_t), s);
+    launch_pdl(k_repos, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, t->skey, t->px, t->py, t->pz, t32, far);
+    launch_pdl(k_tiles1024, nblk(32 * n1024), kT, 0, s, n32, (const Tile *)t32, t1024);
+    launch_pdl(k_extents_ranges, nblk(t->nnodes), kT, 0, s, t->nnodes, t->nlev, t->nbeg, t->nend, t->norg, t->px,
+               t->py, t->pz, (const Tile *)t32, (const Tile *)t1024, t->next_s, t->next_l);
+    launch_pdl(k_extents_top, dim3((unsigned)B), 32, 0, s, n, t->nlev, t->nbeg, t->nend, t->ncbeg, t->nccnt, t->nocc,
+               t->child, t->px, t->py, t->pz, t->nchild, t->norg, t->next_s, t->next_l);
     node_moments(t, nullptr, t->nnodes, mom_scratch, s);
-    extents_bottom_up(t, t->next_s, t->next_l);
     launch_pdl(k_group_fin, stride_grid(t->ngroups), kT, 0, s, n, nullptr, t->ngroups, t->gbeg, t->gend, t->px,
                                                        t->py, t->pz, t->sseg, t->gbox, t->gseg);
     launch_pdl(k_records, stride_grid(t->nchild), kT, 0, s, n, nullptr, t->nchild, t->nchild, t->child, t->px,
@@ -1200,9 +1396,30 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
                                                     t->nccnt, t->nmom, t->ncom, t->crec, t->ctx->d_status);
     launch_pdl(k_ext_records, nblk(t->nchild), kT, 0, s, n, t->nchild, t->child, t->next_s, t->next_l,
                                                  t->cext);
+    uint32_t *h_far = pinned_counts(t->ctx);
+    cudaMemcpyAsync(h_far, far, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
     cudaEventRecord(e1, s);
+    err = cudaStreamSynchronize(s);
+    if (err == cudaSuccess && *h_far) {
+        // a drift of a quarter of the box or more: the extents level by level
+        og_status st = level_lists(t, lcount);
+        if (st) {
+            cudaFreeAsync(scratch, s);
+            cudaEventDestroy(e0);
+            cudaEventDestroy(e1);
+            return st;
+        }
+        extents_bottom_up(t, t->next_s, t->next_l);
+        launch_pdl(k_ext_records, nblk(t->nchild), kT, 0, s, n, t->nchild, t->child, t->next_s, t->next_l, t->cext);
+        cudaEventRecord(e1, s);
+        err = cudaStreamSynchronize(s);
+    }
     cudaFreeAsync(scratch, s);
-    if ((err = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(err, "refit");
+    if (err != cudaSuccess) {
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        return cuda_fail(err, "refit");
+    }
     float ms = 0;
     cudaEventElapsedTime(&ms, e0, e1);
     t->ms_refit = ms;
