@@ -477,73 +477,6 @@ __device__ __forceinline__ bool open_exact(const uint4 &c, const Box &b, double 
     return __dmul_rn(__dmul_rn(p.G, M), l2) > __dmul_rn(arel, __dmul_rn(d2, d2));
 }
 
-// The short form, for a group whose box sides are in [1, 2^29) grid units and
-// whose prune distance is below 2^29: signed differences to the near and far
-// sides, no wrap to tell apart, and one straight line for particles and nodes,
-// so that the two records of a lane overlap.  About 60 instructions a record,
-// where the interval form below takes about 100 in two divergent branches.
-//
-// With a = lo - c and b = c - hi (signed), the gap of c is max(a, b, 0).  It
-// differs from the gap on the circle only where both a and b are positive,
-// i.e. for a c within len of the far side of the circle, where it takes the larger
-// one; both are above 2^31 - 2^29 there (and with len >= 1 they are never both
-// -2^31).  A particle or a cell (half side
-// s2 <= 2^30) there is beyond the prune distance either way.  The centre of mass
-// of a cell that is not pruned is at most 2 s2 further, so it can be there
-// only for a node of level 1; those take the exact branch.
-//
-// A cell's centre is c = (COM with the low 32 - lev bits cleared) + s2 and its
-// gap max(a + 1 - s2, b - s2, 0) = max(max(b - 1, a) - (s2 - 1), 0), as it spans
-// [c - s2, c + s2 - 1].  The level of a particle reads as 32 or more: s2 = 0, and
-// without the ones the cell is the point itself.
-// Boundary check: the box meets the cell enlarged to 0.6 side, max(a, b) <=
-// floor(6 s2 / 5) on every axis; 6/5 = 1.0011 0011..., so for s2 = 2^(31 - lev)
-// that is 0x99999999 >> lev.
-template <int kOpen>
-__device__ __forceinline__ Cls classify_short(const TreeView &T, uint32_t ci, bool has, const Box &b,
-                                              const WalkParams &p, float arelf, double arel) {
-    const uint4 *rec = reinterpret_cast<const uint4 *>(T.crec + (has ? ci : 0u));
-    const uint4 q0 = rec[0], q1 = rec[1];
-    const uint32_t info = q1.z, lev = info >> 26;
-    const bool isnode = (int)info >= 0;
-    const int isn = isnode ? 1 : 0;
-    const uint32_t mask = shr(0xffffffffu, lev), s2 = shr(0x80000000u, lev), blim = shr(0x99999999u, lev);
-    unsigned long long g2 = 0ull;
-    int dc;
-    uint32_t g[3];
-    const uint32_t c[3] = {q0.x, q0.y, q0.z};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const uint32_t cc = (c[k] & ~mask) | s2;
-        const int a = (int)(b.lo[k] - cc), d = (int)(cc - b.hi[k]);
-        dc = k == 0 ? max(a, d) : __vimax3_s32(dc, a, d);
-        const uint32_t cg = (uint32_t)__viaddmax_s32_relu(__viaddmax_s32(d, -isn, a), isn - (int)s2, 0);
-        g2 += sq64(cg);
-        g[k] = (uint32_t)__vimax_s32_relu((int)(b.lo[k] - c[k]), (int)(c[k] - b.hi[k]));
-    }
-    float d2f = dist2f(g[0], g[1], g[2]);
-    const bool keep = has && g2 <= p.rprune;
-    const bool bnear = dc <= (int)blim;
-    const float l2f = __uint_as_float(0x5f800000u - (lev << 24));   // 2^(64 - 2 lev)
-    bool op, sure;
-    if (kOpen == OG_OPEN_BH) {
-        const float q = p.th2f * d2f, t = l2f - q;
-        op = t > 0.0f;
-        sure = fabsf(t) > q * kFilterEps;
-    } else {
-        const float lhs = (p.Gf * __uint_as_float(q0.w)) * l2f, rhs = (arelf * d2f) * d2f, t = lhs - rhs;
-        op = t > 0.0f;
-        sure = fabsf(t) > rhs * kFilterEps && fminf(lhs, rhs) >= 1e-30f && fmaxf(lhs, rhs) <= 1e30f;
-    }
-    if (__builtin_expect(keep && isnode && !bnear && (!sure || lev == 1u), 0)) {
-        const double l2 = __longlong_as_double((long long)(1023 + 64 - 2 * lev) << 52);
-        op = open_exact<kOpen>(q0, b, l2, __hiloint2double((int)q1.y, (int)q1.x), arel, p, d2f);
-    }
-    const bool open = keep && isnode && (bnear || op);
-    // near: in single precision with a margin above its error
-    return Cls{keep && !open, open, isnode, !(d2f >= p.hnear2f), q0, q1.w, info & 0x3ffffffu};
-}
-
 // The general form: intervals on the circle, any box, node extents after a refit.
 template <int kOpen, bool kSplit, bool kRefit>
 __device__ __forceinline__ Cls classify(const TreeView &T, uint32_t ci, bool has, const Box &b,
@@ -627,6 +560,107 @@ __device__ __forceinline__ Cls classify(const TreeView &T, uint32_t ci, bool has
     return Cls{emit, open, isnode, near, ent, push_ref, push_cnt};
 }
 
+// The short form, for a group whose box sides are in [1, 2^29) grid units and
+// whose prune distance is below 2^29: signed differences to the near and far
+// sides, no wrap to tell apart, and one straight line for particles and nodes,
+// so that the two records of a lane overlap.  About 60 instructions a record,
+// where the interval form below takes about 100 in two divergent branches.
+//
+// With a = lo - c and b = c - hi (signed), the gap of c is max(a, b, 0).  It
+// differs from the gap on the circle only where both a and b are positive,
+// i.e. for a c within len of the far side of the circle, where it takes the larger
+// one; both are above 2^31 - 2^29 there (and with len >= 1 they are never both
+// -2^31).  A particle or a cell (half side
+// s2 <= 2^30) there is beyond the prune distance either way.  The centre of mass
+// of a cell that is not pruned is at most 2 s2 further, so it can be there
+// only for a node of level 1; those take the exact branch.
+//
+// A cell's centre is c = (COM with the low 32 - lev bits cleared) + s2 and its
+// gap max(a + 1 - s2, b - s2, 0) = max(max(b - 1, a) - (s2 - 1), 0), as it spans
+// [c - s2, c + s2 - 1].  The level of a particle reads as 32 or more: s2 = 0, and
+// without the ones the cell is the point itself.
+// Boundary check: the box meets the cell enlarged to 0.6 side, max(a, b) <=
+// floor(6 s2 / 5) on every axis; 6/5 = 1.0011 0011..., so for s2 = 2^(31 - lev)
+// that is 0x99999999 >> lev.
+//
+// After a refit (kRefit) a node spans its extent [s, s + l] instead, and the gap is
+// max(lo - (s + l), s - hi, 0); an extent of 2^30 or more on some axis takes the
+// general form.  The centre of mass of members on either side of the box's face is
+// the plain mean of their coordinates, far outside the extent, so its gap is taken
+// on the circle.  200k particles, Barnes-Hut: 384 -> 345 us.
+template <int kOpen, bool kSplit, bool kRefit>
+__device__ __forceinline__ Cls classify_short(const TreeView &T, uint32_t ci, bool has, const Box &b,
+                                              const WalkParams &p, float arelf, double arel) {
+    const uint4 *rec = reinterpret_cast<const uint4 *>(T.crec + (has ? ci : 0u));
+    const uint4 q0 = rec[0], q1 = rec[1];
+    const uint32_t info = q1.z, lev = info >> 26;
+    const bool isnode = (int)info >= 0;
+    unsigned long long g2 = 0ull;
+    int dc;
+    uint32_t g[3], blim, side = 0u;
+    bool odd;                  // a node that the short form does not cover
+    float l2f;
+    const uint32_t c[3] = {q0.x, q0.y, q0.z};
+    if (kRefit) {
+        const uint4 *ext = reinterpret_cast<const uint4 *>(T.cext + (has ? ci : 0u));
+        const uint4 x0 = ext[0], x1 = ext[1];
+        const uint32_t es[3] = {x0.x, x0.y, x0.z}, el[3] = {x1.x, x1.y, x1.z};   // zeros for a particle
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t s = isnode ? es[k] : c[k], cc = s + ((el[k] + 1u) >> 1);
+            const int a = (int)(b.lo[k] - cc), d = (int)(cc - b.hi[k]);
+            dc = k == 0 ? max(a, d) : __vimax3_s32(dc, a, d);
+            g2 += sq64((uint32_t)__vimax_s32_relu((int)(b.lo[k] - (s + el[k])), (int)(s - b.hi[k])));
+            g[k] = point_gap(c[k], b.lo[k], b.hi[k] - b.lo[k]);
+        }
+        side = max(el[0], max(el[1], el[2])) + 1u;
+        odd = side - 1u >= (1u << 30);
+        blim = __umulhi(3u * side, 0xCCCCCCCDu) >> 2;   // floor(3 ell / 5)
+        const float ell = (float)side;
+        l2f = ell * ell;
+    } else {
+        const int isn = isnode ? 1 : 0;
+        const uint32_t mask = shr(0xffffffffu, lev), s2 = shr(0x80000000u, lev);
+        blim = shr(0x99999999u, lev);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t cc = (c[k] & ~mask) | s2;
+            const int a = (int)(b.lo[k] - cc), d = (int)(cc - b.hi[k]);
+            dc = k == 0 ? max(a, d) : __vimax3_s32(dc, a, d);
+            const uint32_t cg = (uint32_t)__viaddmax_s32_relu(__viaddmax_s32(d, -isn, a), isn - (int)s2, 0);
+            g2 += sq64(cg);
+            g[k] = (uint32_t)__vimax_s32_relu((int)(b.lo[k] - c[k]), (int)(c[k] - b.hi[k]));
+        }
+        odd = lev == 1u;
+        l2f = __uint_as_float(0x5f800000u - (lev << 24));   // 2^(64 - 2 lev)
+    }
+    float d2f = dist2f(g[0], g[1], g[2]);
+    const bool keep = has && g2 <= p.rprune;
+    const bool bnear = dc <= (int)blim;
+    bool op, sure;
+    if (kOpen == OG_OPEN_BH) {
+        const float q = p.th2f * d2f, t = l2f - q;
+        op = t > 0.0f;
+        sure = fabsf(t) > q * kFilterEps;
+    } else {
+        const float lhs = (p.Gf * __uint_as_float(q0.w)) * l2f, rhs = (arelf * d2f) * d2f, t = lhs - rhs;
+        op = t > 0.0f;
+        sure = fabsf(t) > rhs * kFilterEps && fminf(lhs, rhs) >= 1e-30f && fmaxf(lhs, rhs) <= 1e30f;
+    }
+    if (kRefit) {
+        if (__builtin_expect(has && isnode && odd, 0))
+            return classify<kOpen, kSplit, kRefit>(T, ci, has, b, p, arelf, arel);
+    }
+    if (__builtin_expect(keep && isnode && !bnear && (!sure || (!kRefit && odd)), 0)) {
+        const double l2 = kRefit ? (double)side * (double)side
+                                 : __longlong_as_double((long long)(1023 + 64 - 2 * lev) << 52);
+        op = open_exact<kOpen>(q0, b, l2, __hiloint2double((int)q1.y, (int)q1.x), arel, p, d2f);
+    }
+    const bool open = keep && isnode && (bnear || op);
+    // near: in single precision with a margin above its error
+    return Cls{keep && !open, open, isnode, !(d2f >= p.hnear2f), q0, q1.w, info & 0x3ffffffu};
+}
+
 // kOneSeg: a single tree of one box, whose parameters come from the launch
 // argument (constant operands) instead of a per-box record in global memory.
 // Registers: at most 96 per thread (64 KB / (96 x 128) gives 5 blocks of 4
@@ -698,7 +732,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             box.hi[k] = T.gbox[6 * g + 3 + k];
         }
         // the short form of the tests (see classify_short)
-        bool compact = kSplit && !kRefit && p.rprune < (1ull << 58);
+        bool compact = kSplit && p.rprune < (1ull << 58);
 #pragma unroll
         for (int k = 0; k < 3; ++k) compact = compact && box.hi[k] - box.lo[k] - 1u < (1u << 29) - 1u;
         // Lane -> (target pair, replica): P lanes hold the group's targets, two
@@ -801,9 +835,9 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             // results merged after a branch cost more than the tests)
             auto take = [&](auto form) {
                 constexpr bool kShort = decltype(form)::value;
-                const Cls c0 = kShort ? classify_short<kOpen>(T, ci0, has0, box, p, arelf, arel)
+                const Cls c0 = kShort ? classify_short<kOpen, kSplit, kRefit>(T, ci0, has0, box, p, arelf, arel)
                                       : classify<kOpen, kSplit, kRefit>(T, ci0, has0, box, p, arelf, arel);
-                const Cls c1 = kShort ? classify_short<kOpen>(T, ci1, has1, box, p, arelf, arel)
+                const Cls c1 = kShort ? classify_short<kOpen, kSplit, kRefit>(T, ci1, has1, box, p, arelf, arel)
                                       : classify<kOpen, kSplit, kRefit>(T, ci1, has1, box, p, arelf, arel);
                 // push opened ranges (k_records has checked that every node has
                 // children, inside the child array)
@@ -848,7 +882,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 return true;
             };
             bool ok;
-            if (kSplit && !kRefit && __builtin_expect(compact, 1)) ok = take(std::integral_constant<bool, true>{});
+            if (kSplit && __builtin_expect(compact, 1)) ok = take(std::integral_constant<bool, true>{});
             else ok = take(std::integral_constant<bool, false>{});
             if (!ok) {
                 overflow = true;

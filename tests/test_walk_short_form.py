@@ -87,6 +87,37 @@ def test_short_form_takes_the_interval_form_decisions(seed):
     assert com_equal[keep & particle].all()
 
 
+@pytest.mark.parametrize("seed", range(4))
+def test_short_form_of_refitted_extents(seed):
+    rng = np.random.default_rng(100 + seed)
+    n = 200_000
+    length = np.clip((rng.random((3, n)) * 2.0 ** rng.integers(0, 30, (3, n))).astype(np.int64), 1, 2 ** 29 - 1)
+    ext = np.minimum((rng.random((3, n)) * 2.0 ** rng.integers(0, 31, (3, n))).astype(np.int64), 2 ** 30 - 1)
+    lo = rng.integers(0, M, (3, n))
+    hi = (lo + length) % M
+    edge = rng.integers(-3, 4, (3, n))
+    off = np.choose(rng.integers(0, 4, (3, n)),
+                    [rng.integers(0, M, (3, n)), length + edge, edge - ext, 2 ** 31 + edge + length * rng.integers(0, 2, (3, n))])
+    s = (lo + off) % M
+    side = ext.max(axis=0) + 1
+    blim = 3 * side // 5
+    assert np.array_equal(((3 * side) * 0xCCCCCCCD >> 32) >> 2, blim)
+    rprune = ((2.0 ** rng.uniform(10, 28.99, n)) ** 2).astype(np.int64)
+    cap = 2 ** 30
+    g2, e2 = np.zeros(n, np.int64), np.zeros(n, np.int64)
+    dc, near = np.full(n, -2 ** 40), np.ones(n, bool)
+    for k in range(3):
+        gap = np.maximum(np.maximum(_s32(lo[k] - (s[k] + ext[k])), _s32(s[k] - hi[k])), 0)
+        g2 += np.minimum(gap, cap) ** 2
+        e2 += np.minimum(_box_gap(lo[k], length[k], s[k], ext[k]), cap) ** 2
+        cc = (s[k] + (ext[k] + 1 >> 1)) % M
+        dc = np.maximum(dc, np.maximum(_s32(lo[k] - cc), _s32(cc - hi[k])))
+        near &= _point_gap(cc, lo[k], length[k]) <= blim
+    keep = e2 <= rprune
+    assert np.array_equal(g2 <= rprune, keep)
+    assert np.array_equal((dc <= blim)[keep], near[keep])
+
+
 @pytest.fixture(scope="module")
 def ctx():
     B.build()
