@@ -101,7 +101,8 @@ def test_short_form_of_refitted_extents(seed):
     s = (lo + off) % M
     side = ext.max(axis=0) + 1
     blim = 3 * side // 5
-    assert np.array_equal(((3 * side) * 0xCCCCCCCD >> 32) >> 2, blim)
+    high = ((3 * side).astype(np.uint64) * np.uint64(0xCCCCCCCD)) >> np.uint64(32)
+    assert np.array_equal((high >> np.uint64(2)).astype(np.int64), blim)
     rprune = ((2.0 ** rng.uniform(10, 28.99, n)) ** 2).astype(np.int64)
     cap = 2 ** 30
     g2, e2 = np.zeros(n, np.int64), np.zeros(n, np.int64)
