@@ -140,7 +140,11 @@ __device__ __forceinline__ float fix_scale(double mtot) {
 // base point, the key's top 3 log2 Ng bits) are contiguous.  Each warp sums the
 // contributions of every such run with a segmented suffix sum (integers: the
 // order does not change the result) and the run's first lane adds the 8 sums,
-// so a dense cell costs 8 atomics per warp instead of 8 per particle.
+// so a dense cell costs 8 atomics per warp instead of 8 per particle.  The sum
+// takes only the steps the warp's longest run needs (none where every particle
+// has a cell of its own).  62 us for 2.1M clustered particles on 256^3 points:
+// the conversions to 64 bits and the shuffles take half of the issue slots,
+// the rest waits for the atomics.
 __global__ void k_pm_deposit(int64_t n, int shift, int ng, const uint32_t *__restrict__ px,
                              const uint32_t *__restrict__ py, const uint32_t *__restrict__ pz,
                              const float *__restrict__ pm32, const NodeMom *__restrict__ root,
@@ -162,6 +166,7 @@ __global__ void k_pm_deposit(int64_t n, int shift, int ng, const uint32_t *__res
     const unsigned heads = __ballot_sync(0xffffffffu, head);
     const unsigned later = lane == 31 ? 0u : heads & (0xfffffffeu << lane);
     const unsigned end = later ? (unsigned)__ffs(later) - 2u : 31u;   // last lane of this run
+    const unsigned reach = __reduce_max_sync(0xffffffffu, end - lane);   // the longest run's span
     const float wx[2] = {1.0f - fx, fx}, wy[2] = {1.0f - fy, fy}, wz[2] = {1.0f - fz, fz};
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
@@ -174,8 +179,7 @@ __global__ void k_pm_deposit(int64_t n, int shift, int ng, const uint32_t *__res
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 unsigned long long v = __float2ull_rn(mab * wz[c]);
-#pragma unroll
-                for (unsigned d = 1; d < 32; d <<= 1) {
+                for (unsigned d = 1; d <= reach; d <<= 1) {
                     const unsigned long long u = __shfl_down_sync(0xffffffffu, v, d);
                     if (lane + d <= end) v += u;
                 }
@@ -185,33 +189,50 @@ __global__ void k_pm_deposit(int64_t n, int shift, int ng, const uint32_t *__res
     }
 }
 
-// density in units of the fixed point -> FP32 (the Green's factor carries the rest)
+// density in units of the fixed point -> FP32 (the Green's factor carries the rest).
+// Bound by memory: four points a thread in vectors (a mesh has at least 8), 30 us
+// for 256^3 points against 48 with one; 201 MB, part of them still in L2.
 __global__ void k_pm_density(int64_t cells, const unsigned long long *__restrict__ fix,
                              float *__restrict__ rho) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= cells) return;
-    rho[i] = __ull2float_rn(fix[i]);
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(fix + i);
+    const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(fix + i + 2);
+    *reinterpret_cast<float4 *>(rho + i) = make_float4(__ull2float_rn(a.x), __ull2float_rn(a.y),
+                                                       __ull2float_rn(b.x), __ull2float_rn(b.y));
 }
 
-// tab[n] = (k_n^2, exp(-k_n^2 r_s^2) / sinc^4(k_n D / 2)) for the full-axis index n
+// tab[n] = (k_n^2, exp(-k_n^2 r_s^2) / sinc^4(k_n D / 2)) for the full-axis index n.
+// A warp per row of modes, the row's factors held by every lane: the index needs no
+// division per mode and a lane has four modes in flight.  135 MB for 256^3
+// points; 30 us against 37 with a thread per mode and two 64-bit divisions.
 __global__ void k_pm_green(int ng, int nzh, const float2 *__restrict__ tab, float cfac,
                            float2 *__restrict__ rk) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t total = (int64_t)ng * ng * nzh;
-    if (idx >= total) return;
-    const int iz = (int)(idx % nzh);
-    const int64_t r = idx / nzh;
-    const int iy = (int)(r % ng), ix = (int)(r / ng);
-    const float2 tx = tab[ix], ty = tab[iy], tz = tab[iz];
-    const float k2 = (tx.x + ty.x) + tz.x;
-    float g = 0.0f;
-    if (idx != 0) g = cfac * ((tx.y * ty.y) * tz.y) / k2;
-    float2 v = rk[idx];
-    v.x *= g;
-    v.y *= g;
-    rk[idx] = v;
+    const int row = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (row >= ng * ng) return;
+    const int ix = row / ng, iy = row & (ng - 1);
+    const float2 tx = tab[ix], ty = tab[iy];
+    const float kxy = tx.x + ty.x, wxy = tx.y * ty.y;
+    float2 *r = rk + (size_t)row * nzh;
+#pragma unroll 4
+    for (int iz = threadIdx.x & 31; iz < nzh; iz += 32) {
+        const float2 tz = tab[iz];
+        const float k2 = kxy + tz.x;
+        float g = 0.0f;
+        if (row + iz != 0) g = cfac * (wxy * tz.y) / k2;
+        float2 v = r[iz];
+        v.x *= g;
+        v.y *= g;
+        r[iz] = v;
+    }
 }
 
+// 56 mesh values a particle: the cell's 8 points, shared by the axes, and per axis
+// four more on each of 4 rows.  Bound by the latency of these gathers and by the
+// first-level cache (58 % of its wavefronts, 77 % hits): 86 us for 2.1M clustered
+// particles on 256^3 points, 95 with the stencil's 96 values each addressed by
+// itself.  Smaller blocks and more resident warps (fewer registers) measured the same
+// or slower.
 __global__ void k_pm_interp(int64_t n, int shift, int ng, const uint32_t *__restrict__ px,
                             const uint32_t *__restrict__ py, const uint32_t *__restrict__ pz,
                             const uint32_t *__restrict__ perm, const float *__restrict__ phi,
@@ -226,25 +247,44 @@ __global__ void k_pm_interp(int64_t n, int shift, int ng, const uint32_t *__rest
     const int ix = (int)(qx >> shift), iy = (int)(qy >> shift), iz = (int)(qz >> shift);
     const float fx = frac_of(qx, shift), fy = frac_of(qy, shift), fz = frac_of(qz, shift);
     const float wx[2] = {1.0f - fx, fx}, wy[2] = {1.0f - fy, fy}, wz[2] = {1.0f - fz, fz};
-    auto at = [&](int x, int y, int z) -> float {
-        return __ldg(&phi[((size_t)(x & m1) * ng + (size_t)(y & m1)) * ng + (size_t)(z & m1)]);
-    };
+    uint32_t X[6], Y[6], Z[6];   // mesh offsets of the stencil's six points on each axis
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        X[k] = (uint32_t)((ix + k - 2) & m1) * (uint32_t)(ng * ng);
+        Y[k] = (uint32_t)((iy + k - 2) & m1) * (uint32_t)ng;
+        Z[k] = (uint32_t)((iz + k - 2) & m1);
+    }
+    // central difference at the row's points 2 and 3
+    auto grad = [](float r0, float r1, float r3, float r4) { return 8.0f * (r3 - r1) - (r4 - r0); };
+    float c[2][2][2];            // the 8 points of the cell, shared by the three axes
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int d = 0; d < 2; ++d) c[a][b][d] = __ldg(&phi[X[2 + a] + Y[2 + b] + Z[2 + d]]);
     float ax = 0.0f, ay = 0.0f, az = 0.0f;
 #pragma unroll
-    for (int a = 0; a < 2; ++a) {
+    for (int u = 0; u < 2; ++u) {
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
+        for (int v = 0; v < 2; ++v) {
+            float r[6];
+            const uint32_t bx = Y[2 + u] + Z[2 + v], by = X[2 + u] + Z[2 + v], bz = X[2 + u] + Y[2 + v];
+            r[2] = c[0][u][v]; r[3] = c[1][u][v];
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int x = ix + a, y = iy + b, z = iz + c;
-                const float w = (wx[a] * wy[b]) * wz[c];
-                const float gx = 8.0f * (at(x + 1, y, z) - at(x - 1, y, z)) - (at(x + 2, y, z) - at(x - 2, y, z));
-                const float gy = 8.0f * (at(x, y + 1, z) - at(x, y - 1, z)) - (at(x, y + 2, z) - at(x, y - 2, z));
-                const float gz = 8.0f * (at(x, y, z + 1) - at(x, y, z - 1)) - (at(x, y, z + 2) - at(x, y, z - 2));
-                ax = fmaf(w, gx, ax);
-                ay = fmaf(w, gy, ay);
-                az = fmaf(w, gz, az);
-            }
+            for (int k : {0, 1, 4, 5}) r[k] = __ldg(&phi[X[k] + bx]);
+            ax = fmaf((wx[0] * wy[u]) * wz[v], grad(r[0], r[1], r[3], r[4]), ax);
+            ax = fmaf((wx[1] * wy[u]) * wz[v], grad(r[1], r[2], r[4], r[5]), ax);
+            r[2] = c[u][0][v]; r[3] = c[u][1][v];
+#pragma unroll
+            for (int k : {0, 1, 4, 5}) r[k] = __ldg(&phi[Y[k] + by]);
+            ay = fmaf((wx[u] * wy[0]) * wz[v], grad(r[0], r[1], r[3], r[4]), ay);
+            ay = fmaf((wx[u] * wy[1]) * wz[v], grad(r[1], r[2], r[4], r[5]), ay);
+            r[2] = c[u][v][0]; r[3] = c[u][v][1];
+#pragma unroll
+            for (int k : {0, 1, 4, 5}) r[k] = __ldg(&phi[Z[k] + bz]);
+            az = fmaf((wx[u] * wy[v]) * wz[0], grad(r[0], r[1], r[3], r[4]), az);
+            az = fmaf((wx[u] * wy[v]) * wz[1], grad(r[1], r[2], r[4], r[5]), az);
         }
     }
     const size_t o = 3 * (size_t)perm[i];
@@ -296,17 +336,7 @@ extern "C" og_status og_tree_pm_force(og_tree *t, int32_t mesh, float *acc) {
     og_status st = plans_for(c, ng, &plans);
     if (st) return st;
     const CufftApi *api = cufft_api();
-    // per-axis table: k_n^2 and exp(-k_n^2 r_s^2) / sinc^4(k_n D / 2), FP64 on the host
     const double L = p.box, D = L / ng, rs = p.r_s;
-    std::vector<float2> h_tab(ng);
-    for (int i = 0; i < ng; ++i) {
-        const int nsig = i < ng / 2 ? i : i - ng;
-        const double k = 2.0 * M_PI * nsig / L;
-        const double x = 0.5 * k * D;
-        const double sinc = nsig == 0 ? 1.0 : std::sin(x) / x;
-        const double s2 = sinc * sinc;
-        h_tab[i] = make_float2((float)(k * k), (float)(std::exp(-k * k * rs * rs) / (s2 * s2)));
-    }
     // buffers: fixed-point mesh (8 B/point), real mesh (4 B/point, density then
     // potential), modes (8 B/mode), the table
     const size_t b_fix = (size_t)cells * 8, b_real = (size_t)cells * 4, b_modes = (size_t)modes * 8;
@@ -336,19 +366,30 @@ extern "C" og_status og_tree_pm_force(og_tree *t, int32_t mesh, float *acc) {
     float2 *rk = reinterpret_cast<float2 *>(buf + off_modes);
     float2 *tab = reinterpret_cast<float2 *>(buf + off_tab);
     float *d_acc = b_out ? reinterpret_cast<float *>(buf + off_out) : acc;
-    cudaMemcpyAsync(tab, h_tab.data(), b_tab, cudaMemcpyHostToDevice, s);
     cudaMemsetAsync(fix, 0, b_fix, s);
     if (n > 0) {
         k_pm_deposit<<<nblk(n), kT, 0, s>>>(n, shift, ng, t->px, t->py, t->pz, t->pm32, t->nmom, fix);
         note_launch();
     }
-    k_pm_density<<<nblk(cells), kT, 0, s>>>(cells, fix, real); note_launch();
+    k_pm_density<<<nblk(cells / 4), kT, 0, s>>>(cells, fix, real); note_launch();
+    // per-axis table: k_n^2 and exp(-k_n^2 r_s^2) / sinc^4(k_n D / 2), FP64 on the
+    // host beside the deposit
+    std::vector<float2> h_tab(ng);
+    for (int i = 0; i < ng; ++i) {
+        const int nsig = i < ng / 2 ? i : i - ng;
+        const double k = 2.0 * M_PI * nsig / L;
+        const double x = 0.5 * k * D;
+        const double sinc = nsig == 0 ? 1.0 : std::sin(x) / x;
+        const double s2 = sinc * sinc;
+        h_tab[i] = make_float2((float)(k * k), (float)(std::exp(-k * k * rs * rs) / (s2 * s2)));
+    }
+    cudaMemcpyAsync(tab, h_tab.data(), b_tab, cudaMemcpyHostToDevice, s);
     cufftResult r = api->set_stream(plans.r2c, s);
     if (r == CUFFT_SUCCESS) r = api->exec_r2c(plans.r2c, real, reinterpret_cast<cufftComplex *>(rk));
     if (r == CUFFT_SUCCESS) {
         // -4 pi G / k^2 of the density (mass / D^3), over Ng^3 for the unnormalised inverse FFT
         const double cfac = -4.0 * M_PI * p.G / (D * D * D) / (double)cells;
-        k_pm_green<<<nblk(modes), kT, 0, s>>>(ng, nzh, tab, (float)cfac, rk); note_launch();
+        k_pm_green<<<nblk((int64_t)ng * ng * 32), kT, 0, s>>>(ng, nzh, tab, (float)cfac, rk); note_launch();
         r = api->set_stream(plans.c2r, s);
     }
     if (r == CUFFT_SUCCESS) r = api->exec_c2r(plans.c2r, reinterpret_cast<cufftComplex *>(rk), real);
