@@ -119,29 +119,48 @@ __device__ __forceinline__ uint32_t quantize(double v, double box, double inv_bo
     return (uint32_t)floor(f * 4294967296.0);
 }
 
-// In a build (d_tot set) it also clears what later kernels accumulate into:
-// the device totals, the masses' set-bit span (empty: lowest 0x7f7f7f7f
-// above highest 0x80808080), the scans' look words and tile counters, and with
-// one box its sorted box indices (all 0).
+// What the first kernel of a build or a refit clears for the later ones, so that they
+// need no memset of their own (each would be a launch of its own between two kernels
+// that could overlap); null: not wanted.
+struct FirstClear {
+    uint32_t *d_tot;                   // the device totals
+    int *mbits;                        // the masses' set-bit span (empty: lowest 0x7f7f7f7f above highest 0x80808080)
+    unsigned long long *scan_look;     // the scans' look words and tile counters
+    int64_t nlook;
+    unsigned long long *sort;          // the sort's histograms, counters and look words
+    int64_t nsort;
+    uint32_t *seg_off;                 // one box: its offsets 0, n
+    uint32_t *sseg;                    // one box: the sorted box indices (all 0)
+    uint32_t *far;                     // a refit's drift flag
+};
+
+// One box: its geometry comes with the launch (g1) and not from the table.
 // Several boxes (pseg set): it also finds and writes the box of every particle of
 // the caller's order, and reads the positions where the box has them (io).
 __global__ void k_quantize_keys(const double *__restrict__ pos, int64_t n, int64_t B,
                                 const uint32_t *__restrict__ seg_off, uint32_t *__restrict__ pseg,
-                                const BoxIO *__restrict__ io, const SegGeom *__restrict__ geom, uint4 *q4, uint64_t *key,
-                                uint64_t *key_copy, uint32_t *idx,
-                                uint32_t *sseg_zero, uint32_t *d_tot, int *mbits,
-                                unsigned long long *scan_look, int64_t nlook, uint32_t *status) {
+                                const BoxIO *__restrict__ io, const SegGeom *__restrict__ geom, const SegGeom g1, uint4 *q4,
+                                uint64_t *key, uint64_t *key_copy, uint32_t *idx, const FirstClear c,
+                                uint32_t *status) {
     pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    // the look words and tile counters of the build's one-kernel scans
-    for (int64_t k = i; k < nlook; k += (int64_t)gridDim.x * blockDim.x) scan_look[k] = 0ull;
-    if (i == 0 && d_tot) {
-        d_tot[0] = d_tot[1] = d_tot[2] = d_tot[3] = 0u;
-        mbits[0] = 0x7f7f7f7f;
-        mbits[1] = (int)0x80808080u;
+    const int64_t all = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t k = i; k < c.nlook; k += all) c.scan_look[k] = 0ull;
+    for (int64_t k = i; k < c.nsort; k += all) c.sort[k] = 0ull;
+    if (i == 0) {
+        if (c.d_tot) {
+            c.d_tot[0] = c.d_tot[1] = c.d_tot[2] = c.d_tot[3] = 0u;
+            c.mbits[0] = 0x7f7f7f7f;
+            c.mbits[1] = (int)0x80808080u;
+        }
+        if (c.seg_off) {
+            c.seg_off[0] = 0u;
+            c.seg_off[1] = (uint32_t)n;
+        }
+        if (c.far) *c.far = 0u;
     }
     if (i >= n) return;
-    if (sseg_zero) sseg_zero[i] = 0u;
+    if (c.sseg) c.sseg[i] = 0u;
     uint32_t seg = 0;
     const double *x3 = pos + 3 * i;
     if (pseg) {
@@ -153,13 +172,14 @@ __global__ void k_quantize_keys(const double *__restrict__ pos, int64_t n, int64
         pseg[i] = seg = (uint32_t)lo;
         if (io) x3 = io[seg].pos + 3 * (i - (int64_t)seg_off[seg]);
     }
-    const SegGeom g = geom[seg];
+    const SegGeom g = pseg ? geom[seg] : g1;
     const double box = g.box, inv_box = g.inv_box;
     const bool pow2 = g.pow2 != 0;
     uint32_t x = quantize(x3[0], box, inv_box, pow2, g.shift, status);
     uint32_t y = quantize(x3[1], box, inv_box, pow2, g.shift, status);
     uint32_t z = quantize(x3[2], box, inv_box, pow2, g.shift, status);
     q4[i] = make_uint4(x, y, z, 0u);   // one 16-byte record: the permute gathers it whole
+    if (!key) return;                  // a refit keeps its keys
     const uint64_t k = (spread21(x >> 11) << 2) | (spread21(y >> 11) << 1) | spread21(z >> 11);
     key[i] = k;
     if (key_copy) key_copy[i] = k;
@@ -1201,6 +1221,17 @@ struct Bump {
     }
 };
 
+// The end of a build: its counts and the status word written to the host's page-locked
+// words (two copies cost more than this launch), and the next walk's counters cleared.
+__global__ void k_report(const uint32_t *__restrict__ d_tot, const uint32_t *__restrict__ status,
+                         unsigned long long *counters, uint32_t *h_tot, uint32_t *h_status) {
+    pdl_wait();
+    const uint32_t i = threadIdx.x;
+    if (i < 3u) h_tot[i] = d_tot[i];
+    if (i == 3u) *h_status = *status;
+    if (i < (uint32_t)kWalkCounters) counters[i] = 0ull;
+}
+
 }  // namespace
 
 // Bytes of the persistent arrays of a forest with n particles in B boxes.
@@ -1360,14 +1391,12 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
     ensure_origins(t);   // from the build's positions, before k_repos moves them
     const size_t mom_bytes = moments_scratch_bytes(n);
     const int64_t n32 = (n + 31) / 32, n1024 = (n32 + 31) / 32;
-    size_t sb = (size_t)n * (16 + 8 + 4 + 4) + 4096 + mom_bytes + 4 * (kLevels + 3) * sizeof(uint32_t) + 256 +
+    size_t sb = (size_t)n * (16 + 4) + 4096 + mom_bytes + 4 * (kLevels + 3) * sizeof(uint32_t) + 256 +
                 (size_t)(n32 + n1024) * sizeof(Tile) + 1024;
     void *scratch = nullptr;
     if ((err = dev_malloc_async(&scratch, sb, s)) != cudaSuccess) return cuda_fail(err, "cudaMallocAsync (refit)");
     Bump W(scratch, sb);
     uint4 *q4 = W.take<uint4>(n);
-    uint64_t *keys = W.take<uint64_t>(n);
-    uint32_t *idx = W.take<uint32_t>(n);
     uint32_t *pseg = W.take<uint32_t>(n);
     uint32_t *lcount = W.take<uint32_t>(4 * (kLevels + 3));
     void *mom_scratch = W.take<char>((int64_t)mom_bytes);
@@ -1377,11 +1406,11 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     cudaEventRecord(e0, s);
+    FirstClear fc{};
+    fc.far = far;
     launch_pdl(k_quantize_keys, nblk(n), kT, 0, s, d_pos, n, B, t->seg_off, B > 1 ? pseg : nullptr,
-                                           (const BoxIO *)nullptr, t->geom, q4,
-                                           keys, nullptr, idx, nullptr, nullptr, nullptr, nullptr, (int64_t)0,
-                                           t->ctx->d_status);
-    cudaMemsetAsync(far, 0, sizeof(uint32_t), s);
+               (const BoxIO *)nullptr, t->geom, t->h_geom[0], q4, (uint64_t *)nullptr, (uint64_t *)nullptr,
+               (uint32_t *)nullptr, fc, t->ctx->d_status);
     launch_pdl(k_repos, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, t->skey, t->px, t->py, t->pz, t32, far);
     launch_pdl(k_tiles1024, nblk(32 * n1024), kT, 0, s, n32, (const Tile *)t32, t1024);
     launch_pdl(k_extents_ranges, nblk(t->nnodes), kT, 0, s, t->nnodes, t->nlev, t->nbeg, t->nend, t->norg, t->px,
@@ -1501,8 +1530,10 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
             hg[b].pow2 = std::frexp(t->seg_prm[b].box, &e2) == 0.5 ? 1 : 0;
             hg[b].shift = 33 - e2;   // box = 2^(e2 - 1): x / box * 2^32 = x * 2^(33 - e2)
         }
-        cudaMemcpyAsync(t->seg_off, t->h_seg_off.data(), (B + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(t->geom, hg.data(), B * sizeof(SegGeom), cudaMemcpyHostToDevice, s);
+        if (B > 1) {                   // one box: k_quantize_keys has both by value
+            cudaMemcpyAsync(t->seg_off, t->h_seg_off.data(), (B + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice, s);
+            cudaMemcpyAsync(t->geom, hg.data(), B * sizeof(SegGeom), cudaMemcpyHostToDevice, s);
+        }
     }
 
     // ---- scratch
@@ -1566,12 +1597,14 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
         keys = t->skey;
         idx = t->perm;
     }
-    launch_pdl(k_quantize_keys, nblk(n), kT, 0, s, d_pos, n, B, t->seg_off, B > 1 ? pseg : nullptr, t->io, t->geom, q4,
-                                           keys, B > 1 ? key0 : nullptr, idx, B > 1 ? nullptr : t->sseg,
-                                           d_tot, t->mbits, scan_look, nlook, status);
+    FirstClear fc{d_tot, t->mbits, scan_look, nlook, nullptr, 0, B > 1 ? nullptr : t->seg_off,
+                  B > 1 ? nullptr : t->sseg, nullptr};
+    fc.sort = radix_sort_clear(n, sort_scratch, &fc.nsort);
+    launch_pdl(k_quantize_keys, nblk(n), kT, 0, s, d_pos, n, B, t->seg_off, B > 1 ? pseg : nullptr, t->io, t->geom,
+               t->h_geom[0], q4, keys, B > 1 ? key0 : nullptr, idx, fc, status);
     // a3: by key, then (several boxes) stably by box
     bool in_alt = false;
-    radix_sort_pairs(keys, idx, keys_alt, idx_alt, n, 63, sort_scratch, s, &in_alt, status);
+    radix_sort_pairs(keys, idx, keys_alt, idx_alt, n, 63, sort_scratch, s, &in_alt, status, true);
     if (B > 1) {
         uint32_t *perm1 = in_alt ? idx_alt : idx;
         uint64_t *segkey = in_alt ? keys : keys_alt;      // the free key buffer
@@ -1646,10 +1679,11 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
     // the counts and the status word, read once the build is complete (its
     // only host synchronisation)
     uint32_t *hc = pinned_counts(t->ctx), *hs = pinned_status(t->ctx);
-    cudaMemcpyAsync(hc, d_tot, 3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(hs, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    launch_pdl(k_report, 1, 32, 0, s, (const uint32_t *)d_tot, (const uint32_t *)status, t->ctx->d_counters, hc, hs);
     cudaFreeAsync(scratch, s);
+    t->ctx->counters_zero = false;
     if ((err = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(err, "build");
+    if (cudaPeekAtLastError() == cudaSuccess) t->ctx->counters_zero = true;
     for (int k = 0; k < 3; ++k) h_tot[k] = hc[k];
     t->build_status = *hs;
     float ms = 0;

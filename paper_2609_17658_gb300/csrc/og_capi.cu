@@ -77,10 +77,23 @@ __global__ void k_gather_aold(int64_t n, const uint32_t *__restrict__ perm,
 // Outputs in caller order, gathered: caller index j reads sorted position
 // inv[j] (the sorted arrays were just written by the walk and sit in L2), and
 // the stores of consecutive j are contiguous.
+// rep: the walk's counters and the status word also go to the host's page-locked words
+// (two copies there cost more), and the counters are cleared for the next walk.
+struct ForceReport {
+    unsigned long long *counters;
+    const uint32_t *status;
+    unsigned long long *h_counters;
+    uint32_t *h_status;
+};
 __global__ void k_unpermute(int64_t n, const uint32_t *__restrict__ inv,
                             const float *__restrict__ acc_sorted,
                             const uint32_t *__restrict__ npp_s, const uint32_t *__restrict__ npn_s,
-                            float *acc, uint32_t *npp, uint32_t *npn) {
+                            float *acc, uint32_t *npp, uint32_t *npn, ForceReport rep) {
+    if (rep.counters && blockIdx.x == 0 && threadIdx.x < (uint32_t)kWalkCounters) {
+        if (threadIdx.x < 3u && rep.h_counters) rep.h_counters[threadIdx.x] = rep.counters[threadIdx.x];
+        if (threadIdx.x == 3u) *rep.h_status = *rep.status;
+        rep.counters[threadIdx.x] = 0ull;
+    }
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     const uint32_t i = inv[j];
@@ -600,35 +613,39 @@ og_status og_tree_force(og_tree *t, const float *a_old, float *acc, uint32_t *n_
         cudaEventDestroy(e1);
         return fail(st);
     }
-    // back to caller order
+    // back to caller order; the last kernel reports the last pass's counters (a pass
+    // with list dumps is not deferred and has read its own)
+    uint32_t *hst = pinned_status(c);
+    const bool last_deferred = t->npend > 0 && !t->h_wp[0].dump;
+    const ForceReport none{}, rep{c->d_counters, c->d_status,
+                                  last_deferred ? pinned_counters(c, t->npend - 1) : nullptr, hst};
     if (!dev && (n_pp || n_pn)) {
         // host outputs: the counts first, their copy on the side stream beside
         // the accelerations' reordering (the copies share the link, the
         // reordering does not)
         k_unpermute<<<nblk(n), kT, 0, s>>>(n, t->inv, t->a_sorted, t->npp_sorted, t->npn_sorted,
-                                           nullptr, d_npp, d_npn); note_launch();
+                                           nullptr, d_npp, d_npn, none); note_launch();
         cudaEventRecord(c->ev_to_side, s);
         cudaStreamWaitEvent(c->copy_stream, c->ev_to_side, 0);
         if (n_pp) cudaMemcpyAsync(n_pp, d_npp, (size_t)n * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->copy_stream);
         if (n_pn) cudaMemcpyAsync(n_pn, d_npn, (size_t)n * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->copy_stream);
         cudaEventRecord(c->ev_from_side, c->copy_stream);
         k_unpermute<<<nblk(n), kT, 0, s>>>(n, t->inv, t->a_sorted, t->npp_sorted, t->npn_sorted,
-                                           d_acc, nullptr, nullptr); note_launch();
+                                           d_acc, nullptr, nullptr, rep); note_launch();
         cudaMemcpyAsync(acc, d_acc, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost, s);
         cudaStreamWaitEvent(s, c->ev_from_side, 0);
         cudaFreeAsync(out_tmp, s);
     } else {
         k_unpermute<<<nblk(n), kT, 0, s>>>(n, t->inv, t->a_sorted, t->npp_sorted, t->npn_sorted,
-                                           d_acc, d_npp, d_npn); note_launch();
+                                           d_acc, d_npp, d_npn, rep); note_launch();
         if (!dev) {
             cudaMemcpyAsync(acc, d_acc, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost, s);
             cudaFreeAsync(out_tmp, s);
         }
     }
     cudaEventRecord(e1, s);
-    uint32_t *hst = pinned_status(c);
-    cudaMemcpyAsync(hst, c->d_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
     e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && cudaPeekAtLastError() == cudaSuccess) c->counters_zero = true;
     st = finish_deferred(t, &ms_walk);
     cudaEventElapsedTime(&ms, e0, e1);
     cudaEventDestroy(e0);
@@ -926,7 +943,7 @@ og_status og_batch_force(og_ctx *c, int64_t nbox, const og_box *boxes, og_batch_
         uint32_t *o_pp = reinterpret_cast<uint32_t *>(o_acc + 3 * total);
         uint32_t *o_pn = o_pp + total;
         k_unpermute<<<nblk(total), kT, 0, s>>>(total, t->inv, t->a_sorted, t->npp_sorted, t->npn_sorted,
-                                               o_acc, o_pp, o_pn); note_launch();
+                                               o_acc, o_pp, o_pn, ForceReport{}); note_launch();
         for (int64_t b = 0; b < nbox; ++b) {
             const int64_t o = t->h_seg_off[b], nb = boxes[b].n;
             cudaMemcpyAsync(boxes[b].acc, o_acc + 3 * o, (size_t)nb * 3 * sizeof(float), cudaMemcpyDeviceToHost, s);

@@ -86,6 +86,7 @@ struct og_ctx {
     cudaStream_t stream = nullptr;
     size_t hbm_budget = 0;
     uint32_t *d_status = nullptr;     // device status word
+    bool counters_zero = false;       // d_counters are known to be zero on the stream
     void *h_pinned = nullptr;         // page-locked host words read back without a sync of
                                       // their own: pass counters, status, build counts
     unsigned long long *d_counters = nullptr;  // scratch counters (work queues, totals)
@@ -203,6 +204,9 @@ inline uint32_t *pinned_status(og_ctx *c) {
 inline uint32_t *pinned_counts(og_ctx *c) {
     return reinterpret_cast<uint32_t *>(static_cast<unsigned long long *>(c->h_pinned) + 9);
 }
+// words of og_ctx::d_counters that a walk counts in: next item, interactions, list
+// cursor, items in parts, next part
+constexpr int kWalkCounters = 5;
 // default launch shape of the walk (og_params.walk_warps / walk_chunk = 0)
 constexpr int kDefaultWalkWarps = 4;
 constexpr int kDefaultWalkChunk = 256;
@@ -288,7 +292,10 @@ void scan_inclusive_max_u32_look(const uint32_t *in, uint32_t *out, int64_t n, u
 size_t radix_sort_scratch_bytes(int64_t n);
 void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt,
                       int64_t n, int bits, void *scratch, cudaStream_t s, bool *result_in_alt,
-                      uint32_t *status);
+                      uint32_t *status, bool cleared = false);
+// the 64-bit words of the scratch that a sort of n pairs wants cleared: a caller whose
+// own kernel clears them passes cleared and saves the memset
+unsigned long long *radix_sort_clear(int64_t n, void *scratch, int64_t *words);
 
 // the same sort with every digit pass run (no histogram read-back, no host
 // synchronisation); with an even pass count the result is back in keys/vals

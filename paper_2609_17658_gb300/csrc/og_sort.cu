@@ -376,26 +376,34 @@ size_t radix_sort_scratch_bytes(int64_t n) {
     return every > one ? every : one;
 }
 
+// word offset of the look words: the digit histograms and 64 tile counters before them
+constexpr int64_t kLookAt = (8 * kRadix * sizeof(uint32_t) + 256) / sizeof(unsigned long long);
+
+unsigned long long *radix_sort_clear(int64_t n, void *scratch, int64_t *words) {
+    const int64_t ntiles = (n + kTile - 1) / kTile;
+    // one-kernel passes: a look word per tile and digit; large sorts: the look words of
+    // the tile counts' one-kernel scans (one tag per pass), the counts follow them
+    *words = kLookAt + (ntiles > kOneSweepMaxTiles ? (int64_t)scan_look_words((int64_t)kRadix * ntiles)
+                                                   : (int64_t)kRadix * ntiles);
+    return reinterpret_cast<unsigned long long *>((reinterpret_cast<uintptr_t>(scratch) + 255) & ~(uintptr_t)255);
+}
+
 void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt,
                       int64_t n, int bits, void *scratch, cudaStream_t s, bool *result_in_alt,
-                      uint32_t *status) {
+                      uint32_t *status, bool cleared) {
     *result_in_alt = false;
     if (n <= 1) return;
     int64_t ntiles = (n + kTile - 1) / kTile;
-    char *p = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(scratch) + 255) & ~(uintptr_t)255);
+    int64_t nclear;
+    unsigned long long *p = radix_sort_clear(n, scratch, &nclear);
     uint32_t *hist8 = reinterpret_cast<uint32_t *>(p);
     uint32_t *tile_ctr = hist8 + 8 * kRadix;
-    unsigned long long *look = reinterpret_cast<unsigned long long *>(p + 8 * kRadix * sizeof(uint32_t) + 256);
-    // large sorts: the look words of the tile counts' one-kernel scans (one
-    // tag per pass), then the counts
+    unsigned long long *look = p + kLookAt;
     const size_t scan_words = scan_look_words((int64_t)kRadix * ntiles);
-    const size_t clear = 8 * kRadix * sizeof(uint32_t) + 256 +
-                         (ntiles > kOneSweepMaxTiles ? scan_words : (size_t)kRadix * ntiles) *
-                             sizeof(unsigned long long);
 
     // the digit histograms of all passes (they give every pass its digit
     // bases and show which passes are trivial); counters and look words cleared
-    cudaMemsetAsync(p, 0, clear, s);
+    if (!cleared) cudaMemsetAsync(p, 0, (size_t)nclear * sizeof(unsigned long long), s);
     int grid = (int)((n + kThreads * 16 - 1) / (kThreads * 16));
     if (grid > 1184) grid = 1184;
     launch_pdl(k_all_digits, grid, kThreads, 0, s, keys, n, hist8);

@@ -1058,8 +1058,8 @@ void launch_walk(const WalkArgs &a, bool dump, bool refit, bool multi, bool pot,
                  cudaStream_t s, int sms) {
     if (pot) {
         // the potential is computed on single trees without list dumps
-        if (refit) launch_walk_t<kOpen, kSplit, false, true, false, true>(a, nitems, s, sms);
-        else launch_walk_t<kOpen, kSplit, false, false, false, true>(a, nitems, s, sms);
+        if (refit) launch_walk_t<kOpen, kSplit, false, true, false, true, true>(a, nitems, s, sms);
+        else launch_walk_t<kOpen, kSplit, false, false, false, true, true>(a, nitems, s, sms);
     } else if (multi) {
         if (refit) launch_walk_t<kOpen, kSplit, false, true, true>(a, nitems, s, sms);
         else launch_walk_t<kOpen, kSplit, false, false, true>(a, nitems, s, sms);
@@ -1148,10 +1148,10 @@ struct PassScratch {
     }
 };
 
-// Per-box parameters of a pass (uploaded) and the tree's view.  The first
+// Per-box parameters of a pass (uploaded if the launch reads them as a table) and the tree's view.  The first
 // pass of the relative criterion is Barnes-Hut with theta_first_pass.
 og_status prepare_view(og_tree *t, int opening, bool first_pass, const float *a_old_sorted,
-                       float *acc_sorted, bool pot, TreeView *v, WalkParams *wp0, PassScratch *sc) {
+                       float *acc_sorted, bool pot, bool table, TreeView *v, WalkParams *wp0, PassScratch *sc) {
     cudaStream_t s = t->ctx->stream;
     const int64_t B = t->nseg;
     t->h_wp.resize((size_t)B);
@@ -1170,8 +1170,10 @@ og_status prepare_view(og_tree *t, int opening, bool first_pass, const float *a_
     sc->axes = pot ? 4u : 3u;
     *wp0 = t->h_wp[0];
     WalkParams *dp = t->segp + (first_pass ? 0 : B);
-    cudaError_t err = cudaMemcpyAsync(dp, t->h_wp.data(), B * sizeof(WalkParams), cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "walk setup");
+    if (table) {
+        cudaError_t err = cudaMemcpyAsync(dp, t->h_wp.data(), B * sizeof(WalkParams), cudaMemcpyHostToDevice, s);
+        if (err != cudaSuccess) return cuda_fail(err, "walk setup");
+    }
     TreeView &w = *v;
     w = TreeView{};
     w.n = t->n;
@@ -1261,6 +1263,13 @@ WalkParams make_walk_params(const og_params &p, int opening, double theta) {
     return w;
 }
 
+// The counters before a walk: cleared here, unless the last build or force call left
+// them at zero (its last kernel clears them, which saves a memset between two kernels).
+static void clear_counters(og_ctx *c) {
+    if (!c->counters_zero) cudaMemsetAsync(c->d_counters, 0, kWalkCounters * sizeof(unsigned long long), c->stream);
+    c->counters_zero = false;
+}
+
 static og_status finish_pass(og_ctx *c, cudaEvent_t e0, cudaEvent_t e1, float *ms_out,
                              unsigned long long h[3]) {
     cudaStream_t s = c->stream;
@@ -1326,8 +1335,10 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
     WalkArgs a{};
     WalkParams wp;
     PassScratch sc;
-    og_status st = prepare_view(t, opening, first_pass, a_old_sorted, acc_sorted, pot_sorted != nullptr, &a.tree0,
-                                &wp, &sc);
+    // one box without list dumps: the parameters come with the launch
+    const bool dump = (t->seg_prm[0].flags & OG_DEBUG_DUMP_LISTS) != 0 && !pot_sorted;
+    og_status st = prepare_view(t, opening, first_pass, a_old_sorted, acc_sorted, pot_sorted != nullptr,
+                                t->nseg > 1 || dump, &a.tree0, &wp, &sc);
     if (st) return st;
     fill_common(a, t->ctx, t);
     a.one_seg = t->nseg == 1 ? 1 : 0;
@@ -1370,18 +1381,20 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
         a.tree0.gorder = t->gorder;
     }
     if (defer && !wp.dump && t->npend < 2) {
-        // no host synchronisation: the counters go to a page-locked slot and
+        // no host synchronisation: the counters go to page-locked slot npend and
         // the times to events, both read by finish_deferred
         const int k = t->npend;
-        cudaMemsetAsync(t->ctx->d_counters, 0, 5 * sizeof(unsigned long long), s);
+        clear_counters(t->ctx);
         cudaEventCreate(&t->pend_e0[k]);
         cudaEventCreate(&t->pend_e1[k]);
         cudaEventRecord(t->pend_e0[k], s);
         a.tree0.pot = pot_sorted;
         launch(a, opening, wp.split, false, t->refit, false, a.tree0.ngroups, s, pot_sorted != nullptr);
         cudaEventRecord(t->pend_e1[k], s);
-        cudaMemcpyAsync(pinned_counters(t->ctx, k), t->ctx->d_counters, 3 * sizeof(unsigned long long),
-                        cudaMemcpyDeviceToHost, s);
+        // the last pass's counters are reported by the caller's last kernel
+        if (first_pass)
+            cudaMemcpyAsync(pinned_counters(t->ctx, k), t->ctx->d_counters, 3 * sizeof(unsigned long long),
+                            cudaMemcpyDeviceToHost, s);
         t->npend = k + 1;
         release();
         // the next pass may take this one's list lengths: stream order makes them ready
@@ -1391,7 +1404,7 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
     }
     unsigned long long h[3] = {0, 0, 0};
     for (int attempt = 0; attempt < 2; ++attempt) {
-        cudaMemsetAsync(t->ctx->d_counters, 0, 5 * sizeof(unsigned long long), s);
+        clear_counters(t->ctx);
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
@@ -1432,7 +1445,7 @@ og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int openi
     for (int64_t k = 0; k < ntrees; ++k) {
         WalkParams wp;
         og_status st = prepare_view(trees[k], opening, false, a_old_sorted ? a_old_sorted[k] : nullptr,
-                                    acc_sorted[k], false, &hv[k], &wp, &sc[k]);
+                                    acc_sorted[k], false, true, &hv[k], &wp, &sc[k]);
         if (st) return st;
         if (k == 0) split = wp.split;
         else if (wp.split != split) {
@@ -1505,7 +1518,7 @@ og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int openi
     }
     a.tree_inter = tint;
     cudaMemsetAsync(tint, 0, (size_t)ntrees * sizeof(unsigned long long), s);
-    cudaMemsetAsync(c->d_counters, 0, 5 * sizeof(unsigned long long), s);
+    clear_counters(c);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
