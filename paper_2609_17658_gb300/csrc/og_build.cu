@@ -9,31 +9,32 @@
 // between two boxes are separators: no node spans them.
 //
 //   a1/a2  k_quantize_keys   f64 positions -> u32 fixed point -> 63-bit Morton key
-//   a3     radix sort (og_sort.cu), k_permute gathers sorted SoA positions/masses
+//   a3     radix sort (og_sort.cu), Permute gathers sorted SoA positions/masses
 //                           and the masses' set-bit span
-//   a4     k_split_tiles    level of every adjacent-key split (shared 3-bit digits)
+//   a4     SplitTiles       level of every adjacent-key split (shared 3-bit digits)
 //          k_split_carry    and, per level threshold, the nearest lower split
 //          k_split_ranges   across tiles; the node a split belongs to: its key
 //                           range (nearest lower splits on both sides) and whether
 //                           it is the node's first split; first splits are
 //                           numbered by a scan
-//          k_node_init      nodes of first splits, node id of every split
-//          k_link           parent of every node, owner node of every particle,
+//          NodeInit         nodes of first splits, node id of every split
+//          Link             parent of every node, owner node of every particle,
 //                           octant-occupancy bits of every node
-//          k_place          child array in key order, grouped by parent
-//          k_threading      nextnode / sibling threading (unified index space)
-//   a5     exact node moments and centres of mass (og_moments.cu): prefix
+//          Place            child array in key order, grouped by parent
+//          Threading        nextnode / sibling threading (unified index space)
+//   a5     exact node moments and centres of mass (og_moments.h): prefix
 //                           sums over the sorted particles, one pass over the nodes
 //          k_level_hist .. k_level_scatter   node ids bucketed by tree level (a
 //                           refit's extents only, made on the first refit)
-//          k_extents_ranges a refit's node extents from ranges of the sorted particles
+//          ExtentRanges    a refit's node extents from ranges of the sorted particles
 //          k_extents_level  the same level by level, for drifts above a quarter of the
 //          k_extents_run    box: a launch per large level, runs of small ones in a block
-//   a6     k_frontier       frontier node, unit and run start mark of every particle
-//          k_groupmark      group starts (then compacted into gbeg by a scan)
-//          k_group_fin      group ends, boxes and box index
-//          k_records        32-byte child records read by the walk
+//   a6     Frontier         frontier node, unit and run start mark of every particle
+//          GroupMark        group starts (then compacted into gbeg by a scan)
+//          GroupFin         group ends, boxes and box index
+//          Records          32-byte child records read by the walk
 //          k_cell_origin    node cell origins, made when extents are first needed
+//   (names without k_ are stages, which k_stages runs alone or side by side)
 //
 // Every decision is integer or exact, so the result is identical to the
 // oracle's recursive construction.
@@ -42,11 +43,44 @@
 #include <vector>
 
 #include "og_internal.h"
+#include "og_moments.h"
 
 namespace og {
 namespace {
 
 constexpr int kT = 256;
+// Stages of a build or a refit that do not depend on each other share a launch up to
+// kShareMax particles: blocks [0, na) are the first one's, the next nb the second's, the
+// rest the third's.  Down there a kernel of the chain takes 3 to 4 us, most of it launch
+// and latency, so a stage beside another one costs little: builds of 4k, 32k, 100k and
+// 200k particles took 122, 139, 162 and 189 us with a launch per stage and 104, 120,
+// 144 and 179 this way.  Above, a stage pays for the registers of the one beside it
+// (400k: 254 and 261 us, 700k: 350 and 377, 2M: 716 and 870), and each has its own launch.
+constexpr int64_t kShareMax = 1 << 18;
+struct NoStage {
+    __device__ void operator()(uint32_t, uint32_t) const {}
+};
+template <int kThreads, class A, class B, class C>
+__global__ void __launch_bounds__(kThreads) k_stages(const A a, uint32_t na, const B b, uint32_t nb, const C c) {
+    pdl_wait();
+    uint32_t bid = blockIdx.x;
+    if (bid < na) {
+        a(bid, na);
+        return;
+    }
+    bid -= na;
+    if (bid < nb) b(bid, nb);
+    else c(bid - nb, gridDim.x - na - nb);
+}
+template <int kThreads, class A>
+void run_stage(cudaStream_t s, unsigned na, const A &a) {
+    launch_pdl(k_stages<kThreads, A, NoStage, NoStage>, na, kThreads, 0, s, a, na, NoStage{}, 0u, NoStage{});
+}
+template <int kThreads, class A, class B, class C = NoStage>
+void run_stages(cudaStream_t s, unsigned na, const A &a, unsigned nb, const B &b, unsigned nc = 0, const C &c = C{}) {
+    launch_pdl(k_stages<kThreads, A, B, C>, na + nb + nc, kThreads, 0, s, a, na, b, nb, c);
+}
+
 constexpr uint8_t kSep = 0xff;  // split level of a boundary between two boxes
 
 __device__ __forceinline__ uint64_t spread21(uint32_t v) {
@@ -210,52 +244,64 @@ __global__ void k_gather_keys(int64_t n, const uint32_t *__restrict__ perm,
 // call gathers its caller-order outputs through it); the masses are checked here, and their
 // set-bit span (the units of the exact moments) is gathered: a block's lowest
 // and highest exponents, merged by atomics only where they widen the span.
-__global__ void __launch_bounds__(kT) k_permute(int64_t n, const uint32_t *__restrict__ perm,
-                                                const uint4 *__restrict__ q4, const double *__restrict__ mass,
-                                                const BoxIO *__restrict__ io, const uint32_t *__restrict__ sseg,
-                                                const uint32_t *__restrict__ seg_off, uint32_t *px, uint32_t *py, uint32_t *pz, float *pm32,
-                                                double *pm64, uint32_t *inv, int *mbits, uint32_t *status) {
-    pdl_wait();
-    __shared__ int wlo[kT / 32], whi[kT / 32];
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int lo = 0x7fffffff, hi = (int)0x80000000;
-    if (i < n) {
-        uint32_t j = perm[i];
-        inv[j] = (uint32_t)i;
-        const uint4 q = q4[j];
-        px[i] = q.x;
-        py[i] = q.y;
-        pz[i] = q.z;
-        double m;
-        if (io) {
-            const uint32_t b = sseg[i];
-            m = io[b].mass[j - seg_off[b]];
-        } else {
-            m = mass[j];
+struct Permute {
+    int64_t n;
+    const uint32_t *__restrict__ perm;
+    const uint4 *__restrict__ q4;
+    const double *__restrict__ mass;
+    const BoxIO *__restrict__ io;
+    const uint32_t *__restrict__ sseg;
+    const uint32_t *__restrict__ seg_off;
+    uint32_t *px;
+    uint32_t *py;
+    uint32_t *pz;
+    float *pm32;
+    double *pm64;
+    uint32_t *inv;
+    int *mbits;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        __shared__ int wlo[32], whi[32];
+        int64_t i = (int64_t)bid * blockDim.x + threadIdx.x;
+        int lo = 0x7fffffff, hi = (int)0x80000000;
+        if (i < n) {
+            uint32_t j = perm[i];
+            inv[j] = (uint32_t)i;
+            const uint4 q = q4[j];
+            px[i] = q.x;
+            py[i] = q.y;
+            pz[i] = q.z;
+            double m;
+            if (io) {
+                const uint32_t b = sseg[i];
+                m = io[b].mass[j - seg_off[b]];
+            } else {
+                m = mass[j];
+            }
+            if (!isfinite(m) || m < 0.0) atomicOr(status, ST_BAD_INPUT);
+            pm64[i] = m;
+            pm32[i] = __double2float_rn(m);
+            mass_bit_span(m, lo, hi);
         }
-        if (!isfinite(m) || m < 0.0) atomicOr(status, ST_BAD_INPUT);
-        pm64[i] = m;
-        pm32[i] = __double2float_rn(m);
-        mass_bit_span(m, lo, hi);
-    }
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if ((threadIdx.x & 31u) == 0u) {
-        wlo[threadIdx.x >> 5] = lo;
-        whi[threadIdx.x >> 5] = hi;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < kT / 32; ++w) {
-            lo = min(lo, wlo[w]);
-            hi = max(hi, whi[w]);
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if ((threadIdx.x & 31u) == 0u) {
+            wlo[threadIdx.x >> 5] = lo;
+            whi[threadIdx.x >> 5] = hi;
         }
-        if (lo <= hi) {
-            if (lo < __ldcg(&mbits[0])) atomicMin(&mbits[0], lo);
-            if (hi > __ldcg(&mbits[1])) atomicMax(&mbits[1], hi);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (uint32_t w = 1; w < blockDim.x / 32; ++w) {
+                lo = min(lo, wlo[w]);
+                hi = max(hi, whi[w]);
+            }
+            if (lo <= hi) {
+                if (lo < __ldcg(&mbits[0])) atomicMin(&mbits[0], lo);
+                if (hi > __ldcg(&mbits[1])) atomicMax(&mbits[1], hi);
+            }
         }
     }
-}
+};
 
 // The node of a split of level L is the key range around it whose adjacent
 // splits all have levels >= L (the lcp of two sorted keys is the smallest
@@ -298,49 +344,54 @@ __device__ __forceinline__ unsigned lanes_below(const WarpLevels &w, int t) {
 }
 
 // levels of all splits; per tile and threshold, its last and first split below t
-__global__ void __launch_bounds__(kSplitTile) k_split_tiles(const uint64_t *__restrict__ skey,
-                                                            const uint32_t *__restrict__ sseg, int64_t nsplit,
-                                                            uint8_t *lv, int *tlast, int *tfirst) {
-    pdl_wait();
-    __shared__ int wl[32][kNT], wf[32][kNT];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * kSplitTile + threadIdx.x;
-    int v = kNT;  // past the last split: below no threshold
-    // key i and box i of every lane (i <= nsplit = n - 1 is a particle); the
-    // next particle's from the lane above, the warp's last lane loads its own
-    const int64_t ic = i <= nsplit ? i : nsplit;
-    const uint64_t k0 = skey[ic];
-    const uint32_t s0 = sseg[ic];
-    uint64_t k1 = __shfl_down_sync(0xffffffffu, k0, 1);
-    uint32_t s1 = __shfl_down_sync(0xffffffffu, s0, 1);
-    if (lane == 31 && i < nsplit) {
-        k1 = skey[i + 1];
-        s1 = sseg[i + 1];
-    }
-    if (i < nsplit) {
-        const uint8_t l = (s0 != s1) ? kSep : (uint8_t)lcp_levels(k0, k1);
-        lv[i] = l;
-        v = split_rank(l);
-    }
-    // lane t < kNT: this warp's last and first split below threshold t
-    const int64_t base = (int64_t)blockIdx.x * kSplitTile + warp * 32;
-    const unsigned m = lanes_below(warp_levels(v), lane < kNT ? lane : 0);
-    if (lane < kNT) {
-        wl[warp][lane] = m ? (int)(base + 31 - __clz(m)) : -1;
-        wf[warp][lane] = m ? (int)(base + __ffs(m) - 1) : kNone;
-    }
-    __syncthreads();
-    // warp t folds threshold t over the 32 warps of the tile
-    if (warp < kNT) {
-        int l = wl[lane][warp], f = wf[lane][warp];
-        l = __reduce_max_sync(0xffffffffu, l);
-        f = __reduce_min_sync(0xffffffffu, f);
-        if (lane == 0) {
-            tlast[blockIdx.x * kNT + warp] = l;
-            tfirst[blockIdx.x * kNT + warp] = f;
+struct SplitTiles {
+    const uint64_t *__restrict__ skey;
+    const uint32_t *__restrict__ sseg;
+    int64_t nsplit;
+    uint8_t *lv;
+    int *tlast;
+    int *tfirst;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        __shared__ int wl[32][kNT], wf[32][kNT];
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const int64_t i = (int64_t)bid * kSplitTile + threadIdx.x;
+        int v = kNT;  // past the last split: below no threshold
+        // key i and box i of every lane (i <= nsplit = n - 1 is a particle); the
+        // next particle's from the lane above, the warp's last lane loads its own
+        const int64_t ic = i <= nsplit ? i : nsplit;
+        const uint64_t k0 = skey[ic];
+        const uint32_t s0 = sseg[ic];
+        uint64_t k1 = __shfl_down_sync(0xffffffffu, k0, 1);
+        uint32_t s1 = __shfl_down_sync(0xffffffffu, s0, 1);
+        if (lane == 31 && i < nsplit) {
+            k1 = skey[i + 1];
+            s1 = sseg[i + 1];
+        }
+        if (i < nsplit) {
+            const uint8_t l = (s0 != s1) ? kSep : (uint8_t)lcp_levels(k0, k1);
+            lv[i] = l;
+            v = split_rank(l);
+        }
+        // lane t < kNT: this warp's last and first split below threshold t
+        const int64_t base = (int64_t)bid * kSplitTile + warp * 32;
+        const unsigned m = lanes_below(warp_levels(v), lane < kNT ? lane : 0);
+        if (lane < kNT) {
+            wl[warp][lane] = m ? (int)(base + 31 - __clz(m)) : -1;
+            wf[warp][lane] = m ? (int)(base + __ffs(m) - 1) : kNone;
+        }
+        __syncthreads();
+        // warp t folds threshold t over the 32 warps of the tile
+        if (warp < kNT) {
+            int l = wl[lane][warp], f = wf[lane][warp];
+            l = __reduce_max_sync(0xffffffffu, l);
+            f = __reduce_min_sync(0xffffffffu, f);
+            if (lane == 0) {
+                tlast[bid * kNT + warp] = l;
+                tfirst[bid * kNT + warp] = f;
+            }
         }
     }
-}
+};
 
 // per tile and threshold t: the last split below t in the tiles before it and
 // the first one in the tiles after it (one block per threshold)
@@ -490,49 +541,63 @@ __global__ void __launch_bounds__(kSplitTile) k_split_ranges(const uint8_t *__re
 // Roots, the nodes of first splits (level, key range), cleared
 // per-node accumulators, and the node id of every split: its box's root at level 0, else the node of the
 // first split reached along prevle (at most 7 steps).
-__global__ void k_node_init(int64_t n, int64_t B, const uint32_t *__restrict__ seg_off,
-                            const uint32_t *__restrict__ first, const uint32_t *__restrict__ nid,
-                            const uint8_t *__restrict__ lv, const uint32_t *__restrict__ sb,
-                            const uint32_t *__restrict__ se, const uint32_t *__restrict__ prevle,
-                            const uint32_t *__restrict__ sseg,
-                            uint8_t *nlev, uint32_t *nbeg, uint32_t *nend, uint32_t *sid,
-                            int64_t mcap, uint32_t *occ, uint32_t *nnc, uint32_t *nccnt, uint32_t *status) {
-    pdl_wait();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < mcap) {  // per-node accumulators of the kernels that follow
-        occ[i] = 0u;
-        nnc[i] = 0u;
-        nccnt[i] = 0u;
-    }
-    if (i < B) {  // the root of box i covers the whole box
-        nlev[i] = 0;
-        nbeg[i] = seg_off[i];
-        nend[i] = seg_off[i + 1];
-    }
-    if (i >= n - 1) return;
-    const int L = lv[i];
-    if (L == kSep) { sid[i] = 0xffffffffu; return; }
-    if (L == 0) { sid[i] = sseg[i]; return; }  // the root of this box
-    if (first[i]) {
-        const uint32_t id = (uint32_t)B + nid[i];
-        sid[i] = id;
-        nlev[id] = (uint8_t)L;
-        nbeg[id] = sb[i];
-        nend[id] = se[i];
-        return;
-    }
-    uint32_t j = prevle[i];
-    for (int guard = 0;; ++guard) {
-        if (guard > 7 || (int64_t)j >= n - 1) {
-            atomicOr(status, ST_INTERNAL);
-            sid[i] = sseg[i];
+struct NodeInit {
+    int64_t n;
+    int64_t B;
+    const uint32_t *__restrict__ seg_off;
+    const uint32_t *__restrict__ first;
+    const uint32_t *__restrict__ nid;
+    const uint8_t *__restrict__ lv;
+    const uint32_t *__restrict__ sb;
+    const uint32_t *__restrict__ se;
+    const uint32_t *__restrict__ prevle;
+    const uint32_t *__restrict__ sseg;
+    uint8_t *nlev;
+    uint32_t *nbeg;
+    uint32_t *nend;
+    uint32_t *sid;
+    int64_t mcap;
+    uint32_t *occ;
+    uint32_t *nnc;
+    uint32_t *nccnt;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        int64_t i = (int64_t)bid * blockDim.x + threadIdx.x;
+        if (i < mcap) {  // per-node accumulators of the kernels that follow
+            occ[i] = 0u;
+            nnc[i] = 0u;
+            nccnt[i] = 0u;
+        }
+        if (i < B) {  // the root of box i covers the whole box
+            nlev[i] = 0;
+            nbeg[i] = seg_off[i];
+            nend[i] = seg_off[i + 1];
+        }
+        if (i >= n - 1) return;
+        const int L = lv[i];
+        if (L == kSep) { sid[i] = 0xffffffffu; return; }
+        if (L == 0) { sid[i] = sseg[i]; return; }  // the root of this box
+        if (first[i]) {
+            const uint32_t id = (uint32_t)B + nid[i];
+            sid[i] = id;
+            nlev[id] = (uint8_t)L;
+            nbeg[id] = sb[i];
+            nend[id] = se[i];
             return;
         }
-        if (first[j]) break;
-        j = prevle[j];
+        uint32_t j = prevle[i];
+        for (int guard = 0;; ++guard) {
+            if (guard > 7 || (int64_t)j >= n - 1) {
+                atomicOr(status, ST_INTERNAL);
+                sid[i] = sseg[i];
+                return;
+            }
+            if (first[j]) break;
+            j = prevle[j];
+        }
+        sid[i] = (uint32_t)B + nid[j];
     }
-    sid[i] = (uint32_t)B + nid[j];
-}
+};
 
 __device__ __forceinline__ int split_at(const uint8_t *lv, int64_t j, int64_t n) {
     if (j < 0 || j >= n - 1) return -1;
@@ -541,121 +606,155 @@ __device__ __forceinline__ int split_at(const uint8_t *lv, int64_t j, int64_t n)
 }
 
 // parent of every non-root node, owner of every particle, octant occupancy
-__global__ void k_link(int64_t n, const uint32_t *__restrict__ nsplit, int64_t B,
-                       const uint64_t *__restrict__ skey,
-                       const uint8_t *__restrict__ lv, const uint32_t *__restrict__ sid,
-                       const uint32_t *__restrict__ sseg, const uint8_t *__restrict__ nlev,
-                       const uint32_t *__restrict__ nbeg, const uint32_t *__restrict__ nend,
-                       int32_t *npar, uint32_t *owner, uint32_t *occ, uint32_t *nnc,
-                       uint32_t *status) {
-    pdl_wait();
-    const int64_t m = B + (int64_t)*nsplit;  // nodes: the roots and one per first split
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) {
-        const int64_t p = t;
-        const int dl = split_at(lv, p - 1, n), dr = split_at(lv, p, n);
-        uint32_t own;
-        if (dl < 0 && dr < 0) own = sseg[p];  // alone in its box: hangs from the root
-        else own = sid[dl >= dr ? p - 1 : p];
-        if (own >= (uint32_t)m) {
-            atomicOr(status, ST_INTERNAL);
-            own = sseg[p];
+struct Link {
+    int64_t n;
+    const uint32_t *__restrict__ nsplit;
+    int64_t B;
+    const uint64_t *__restrict__ skey;
+    const uint8_t *__restrict__ lv;
+    const uint32_t *__restrict__ sid;
+    const uint32_t *__restrict__ sseg;
+    const uint8_t *__restrict__ nlev;
+    const uint32_t *__restrict__ nbeg;
+    const uint32_t *__restrict__ nend;
+    int32_t *npar;
+    uint32_t *owner;
+    uint32_t *occ;
+    uint32_t *nnc;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        const int64_t m = B + (int64_t)*nsplit;  // nodes: the roots and one per first split
+        int64_t t = (int64_t)bid * blockDim.x + threadIdx.x;
+        if (t < n) {
+            const int64_t p = t;
+            const int dl = split_at(lv, p - 1, n), dr = split_at(lv, p, n);
+            uint32_t own;
+            if (dl < 0 && dr < 0) own = sseg[p];  // alone in its box: hangs from the root
+            else own = sid[dl >= dr ? p - 1 : p];
+            if (own >= (uint32_t)m) {
+                atomicOr(status, ST_INTERNAL);
+                own = sseg[p];
+            }
+            owner[p] = own;
+            int lo = nlev[own];
+            if (lo < kLevels) atomicOr(&occ[own], 1u << digit_at(skey[p], lo + 1));
+        } else if (t < n + (m - B)) {
+            const int64_t id = B + (t - n);
+            const int64_t b = nbeg[id], e = nend[id];
+            const int dl = split_at(lv, b - 1, n), dr = split_at(lv, e - 1, n);
+            uint32_t par;
+            if (dl < 0 && dr < 0) par = sseg[b];  // the whole box: child of its root
+            else par = sid[dl >= dr ? b - 1 : e - 1];
+            npar[id] = (int32_t)par;
+            if (par >= (uint32_t)m || nlev[par] >= nlev[id] || nlev[par] >= kLevels) {
+                atomicOr(status, ST_INTERNAL);
+                return;
+            }
+            atomicOr(&occ[par], 1u << digit_at(skey[b], nlev[par] + 1));
+            atomicAdd(&nnc[par], 1u);
+        } else if (t < n + m) {
+            npar[t - n - (m - B)] = -1;  // roots
         }
-        owner[p] = own;
-        int lo = nlev[own];
-        if (lo < kLevels) atomicOr(&occ[own], 1u << digit_at(skey[p], lo + 1));
-    } else if (t < n + (m - B)) {
-        const int64_t id = B + (t - n);
-        const int64_t b = nbeg[id], e = nend[id];
-        const int dl = split_at(lv, b - 1, n), dr = split_at(lv, e - 1, n);
-        uint32_t par;
-        if (dl < 0 && dr < 0) par = sseg[b];  // the whole box: child of its root
-        else par = sid[dl >= dr ? b - 1 : e - 1];
-        npar[id] = (int32_t)par;
-        if (par >= (uint32_t)m || nlev[par] >= nlev[id] || nlev[par] >= kLevels) {
-            atomicOr(status, ST_INTERNAL);
-            return;
+    }
+};
+
+struct ChildCount {
+    const uint32_t *__restrict__ nsplit;
+    int64_t B;
+    const uint8_t *__restrict__ nlev;
+    const uint32_t *__restrict__ nbeg;
+    const uint32_t *__restrict__ nend;
+    const uint32_t *__restrict__ occ;
+    uint32_t *nccnt;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        const int64_t m = B + (int64_t)*nsplit;
+        int64_t id = (int64_t)bid * blockDim.x + threadIdx.x;
+        if (id >= m) return;
+        nccnt[id] = nlev[id] == kLevels ? nend[id] - nbeg[id] : (uint32_t)__popc(occ[id]);
+    }
+};
+
+struct Place {
+    int64_t n;
+    const uint32_t *__restrict__ nsplit;
+    int64_t B;
+    const uint64_t *__restrict__ skey;
+    const uint8_t *__restrict__ nlev;
+    const uint32_t *__restrict__ nbeg;
+    const uint32_t *__restrict__ ncbeg;
+    const uint32_t *__restrict__ occ;
+    const int32_t *__restrict__ npar;
+    const uint32_t *__restrict__ owner;
+    uint32_t *child;
+    uint32_t *npos;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        const int64_t m = B + (int64_t)*nsplit;
+        const int64_t nchild = n + (m - B);
+        int64_t t = (int64_t)bid * blockDim.x + threadIdx.x;
+        if (t < n) {
+            const int64_t p = t;
+            uint32_t own = owner[p];
+            int lo = nlev[own];
+            uint32_t slot;
+            if (lo == kLevels) {
+                slot = ncbeg[own] + (uint32_t)(p - nbeg[own]);
+            } else {
+                int d = digit_at(skey[p], lo + 1);
+                slot = ncbeg[own] + __popc(occ[own] & ((1u << d) - 1u));
+            }
+            if (slot >= (uint64_t)nchild) { atomicOr(status, ST_INTERNAL); return; }
+            child[slot] = (uint32_t)p;
+        } else if (t < n + m - B) {
+            const int64_t id = B + (t - n);
+            uint32_t par = (uint32_t)npar[id];
+            int d = digit_at(skey[nbeg[id]], nlev[par] + 1);
+            uint32_t slot = ncbeg[par] + __popc(occ[par] & ((1u << d) - 1u));
+            if (slot >= (uint64_t)nchild) { atomicOr(status, ST_INTERNAL); return; }
+            child[slot] = (uint32_t)(n + id);
+            npos[id] = slot;
         }
-        atomicOr(&occ[par], 1u << digit_at(skey[b], nlev[par] + 1));
-        atomicAdd(&nnc[par], 1u);
-    } else if (t < n + m) {
-        npar[t - n - (m - B)] = -1;  // roots
     }
-}
+};
 
-__global__ void k_ccnt(const uint32_t *__restrict__ nsplit, int64_t B, const uint8_t *__restrict__ nlev,
-                       const uint32_t *__restrict__ nbeg, const uint32_t *__restrict__ nend,
-                       const uint32_t *__restrict__ occ, uint32_t *nccnt) {
-    pdl_wait();
-    const int64_t m = B + (int64_t)*nsplit;
-    int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= m) return;
-    nccnt[id] = nlev[id] == kLevels ? nend[id] - nbeg[id] : (uint32_t)__popc(occ[id]);
-}
-
-__global__ void k_place(int64_t n, const uint32_t *__restrict__ nsplit, int64_t B,
-                        const uint64_t *__restrict__ skey,
-                        const uint8_t *__restrict__ nlev, const uint32_t *__restrict__ nbeg,
-                        const uint32_t *__restrict__ ncbeg, const uint32_t *__restrict__ occ,
-                        const int32_t *__restrict__ npar, const uint32_t *__restrict__ owner,
-                        uint32_t *child, uint32_t *npos, uint32_t *status) {
-    pdl_wait();
-    const int64_t m = B + (int64_t)*nsplit;
-    const int64_t nchild = n + (m - B);
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) {
-        const int64_t p = t;
-        uint32_t own = owner[p];
-        int lo = nlev[own];
-        uint32_t slot;
-        if (lo == kLevels) {
-            slot = ncbeg[own] + (uint32_t)(p - nbeg[own]);
-        } else {
-            int d = digit_at(skey[p], lo + 1);
-            slot = ncbeg[own] + __popc(occ[own] & ((1u << d) - 1u));
+struct Threading {
+    int64_t n;
+    const uint32_t *__restrict__ nsplit;
+    int64_t B;
+    const uint32_t *__restrict__ child;
+    const uint32_t *__restrict__ ncbeg;
+    const uint32_t *__restrict__ nccnt;
+    const int32_t *__restrict__ npar;
+    const uint32_t *__restrict__ npos;
+    const uint32_t *__restrict__ owner;
+    int32_t *nnext;
+    int32_t *nsib;
+    int32_t *pnext;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        const int64_t m = B + (int64_t)*nsplit;
+        const int64_t nchild = n + (m - B);
+        int64_t c = (int64_t)bid * blockDim.x + threadIdx.x;
+        if (c < m) {
+            nnext[c] = (int32_t)child[ncbeg[c]];
+            if (c < B) nsib[c] = -1;  // a root ends its box's threading
         }
-        if (slot >= (uint64_t)nchild) { atomicOr(status, ST_INTERNAL); return; }
-        child[slot] = (uint32_t)p;
-    } else if (t < n + m - B) {
-        const int64_t id = B + (t - n);
-        uint32_t par = (uint32_t)npar[id];
-        int d = digit_at(skey[nbeg[id]], nlev[par] + 1);
-        uint32_t slot = ncbeg[par] + __popc(occ[par] & ((1u << d) - 1u));
-        if (slot >= (uint64_t)nchild) { atomicOr(status, ST_INTERNAL); return; }
-        child[slot] = (uint32_t)(n + id);
-        npos[id] = slot;
+        if (c >= nchild) return;
+        const uint32_t item = child[c];
+        int64_t par = item < n ? (int64_t)owner[item] : (int64_t)npar[item - n];
+        int64_t cc = c;
+        int32_t after = -1;
+        for (int guard = 0;; ++guard) {
+            if (guard > 2 * kLevels + 2 || par < 0 || par >= m) { atomicOr(status, ST_INTERNAL); break; }
+            if (cc + 1 < (int64_t)ncbeg[par] + nccnt[par]) { after = (int32_t)child[cc + 1]; break; }
+            if (par < B) { after = -1; break; }
+            cc = npos[par];
+            par = npar[par];
+        }
+        if (item < n) pnext[item] = after;
+        else nsib[item - n] = after;
     }
-}
-
-__global__ void k_threading(int64_t n, const uint32_t *__restrict__ nsplit, int64_t B,
-                            const uint32_t *__restrict__ child,
-                            const uint32_t *__restrict__ ncbeg, const uint32_t *__restrict__ nccnt,
-                            const int32_t *__restrict__ npar, const uint32_t *__restrict__ npos,
-                            const uint32_t *__restrict__ owner, int32_t *nnext, int32_t *nsib,
-                            int32_t *pnext, uint32_t *status) {
-    pdl_wait();
-    const int64_t m = B + (int64_t)*nsplit;
-    const int64_t nchild = n + (m - B);
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < m) {
-        nnext[c] = (int32_t)child[ncbeg[c]];
-        if (c < B) nsib[c] = -1;  // a root ends its box's threading
-    }
-    if (c >= nchild) return;
-    const uint32_t item = child[c];
-    int64_t par = item < n ? (int64_t)owner[item] : (int64_t)npar[item - n];
-    int64_t cc = c;
-    int32_t after = -1;
-    for (int guard = 0;; ++guard) {
-        if (guard > 2 * kLevels + 2 || par < 0 || par >= m) { atomicOr(status, ST_INTERNAL); break; }
-        if (cc + 1 < (int64_t)ncbeg[par] + nccnt[par]) { after = (int32_t)child[cc + 1]; break; }
-        if (par < B) { after = -1; break; }
-        cc = npos[par];
-        par = npar[par];
-    }
-    if (item < n) pnext[item] = after;
-    else nsib[item - n] = after;
-}
+};
 
 // Node ids bucketed by tree level, for the bottom-up pass of a refit's
 // extents (a node's extent joins its children's).
@@ -849,40 +948,55 @@ __device__ __forceinline__ uint32_t frontier_of(int64_t p, int64_t B, int G, con
 // frontier node and unit of every particle, and the run marks: p where the
 // frontier node changes (else 0), for the maximum scan that gives each
 // particle the start of its run
-__global__ void k_frontier(int64_t n, int64_t B, int G, const uint32_t *__restrict__ owner,
-                           const int32_t *__restrict__ npar, const uint32_t *__restrict__ nbeg,
-                           const uint32_t *__restrict__ nend, uint32_t *fp, uint32_t *unit, uint32_t *rs) {
-    pdl_wait();
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t pc = p < n ? p : n - 1;          // every lane takes part in the shuffle
-    int64_t prev;
-    const uint32_t f = frontier_of(pc, B, G, owner, npar, nbeg, nend, prev);
-    uint32_t fl = __shfl_up_sync(0xffffffffu, f, 1);
-    if ((threadIdx.x & 31) == 0 && pc > 0) {
-        int64_t unused;
-        fl = frontier_of(pc - 1, B, G, owner, npar, nbeg, nend, unused);
+struct Frontier {
+    int64_t n;
+    int64_t B;
+    int G;
+    const uint32_t *__restrict__ owner;
+    const int32_t *__restrict__ npar;
+    const uint32_t *__restrict__ nbeg;
+    const uint32_t *__restrict__ nend;
+    uint32_t *fp;
+    uint32_t *unit;
+    uint32_t *rs;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        const int64_t p = (int64_t)bid * blockDim.x + threadIdx.x;
+        const int64_t pc = p < n ? p : n - 1;          // every lane takes part in the shuffle
+        int64_t prev;
+        const uint32_t f = frontier_of(pc, B, G, owner, npar, nbeg, nend, prev);
+        uint32_t fl = __shfl_up_sync(0xffffffffu, f, 1);
+        if ((threadIdx.x & 31) == 0 && pc > 0) {
+            int64_t unused;
+            fl = frontier_of(pc - 1, B, G, owner, npar, nbeg, nend, unused);
+        }
+        if (p >= n) return;
+        fp[p] = f;
+        unit[p] = prev < 0 ? (uint32_t)p : nbeg[prev];
+        rs[p] = (p == 0 || f != fl) ? (uint32_t)p : 0u;
     }
-    if (p >= n) return;
-    fp[p] = f;
-    unit[p] = prev < 0 ? (uint32_t)p : nbeg[prev];
-    rs[p] = (p == 0 || f != fl) ? (uint32_t)p : 0u;
-}
+};
 
 // group starts: inside a frontier node of at most 8G particles, runs of
 // consecutive particles are cut every G; inside a larger frontier node every
 // unit (a small child node or a single particle) starts a group of its own
-__global__ void k_groupmark(int64_t n, int G, const uint32_t *__restrict__ runstart,
-                            const uint32_t *__restrict__ fp, const uint32_t *__restrict__ unit,
-                            const uint32_t *__restrict__ nbeg, const uint32_t *__restrict__ nend,
-                            uint32_t *gs) {
-    pdl_wait();
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const uint32_t f = fp[p];
-    const bool merge = (uint64_t)(nend[f] - nbeg[f]) <= 8ull * (uint64_t)G;
-    if (merge) gs[p] = ((p - runstart[p]) % G == 0) ? 1u : 0u;
-    else gs[p] = (unit[p] == (uint32_t)p) ? 1u : 0u;
-}
+struct GroupMark {
+    int64_t n;
+    int G;
+    const uint32_t *__restrict__ runstart;
+    const uint32_t *__restrict__ fp;
+    const uint32_t *__restrict__ unit;
+    const uint32_t *__restrict__ nbeg;
+    const uint32_t *__restrict__ nend;
+    uint32_t *gs;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        int64_t p = (int64_t)bid * blockDim.x + threadIdx.x;
+        if (p >= n) return;
+        const uint32_t f = fp[p];
+        const bool merge = (uint64_t)(nend[f] - nbeg[f]) <= 8ull * (uint64_t)G;
+        if (merge) gs[p] = ((p - runstart[p]) % G == 0) ? 1u : 0u;
+        else gs[p] = (unit[p] == (uint32_t)p) ? 1u : 0u;
+    }
+};
 
 __device__ __forceinline__ void group_box(int64_t n, int64_t ng, int64_t g,
                                           const uint32_t *__restrict__ gbeg, uint32_t *gend,
@@ -916,34 +1030,47 @@ __device__ __forceinline__ void group_box(int64_t n, int64_t ng, int64_t g,
 
 // group ends and boxes; the group count is *d_ng (the build, before the host
 // knows it) or ng (a refit)
-__global__ void k_group_fin(int64_t n, const uint32_t *__restrict__ d_ng, int64_t ng_host,
-                            const uint32_t *__restrict__ gbeg, uint32_t *gend,
-                            const uint32_t *__restrict__ px, const uint32_t *__restrict__ py,
-                            const uint32_t *__restrict__ pz, const uint32_t *__restrict__ sseg,
-                            uint32_t *gbox, uint32_t *gseg) {
-    pdl_wait();
-    int64_t ng = d_ng ? (int64_t)*d_ng : ng_host;
-    if (ng > n) ng = n;                        // the host reports a bad count
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < ng;
-         g += (int64_t)gridDim.x * blockDim.x)
-        group_box(n, ng, g, gbeg, gend, px, py, pz, sseg, gbox, gseg);
-}
-
-__global__ void k_ext_records(int64_t n, int64_t nchild, const uint32_t *__restrict__ child,
-                              const uint32_t *__restrict__ ext_s, const uint32_t *__restrict__ ext_l,
-                              CExt *cext) {
-    pdl_wait();
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= nchild) return;
-    const uint32_t item = child[c];
-    CExt x = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-    if (item >= n) {
-        const int64_t j = item - n;
-        x = {ext_s[3 * j], ext_s[3 * j + 1], ext_s[3 * j + 2], 0u,
-             ext_l[3 * j], ext_l[3 * j + 1], ext_l[3 * j + 2], 0u};
+struct GroupFin {
+    int64_t n;
+    const uint32_t *__restrict__ d_ng;
+    int64_t ng_host;
+    const uint32_t *__restrict__ gbeg;
+    uint32_t *gend;
+    const uint32_t *__restrict__ px;
+    const uint32_t *__restrict__ py;
+    const uint32_t *__restrict__ pz;
+    const uint32_t *__restrict__ sseg;
+    uint32_t *gbox;
+    uint32_t *gseg;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        int64_t ng = d_ng ? (int64_t)*d_ng : ng_host;
+        if (ng > n) ng = n;                        // the host reports a bad count
+        for (int64_t g = (int64_t)bid * blockDim.x + threadIdx.x; g < ng;
+             g += (int64_t)nb * blockDim.x)
+            group_box(n, ng, g, gbeg, gend, px, py, pz, sseg, gbox, gseg);
     }
-    cext[c] = x;
-}
+};
+
+struct ExtRecords {
+    int64_t n;
+    int64_t nchild;
+    const uint32_t *__restrict__ child;
+    const uint32_t *__restrict__ ext_s;
+    const uint32_t *__restrict__ ext_l;
+    CExt *cext;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        int64_t c = (int64_t)bid * blockDim.x + threadIdx.x;
+        if (c >= nchild) return;
+        const uint32_t item = child[c];
+        CExt x = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+        if (item >= n) {
+            const int64_t j = item - n;
+            x = {ext_s[3 * j], ext_s[3 * j + 1], ext_s[3 * j + 2], 0u,
+                 ext_l[3 * j], ext_l[3 * j + 1], ext_l[3 * j + 2], 0u};
+        }
+        cext[c] = x;
+    }
+};
 
 // a built tree's node extents: its cells
 __global__ void k_cell_ext(int64_t m, const uint8_t *__restrict__ nlev, const uint32_t *__restrict__ norg,
@@ -978,7 +1105,6 @@ __device__ __forceinline__ uint32_t gather21(uint64_t x) {
 // A position counts from the key's cell the particle had in the build, X = origin
 // + signed drift, so it does not wrap where it leaves the box; a drift of a
 // quarter of the box or more is left to the level-by-level form.
-constexpr int kTile32 = 32, kTile1024 = 1024;
 struct Tile {
     long long lo[3], hi[3];
 };
@@ -1043,20 +1169,24 @@ __global__ void k_repos(int64_t n, const uint32_t *__restrict__ perm, const uint
 }
 
 // tiles of 1024 from the tiles of 32, a warp each
-__global__ void k_tiles1024(int64_t n32, const Tile *__restrict__ t32, Tile *__restrict__ t1024) {
-    pdl_wait();
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (32 * w >= n32) return;
-    const int64_t k = 32 * w + lane;
-    Tile t;
+struct Tiles1024 {
+    int64_t n32;
+    const Tile *__restrict__ t32;
+    Tile *__restrict__ t1024;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        const int64_t w = ((int64_t)bid * blockDim.x + threadIdx.x) >> 5;
+        const int lane = threadIdx.x & 31;
+        if (32 * w >= n32) return;
+        const int64_t k = 32 * w + lane;
+        Tile t;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        t.lo[a] = warp_min(k < n32 ? t32[k].lo[a] : kNoMin);
-        t.hi[a] = warp_max(k < n32 ? t32[k].hi[a] : kNoMax);
+        for (int a = 0; a < 3; ++a) {
+            t.lo[a] = warp_min(k < n32 ? t32[k].lo[a] : kNoMin);
+            t.hi[a] = warp_max(k < n32 ? t32[k].hi[a] : kNoMax);
+        }
+        if (lane == 0) t1024[w] = t;
     }
-    if (lane == 0) t1024[w] = t;
-}
+};
 
 // extent [lo, hi] (offsets from the cell origin o) of a node, stored
 __device__ __forceinline__ void store_extent(uint32_t node, const uint32_t *o, const long long *lo, const long long *hi,
@@ -1075,135 +1205,162 @@ __device__ __forceinline__ void store_extent(uint32_t node, const uint32_t *o, c
 // extents of the nodes of level 2 and deeper: up to kThreadNode particles by one
 // thread, more by its warp
 constexpr uint32_t kThreadNode = 48;
-__global__ void __launch_bounds__(kT) k_extents_ranges(int64_t m, const uint8_t *__restrict__ nlev,
-                                                       const uint32_t *__restrict__ nbeg,
-                                                       const uint32_t *__restrict__ nend,
-                                                       const uint32_t *__restrict__ norg,
-                                                       const uint32_t *__restrict__ px,
-                                                       const uint32_t *__restrict__ py,
-                                                       const uint32_t *__restrict__ pz,
-                                                       const Tile *__restrict__ t32, const Tile *__restrict__ t1024,
-                                                       uint32_t *ext_s, uint32_t *ext_l) {
-    pdl_wait();
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    const int lev = j < m ? nlev[j] : 0;
-    const uint32_t b = lev >= 2 ? nbeg[j] : 0u, e = lev >= 2 ? nend[j] : 0u;
-    auto point = [&](uint32_t q, const uint32_t *o, long long *lo, long long *hi) {
-        const int d[3] = {(int)(px[q] - o[0]), (int)(py[q] - o[1]), (int)(pz[q] - o[2])};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = d[a] < lo[a] ? d[a] : lo[a];
-            hi[a] = d[a] > hi[a] ? d[a] : hi[a];
-        }
-    };
-    if (lev >= 2 && e - b <= kThreadNode) {
-        const uint32_t o[3] = {norg[3 * j], norg[3 * j + 1], norg[3 * j + 2]};
-        const long long side = 1ll << (32 - lev);
-        long long lo[3] = {0, 0, 0}, hi[3] = {side - 1, side - 1, side - 1};
-        for (uint32_t q = b; q < e; ++q) point(q, o, lo, hi);
-        store_extent((uint32_t)j, o, lo, hi, ext_s, ext_l);
-    }
-    for (unsigned todo = __ballot_sync(0xffffffffu, lev >= 2 && e - b > kThreadNode); todo; todo &= todo - 1u) {
-        const int src = __ffs((int)todo) - 1;
-        const uint32_t node = (uint32_t)(j - lane + src);
-        const uint32_t b0 = __shfl_sync(0xffffffffu, b, src), e0 = __shfl_sync(0xffffffffu, e, src);
-        const int L = __shfl_sync(0xffffffffu, lev, src);
-        const uint32_t o[3] = {norg[3 * node], norg[3 * node + 1], norg[3 * node + 2]};
-        const long long side = 1ll << (32 - L);
-        long long lo[3] = {0, 0, 0}, hi[3] = {side - 1, side - 1, side - 1};
-        // [b0, e0) = particles, tiles of 32 [p, q), tiles of 1024 [r, s) inside them
-        const uint32_t p = (b0 + 31u) / 32u, q = e0 / 32u;
-        auto tile = [&](const Tile &t) {
+struct ExtentRanges {
+    int64_t m;
+    const uint8_t *__restrict__ nlev;
+    const uint32_t *__restrict__ nbeg;
+    const uint32_t *__restrict__ nend;
+    const uint32_t *__restrict__ norg;
+    const uint32_t *__restrict__ px;
+    const uint32_t *__restrict__ py;
+    const uint32_t *__restrict__ pz;
+    const Tile *__restrict__ t32;
+    const Tile *__restrict__ t1024;
+    uint32_t *ext_s;
+    uint32_t *ext_l;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        const int64_t j = (int64_t)bid * blockDim.x + threadIdx.x;
+        const int lane = threadIdx.x & 31;
+        const int lev = j < m ? nlev[j] : 0;
+        const uint32_t b = lev >= 2 ? nbeg[j] : 0u, e = lev >= 2 ? nend[j] : 0u;
+        auto point = [&](uint32_t q, const uint32_t *o, long long *lo, long long *hi) {
+            const int d[3] = {(int)(px[q] - o[0]), (int)(py[q] - o[1]), (int)(pz[q] - o[2])};
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                const long long l = t.lo[a] - (long long)o[a], h = t.hi[a] - (long long)o[a];
-                lo[a] = l < lo[a] ? l : lo[a];
-                hi[a] = h > hi[a] ? h : hi[a];
+                lo[a] = d[a] < lo[a] ? d[a] : lo[a];
+                hi[a] = d[a] > hi[a] ? d[a] : hi[a];
             }
         };
-        if (b0 + lane < 32u * p) point(b0 + lane, o, lo, hi);
-        if (32u * q + lane < e0) point(32u * q + lane, o, lo, hi);
-        const uint32_t r = (p + 31u) / 32u, s = q / 32u;
-        if (r < s) {
-            if (p + lane < 32u * r) tile(t32[p + lane]);
-            if (32u * s + lane < q) tile(t32[32u * s + lane]);
-            for (uint32_t k = r + (uint32_t)lane; k < s; k += 32u) tile(t1024[k]);
-        } else {
-            for (uint32_t k = p + (uint32_t)lane; k < q; k += 32u) tile(t32[k]);
+        if (lev >= 2 && e - b <= kThreadNode) {
+            const uint32_t o[3] = {norg[3 * j], norg[3 * j + 1], norg[3 * j + 2]};
+            const long long side = 1ll << (32 - lev);
+            long long lo[3] = {0, 0, 0}, hi[3] = {side - 1, side - 1, side - 1};
+            for (uint32_t q = b; q < e; ++q) point(q, o, lo, hi);
+            store_extent((uint32_t)j, o, lo, hi, ext_s, ext_l);
         }
+        for (unsigned todo = __ballot_sync(0xffffffffu, lev >= 2 && e - b > kThreadNode); todo; todo &= todo - 1u) {
+            const int src = __ffs((int)todo) - 1;
+            const uint32_t node = (uint32_t)(j - lane + src);
+            const uint32_t b0 = __shfl_sync(0xffffffffu, b, src), e0 = __shfl_sync(0xffffffffu, e, src);
+            const int L = __shfl_sync(0xffffffffu, lev, src);
+            const uint32_t o[3] = {norg[3 * node], norg[3 * node + 1], norg[3 * node + 2]};
+            const long long side = 1ll << (32 - L);
+            long long lo[3] = {0, 0, 0}, hi[3] = {side - 1, side - 1, side - 1};
+            // [b0, e0) = particles, tiles of 32 [p, q), tiles of 1024 [r, s) inside them
+            const uint32_t p = (b0 + 31u) / 32u, q = e0 / 32u;
+            auto tile = [&](const Tile &t) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = warp_min(lo[a]);
-            hi[a] = warp_max(hi[a]);
+                for (int a = 0; a < 3; ++a) {
+                    const long long l = t.lo[a] - (long long)o[a], h = t.hi[a] - (long long)o[a];
+                    lo[a] = l < lo[a] ? l : lo[a];
+                    hi[a] = h > hi[a] ? h : hi[a];
+                }
+            };
+            if (b0 + lane < 32u * p) point(b0 + lane, o, lo, hi);
+            if (32u * q + lane < e0) point(32u * q + lane, o, lo, hi);
+            const uint32_t r = (p + 31u) / 32u, s = q / 32u;
+            if (r < s) {
+                if (p + lane < 32u * r) tile(t32[p + lane]);
+                if (32u * s + lane < q) tile(t32[32u * s + lane]);
+                for (uint32_t k = r + (uint32_t)lane; k < s; k += 32u) tile(t1024[k]);
+            } else {
+                for (uint32_t k = p + (uint32_t)lane; k < q; k += 32u) tile(t32[k]);
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                lo[a] = warp_min(lo[a]);
+                hi[a] = warp_max(hi[a]);
+            }
+            if (lane == 0) store_extent(node, o, lo, hi, ext_s, ext_l);
         }
-        if (lane == 0) store_extent(node, o, lo, hi, ext_s, ext_l);
     }
-}
+};
 
 // levels 1 and 0, where an offset may not fit 32 bits and takes the joined form:
 // a block per box, its nodes of level 1 and then the root
-__global__ void k_extents_top(int64_t n, const uint8_t *__restrict__ nlev, const uint32_t *__restrict__ nbeg,
-                              const uint32_t *__restrict__ nend, const uint32_t *__restrict__ ncbeg,
-                              const uint32_t *__restrict__ nccnt, const uint32_t *__restrict__ occ,
-                              const uint32_t *__restrict__ child, const uint32_t *__restrict__ px,
-                              const uint32_t *__restrict__ py, const uint32_t *__restrict__ pz, int64_t nchild,
-                              const uint32_t *__restrict__ norg, uint32_t *ext_s, uint32_t *ext_l) {
-    pdl_wait();
-    const uint32_t root = blockIdx.x;
-    const uint32_t slot = ncbeg[root] + threadIdx.x;
-    if (threadIdx.x < nccnt[root] && slot < (uint64_t)nchild && child[slot] >= n) {
-        const uint32_t j = (uint32_t)(child[slot] - n);
-        if (nlev[j] == 1) extent_node(n, nbeg, nend, ncbeg, occ, child, px, py, pz, nchild, norg, ext_s, ext_l, j, 1);
+struct ExtentTop {
+    int64_t n;
+    const uint8_t *__restrict__ nlev;
+    const uint32_t *__restrict__ nbeg;
+    const uint32_t *__restrict__ nend;
+    const uint32_t *__restrict__ ncbeg;
+    const uint32_t *__restrict__ nccnt;
+    const uint32_t *__restrict__ occ;
+    const uint32_t *__restrict__ child;
+    const uint32_t *__restrict__ px;
+    const uint32_t *__restrict__ py;
+    const uint32_t *__restrict__ pz;
+    int64_t nchild;
+    const uint32_t *__restrict__ norg;
+    uint32_t *ext_s;
+    uint32_t *ext_l;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        const uint32_t root = bid;
+        const uint32_t slot = ncbeg[root] + threadIdx.x;
+        if (threadIdx.x < nccnt[root] && slot < (uint64_t)nchild && child[slot] >= n) {
+            const uint32_t j = (uint32_t)(child[slot] - n);
+            if (nlev[j] == 1) extent_node(n, nbeg, nend, ncbeg, occ, child, px, py, pz, nchild, norg, ext_s, ext_l, j, 1);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0)
+            extent_node(n, nbeg, nend, ncbeg, occ, child, px, py, pz, nchild, norg, ext_s, ext_l, root, 0);
     }
-    __syncthreads();
-    if (threadIdx.x == 0)
-        extent_node(n, nbeg, nend, ncbeg, occ, child, px, py, pz, nchild, norg, ext_s, ext_l, root, 0);
-}
+};
 
 // the walk's child records; the child count is *d_nchild (the build) or
 // nchild_host (a refit), at most ccap
-__global__ void k_records(int64_t n, const uint32_t *__restrict__ d_nchild, int64_t nchild_host,
-                          int64_t ccap, const uint32_t *__restrict__ child,
-                          const uint32_t *__restrict__ px, const uint32_t *__restrict__ py,
-                          const uint32_t *__restrict__ pz, const float *__restrict__ pm32,
-                          const double *__restrict__ pm64, const uint8_t *__restrict__ nlev,
-                          const uint32_t *__restrict__ ncbeg, const uint32_t *__restrict__ nccnt,
-                          const NodeMom *__restrict__ nmom, const uint32_t *__restrict__ ncom,
-                          CRec *crec, uint32_t *status) {
-    pdl_wait();
-    int64_t nchild = d_nchild ? (int64_t)*d_nchild : nchild_host;
-    if (nchild > ccap) nchild = ccap;          // the host reports a bad count
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nchild;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t item = child[c];
-        CRec r;
-        if (item < n) {
-            r.x = px[item];
-            r.y = py[item];
-            r.z = pz[item];
-            r.m = pm32[item];
-            r.M = pm64[item];
-            r.info = 1u << 31;
-            r.ref = item;
-        } else {
-            int64_t j = item - n;
-            r.x = ncom[3 * j + 0];
-            r.y = ncom[3 * j + 1];
-            r.z = ncom[3 * j + 2];
-            r.M = nmom[j].M;
-            r.m = __double2float_rn(r.M);
-            r.info = ((uint32_t)nlev[j] << 26) | (nccnt[j] & 0x3ffffffu);
-            r.ref = ncbeg[j];
-            // the walk pushes (ref, count) unchecked: a node has children, inside
-            // the child array, and is never a root
-            if (nccnt[j] == 0u || nccnt[j] > 0x3ffffffu || nlev[j] == 0u || nlev[j] > kLevels ||
-                (uint64_t)ncbeg[j] + nccnt[j] > (uint64_t)nchild)
-                atomicOr(status, ST_INTERNAL);
+struct Records {
+    int64_t n;
+    const uint32_t *__restrict__ d_nchild;
+    int64_t nchild_host;
+    int64_t ccap;
+    const uint32_t *__restrict__ child;
+    const uint32_t *__restrict__ px;
+    const uint32_t *__restrict__ py;
+    const uint32_t *__restrict__ pz;
+    const float *__restrict__ pm32;
+    const double *__restrict__ pm64;
+    const uint8_t *__restrict__ nlev;
+    const uint32_t *__restrict__ ncbeg;
+    const uint32_t *__restrict__ nccnt;
+    const NodeMom *__restrict__ nmom;
+    const uint32_t *__restrict__ ncom;
+    CRec *crec;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        int64_t nchild = d_nchild ? (int64_t)*d_nchild : nchild_host;
+        if (nchild > ccap) nchild = ccap;          // the host reports a bad count
+        for (int64_t c = (int64_t)bid * blockDim.x + threadIdx.x; c < nchild;
+             c += (int64_t)nb * blockDim.x) {
+            uint32_t item = child[c];
+            CRec r;
+            if (item < n) {
+                r.x = px[item];
+                r.y = py[item];
+                r.z = pz[item];
+                r.m = pm32[item];
+                r.M = pm64[item];
+                r.info = 1u << 31;
+                r.ref = item;
+            } else {
+                int64_t j = item - n;
+                r.x = ncom[3 * j + 0];
+                r.y = ncom[3 * j + 1];
+                r.z = ncom[3 * j + 2];
+                r.M = nmom[j].M;
+                r.m = __double2float_rn(r.M);
+                r.info = ((uint32_t)nlev[j] << 26) | (nccnt[j] & 0x3ffffffu);
+                r.ref = ncbeg[j];
+                // the walk pushes (ref, count) unchecked: a node has children, inside
+                // the child array, and is never a root
+                if (nccnt[j] == 0u || nccnt[j] > 0x3ffffffu || nlev[j] == 0u || nlev[j] > kLevels ||
+                    (uint64_t)ncbeg[j] + nccnt[j] > (uint64_t)nchild)
+                    atomicOr(status, ST_INTERNAL);
+            }
+            crec[c] = r;
         }
-        crec[c] = r;
     }
-}
+};
 
 inline unsigned nblk(int64_t n) { return (unsigned)((n + kT - 1) / kT); }
 
@@ -1368,8 +1525,7 @@ og_status cell_extents(og_tree *t) {
     ensure_origins(t);
     cudaStream_t s = t->ctx->stream;
     launch_pdl(k_cell_ext, nblk(t->nnodes), kT, 0, s, t->nnodes, t->nlev, t->norg, t->next_s, t->next_l);
-    launch_pdl(k_ext_records, nblk(t->nchild), kT, 0, s, t->n, t->nchild, t->child, t->next_s, t->next_l,
-                                                 t->cext);
+    run_stage<kT>(s, nblk(t->nchild), ExtRecords{t->n, t->nchild, t->child, t->next_s, t->next_l, t->cext});
     return OG_OK;
 }
 
@@ -1412,19 +1568,37 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
                (const BoxIO *)nullptr, t->geom, t->h_geom[0], q4, (uint64_t *)nullptr, (uint64_t *)nullptr,
                (uint32_t *)nullptr, fc, t->ctx->d_status);
     launch_pdl(k_repos, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, t->skey, t->px, t->py, t->pz, t32, far);
-    launch_pdl(k_tiles1024, nblk(32 * n1024), kT, 0, s, n32, (const Tile *)t32, t1024);
-    launch_pdl(k_extents_ranges, nblk(t->nnodes), kT, 0, s, t->nnodes, t->nlev, t->nbeg, t->nend, t->norg, t->px,
-               t->py, t->pz, (const Tile *)t32, (const Tile *)t1024, t->next_s, t->next_l);
-    launch_pdl(k_extents_top, dim3((unsigned)B), 32, 0, s, n, t->nlev, t->nbeg, t->nend, t->ncbeg, t->nccnt, t->nocc,
-               t->child, t->px, t->py, t->pz, t->nchild, t->norg, t->next_s, t->next_l);
-    node_moments(t, nullptr, t->nnodes, mom_scratch, s);
-    launch_pdl(k_group_fin, stride_grid(t->ngroups), kT, 0, s, n, nullptr, t->ngroups, t->gbeg, t->gend, t->px,
-                                                       t->py, t->pz, t->sseg, t->gbox, t->gseg);
-    launch_pdl(k_records, stride_grid(t->nchild), kT, 0, s, n, nullptr, t->nchild, t->nchild, t->child, t->px,
-                                                    t->py, t->pz, t->pm32, t->pm64, t->nlev, t->ncbeg,
-                                                    t->nccnt, t->nmom, t->ncom, t->crec, t->ctx->d_status);
-    launch_pdl(k_ext_records, nblk(t->nchild), kT, 0, s, n, t->nchild, t->child, t->next_s, t->next_l,
-                                                 t->cext);
+    const Moments mom(t, mom_scratch);
+    const Tiles1024 tiles1024{n32, t32, t1024};
+    const ExtentRanges ranges{t->nnodes, t->nlev, t->nbeg, t->nend, t->norg, t->px, t->py, t->pz, t32, t1024,
+                              t->next_s, t->next_l};
+    const ExtentTop top{n, t->nlev, t->nbeg, t->nend, t->ncbeg, t->nccnt, t->nocc, t->child, t->px, t->py, t->pz,
+                        t->nchild, t->norg, t->next_s, t->next_l};
+    const GroupFin group_fin{n, nullptr, t->ngroups, t->gbeg, t->gend, t->px, t->py, t->pz, t->sseg, t->gbox, t->gseg};
+    const Records records{n, nullptr, t->nchild, t->nchild, t->child, t->px, t->py, t->pz, t->pm32, t->pm64, t->nlev,
+                          t->ncbeg, t->nccnt, t->nmom, t->ncom, t->crec, t->ctx->d_status};
+    const ExtRecords ext_records{n, t->nchild, t->child, t->next_s, t->next_l, t->cext};
+    if (n <= kShareMax) {
+        run_stages<kT>(s, (unsigned)mom.ntiles, mom.tiles(), nblk(32 * n1024), tiles1024, stride_grid(t->ngroups),
+                       group_fin);
+        run_stages<kT>(s, (unsigned)mom.nblocks, mom.scan1(), nblk(t->nnodes), ranges);
+        run_stages<kT>(s, 1, mom.scan2(), (unsigned)B, top);
+        mom.prefix(s);
+        run_stage<kT>(s, Moments::node_blocks(t->nnodes), mom.nodes(nullptr, t->nnodes));
+        run_stages<kT>(s, stride_grid(t->nchild), records, nblk(t->nchild), ext_records);
+    } else {
+        run_stage<kT>(s, nblk(32 * n1024), tiles1024);
+        run_stage<kT>(s, nblk(t->nnodes), ranges);
+        run_stage<kT>(s, (unsigned)B, top);
+        run_stage<kT>(s, (unsigned)mom.ntiles, mom.tiles());
+        run_stage<kT>(s, (unsigned)mom.nblocks, mom.scan1());
+        run_stage<kT>(s, 1, mom.scan2());
+        mom.prefix(s);
+        run_stage<kT>(s, Moments::node_blocks(t->nnodes), mom.nodes(nullptr, t->nnodes));
+        run_stage<kT>(s, stride_grid(t->ngroups), group_fin);
+        run_stage<kT>(s, stride_grid(t->nchild), records);
+        run_stage<kT>(s, nblk(t->nchild), ext_records);
+    }
     uint32_t *h_far = pinned_counts(t->ctx);
     cudaMemcpyAsync(h_far, far, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
     cudaEventRecord(e1, s);
@@ -1439,7 +1613,7 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
             return st;
         }
         extents_bottom_up(t, t->next_s, t->next_l);
-        launch_pdl(k_ext_records, nblk(t->nchild), kT, 0, s, n, t->nchild, t->child, t->next_s, t->next_l, t->cext);
+        run_stage<kT>(s, nblk(t->nchild), ExtRecords{n, t->nchild, t->child, t->next_s, t->next_l, t->cext});
         cudaEventRecord(e1, s);
         err = cudaStreamSynchronize(s);
     }
@@ -1544,7 +1718,7 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
         add(8, n); add(4, n); add(8, n); add(4, n); add(8, n); add(4, n);  // keys, idx, alt, key copy, pseg
         add(1, n); add(4, n); add(4, n); add(4, n); add(4, n); add(4, n);  // lv sb se first nid sid
         add(4, 4 * kNT * ((n + kSplitTile - 1) / kSplitTile));  // split tile summaries
-        add(8, (int64_t)scan_look_words(n + B) + 2);            // scans' look words, counters
+        add(8, 2 * (int64_t)scan_look_words(n + B) + 2);            // scans' look words, counters
         add(4, n + B);                  // nnc
         add(4, n); add(4, n); add(4, n); add(4, n);  // fp rs gs unit
         sb_bytes += radix_sort_scratch_bytes(n) + scan_scratch_bytes(2 * n + B + 8) +
@@ -1566,15 +1740,17 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
     uint32_t *sbeg = W.take<uint32_t>(n), *send = W.take<uint32_t>(n);
     uint32_t *first = W.take<uint32_t>(n), *nid = W.take<uint32_t>(n), *sid = W.take<uint32_t>(n);
     int *tsum = W.take<int>(4 * kNT * ((n + kSplitTile - 1) / kSplitTile));
-    // the four one-kernel scans of the build share these look words (tags 1-4);
-    // their tile counters are the last two words (four 32-bit counters)
+    // the four one-kernel scans of the build share these look words (tags 1-4; the
+    // maximum scan, which runs beside a sum, has its own); their tile counters are
+    // the last two words (four 32-bit counters)
     const int64_t nlook_w = (int64_t)scan_look_words(n + B);
-    unsigned long long *scan_look = W.take<unsigned long long>(nlook_w + 2);
-    const int64_t nlook = nlook_w + 2;
-    uint32_t *scan_ctr = reinterpret_cast<uint32_t *>(scan_look + nlook_w);
+    unsigned long long *scan_look = W.take<unsigned long long>(2 * nlook_w + 2);
+    unsigned long long *scan_look_max = scan_look + nlook_w;
+    const int64_t nlook = 2 * nlook_w + 2;
+    uint32_t *scan_ctr = reinterpret_cast<uint32_t *>(scan_look + 2 * nlook_w);
     uint32_t *occ = t->nocc, *nnc = W.take<uint32_t>(n + B);
     uint32_t *fp = W.take<uint32_t>(n), *rs = W.take<uint32_t>(n), *gs = W.take<uint32_t>(n);
-    // a split's previous split in its node: needed only until k_node_init,
+    // a split's previous split in its node: needed only until NodeInit,
     // long before the groups' first use of fp
     uint32_t *prevle = fp;
     uint32_t *unit = W.take<uint32_t>(n);
@@ -1590,7 +1766,7 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
     cudaEventRecord(e0, s);
 
     // a1, a2
-    // the masses are checked where they are first read (k_permute), so that a
+    // the masses are checked where they are first read (Permute), so that a
     // host copy of them can still be in flight here
     // one box: the keys and the permutation are sorted in place in the tree
     if (B == 1) {
@@ -1624,8 +1800,9 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
         cudaMemcpyAsync(t->perm, idx_alt, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
     }
     if (t->mass_ready) cudaStreamWaitEvent(s, t->mass_ready, 0);
-    launch_pdl(k_permute, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, d_mass, t->io, t->sseg, t->seg_off, t->px, t->py, t->pz, t->pm32,
-                                     t->pm64, t->inv, t->mbits, status);
+    const bool share = n <= kShareMax;
+    const Permute permute{n, t->perm, q4, d_mass, t->io, t->sseg, t->seg_off, t->px, t->py, t->pz, t->pm32, t->pm64,
+                          t->inv, t->mbits, status};
     // a4: nodes from splits.  The node count stays on the device (d_tot[0]
     // counts the first splits, m = B + that): the kernels up to the groups
     // read it there and are sized for the most nodes a tree can have, so the
@@ -1636,45 +1813,77 @@ og_status build_tree(og_tree *t, const double *d_pos, const double *d_mass) {
         const int64_t ntiles = (nsplit + kSplitTile - 1) / kSplitTile;
         int *tlast = tsum, *tfirst = tsum + ntiles * kNT;
         int *clast = tsum + 2 * ntiles * kNT, *cfirst = tsum + 3 * ntiles * kNT;
-        launch_pdl(k_split_tiles, dim3((unsigned)ntiles), kSplitTile, 0, s, t->skey, t->sseg, nsplit, lv, tlast,
-                   tfirst);
+        const SplitTiles tiles{t->skey, t->sseg, nsplit, lv, tlast, tfirst};
+        if (share) {
+            run_stages<kSplitTile>(s, (unsigned)((n + kSplitTile - 1) / kSplitTile), permute, (unsigned)ntiles, tiles);
+        } else {
+            run_stage<kT>(s, nblk(n), permute);
+            run_stage<kSplitTile>(s, (unsigned)ntiles, tiles);
+        }
         launch_pdl(k_split_carry, dim3(kNT), kSplitTile, 0, s, ntiles, (const int *)tlast, (const int *)tfirst,
                    clast, cfirst);
         launch_pdl(k_split_ranges, dim3((unsigned)ntiles), kSplitTile, 0, s, (const uint8_t *)lv, nsplit,
                    (const int *)clast, (const int *)cfirst, sbeg, send, first, prevle);
         scan_exclusive_u32_look(first, nid, nsplit, d_tot, scan_look, scan_ctr + 0, 1, status, scan_scratch, s);
+    } else {
+        run_stage<kT>(s, nblk(n), permute);
     }
     const uint32_t *nsp = d_tot;
     // (mcap = n + B covers the splits and the roots too.)  Child counts beyond
     // the last node stay 0, so the scan over mcap entries gives the nodes'
     // child offsets and, as its total, the child entries.
-    launch_pdl(k_node_init, nblk(mcap), kT, 0, s, n, B, t->seg_off, first, nid, lv, sbeg, send, prevle,
-               t->sseg, t->nlev, t->nbeg, t->nend, sid, mcap, occ, nnc, t->nccnt,
-               status);
-    launch_pdl(k_link, nblk(n + mcap), kT, 0, s, n, nsp, B, t->skey, lv, sid, t->sseg, t->nlev, t->nbeg,
-                                         t->nend, t->npar, t->owner, occ, nnc, status);
-    launch_pdl(k_ccnt, nblk(mcap), kT, 0, s, nsp, B, t->nlev, t->nbeg, t->nend, occ, t->nccnt);
-    scan_exclusive_u32_look(t->nccnt, t->ncbeg, mcap, d_tot + 1, scan_look, scan_ctr + 1, 2, status, scan_scratch, s);
-    launch_pdl(k_place, nblk(n + mcap), kT, 0, s, n, nsp, B, t->skey, t->nlev, t->nbeg, t->ncbeg, occ,
-                                          t->npar, t->owner, t->child, t->npos, status);
-    launch_pdl(k_threading, nblk(ccap), kT, 0, s, n, nsp, B, t->child, t->ncbeg, t->nccnt, t->npar,
-                                          t->npos, t->owner, t->nnext, t->nsib, t->pnext, status);
+    const NodeInit node_init{n, B, t->seg_off, first, nid, lv, sbeg, send, prevle, t->sseg, t->nlev, t->nbeg, t->nend,
+                             sid, mcap, occ, nnc, t->nccnt, status};
+    const Link link{n, nsp, B, t->skey, lv, sid, t->sseg, t->nlev, t->nbeg, t->nend, t->npar, t->owner, occ, nnc,
+                    status};
+    const ChildCount child_count{nsp, B, t->nlev, t->nbeg, t->nend, occ, t->nccnt};
+    const Place place{n, nsp, B, t->skey, t->nlev, t->nbeg, t->ncbeg, occ, t->npar, t->owner, t->child, t->npos,
+                      status};
+    const Threading threading{n, nsp, B, t->child, t->ncbeg, t->nccnt, t->npar, t->npos, t->owner, t->nnext, t->nsib,
+                              t->pnext, status};
     // a5: exact moments and centres of mass of every node (in units fixed by
-    // the masses' set-bit span, which k_permute gathered)
-    node_moments(t, nsp, mcap, mom_scratch, s);
+    // the masses' set-bit span, which Permute gathered)
+    const Moments mom(t, mom_scratch);
     // a6: groups (one group size for the whole forest)
     const int G = t->prm.group_max;
-    launch_pdl(k_frontier, nblk(n), kT, 0, s, n, B, G, t->owner, t->npar, t->nbeg, t->nend, fp, unit, rs);
-    scan_inclusive_max_u32_look(rs, rs, n, scan_look, scan_ctr + 2, 3, status, scan_scratch, s);
-    launch_pdl(k_groupmark, nblk(n), kT, 0, s, n, G, rs, fp, unit, t->nbeg, t->nend, gs);
-    // group starts, compacted into gbeg; their count to d_tot[2]
-    scan_compact_u32_look(gs, t->gbeg, n, d_tot + 2, scan_look, scan_ctr + 3, 4, status, scan_scratch, s);
-    // group count (d_tot[2]) and child count (d_tot[1]) from the device
-    launch_pdl(k_group_fin, stride_grid(n), kT, 0, s, n, d_tot + 2, 0, t->gbeg, t->gend, t->px, t->py, t->pz,
-                                              t->sseg, t->gbox, t->gseg);
-    launch_pdl(k_records, stride_grid(ccap), kT, 0, s, n, d_tot + 1, 0, ccap, t->child, t->px, t->py, t->pz,
-                                               t->pm32, t->pm64, t->nlev, t->ncbeg, t->nccnt, t->nmom,
-                                               t->ncom, t->crec, status);
+    const Frontier frontier{n, B, G, t->owner, t->npar, t->nbeg, t->nend, fp, unit, rs};
+    const GroupMark group_mark{n, G, rs, fp, unit, t->nbeg, t->nend, gs};
+    // the group count (d_tot[2]) and child count (d_tot[1]) from the device
+    const GroupFin group_fin{n, d_tot + 2, 0, t->gbeg, t->gend, t->px, t->py, t->pz, t->sseg, t->gbox, t->gseg};
+    const Records records{n, d_tot + 1, 0, ccap, t->child, t->px, t->py, t->pz, t->pm32, t->pm64, t->nlev, t->ncbeg,
+                          t->nccnt, t->nmom, t->ncom, t->crec, status};
+    if (share) {
+        run_stages<kT>(s, nblk(mcap), node_init, (unsigned)mom.ntiles, mom.tiles());
+        run_stages<kT>(s, nblk(n + mcap), link, (unsigned)mom.nblocks, mom.scan1());
+        run_stages<kT>(s, 1, mom.scan2(), nblk(n), frontier, nblk(mcap), child_count);
+        scan_sum_and_max_u32_look(t->nccnt, t->ncbeg, mcap, d_tot + 1, scan_ctr + 1, 2, rs, rs, n, scan_ctr + 2, 3,
+                                  scan_look, scan_look_max, status, scan_scratch, s);
+        run_stages<kT>(s, nblk(n + mcap), place, nblk(n), group_mark);
+        mom.prefix(s);
+        // group starts, compacted into gbeg; their count to d_tot[2]
+        scan_compact_u32_look(gs, t->gbeg, n, d_tot + 2, scan_look, scan_ctr + 3, 4, status, scan_scratch, s);
+        run_stages<kT>(s, Moments::node_blocks(mcap), mom.nodes(nsp, mcap), nblk(ccap), threading);
+        run_stages<kT>(s, stride_grid(ccap), records, stride_grid(n), group_fin);
+    } else {
+        run_stage<kT>(s, nblk(mcap), node_init);
+        run_stage<kT>(s, nblk(n + mcap), link);
+        run_stage<kT>(s, nblk(mcap), child_count);
+        scan_exclusive_u32_look(t->nccnt, t->ncbeg, mcap, d_tot + 1, scan_look, scan_ctr + 1, 2, status, scan_scratch,
+                                s);
+        run_stage<kT>(s, nblk(n + mcap), place);
+        run_stage<kT>(s, nblk(ccap), threading);
+        run_stage<kT>(s, (unsigned)mom.ntiles, mom.tiles());
+        run_stage<kT>(s, (unsigned)mom.nblocks, mom.scan1());
+        run_stage<kT>(s, 1, mom.scan2());
+        mom.prefix(s);
+        run_stage<kT>(s, Moments::node_blocks(mcap), mom.nodes(nsp, mcap));
+        run_stage<kT>(s, nblk(n), frontier);
+        scan_inclusive_max_u32_look(rs, rs, n, scan_look, scan_ctr + 2, 3, status, scan_scratch, s);
+        run_stage<kT>(s, nblk(n), group_mark);
+        scan_compact_u32_look(gs, t->gbeg, n, d_tot + 2, scan_look, scan_ctr + 3, 4, status, scan_scratch, s);
+        run_stage<kT>(s, stride_grid(n), group_fin);
+        run_stage<kT>(s, stride_grid(ccap), records);
+    }
     cudaEventRecord(e1, s);
     // the counts and the status word, read once the build is complete (its
     // only host synchronisation)

@@ -288,6 +288,13 @@ void scan_inclusive_max_u32_look(const uint32_t *in, uint32_t *out, int64_t n, u
                                  uint32_t *ctr, uint32_t tag, uint32_t *status, void *scratch,
                                  cudaStream_t s);
 
+// the sum scan and the maximum scan above of two arrays, in one launch where both take
+// the one-kernel form (its 2 to 4 us are mostly launch and latency); each its own look words
+void scan_sum_and_max_u32_look(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *d_total, uint32_t *ctr,
+                               uint32_t tag, const uint32_t *in2, uint32_t *out2, int64_t n2, uint32_t *ctr2,
+                               uint32_t tag2, unsigned long long *look, unsigned long long *look2, uint32_t *status,
+                               void *scratch, cudaStream_t s);
+
 // radix sort of (key, value) pairs, stable, keys of `bits` significant bits
 size_t radix_sort_scratch_bytes(int64_t n);
 void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt,
@@ -302,14 +309,6 @@ unsigned long long *radix_sort_clear(int64_t n, void *scratch, int64_t *words);
 void radix_sort_pairs_every_pass(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt,
                                  uint32_t *vals_alt, int64_t n, int bits, void *scratch,
                                  cudaStream_t s);
-
-// exact node moments (og_moments.cu): prefix sums over the sorted particles,
-// then every node's mass, sums and centre of mass.  The node count is
-// B + *d_nsplit (device) or, with d_nsplit null, t->nnodes; at most mcap.
-size_t moments_scratch_bytes(int64_t n);
-// t->mbits holds the lowest and highest set-bit exponents over the masses
-// (gathered by the build's k_permute with mass_bit_span)
-void node_moments(og_tree *t, const uint32_t *d_nsplit, int64_t mcap, void *scratch, cudaStream_t s);
 
 // lowest and highest set-bit exponents of a mass: m = s 2^e (s < 2^53) has
 // bits from 2^lo to below 2^hi; zero, negative and non-finite masses have none

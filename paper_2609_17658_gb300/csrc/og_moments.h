@@ -1,3 +1,4 @@
+#pragma once
 // a5: node moments (mass, sum of m x per axis) and centres of mass, exact.
 //
 // Monopole moments in double precision from the particles up (paper Sect.
@@ -16,13 +17,13 @@
 // tree level.
 //
 //   (the lowest and highest set bit over all masses come from the build's
-//   k_permute, which reads the masses first)
-//   k_mom_tiles      per tile of 512 sorted particles: the sums of the tile
-//   k_mom_scan_l1/2  exclusive prefix over the tiles, in two levels (blocks of
+//   Permute, which reads the masses first)
+//   MomTiles         per tile of 512 sorted particles: the sums of the tile
+//   MomScan1, 2      exclusive prefix over the tiles, in two levels (blocks of
 //                    256 tiles, then the block totals)
 //   k_mom_prefix     per particle: exclusive prefix P[i] = sum over q < i,
 //                    and P[n], 96 bytes per entry
-//   k_node_moments   per node: P[end] - P[begin], rounded to FP64, and the
+//   NodeMoments      per node: P[end] - P[begin], rounded to FP64, and the
 //                    rounded ratio for the centre of mass
 #include "og_internal.h"
 
@@ -33,7 +34,7 @@ constexpr int kMomThreads = 256;
 constexpr int kMomItems = 2;                        // consecutive particles per thread
 constexpr int kMomTile = kMomThreads * kMomItems;   // 512
 constexpr int kScanBlock = 256;                      // tiles per block of the first scan level
-constexpr int kScanTop = 512;                        // threads of the second level
+constexpr int kScanTop = 256;                        // threads of the second level
 // a warp's 64 prefix records staged in shared memory before they are written
 // out as contiguous 512-byte runs: 2 records per lane, 16 bytes of padding per
 // lane so that the lanes' 16-byte stores fall in distinct banks
@@ -274,10 +275,10 @@ __device__ __forceinline__ void block_scan(const Mom192 &x, Mom192 &excl, Mom192
     __syncthreads();                           // wsum may be reused by the caller
 }
 
-__device__ __forceinline__ bool span_ok(const int *mbits, uint32_t *status) {
+__device__ __forceinline__ bool span_ok(const int *mbits, uint32_t *status, uint32_t bid) {
     const int lo = mbits[0], hi = mbits[1];
     if (hi >= lo && hi - lo > kMassSpanMax) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, ST_MASS_RANGE);
+        if (bid == 0 && threadIdx.x == 0) atomicOr(status, ST_MASS_RANGE);
         return false;
     }
     return true;
@@ -308,80 +309,93 @@ __device__ __forceinline__ void load_pair(int64_t n, int64_t q0, const double *_
 }
 
 // the sums of one tile (the order of the additions does not matter: exact)
-__global__ void __launch_bounds__(kMomThreads) k_mom_tiles(int64_t n, const double *__restrict__ pm64,
-                                                           const uint32_t *__restrict__ px,
-                                                           const uint32_t *__restrict__ py,
-                                                           const uint32_t *__restrict__ pz,
-                                                           const int *__restrict__ mbits,
-                                                           Mom192 *tile_sum, uint32_t *status) {
-    pdl_wait();
-    if (!span_ok(mbits, status)) return;
-    const int b = mbits[0];
-    const int64_t q0 = (int64_t)blockIdx.x * kMomTile + (int64_t)threadIdx.x * kMomItems;
-    __shared__ Mom192 wsum[kMomThreads / 32];
-    Mom192 v0, v1;
-    load_pair(n, q0, pm64, px, py, pz, b, v0, v1);
-    mom_add(v0, v1);
-    // the tile's total: a butterfly over the warp (sums modulo 2^192 do not
-    // depend on the order), then the warps' totals
+struct MomTiles {
+    int64_t n;
+    const double *__restrict__ pm64;
+    const uint32_t *__restrict__ px;
+    const uint32_t *__restrict__ py;
+    const uint32_t *__restrict__ pz;
+    const int *__restrict__ mbits;
+    Mom192 *tile_sum;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        if (!span_ok(mbits, status, bid)) return;
+        const int b = mbits[0];
+        const int64_t q0 = (int64_t)bid * kMomTile + (int64_t)threadIdx.x * kMomItems;
+        __shared__ Mom192 wsum[kMomThreads / 32];
+        Mom192 v0, v1;
+        load_pair(n, q0, pm64, px, py, pz, b, v0, v1);
+        mom_add(v0, v1);
+        // the tile's total: a butterfly over the warp (sums modulo 2^192 do not
+        // depend on the order), then the warps' totals
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        Mom192 o;
+        for (int d = 16; d > 0; d >>= 1) {
+            Mom192 o;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            o.q[k].w0 = __shfl_xor_sync(0xffffffffu, v0.q[k].w0, d);
-            o.q[k].w1 = __shfl_xor_sync(0xffffffffu, v0.q[k].w1, d);
-            o.q[k].w2 = __shfl_xor_sync(0xffffffffu, v0.q[k].w2, d);
+            for (int k = 0; k < 4; ++k) {
+                o.q[k].w0 = __shfl_xor_sync(0xffffffffu, v0.q[k].w0, d);
+                o.q[k].w1 = __shfl_xor_sync(0xffffffffu, v0.q[k].w1, d);
+                o.q[k].w2 = __shfl_xor_sync(0xffffffffu, v0.q[k].w2, d);
+            }
+            mom_add(v0, o);
         }
-        mom_add(v0, o);
-    }
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        Mom192 t = wsum[0];
+        if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v0;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            Mom192 t = wsum[0];
 #pragma unroll
-        for (int w = 1; w < kMomThreads / 32; ++w) mom_add(t, wsum[w]);
-        store_mom(&tile_sum[blockIdx.x], t);
+            for (int w = 1; w < kMomThreads / 32; ++w) mom_add(t, wsum[w]);
+            store_mom(&tile_sum[bid], t);
+        }
     }
-}
+};
 
 // first level: each block turns its kScanBlock tile sums into exclusive
 // prefixes within the block (in place) and stores its total
-__global__ void __launch_bounds__(kScanBlock) k_mom_scan_l1(int64_t ntiles, const int *__restrict__ mbits,
-                                                            Mom192 *tile_sum, Mom192 *block_sum,
-                                                            uint32_t *status) {
-    pdl_wait();
-    if (!span_ok(mbits, status)) return;
-    const int64_t k = (int64_t)blockIdx.x * kScanBlock + threadIdx.x;
-    Mom192 v, excl, total;
-    if (k < ntiles) v = load_mom(&tile_sum[k]);
-    else mom_zero(v);
-    block_scan<kScanBlock>(v, excl, total);
-    if (k < ntiles) store_mom(&tile_sum[k], excl);
-    if (threadIdx.x == 0) store_mom(&block_sum[blockIdx.x], total);
-}
+struct MomScan1 {
+    int64_t ntiles;
+    const int *__restrict__ mbits;
+    Mom192 *tile_sum;
+    Mom192 *block_sum;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        if (!span_ok(mbits, status, bid)) return;
+        const int64_t k = (int64_t)bid * kScanBlock + threadIdx.x;
+        Mom192 v, excl, total;
+        if (k < ntiles) v = load_mom(&tile_sum[k]);
+        else mom_zero(v);
+        block_scan<kScanBlock>(v, excl, total);
+        if (k < ntiles) store_mom(&tile_sum[k], excl);
+        if (threadIdx.x == 0) store_mom(&block_sum[bid], total);
+    }
+};
 
 // second level: exclusive prefixes of the block totals (in place, several
 // per thread when there are more than kScanTop), the grand total to P[n]
-__global__ void __launch_bounds__(kScanTop) k_mom_scan_l2(int64_t nblocks, const int *__restrict__ mbits,
-                                                          Mom192 *block_sum, unsigned char *P, int64_t n,
-                                                          uint32_t *status) {
-    pdl_wait();
-    if (!span_ok(mbits, status)) return;
-    const int64_t per = (nblocks + kScanTop - 1) / kScanTop;
-    const int64_t k0 = (int64_t)threadIdx.x * per;
-    const int64_t k1 = k0 + per < nblocks ? k0 + per : nblocks;
-    Mom192 s, excl, total;
-    mom_zero(s);
-    for (int64_t k = k0; k < k1; ++k) mom_add(s, load_mom(&block_sum[k]));
-    block_scan<kScanTop>(s, excl, total);
-    for (int64_t k = k0; k < k1; ++k) {
-        const Mom192 v = load_mom(&block_sum[k]);
-        store_mom(&block_sum[k], excl);
-        mom_add(excl, v);
+struct MomScan2 {
+    int64_t nblocks;
+    const int *__restrict__ mbits;
+    Mom192 *block_sum;
+    unsigned char *P;
+    int64_t n;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        if (!span_ok(mbits, status, bid)) return;
+        const int64_t per = (nblocks + kScanTop - 1) / kScanTop;
+        const int64_t k0 = (int64_t)threadIdx.x * per;
+        const int64_t k1 = k0 + per < nblocks ? k0 + per : nblocks;
+        Mom192 s, excl, total;
+        mom_zero(s);
+        for (int64_t k = k0; k < k1; ++k) mom_add(s, load_mom(&block_sum[k]));
+        block_scan<kScanTop>(s, excl, total);
+        for (int64_t k = k0; k < k1; ++k) {
+            const Mom192 v = load_mom(&block_sum[k]);
+            store_mom(&block_sum[k], excl);
+            mom_add(excl, v);
+        }
+        if (threadIdx.x == 0) store_prefix(P, n, total, short_prefix(mbits));
     }
-    if (threadIdx.x == 0) store_prefix(P, n, total, short_prefix(mbits));
-}
+};
 
 // Per particle the exclusive prefix: the tile's offset (both scan levels)
 // plus the prefix within the tile.  Thread t owns the items 2t, 2t + 1 of the
@@ -398,7 +412,7 @@ __global__ void __launch_bounds__(kMomThreads) k_mom_prefix(int64_t n, const dou
                                                             unsigned char *P, uint32_t *status) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char stage_all[];
-    if (!span_ok(mbits, status)) return;
+    if (!span_ok(mbits, status, blockIdx.x)) return;
     const int b = mbits[0];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t tile0 = (int64_t)blockIdx.x * kMomTile;
@@ -550,84 +564,106 @@ __device__ __forceinline__ uint32_t round_ratio(const U192 &S, const U192 &M, in
 }
 
 // one thread per node; m = B + *nsplit (the build) or m_host (a refit)
-__global__ void __launch_bounds__(kMomThreads) k_node_moments(
-    const uint32_t *__restrict__ nsplit, int64_t B, int64_t m_host, int64_t mcap,
-    const uint32_t *__restrict__ nbeg, const uint32_t *__restrict__ nend,
-    const uint8_t *__restrict__ nlev, const uint32_t *__restrict__ px,
-    const uint32_t *__restrict__ py, const uint32_t *__restrict__ pz,
-    const unsigned char *__restrict__ P, const int *__restrict__ mbits, NodeMom *nmom, uint32_t *ncom,
-    uint32_t *status) {
-    pdl_wait();
-    if (!span_ok(mbits, status)) return;
-    int64_t m = nsplit ? B + (int64_t)*nsplit : m_host;
-    if (m > mcap) m = mcap;                    // the host reports the overflow
-    const int b = mbits[0];
-    const bool shrt = short_prefix(mbits);
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t q0 = nbeg[j], q1 = nend[j];
-        const Mom192 D = prefix_diff(P, q0, q1, shrt);
-        nmom[j] = NodeMom{to_double(D.q[0], b), to_double(D.q[1], b), to_double(D.q[2], b),
-                          to_double(D.q[3], b)};
-        uint32_t c[3];
-        if (!is_zero192(D.q[0])) {
-            const int pM = top192(D.q[0]);
-            const float rM = rcp_approx(top24(D.q[0], pM));
-            c[0] = round_ratio(D.q[1], D.q[0], pM, rM, status);
-            c[1] = round_ratio(D.q[2], D.q[0], pM, rM, status);
-            c[2] = round_ratio(D.q[3], D.q[0], pM, rM, status);
-        } else {
-            // massless node: the cell centre
-            const int level = nlev[j];
-            const uint64_t mask = level == 0 ? 0ull : ~((1ull << (32 - level)) - 1ull);
-            const uint32_t pc[3] = {px[q0], py[q0], pz[q0]};
-            for (int a = 0; a < 3; ++a)
-                c[a] = (uint32_t)(((uint64_t)pc[a] & mask) + (1ull << (31 - level)));
+struct NodeMoments {
+    const uint32_t *__restrict__ nsplit;
+    int64_t B;
+    int64_t m_host;
+    int64_t mcap;
+    const uint32_t *__restrict__ nbeg;
+    const uint32_t *__restrict__ nend;
+    const uint8_t *__restrict__ nlev;
+    const uint32_t *__restrict__ px;
+    const uint32_t *__restrict__ py;
+    const uint32_t *__restrict__ pz;
+    const unsigned char *__restrict__ P;
+    const int *__restrict__ mbits;
+    NodeMom *nmom;
+    uint32_t *ncom;
+    uint32_t *status;
+    __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        if (!span_ok(mbits, status, bid)) return;
+        int64_t m = nsplit ? B + (int64_t)*nsplit : m_host;
+        if (m > mcap) m = mcap;                    // the host reports the overflow
+        const int b = mbits[0];
+        const bool shrt = short_prefix(mbits);
+        for (int64_t j = (int64_t)bid * blockDim.x + threadIdx.x; j < m;
+             j += (int64_t)nb * blockDim.x) {
+            const uint32_t q0 = nbeg[j], q1 = nend[j];
+            const Mom192 D = prefix_diff(P, q0, q1, shrt);
+            nmom[j] = NodeMom{to_double(D.q[0], b), to_double(D.q[1], b), to_double(D.q[2], b),
+                              to_double(D.q[3], b)};
+            uint32_t c[3];
+            if (!is_zero192(D.q[0])) {
+                const int pM = top192(D.q[0]);
+                const float rM = rcp_approx(top24(D.q[0], pM));
+                c[0] = round_ratio(D.q[1], D.q[0], pM, rM, status);
+                c[1] = round_ratio(D.q[2], D.q[0], pM, rM, status);
+                c[2] = round_ratio(D.q[3], D.q[0], pM, rM, status);
+            } else {
+                // massless node: the cell centre
+                const int level = nlev[j];
+                const uint64_t mask = level == 0 ? 0ull : ~((1ull << (32 - level)) - 1ull);
+                const uint32_t pc[3] = {px[q0], py[q0], pz[q0]};
+                for (int a = 0; a < 3; ++a)
+                    c[a] = (uint32_t)(((uint64_t)pc[a] & mask) + (1ull << (31 - level)));
+            }
+            ncom[3 * j + 0] = c[0];
+            ncom[3 * j + 1] = c[1];
+            ncom[3 * j + 2] = c[2];
         }
-        ncom[3 * j + 0] = c[0];
-        ncom[3 * j + 1] = c[1];
-        ncom[3 * j + 2] = c[2];
     }
-}
+};
 
-inline int64_t mom_tiles(int64_t n) { return (n + kMomTile - 1) / kMomTile; }
+inline int64_t mom_ntiles(int64_t n) { return (n + kMomTile - 1) / kMomTile; }
 
-}  // namespace
-
-size_t moments_scratch_bytes(int64_t n) {
+// scratch of the moments of n particles
+inline size_t moments_scratch_bytes(int64_t n) {
     const auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t nt = (size_t)(mom_tiles(n) > 0 ? mom_tiles(n) : 1);
+    const size_t nt = (size_t)(mom_ntiles(n) > 0 ? mom_ntiles(n) : 1);
     const size_t nb = (nt + kScanBlock - 1) / kScanBlock;
     return up((size_t)(n + 1) * sizeof(Mom192)) + up(nt * sizeof(Mom192)) + up(nb * sizeof(Mom192)) + 256;
 }
 
-void node_moments(og_tree *t, const uint32_t *d_nsplit, int64_t mcap, void *scratch, cudaStream_t s) {
-    const int64_t n = t->n;
-    const int64_t ntiles = mom_tiles(n);
-    const int64_t nblocks = (ntiles + kScanBlock - 1) / kScanBlock;
-    const auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    char *q = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(scratch) + 255) & ~(uintptr_t)255);
-    unsigned char *P = reinterpret_cast<unsigned char *>(q);   // 64- or 96-byte records
-    q += up((size_t)(n + 1) * sizeof(Mom192));
-    Mom192 *tiles = reinterpret_cast<Mom192 *>(q);
-    q += up((size_t)ntiles * sizeof(Mom192));
-    Mom192 *blocks = reinterpret_cast<Mom192 *>(q);
-    uint32_t *status = t->ctx->d_status;
-    launch_pdl(k_mom_tiles, (unsigned)ntiles, kMomThreads, 0, s, n, t->pm64, t->px, t->py, t->pz, t->mbits,
-                                                         tiles, status);
-    launch_pdl(k_mom_scan_l1, (unsigned)nblocks, kScanBlock, 0, s, ntiles, t->mbits, tiles, blocks, status);
-    launch_pdl(k_mom_scan_l2, 1, kScanTop, 0, s, nblocks, t->mbits, blocks, P, n, status);
-    // the stage is above the default 48 KB of shared memory (set per call: the
-    // attribute belongs to the current device)
-    cudaFuncSetAttribute(k_mom_prefix, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (kMomThreads / 32) * kWarpStage);
-    launch_pdl(k_mom_prefix, (unsigned)ntiles, kMomThreads, (kMomThreads / 32) * kWarpStage, s, 
-        n, t->pm64, t->px, t->py, t->pz, t->mbits, tiles, blocks, P, status);
-    const int64_t mb = (mcap + kMomThreads - 1) / kMomThreads;
-    const unsigned grid = (unsigned)(mb < 4096 ? (mb > 0 ? mb : 1) : 4096);
-    launch_pdl(k_node_moments, grid, kMomThreads, 0, s, d_nsplit, t->nseg, t->nnodes, mcap, t->nbeg, t->nend,
-                                                t->nlev, t->px, t->py, t->pz, P, t->mbits, t->nmom,
-                                                t->ncom, status);
-}
+// The stages in order (tiles, scan1, scan2, prefix, nodes), for the build's and the
+// refit's chains to place beside kernels that do not depend on them.
+struct Moments {
+    og_tree *t;
+    int64_t n, ntiles, nblocks;
+    unsigned char *P;                // 64- or 96-byte records
+    Mom192 *tile, *block;
+    uint32_t *status;
+    Moments(og_tree *tree, void *scratch) : t(tree), n(tree->n), ntiles(mom_ntiles(tree->n)) {
+        nblocks = (ntiles + kScanBlock - 1) / kScanBlock;
+        const auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+        char *q = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(scratch) + 255) & ~(uintptr_t)255);
+        P = reinterpret_cast<unsigned char *>(q);
+        q += up((size_t)(n + 1) * sizeof(Mom192));
+        tile = reinterpret_cast<Mom192 *>(q);
+        q += up((size_t)ntiles * sizeof(Mom192));
+        block = reinterpret_cast<Mom192 *>(q);
+        status = t->ctx->d_status;
+    }
+    MomTiles tiles() const { return {n, t->pm64, t->px, t->py, t->pz, t->mbits, tile, status}; }
+    MomScan1 scan1() const { return {ntiles, t->mbits, tile, block, status}; }
+    MomScan2 scan2() const { return {nblocks, t->mbits, block, P, n, status}; }
+    void prefix(cudaStream_t s) const {
+        // the stage is above the default 48 KB of shared memory (set per call: the
+        // attribute belongs to the current device)
+        const int smem = (kMomThreads / 32) * kWarpStage;
+        cudaFuncSetAttribute(k_mom_prefix, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        launch_pdl(k_mom_prefix, (unsigned)ntiles, kMomThreads, smem, s, n, t->pm64, t->px, t->py, t->pz, t->mbits,
+                   tile, block, P, status);
+    }
+    // m = nseg + *d_nsplit nodes (the build, before the host knows it) or mcap (a refit)
+    NodeMoments nodes(const uint32_t *d_nsplit, int64_t mcap) const {
+        return {d_nsplit, t->nseg, t->nnodes, mcap, t->nbeg, t->nend, t->nlev, t->px, t->py, t->pz,
+                P, t->mbits, t->nmom, t->ncom, status};
+    }
+    static unsigned node_blocks(int64_t mcap) {
+        const int64_t mb = (mcap + kMomThreads - 1) / kMomThreads;
+        return (unsigned)(mb < 4096 ? (mb > 0 ? mb : 1) : 4096);
+    }
+};
 
+}  // namespace
 }  // namespace og

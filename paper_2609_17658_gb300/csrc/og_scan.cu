@@ -159,11 +159,9 @@ template <>
 __device__ __forceinline__ uint32_t warp_fold<OpMax>(uint32_t v) { return __reduce_max_sync(0xffffffffu, v); }
 
 template <class Op, bool kExclusive>
-__global__ void __launch_bounds__(kScanThreads) k_scan_look(const uint32_t *in, uint32_t *out, int64_t n,
-                                                            unsigned long long *look, uint32_t *ctr,
-                                                            unsigned long long tag, uint32_t *d_total,
-                                                            uint32_t *compact, uint32_t *status) {
-    pdl_wait();
+__device__ __forceinline__ void scan_look(const uint32_t *in, uint32_t *out, int64_t n, unsigned long long *look,
+                                          uint32_t *ctr, unsigned long long tag, uint32_t *d_total,
+                                          uint32_t *compact, uint32_t *status) {
     __shared__ uint32_t s_items[kScanTile];
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_tile, s_pre;
@@ -251,6 +249,32 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_look(const uint32_t *in, 
 }
 
 template <class Op, bool kExclusive>
+__global__ void __launch_bounds__(kScanThreads) k_scan_look(const uint32_t *in, uint32_t *out, int64_t n,
+                                                            unsigned long long *look, uint32_t *ctr,
+                                                            unsigned long long tag, uint32_t *d_total,
+                                                            uint32_t *compact, uint32_t *status) {
+    pdl_wait();
+    scan_look<Op, kExclusive>(in, out, n, look, ctr, tag, d_total, compact, status);
+}
+
+// two independent scans in one launch: blocks [0, na) the sums, the rest the maxima
+struct ScanJob {
+    const uint32_t *in;
+    uint32_t *out;
+    int64_t n;
+    unsigned long long *look;
+    uint32_t *ctr;
+    unsigned long long tag;
+    uint32_t *d_total;
+};
+__global__ void __launch_bounds__(kScanThreads) k_scan_look_two(const ScanJob a, uint32_t na, const ScanJob b,
+                                                                uint32_t *status) {
+    pdl_wait();
+    if (blockIdx.x < na) scan_look<OpSum, true>(a.in, a.out, a.n, a.look, a.ctr, a.tag, a.d_total, nullptr, status);
+    else scan_look<OpMax, false>(b.in, b.out, b.n, b.look, b.ctr, b.tag, b.d_total, nullptr, status);
+}
+
+template <class Op, bool kExclusive>
 void scan_impl(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *d_total, void *scratch,
                cudaStream_t s, uint32_t *compact = nullptr) {
     if (n <= 0) {
@@ -313,6 +337,21 @@ void scan_inclusive_max_u32_look(const uint32_t *in, uint32_t *out, int64_t n, u
     }
     launch_pdl(k_scan_look<OpMax, false>, (unsigned)ntiles, kScanThreads, 0, s, in, out, n, look, ctr,
                (unsigned long long)tag, (uint32_t *)nullptr, (uint32_t *)nullptr, status);
+}
+
+void scan_sum_and_max_u32_look(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *d_total, uint32_t *ctr,
+                               uint32_t tag, const uint32_t *in2, uint32_t *out2, int64_t n2, uint32_t *ctr2,
+                               uint32_t tag2, unsigned long long *look, unsigned long long *look2, uint32_t *status,
+                               void *scratch, cudaStream_t s) {
+    const int64_t na = (n + kScanTile - 1) / kScanTile, nb = (n2 + kScanTile - 1) / kScanTile;
+    if (na < 1 || nb < 1 || na > kScanLookMaxTiles || nb > kScanLookMaxTiles) {
+        scan_exclusive_u32_look(in, out, n, d_total, look, ctr, tag, status, scratch, s);
+        scan_inclusive_max_u32_look(in2, out2, n2, look2, ctr2, tag2, status, scratch, s);
+        return;
+    }
+    launch_pdl(k_scan_look_two, (unsigned)(na + nb), kScanThreads, 0, s,
+               ScanJob{in, out, n, look, ctr, (unsigned long long)tag, d_total}, (uint32_t)na,
+               ScanJob{in2, out2, n2, look2, ctr2, (unsigned long long)tag2, nullptr}, status);
 }
 
 og_status scan_wait_timeout_probe(og_ctx *c, int64_t n) {

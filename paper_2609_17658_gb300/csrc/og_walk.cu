@@ -839,7 +839,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                                       : classify<kOpen, kSplit, kRefit>(T, ci0, has0, box, p, arelf, arel);
                 const Cls c1 = kShort ? classify_short<kOpen, kSplit, kRefit>(T, ci1, has1, box, p, arelf, arel)
                                       : classify<kOpen, kSplit, kRefit>(T, ci1, has1, box, p, arelf, arel);
-                // push opened ranges (k_records has checked that every node has
+                // push opened ranges (the stage Records has checked that every node has
                 // children, inside the child array)
                 const unsigned bo0 = __ballot_sync(FULL, c0.open), bo1 = __ballot_sync(FULL, c1.open);
                 const int np0 = __popc(bo0), npush = np0 + __popc(bo1);
