@@ -301,7 +301,8 @@ void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32
                       int64_t n, int bits, void *scratch, cudaStream_t s, bool *result_in_alt,
                       uint32_t *status, bool cleared = false);
 // the 64-bit words of the scratch that a sort of n pairs wants cleared: a caller whose
-// own kernel clears them passes cleared and saves the memset
+// own kernel clears them passes cleared and saves the memset (none where the sort is one
+// launch of a cluster)
 unsigned long long *radix_sort_clear(int64_t n, void *scratch, int64_t *words);
 
 // the same sort with every digit pass run (no histogram read-back, no host

@@ -15,7 +15,11 @@
 // copy their input.  Sorts of at most kOneSweepMaxTiles tiles (small sorts
 // are bound by launch latency) run each pass as one kernel instead: the
 // global digit bases come from that histogram, and a tile's offsets within
-// its digit from a look-back over the counts the tiles before it publish.
+// its digit from a look-back over the counts the tiles before it publish.  Up to
+// kClusterMax keys all passes are one launch (k_cluster_sort).
+#include <map>
+#include <mutex>
+
 #include "og_internal.h"
 
 namespace og {
@@ -358,6 +362,299 @@ __global__ void __launch_bounds__(kThreads, 4) k_onesweep(const uint64_t *__rest
     }
 }
 
+// ---- small sorts: all passes in one kernel of one cluster
+//
+// A pass of a small sort is a chain of latencies (launch, tile ticket, loads, ranking,
+// look-back, stores) of some 7 us that does not get shorter with fewer keys.  Up to
+// kClusterMax keys the whole sort is one launch of a cluster of 16 blocks: the keys
+// stay in the blocks' shared memory, a block sends its digit counts and then its keys
+// into the others' (asynchronous stores to distributed shared memory, counted by a
+// barrier of the receiver), and 9-bit digits take 63-bit keys in 7 passes instead
+// of 8.  Block c owns the slots [c slice, (c + 1) slice) of every pass's input.
+// Builds of 4k, 10k, 32k and 65k particles: 107, 114, 122 and 133 us with the passes,
+// 76, 81, 97 and 124 this way (the sort itself 22 us at 4k, 41 at 32k).  A pass's
+// latencies are 2 us (ranking 0.4, the exchange of counts and of keys 0.4 each); above
+// 16k keys 16 SMs' ranking and sending take over, and from some 90k on the passes on
+// the whole chip win.
+// Tried: keys through global memory with two cluster barriers per pass (46 us at 4k;
+// the barrier's release waits for the stores), synchronous remote stores (28 us).
+//
+// What keeps a block from writing where another still reads: it sends counts of
+// pass p + 2, which go where those of pass p were, after it has all counts of pass
+// p + 1, and a block sends those after it has read the ones of pass p; it sends
+// keys of pass p after it has all counts of pass p, and a block sends those after it
+// has sent on the keys of pass p - 1, whose buffer the new ones take.
+constexpr int kClBlocks = 16, kClThreads = 1024, kClWarps = kClThreads / 32;
+constexpr int kClBits = 9, kClRadix = 1 << kClBits, kClPairs = kClRadix / 2;
+constexpr int kClMaxRounds = 4;        // keys per thread
+constexpr int64_t kClusterMax = (int64_t)kClBlocks * kClThreads * kClMaxRounds;
+constexpr int kClWaitLimit = 1 << 16;
+static_assert(kClThreads == 4 * kClPairs && kClThreads == kClBlocks * kClPairs / 4 &&
+                  kClThreads * kClMaxRounds < 65536,
+              "a thread per digit pair and quarter, and per four pairs and block");
+
+template <int kIt>
+struct ClusterSmem {
+    uint4 rec[2][kClThreads * kIt];                // key, value: this pass's input, the next one's
+    uint32_t cnt[2][kClBlocks][kClPairs];          // every block's digit counts (pairs of 16 bits), by parity of the pass
+    uint32_t wcnt[kClWarps][kClPairs];             // per warp: counts, then offsets within the quarter's 8 warps
+    uint32_t quarter[4][kClPairs];                 // per 8 warps: counts
+    uint32_t qpre[4][kClPairs];                    // those of the quarters before
+    uint32_t own[kClPairs];                        // this block's counts
+    uint32_t base[kClRadix];                       // where this block's keys of the digit go
+    uint32_t wsum[kClPairs / 32];
+    unsigned long long cnt_bar[2], rec_bar;        // received counts, by parity; received keys
+};
+
+__device__ __forceinline__ uint32_t shared_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// the same place in block `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(shared_addr(p)), "r"(rank));
+    return a;
+}
+// 16 bytes into another block, counted by a barrier of that block
+__device__ __forceinline__ void cluster_send(uint32_t a, uint32_t bar, uint4 v) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(a),
+                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void bar_expect(void *bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(shared_addr(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bar_wait(void *bar, uint32_t phase, uint32_t *status) {
+    const uint32_t a = shared_addr(bar);
+    for (int it = 0; it < kClWaitLimit; ++it) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok)
+                     : "r"(a), "r"(phase)
+                     : "memory");
+        if (ok) return;
+    }
+    atomicOr(status, ST_TIMEOUT);                  // gives up: what follows stays in bounds
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// in place: keys, vals
+template <int kIt>
+__global__ void __launch_bounds__(kClThreads, 1) k_cluster_sort(uint64_t *keys, uint32_t *vals, uint32_t n,
+                                                                uint32_t slice, int rounds, int npasses,
+                                                                uint32_t *status) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ClusterSmem<kIt> &S = *reinterpret_cast<ClusterSmem<kIt> *>(smem_raw);
+    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    uint32_t cta;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(cta));
+    const uint32_t lo = cta * slice;
+    const uint32_t mine = lo < n ? (n - lo < slice ? n - lo : slice) : 0u;   // keys of this block
+    const uint32_t wfirst = warp * 32u * (uint32_t)rounds;                   // the warp's first slot
+    const uint32_t pair = t & (kClPairs - 1u), qt = t / kClPairs;            // of the per-digit work
+    if (t == 0) {
+        for (void *b : {(void *)&S.cnt_bar[0], (void *)&S.cnt_bar[1], (void *)&S.rec_bar})
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(shared_addr(b)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    cluster_sync();                                // every block has started and its barriers are there
+    pdl_wait();
+    for (uint32_t r = t; r < mine; r += kClThreads) {
+        const uint64_t k = keys[lo + r];
+        S.rec[0][r] = make_uint4((uint32_t)k, (uint32_t)(k >> 32), vals[lo + r], 0u);
+    }
+    int cur = 0;
+    uint32_t moved = 0;                            // passes that moved the keys
+    bool stored = false;
+    for (int pass = 0; pass < npasses; ++pass) {
+        const int shift = kClBits * pass, par = pass & 1;
+        for (uint32_t i = t; i < kClWarps * kClPairs; i += kClThreads) (&S.wcnt[0][0])[i] = 0u;
+        if (t == 0) bar_expect(&S.cnt_bar[par], kClBlocks * kClPairs * 4u);
+        if (moved) bar_wait(&S.rec_bar, (moved - 1u) & 1u, status);
+        __syncthreads();
+        uint16_t *wc = reinterpret_cast<uint16_t *>(S.wcnt[warp]);
+        uint4 rec[kIt];
+        uint32_t rank[kIt];
+        // rank of every key among its warp's keys of the same digit
+#pragma unroll
+        for (int r = 0; r < kIt; ++r) {
+            if (r >= rounds || wfirst + 32u * (uint32_t)r >= mine) break;
+            const uint32_t p = wfirst + 32u * (uint32_t)r + lane;
+            const bool ok = p < mine;
+            rec[r] = ok ? S.rec[cur][p] : make_uint4(0u, 0u, 0u, 0u);
+            const uint64_t key = rec[r].x | (uint64_t)rec[r].y << 32;
+            const uint32_t d = (uint32_t)(key >> shift) & (kClRadix - 1u);
+            unsigned peers = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+            for (int bit = 0; bit < kClBits; ++bit) {
+                const bool on = (d >> bit) & 1u;
+                const unsigned bb = __ballot_sync(0xffffffffu, on);
+                peers &= on ? bb : ~bb;
+            }
+            const uint32_t before = wc[d];
+            __syncwarp();
+            if (ok && (peers & lt_mask) == 0u) wc[d] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+            rank[r] = before + __popc(peers & lt_mask);
+        }
+        __syncthreads();
+        // offsets of the warps within their quarter (pairs of 16-bit sums: a block has
+        // fewer than 2^16 keys), the quarters' counts
+        {
+            uint32_t c[8], run = 0;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) c[w] = S.wcnt[qt * 8 + w][pair];
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                S.wcnt[qt * 8 + w][pair] = run;
+                run += c[w];
+            }
+            S.quarter[qt][pair] = run;
+        }
+        __syncthreads();
+        {
+            uint32_t own = 0, pre = 0;
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                const uint32_t c = S.quarter[q][pair];
+                pre += q < qt ? c : 0u;
+                own += c;
+            }
+            S.qpre[qt][pair] = pre;
+            if (qt == 0) S.own[pair] = own;
+        }
+        __syncthreads();
+        {
+            // four pairs to one block
+            const uint32_t b = t / (kClPairs / 4), q = 4u * (t & (kClPairs / 4 - 1u));
+            cluster_send(cluster_addr(&S.cnt[par][cta][q], b), cluster_addr(&S.cnt_bar[par], b),
+                         *reinterpret_cast<const uint4 *>(&S.own[q]));
+        }
+        bar_wait(&S.cnt_bar[par], (uint32_t)(pass >> 1) & 1u, status);
+        // the digits' counts in all blocks and in those before this one, and their scan
+        uint32_t all_lo = 0, all_hi = 0, bef_lo = 0, bef_hi = 0, sum = 0;
+        if (qt == 0) {
+#pragma unroll
+            for (uint32_t b = 0; b < kClBlocks; ++b) {
+                const uint32_t c = S.cnt[par][b][pair];
+                all_lo += c & 0xffffu;
+                all_hi += c >> 16;
+                bef_lo += b < cta ? c & 0xffffu : 0u;
+                bef_hi += b < cta ? c >> 16 : 0u;
+            }
+            sum = all_lo + all_hi;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, sum, d);
+                if (lane >= (uint32_t)d) sum += o;
+            }
+            if (lane == 31u) S.wsum[warp] = sum;
+        }
+        // one digit holds every key: the order stays
+        stored = !__syncthreads_or(all_lo == n || all_hi == n);
+        if (!stored) continue;
+        const bool last = pass == npasses - 1;
+        if (t == 0 && !last) bar_expect(&S.rec_bar, mine * 16u);
+        if (qt == 0) {
+            uint32_t at = sum - all_lo - all_hi;
+#pragma unroll
+            for (uint32_t w = 0; w < kClPairs / 32; ++w) at += w < warp ? S.wsum[w] : 0u;
+            S.base[2 * pair] = at + bef_lo;
+            S.base[2 * pair + 1] = at + all_lo + bef_hi;
+        }
+        __syncthreads();
+        const uint16_t *qp = reinterpret_cast<const uint16_t *>(S.qpre[warp >> 3]);
+#pragma unroll
+        for (int r = 0; r < kIt; ++r) {
+            if (r >= rounds || wfirst + 32u * (uint32_t)r + lane >= mine) break;
+            const uint64_t key = rec[r].x | (uint64_t)rec[r].y << 32;
+            const uint32_t d = (uint32_t)(key >> shift) & (kClRadix - 1u);
+            const uint32_t g = S.base[d] + qp[d] + wc[d] + rank[r];
+            if (g >= n) {                          // only after a wait that gave up
+                atomicOr(status, ST_TIMEOUT);
+            } else if (last) {
+                keys[g] = key;
+                vals[g] = rec[r].z;
+            } else {
+                const uint32_t b = g / slice;
+                cluster_send(cluster_addr(&S.rec[cur ^ 1][g - b * slice], b), cluster_addr(&S.rec_bar, b), rec[r]);
+            }
+        }
+        cur ^= 1;
+        ++moved;
+        // the next pass clears the warps' counts, which every thread has read
+        __syncthreads();
+    }
+    if (!stored) {
+        // the last pass had nothing to move: the keys are here, or still on their way
+        if (moved) bar_wait(&S.rec_bar, (moved - 1u) & 1u, status);
+        for (uint32_t r = t; r < mine; r += kClThreads) {
+            const uint4 v = S.rec[cur][r];
+            keys[lo + r] = v.x | (uint64_t)v.y << 32;
+            vals[lo + r] = v.z;
+        }
+    }
+    cluster_sync();                                // no block ends while others may send to it
+}
+
+struct ClusterLaunch {
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg;
+    ClusterLaunch(size_t smem, cudaStream_t s) : attr(), cfg() {
+        cfg.gridDim = kClBlocks;
+        cfg.blockDim = kClThreads;
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim = {kClBlocks, 1, 1};
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+    }
+};
+
+template <int kIt>
+bool cluster_prepare() {
+    auto kern = k_cluster_sort<kIt>;
+    const size_t smem = sizeof(ClusterSmem<kIt>);
+    ClusterLaunch l(smem, nullptr);
+    l.cfg.numAttrs = 1;
+    int count = 0;
+    const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&count, kern, &l.cfg) == cudaSuccess && count > 0;
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
+// whether a sort of n pairs takes the cluster kernel: asked once per device, since
+// one without room for such a cluster takes the passes
+bool cluster_fits(int64_t n) {
+    if (n > kClusterMax) return false;
+    static std::mutex mu;
+    static std::map<int, bool> fits;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = fits.find(dev);
+    if (it == fits.end())
+        it = fits.emplace(dev, cluster_prepare<1>() && cluster_prepare<2>() && cluster_prepare<4>()).first;
+    return it->second;
+}
+
+template <int kIt>
+void cluster_sort(uint64_t *keys, uint32_t *vals, int64_t n, int rounds, int npasses, uint32_t *status, cudaStream_t s) {
+    ClusterLaunch l(sizeof(ClusterSmem<kIt>), s);
+    const int64_t chunk = 32 * rounds;     // a warp's keys
+    const uint32_t slice = (uint32_t)((((n + kClBlocks - 1) / kClBlocks + chunk - 1) / chunk) * chunk);
+    cudaLaunchKernelEx(&l.cfg, k_cluster_sort<kIt>, keys, vals, (uint32_t)n, slice, rounds, npasses, status);
+    note_launch();
+}
+
 }  // namespace
 
 size_t radix_sort_scratch_bytes(int64_t n) {
@@ -381,6 +678,10 @@ constexpr int64_t kLookAt = (8 * kRadix * sizeof(uint32_t) + 256) / sizeof(unsig
 
 unsigned long long *radix_sort_clear(int64_t n, void *scratch, int64_t *words) {
     const int64_t ntiles = (n + kTile - 1) / kTile;
+    if (cluster_fits(n)) {
+        *words = 0;
+        return nullptr;
+    }
     // one-kernel passes: a look word per tile and digit; large sorts: the look words of
     // the tile counts' one-kernel scans (one tag per pass), the counts follow them
     *words = kLookAt + (ntiles > kOneSweepMaxTiles ? (int64_t)scan_look_words((int64_t)kRadix * ntiles)
@@ -393,6 +694,14 @@ void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32
                       uint32_t *status, bool cleared) {
     *result_in_alt = false;
     if (n <= 1) return;
+    if (cluster_fits(n)) {
+        const int rounds = (int)((n + kClBlocks * kClThreads - 1) / (kClBlocks * kClThreads));
+        const int np = (bits + kClBits - 1) / kClBits;
+        if (rounds <= 1) cluster_sort<1>(keys, vals, n, rounds, np, status, s);
+        else if (rounds <= 2) cluster_sort<2>(keys, vals, n, rounds, np, status, s);
+        else cluster_sort<4>(keys, vals, n, rounds, np, status, s);
+        return;
+    }
     int64_t ntiles = (n + kTile - 1) / kTile;
     int64_t nclear;
     unsigned long long *p = radix_sort_clear(n, scratch, &nclear);
