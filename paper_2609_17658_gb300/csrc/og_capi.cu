@@ -385,7 +385,7 @@ og_status og_create(og_ctx **out, int device, size_t hbm_budget_bytes) {
         return cuda_fail(e, "cudaMalloc");
     }
     c->d_counters = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(c->d_status) + 64);
-    if ((e = cudaMallocHost(&c->h_pinned, 256)) != cudaSuccess) {
+    if ((e = cudaMallocHost(&c->h_pinned, kPinnedWords + kStageBytes)) != cudaSuccess) {
         cudaFree(c->d_status);
         cudaEventDestroy(c->ev_to_side);
         cudaEventDestroy(c->ev_from_side);
@@ -394,7 +394,7 @@ og_status og_create(og_ctx **out, int device, size_t hbm_budget_bytes) {
         delete c;
         return cuda_fail(e, "cudaMallocHost");
     }
-    memset(c->h_pinned, 0, 256);
+    memset(c->h_pinned, 0, kPinnedWords);
     cudaMemset(c->d_status, 0, 256);
     cudaDeviceSynchronize();
     *out = c;
@@ -463,16 +463,25 @@ og_status og_tree_build(og_ctx *c, const double *pos, const double *mass, int64_
             return cuda_fail(e, "cudaMallocAsync (inputs)");
         }
         double *dp = static_cast<double *>(staging);
-        cudaMemcpyAsync(dp, pos, (size_t)n * 3 * sizeof(double), cudaMemcpyHostToDevice, s);
-        // the masses follow on the side stream once the positions are in (the
-        // link is not shared with them), beside the quantization and the sort;
-        // the build waits for them before it first reads them
-        cudaEventRecord(c->ev_to_side, s);
-        cudaStreamWaitEvent(c->copy_stream, c->ev_to_side, 0);
-        cudaMemcpyAsync(dp + 3 * n, mass, (size_t)n * sizeof(double), cudaMemcpyHostToDevice,
-                        c->copy_stream);
-        cudaEventRecord(c->ev_from_side, c->copy_stream);
-        t->mass_ready = c->ev_from_side;
+        if (bytes <= kStageBytes) {
+            // small: through the context's page-locked memory in one copy (the build
+            // synchronises, so no copy of an earlier call still reads it)
+            char *h = pinned_stage(c);
+            memcpy(h, pos, (size_t)n * 3 * sizeof(double));
+            memcpy(h + (size_t)n * 3 * sizeof(double), mass, (size_t)n * sizeof(double));
+            cudaMemcpyAsync(dp, h, bytes, cudaMemcpyHostToDevice, s);
+        } else {
+            cudaMemcpyAsync(dp, pos, (size_t)n * 3 * sizeof(double), cudaMemcpyHostToDevice, s);
+            // the masses follow on the side stream once the positions are in (the
+            // link is not shared with them), beside the quantization and the sort;
+            // the build waits for them before it first reads them
+            cudaEventRecord(c->ev_to_side, s);
+            cudaStreamWaitEvent(c->copy_stream, c->ev_to_side, 0);
+            cudaMemcpyAsync(dp + 3 * n, mass, (size_t)n * sizeof(double), cudaMemcpyHostToDevice,
+                            c->copy_stream);
+            cudaEventRecord(c->ev_from_side, c->copy_stream);
+            t->mass_ready = c->ev_from_side;
+        }
         d_pos = dp;
         d_mass = dp + 3 * n;
     }
@@ -601,7 +610,14 @@ og_status og_tree_force(og_tree *t, const float *a_old, float *acc, uint32_t *n_
     float *d_acc = acc;
     uint32_t *d_npp = n_pp, *d_npn = n_pn;
     void *out_tmp = nullptr;
-    if (st == OG_OK && !dev) {
+    // small host outputs: the last kernel writes them to the context's page-locked
+    // memory, and the host copies them on after the call's synchronisation
+    const bool staged = !dev && (size_t)n * 20 <= kStageBytes;
+    if (staged) {
+        d_acc = reinterpret_cast<float *>(pinned_stage(c));
+        d_npp = n_pp ? reinterpret_cast<uint32_t *>(d_acc + 3 * n) : nullptr;
+        d_npn = n_pn ? reinterpret_cast<uint32_t *>(d_acc + 3 * n) + n : nullptr;
+    } else if (st == OG_OK && !dev) {
         size_t bytes = (size_t)n * 3 * sizeof(float) + 2 * (size_t)n * sizeof(uint32_t) + 512;
         if ((e = dev_malloc_async(&out_tmp, bytes, s)) != cudaSuccess) st = cuda_fail(e, "cudaMallocAsync (out)");
         d_acc = static_cast<float *>(out_tmp);
@@ -619,7 +635,7 @@ og_status og_tree_force(og_tree *t, const float *a_old, float *acc, uint32_t *n_
     const bool last_deferred = t->npend > 0 && !t->h_wp[0].dump;
     const ForceReport none{}, rep{c->d_counters, c->d_status,
                                   last_deferred ? pinned_counters(c, t->npend - 1) : nullptr, hst};
-    if (!dev && (n_pp || n_pn)) {
+    if (!dev && !staged && (n_pp || n_pn)) {
         // host outputs: the counts first, their copy on the side stream beside
         // the accelerations' reordering (the copies share the link, the
         // reordering does not)
@@ -638,7 +654,7 @@ og_status og_tree_force(og_tree *t, const float *a_old, float *acc, uint32_t *n_
     } else {
         k_unpermute<<<nblk(n), kT, 0, s>>>(n, t->inv, t->a_sorted, t->npp_sorted, t->npn_sorted,
                                            d_acc, d_npp, d_npn, rep); note_launch();
-        if (!dev) {
+        if (!dev && !staged) {
             cudaMemcpyAsync(acc, d_acc, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost, s);
             cudaFreeAsync(out_tmp, s);
         }
@@ -652,6 +668,11 @@ og_status og_tree_force(og_tree *t, const float *a_old, float *acc, uint32_t *n_
     cudaEventDestroy(e1);
     if (e != cudaSuccess) return cuda_fail(e, "force");
     if (st != OG_OK) return st;
+    if (staged) {
+        memcpy(acc, d_acc, (size_t)n * 3 * sizeof(float));
+        if (n_pp) memcpy(n_pp, d_npp, (size_t)n * sizeof(uint32_t));
+        if (n_pn) memcpy(n_pn, d_npn, (size_t)n * sizeof(uint32_t));
+    }
     t->ms_force = ms;
     t->ms_walk = ms_walk;
     return status_from(c, *hst);

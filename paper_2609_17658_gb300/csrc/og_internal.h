@@ -207,6 +207,13 @@ inline uint32_t *pinned_counts(og_ctx *c) {
 // words of og_ctx::d_counters that a walk counts in: next item, interactions, list
 // cursor, items in parts, next part
 constexpr int kWalkCounters = 5;
+// Page-locked staging of the host arrays of small calls, behind those words: a copy from
+// or to pageable memory costs some 10 us whatever its size, and a call has two or
+// three each way.  Host arrays, build and force: 1k particles 255 -> 218 us, 4k 282 ->
+// 242, 8k 313 -> 282, 16k 350 -> 322; with 24k (768 KB in, 480 KB out) even, with 32k
+// 382 -> 412, where the host's own copy costs more than it saves.
+constexpr size_t kPinnedWords = 256, kStageBytes = 512 * 1024;
+inline char *pinned_stage(og_ctx *c) { return static_cast<char *>(c->h_pinned) + kPinnedWords; }
 // default launch shape of the walk (og_params.walk_warps / walk_chunk = 0)
 constexpr int kDefaultWalkWarps = 4;
 constexpr int kDefaultWalkChunk = 256;
