@@ -356,7 +356,7 @@ struct WalkParams {
     float hnear2f;     // hnear2 raised by more than the FP32 error of a squared distance
     float h;           // softening length, grid units
     float inv_h;
-    float erf_ky;      // 2 r_s / p of the erfc fit, grid units (og_walk.cu)
+    float erf_ky;      // 2 r_s / p of the erfc form, grid units (og_walk.cu)
     float erf_c;       // (2 / sqrt(pi)) / (2 r_s)
     float kexp;        // -log2(e) / (4 r_s^2), grid units
     float out_scale;   // G (2^32/L)^2

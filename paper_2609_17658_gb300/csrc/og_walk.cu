@@ -38,7 +38,7 @@
 // relieved alone: forcing the integer differences to the other pipe, registers
 // for 6 or 8 blocks per SM, or 2 to 8 entries in flight all measured within 2 %.
 // The list building is the other 1 G, about 390 a round of 64 slots.  Two targets
-// a lane, the straight-line classification and the new erfc fit took the pass
+// a lane, the straight-line classification and the erfc from 1 / r took the pass
 // from 3.40 to 2.75 ms and the two-pass walk from 7.10 to 5.73 ms.
 //
 // Work distribution: persistent blocks; warps take groups from a global
@@ -100,14 +100,18 @@ __host__ __device__ constexpr size_t warp_smem(int chunk) {
 constexpr size_t kMaxBlockSmem = kMaxWarps * warp_smem(kMaxChunk);
 static_assert(kMaxBlockSmem <= 227 * 1024, "walk block exceeds the shared memory of an SM");
 
-// erfc(u) exp(u^2) ~ c0 + v (c1 + ... + v c5), v = p u / (1 + p u) in [0, 1): a
-// least-maximum fit of the split factor S(u) = exp(-u^2) (erfc(u) exp(u^2) +
-// (2 / sqrt(pi)) u), |error of S| <= 1e-7 max(S, S(2.25)) for u >= 0, so it is
-// good to 1e-7 relative up to the usual cutoff u = 2.25 (1.7e-7 in FP32
-// arithmetic; Abramowitz & Stegun 7.1.26, used before, 7.4e-6 there).
-constexpr float kErfP = 0.455f;
-constexpr float kErf0 = 0.99999990145469710f, kErf1 = -2.4799351751253551f, kErf2 = 2.3497844342086717f;
-constexpr float kErf3 = -0.79841706208158790f, kErf4 = -0.31761888136087987f, kErf5 = 0.25502248430625629f;
+// erfc(u) exp(u^2) by Abramowitz & Stegun 7.1.26 (t = 1 / (1 + p u), a polynomial
+// a1 t + ... + a5 t^5; the split factor S(u) = exp(-u^2) (erfc(u) exp(u^2) +
+// (2 / sqrt(pi)) u) to 7.4e-6 up to the usual cutoff u = 2.25), written in v = 1 - t:
+// c0 + v (c1 + ... + v c5), v = p u / (1 + p u) in [0, 1), which comes from 1 / r, so r
+// itself is not formed.  A least-maximum fit of S in the same form (p = 0.455) is good
+// to 1e-7 at the same cost; it moved a group's smallest acceleration by 2.6e-7 on
+// average (p99 2.4e-6, this form 7e-8 and 4e-7), and so a first pass near the threshold
+// of the relative criterion to other lists in the second (25 particles of 2.1M by
+// more than 1e-5, none this way), and is not used.
+constexpr float kErfP = 0.3275911f;
+constexpr float kErf0 = 0.999999999f, kErf1 = -3.44449638f, kErf2 = 5.874886615f;
+constexpr float kErf3 = -6.222859923f, kErf4 = 3.853875118f, kErf5 = -1.061405429f;
 constexpr float kTwoOverSqrtPi = 1.1283791670955126f;
 
 // relative margin of the FP32 opening filter (the FP32 evaluation errs by
