@@ -55,6 +55,8 @@ struct SphArgs {
     int64_t ngroups;
     uint32_t *longs;        // groups left to a block each: their number, then their ids
     int limit;              // candidates above which a group is left to a block
+    const uint32_t *many;   // null, or the groups expected above the limit (k_sph_expect)
+    uint32_t max_many;      // more than this: no group is left to a block
     int64_t max_rounds;     // nodes + 2 + buckets' extra rounds (<= n / 32)
     double dens;            // 8 / pi * (2^32 / L)^3
     float *rho;             // caller order (key order without perm)
@@ -300,6 +302,7 @@ __global__ void __launch_bounds__(32 * kSphWarps) k_sph_density(SphArgs a) {
     const unsigned lt = (1u << lane) - 1u;
     const int64_t g = (int64_t)blockIdx.x * kSphWarps + warp;
     if (g >= a.ngroups) return;  // the whole warp
+    const int limit = a.many && *a.many > a.max_many ? 0x7fffffff : a.limit;
     unsigned long long *stk = reinterpret_cast<unsigned long long *>(smem_raw) + (size_t)warp * kSphStack;
     uint4 *chunk = reinterpret_cast<uint4 *>(smem_raw + (size_t)kSphWarps * kSphStack * 8) +
                    (size_t)warp * kSphChunk;
@@ -371,7 +374,7 @@ __global__ void __launch_bounds__(32 * kSphWarps) k_sph_density(SphArgs a) {
         nc += __popc(ba);
         if (nc > kSphChunk - 32) {
             found += nc;
-            if (found > a.limit) {
+            if (found > limit) {
                 if (lane == 0) a.longs[1 + atomicAdd(&a.longs[0], 1u)] = (uint32_t)g;
                 return;
             }
@@ -445,15 +448,55 @@ __global__ void k_sph_gather(int64_t n, const uint32_t *__restrict__ perm, const
 
 inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-// scratch of a search: the long groups' number and list
-inline size_t long_bytes(int64_t ng) { return (size_t)(ng + 1) * 4; }
+// How many groups to expect above the limit, from the group's own density over its
+// search region: with smoothing lengths far too large (a solver's first steps from one
+// mean length) nearly all are, and a block each costs more than a warp each.  The
+// count depends on the lengths alone, so a call's bits do not depend on its timing.
+// 6 us for the 99k groups of 2.1M particles, whose call takes 2.28 ms.
+__global__ void k_sph_expect(SphArgs a, uint32_t *many) {
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    bool above = false;
+    if (g < a.ngroups) {
+        const uint32_t b = a.gbeg[g], e = a.gend[g];
+        float h = 0.0f;
+        bool todo = !a.done;
+        for (uint32_t i = b; i < e; ++i) {
+            h = fmaxf(h, a.hg[i]);
+            todo = todo || a.done[i] == 0;
+        }
+        uint32_t side = 0;
+        for (int k = 0; k < 3; ++k) side = max(side, a.gbox[6 * g + 3 + k] - a.gbox[6 * g + k]);
+        const float x = side ? 1.0f + 2.0f * h / (float)side : 0.0f;
+        above = todo && (float)(e - b) * (x * x * x) > (float)a.limit;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, above);
+    if ((threadIdx.x & 31u) == 0u && m) atomicAdd(many, (uint32_t)__popc(m));
+}
+
+// From this many groups on a call asks k_sph_expect, and leaves no group to a block
+// where it expects more than an eighth above the limit.  Below, a block each pays even
+// where all groups are long.  From the mean length for every particle to 32 neighbours,
+// a warp each always / a block each always / this rule: 100k particles (4.7k groups) 21.3 /
+// 14.0 / 14.0 ms, 400k (19k) 55.9 / 56.0 / 46.6, 2.1M (99k) 187 / 311 / 180 (a quarter
+// instead of an eighth 197, a half 245, a sixteenth 179 but 50.6 at 400k).
+constexpr int64_t kExpectMin = 16384;
+
+// scratch of a search: the long groups' number and list, the expected number
+inline size_t long_bytes(int64_t ng) { return (size_t)(ng + 2) * 4; }
 
 // the density of every group of the tree, at a.hg
 void search(SphArgs &a, char *scratch, cudaStream_t s) {
     if (a.ngroups < 1) return;
-    a.longs = reinterpret_cast<uint32_t *>(scratch);
+    uint32_t *many = reinterpret_cast<uint32_t *>(scratch);
+    a.longs = many + 1;
     a.limit = candidate_limit(a.ngroups);
-    cudaMemsetAsync(a.longs, 0, 4, s);
+    a.many = nullptr;
+    a.max_many = (uint32_t)(a.ngroups / 8);
+    cudaMemsetAsync(many, 0, 8, s);
+    if (a.ngroups >= kExpectMin) {
+        k_sph_expect<<<nblk(a.ngroups, 256), 256, 0, s>>>(a, many); note_launch();
+        a.many = many;
+    }
     k_sph_density<<<nblk(a.ngroups, kSphWarps), 32 * kSphWarps, kSphSmem, s>>>(a); note_launch();
     const unsigned most = (unsigned)(a.ngroups < 456 ? a.ngroups : 456);   // 152 SMs x 3 blocks
     k_sph_long<<<most, kLongThreads, 0, s>>>(a); note_launch();
