@@ -452,7 +452,7 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 // search region: with smoothing lengths far too large (a solver's first steps from one
 // mean length) nearly all are, and a block each costs more than a warp each.  The
 // count depends on the lengths alone, so a call's bits do not depend on its timing.
-// 6 us for the 99k groups of 2.1M particles, whose call takes 2.28 ms.
+// 11 us from a cold cache for the 99k groups of 2.1M particles, whose call takes 2.26 ms.
 __global__ void k_sph_expect(SphArgs a, uint32_t *many) {
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool above = false;
