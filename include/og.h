@@ -52,7 +52,8 @@ typedef enum {
     OG_ERR_CUDA = -3,        /* a CUDA runtime call failed */
     OG_ERR_TIMEOUT = -4,     /* a bounded device-side wait ran out: a tile of a one-kernel
                                 sort pass or scan waited too long for the count of an
-                                earlier tile (the context stays usable) */
+                                earlier tile, or a block of the one-launch sort for
+                                another's (the context stays usable) */
     OG_ERR_BUDGET = -5,      /* the request does not fit the HBM budget */
     OG_ERR_OVERFLOW = -6,    /* a fixed-capacity device buffer overflowed */
     OG_ERR_STATE = -7,       /* call not valid in the handle's state */
@@ -531,6 +532,14 @@ og_status og_debug_fail_allocations(int32_t skip, int32_t count);
  * and frees its own scratch.  OG_ERR_ARG for a NULL context or n out of
  * range. */
 og_status og_debug_scan_wait_timeout(og_ctx *c, int64_t n);
+
+/* The same for the one-launch sort of small systems, whose 16 blocks wait for
+ * each other's digit counts and keys: a sort of n pairs (16 <= n <= 65536) in
+ * which one block keeps back its counts, or with keys_held its keys, so that
+ * the others' waits run out.  They give up, finish, and the call returns
+ * OG_ERR_TIMEOUT if every pair left behind is one that came in (OG_ERR_STATE
+ * otherwise); the context is usable as before. */
+og_status og_debug_sort_wait_timeout(og_ctx *c, int64_t n, int32_t keys_held);
 
 #ifdef __cplusplus
 }

@@ -226,7 +226,8 @@ __global__ void k_seg_keys(int64_t n, const uint32_t *__restrict__ idx,
     pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    segkey[i] = pseg[idx[i]];
+    const uint32_t j = idx[i];
+    segkey[i] = j < n ? pseg[j] : 0u;      // beyond: only after a sort whose wait ran out
 }
 
 __global__ void k_gather_keys(int64_t n, const uint32_t *__restrict__ perm,
@@ -235,7 +236,7 @@ __global__ void k_gather_keys(int64_t n, const uint32_t *__restrict__ perm,
     pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const uint32_t j = perm[i];
+    const uint32_t j = perm[i] < n ? perm[i] : 0u;
     skey[i] = key0[j];
     sseg[i] = pseg[j];
 }
@@ -266,6 +267,10 @@ struct Permute {
         int lo = 0x7fffffff, hi = (int)0x80000000;
         if (i < n) {
             uint32_t j = perm[i];
+            if (j >= n) {                  // only after a sort whose wait ran out
+                atomicOr(status, ST_INTERNAL);
+                j = 0u;
+            }
             inv[j] = (uint32_t)i;
             const uint4 q = q4[j];
             px[i] = q.x;
@@ -741,6 +746,10 @@ struct Threading {
         }
         if (c >= nchild) return;
         const uint32_t item = child[c];
+        if (item >= n + m) {               // a slot nothing was placed in
+            atomicOr(status, ST_INTERNAL);
+            return;
+        }
         int64_t par = item < n ? (int64_t)owner[item] : (int64_t)npar[item - n];
         int64_t cc = c;
         int32_t after = -1;

@@ -249,7 +249,7 @@ og_status status_from(og_ctx *c, uint32_t st) {
     }
     if (st & ST_TIMEOUT) {
         set_error("a device-side wait on another block ran out (the look-back of a one-kernel sort "
-                  "pass or scan)");
+                  "pass or scan, or the one-launch sort)");
         return OG_ERR_TIMEOUT;
     }
     set_error("internal consistency check failed (status 0x%x)", st);
@@ -300,6 +300,15 @@ og_status og_debug_scan_wait_timeout(og_ctx *c, int64_t n) {
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "og_debug_scan_wait_timeout");
     return status_from(c, *h);
+}
+
+og_status og_debug_sort_wait_timeout(og_ctx *c, int64_t n, int32_t keys_held) {
+    if (!c) { set_error("og_debug_sort_wait_timeout: NULL context"); return OG_ERR_ARG; }
+    cudaSetDevice(c->device);
+    const og_status probe = sort_wait_timeout_probe(c, n, keys_held != 0);
+    if (probe != OG_OK && probe != OG_ERR_STATE) return probe;
+    const og_status st = check_status(c);        // clears the status word
+    return probe != OG_OK ? probe : st;
 }
 
 og_status og_debug_fail_allocations(int32_t skip, int32_t count) {

@@ -278,7 +278,7 @@ void scan_inclusive_max_u32(const uint32_t *in, uint32_t *out, int64_t n, void *
 // scan_scratch_bytes(n)).  look holds scan_look_words(n) words, cleared before
 // their first use; tag (1 .. 2^30 - 1) must differ between uses of the same
 // words; ctr is a word that is 0 before the call.  A look-back that waits too
-// long sets ST_INTERNAL in *status.
+// long sets ST_TIMEOUT in *status.
 size_t scan_look_words(int64_t n);
 // test hook: a one-kernel scan whose first tile never publishes (see
 // og_debug_scan_wait_timeout); returns the status word's bits
@@ -302,7 +302,8 @@ void scan_sum_and_max_u32_look(const uint32_t *in, uint32_t *out, int64_t n, uin
                                uint32_t tag2, unsigned long long *look, unsigned long long *look2, uint32_t *status,
                                void *scratch, cudaStream_t s);
 
-// radix sort of (key, value) pairs, stable, keys of `bits` significant bits
+// radix sort of (key, value) pairs, stable, keys of `bits` significant bits, values
+// below n.  A wait that runs out sets ST_TIMEOUT; the order is then undefined.
 size_t radix_sort_scratch_bytes(int64_t n);
 void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt,
                       int64_t n, int bits, void *scratch, cudaStream_t s, bool *result_in_alt,
@@ -311,6 +312,11 @@ void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32
 // own kernel clears them passes cleared and saves the memset (none where the sort is one
 // launch of a cluster)
 unsigned long long *radix_sort_clear(int64_t n, void *scratch, int64_t *words);
+
+// test hook: a one-launch sort of n pairs in which a block keeps back its counts or its
+// keys, so that the others' waits run out (see og_debug_sort_wait_timeout); OG_OK when
+// what it left are pairs that came in
+og_status sort_wait_timeout_probe(og_ctx *c, int64_t n, bool keys_held);
 
 // the same sort with every digit pass run (no histogram read-back, no host
 // synchronisation); with an even pass count the result is back in keys/vals

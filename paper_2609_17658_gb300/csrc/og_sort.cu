@@ -19,6 +19,7 @@
 // kClusterMax keys all passes are one launch (k_cluster_sort).
 #include <map>
 #include <mutex>
+#include <vector>
 
 #include "og_internal.h"
 
@@ -384,11 +385,24 @@ __global__ void __launch_bounds__(kThreads, 4) k_onesweep(const uint64_t *__rest
 // p + 1, and a block sends those after it has read the ones of pass p; it sends
 // keys of pass p after it has all counts of pass p, and a block sends those after it
 // has sent on the keys of pass p - 1, whose buffer the new ones take.
+//
+// A wait that runs out: the block sends and stores nothing from then on, so no block
+// takes a record that never arrived (those it would have reached run out in turn), and
+// what it leaves in keys and vals are the pairs that came in.  It still takes part in
+// the last cluster barrier, after which nothing more is sent to it, and then waits
+// (again with a limit) for what is on its way into its own shared memory.
 constexpr int kClBlocks = 16, kClThreads = 1024, kClWarps = kClThreads / 32;
 constexpr int kClBits = 9, kClRadix = 1 << kClBits, kClPairs = kClRadix / 2;
 constexpr int kClMaxRounds = 4;        // keys per thread
 constexpr int64_t kClusterMax = (int64_t)kClBlocks * kClThreads * kClMaxRounds;
+// tries of a wait; each suspends the thread for about kClTryNs at most, so a wait that runs
+// out takes some 65 ms
 constexpr int kClWaitLimit = 1 << 16;
+constexpr uint32_t kClTryNs = 1000;
+constexpr int kClDrainLimit = 1 << 10;
+// test hook (sort_wait_timeout_probe): the block that keeps back its counts of the first
+// pass, or with kHoldKeys its keys
+constexpr uint32_t kHoldNone = 0xffffffffu, kHoldKeys = 0x100u;
 static_assert(kClThreads == 4 * kClPairs && kClThreads == kClBlocks * kClPairs / 4 &&
                   kClThreads * kClMaxRounds < 65536,
               "a thread per digit pair and quarter, and per four pairs and block");
@@ -403,6 +417,7 @@ struct ClusterSmem {
     uint32_t own[kClPairs];                        // this block's counts
     uint32_t base[kClRadix];                       // where this block's keys of the digit go
     uint32_t wsum[kClPairs / 32];
+    uint32_t gave_up;                              // a wait for counts ran out
     unsigned long long cnt_bar[2], rec_bar;        // received counts, by parity; received keys
 };
 
@@ -422,29 +437,30 @@ __device__ __forceinline__ void cluster_send(uint32_t a, uint32_t bar, uint4 v) 
 __device__ __forceinline__ void bar_expect(void *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(shared_addr(bar)), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void bar_wait(void *bar, uint32_t phase, uint32_t *status) {
+// false: the wait ran out
+__device__ __forceinline__ bool bar_wait(void *bar, uint32_t phase, int limit = kClWaitLimit) {
     const uint32_t a = shared_addr(bar);
-    for (int it = 0; it < kClWaitLimit; ++it) {
+    for (int it = 0; it < limit; ++it) {
         uint32_t ok;
         asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(ok)
-                     : "r"(a), "r"(phase)
+                     : "r"(a), "r"(phase), "r"(kClTryNs)
                      : "memory");
-        if (ok) return;
+        if (ok) return true;
     }
-    atomicOr(status, ST_TIMEOUT);                  // gives up: what follows stays in bounds
+    return false;
 }
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// in place: keys, vals
+// in place: keys, vals (indices below n)
 template <int kIt>
 __global__ void __launch_bounds__(kClThreads, 1) k_cluster_sort(uint64_t *keys, uint32_t *vals, uint32_t n,
                                                                 uint32_t slice, int rounds, int npasses,
-                                                                uint32_t *status) {
+                                                                uint32_t *status, uint32_t hold) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ClusterSmem<kIt> &S = *reinterpret_cast<ClusterSmem<kIt> *>(smem_raw);
     const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
@@ -456,6 +472,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_sort(uint64_t *keys, 
     const uint32_t wfirst = warp * 32u * (uint32_t)rounds;                   // the warp's first slot
     const uint32_t pair = t & (kClPairs - 1u), qt = t / kClPairs;            // of the per-digit work
     if (t == 0) {
+        S.gave_up = 0u;
         for (void *b : {(void *)&S.cnt_bar[0], (void *)&S.cnt_bar[1], (void *)&S.rec_bar})
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(shared_addr(b)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -468,13 +485,14 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_sort(uint64_t *keys, 
     }
     int cur = 0;
     uint32_t moved = 0;                            // passes that moved the keys
-    bool stored = false;
-    for (int pass = 0; pass < npasses; ++pass) {
+    bool stored = false, gave_up = false;
+    int pass = 0;
+    for (; pass < npasses; ++pass) {
         const int shift = kClBits * pass, par = pass & 1;
         for (uint32_t i = t; i < kClWarps * kClPairs; i += kClThreads) (&S.wcnt[0][0])[i] = 0u;
         if (t == 0) bar_expect(&S.cnt_bar[par], kClBlocks * kClPairs * 4u);
-        if (moved) bar_wait(&S.rec_bar, (moved - 1u) & 1u, status);
-        __syncthreads();
+        gave_up = __syncthreads_or(moved && !bar_wait(&S.rec_bar, (moved - 1u) & 1u));
+        if (gave_up) break;
         uint16_t *wc = reinterpret_cast<uint16_t *>(S.wcnt[warp]);
         uint4 rec[kIt];
         uint32_t rank[kIt];
@@ -530,10 +548,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_sort(uint64_t *keys, 
         {
             // four pairs to one block
             const uint32_t b = t / (kClPairs / 4), q = 4u * (t & (kClPairs / 4 - 1u));
-            cluster_send(cluster_addr(&S.cnt[par][cta][q], b), cluster_addr(&S.cnt_bar[par], b),
+            if (hold != cta) cluster_send(cluster_addr(&S.cnt[par][cta][q], b), cluster_addr(&S.cnt_bar[par], b),
                          *reinterpret_cast<const uint4 *>(&S.own[q]));
         }
-        bar_wait(&S.cnt_bar[par], (uint32_t)(pass >> 1) & 1u, status);
+        if (!bar_wait(&S.cnt_bar[par], (uint32_t)(pass >> 1) & 1u)) S.gave_up = 1u;
         // the digits' counts in all blocks and in those before this one, and their scan
         uint32_t all_lo = 0, all_hi = 0, bef_lo = 0, bef_hi = 0, sum = 0;
         if (qt == 0) {
@@ -555,6 +573,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_sort(uint64_t *keys, 
         }
         // one digit holds every key: the order stays
         stored = !__syncthreads_or(all_lo == n || all_hi == n);
+        gave_up = S.gave_up != 0u;                 // written before the barrier only
+        if (gave_up) break;
         if (!stored) continue;
         const bool last = pass == npasses - 1;
         if (t == 0 && !last) bar_expect(&S.rec_bar, mine * 16u);
@@ -573,12 +593,12 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_sort(uint64_t *keys, 
             const uint64_t key = rec[r].x | (uint64_t)rec[r].y << 32;
             const uint32_t d = (uint32_t)(key >> shift) & (kClRadix - 1u);
             const uint32_t g = S.base[d] + qp[d] + wc[d] + rank[r];
-            if (g >= n) {                          // only after a wait that gave up
-                atomicOr(status, ST_TIMEOUT);
+            if (g >= n) {                          // cannot be: the counts are whole
+                atomicOr(status, ST_INTERNAL);
             } else if (last) {
                 keys[g] = key;
                 vals[g] = rec[r].z;
-            } else {
+            } else if (hold != (cta | kHoldKeys)) {
                 const uint32_t b = g / slice;
                 cluster_send(cluster_addr(&S.rec[cur ^ 1][g - b * slice], b), cluster_addr(&S.rec_bar, b), rec[r]);
             }
@@ -588,9 +608,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_sort(uint64_t *keys, 
         // the next pass clears the warps' counts, which every thread has read
         __syncthreads();
     }
-    if (!stored) {
-        // the last pass had nothing to move: the keys are here, or still on their way
-        if (moved) bar_wait(&S.rec_bar, (moved - 1u) & 1u, status);
+    if (gave_up) {
+        if (t == 0) atomicOr(status, ST_TIMEOUT);
+    } else if (!stored) {
+        // the last pass had nothing to move: the keys are here
         for (uint32_t r = t; r < mine; r += kClThreads) {
             const uint4 v = S.rec[cur][r];
             keys[lo + r] = v.x | (uint64_t)v.y << 32;
@@ -598,6 +619,20 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_sort(uint64_t *keys, 
         }
     }
     cluster_sync();                                // no block ends while others may send to it
+    if (gave_up && t == 0) {
+        // What others sent before they stopped: a barrier that never completes only
+        // takes the limit.  The wait that ran out was for the keys of the pass before
+        // (then this pass's counts may be on their way) ...
+        if (!S.gave_up) bar_wait(&S.rec_bar, (moved - 1u) & 1u, kClDrainLimit);
+        bar_wait(&S.cnt_bar[pass & 1], (uint32_t)(pass >> 1) & 1u, kClDrainLimit);
+        if (S.gave_up) {
+            // ... or for this pass's counts (then its keys and the next one's counts)
+            bar_expect(&S.rec_bar, mine * 16u);
+            bar_wait(&S.rec_bar, moved & 1u, kClDrainLimit);
+            bar_expect(&S.cnt_bar[(pass + 1) & 1], kClBlocks * kClPairs * 4u);
+            bar_wait(&S.cnt_bar[(pass + 1) & 1], (uint32_t)((pass + 1) >> 1) & 1u, kClDrainLimit);
+        }
+    }
 }
 
 struct ClusterLaunch {
@@ -647,15 +682,57 @@ bool cluster_fits(int64_t n) {
 }
 
 template <int kIt>
-void cluster_sort(uint64_t *keys, uint32_t *vals, int64_t n, int rounds, int npasses, uint32_t *status, cudaStream_t s) {
+void cluster_sort(uint64_t *keys, uint32_t *vals, int64_t n, int rounds, int npasses, uint32_t *status, cudaStream_t s,
+                  uint32_t hold = kHoldNone) {
     ClusterLaunch l(sizeof(ClusterSmem<kIt>), s);
     const int64_t chunk = 32 * rounds;     // a warp's keys
     const uint32_t slice = (uint32_t)((((n + kClBlocks - 1) / kClBlocks + chunk - 1) / chunk) * chunk);
-    cudaLaunchKernelEx(&l.cfg, k_cluster_sort<kIt>, keys, vals, (uint32_t)n, slice, rounds, npasses, status);
+    cudaLaunchKernelEx(&l.cfg, k_cluster_sort<kIt>, keys, vals, (uint32_t)n, slice, rounds, npasses, status,
+                       hold);
     note_launch();
 }
 
 }  // namespace
+
+og_status sort_wait_timeout_probe(og_ctx *c, int64_t n, bool keys_held) {
+    if (n < kClBlocks || !cluster_fits(n)) {
+        set_error("og_debug_sort_wait_timeout: n must lie in [%d, %lld], on a device with room for the cluster",
+                  kClBlocks, (long long)kClusterMax);
+        return OG_ERR_ARG;
+    }
+    cudaStream_t s = c->stream;
+    std::vector<uint64_t> k((size_t)n), k_in((size_t)n);
+    std::vector<uint32_t> v((size_t)n);
+    for (int64_t i = 0; i < n; ++i) {
+        k_in[(size_t)i] = k[(size_t)i] = ((uint64_t)(i + 1) * 0x9e3779b97f4a7c15ull) >> 1;
+        v[(size_t)i] = (uint32_t)i;
+    }
+    void *buf = nullptr;
+    cudaError_t e = dev_malloc_async(&buf, (size_t)n * 12, s);
+    if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? OG_ERR_OOM : cuda_fail(e, "cudaMallocAsync (probe)");
+    uint64_t *dk = static_cast<uint64_t *>(buf);
+    uint32_t *dv = reinterpret_cast<uint32_t *>(dk + n);
+    cudaMemcpyAsync(dk, k.data(), (size_t)n * 8, cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(dv, v.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s);
+    const uint32_t hold = keys_held ? kHoldKeys : 0u;   // block 0 has keys at any n
+    const int rounds = (int)((n + kClBlocks * kClThreads - 1) / (kClBlocks * kClThreads));
+    const int np = (63 + kClBits - 1) / kClBits;
+    if (rounds <= 1) cluster_sort<1>(dk, dv, n, rounds, np, c->d_status, s, hold);
+    else if (rounds <= 2) cluster_sort<2>(dk, dv, n, rounds, np, c->d_status, s, hold);
+    else cluster_sort<4>(dk, dv, n, rounds, np, c->d_status, s, hold);
+    cudaMemcpyAsync(k.data(), dk, (size_t)n * 8, cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(v.data(), dv, (size_t)n * 4, cudaMemcpyDeviceToHost, s);
+    cudaFreeAsync(buf, s);
+    e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_fail(e, "sort probe");
+    // whatever was moved: pairs that came in, at places inside the arrays
+    for (int64_t i = 0; i < n; ++i)
+        if (v[(size_t)i] >= n || k[(size_t)i] != k_in[v[(size_t)i]]) {
+            set_error("og_debug_sort_wait_timeout: pair %lld is none of those sorted", (long long)i);
+            return OG_ERR_STATE;
+        }
+    return OG_OK;
+}
 
 size_t radix_sort_scratch_bytes(int64_t n) {
     int64_t ntiles = (n + kTile - 1) / kTile;

@@ -713,7 +713,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             part = it.y & 0xffu;
             if (kMulti) ti = it.y >> 8;
         } else if (kMulti) {
-            const uint64_t it = a.items ? a.items[item] : item;
+            const uint64_t it = a.items ? min(a.items[item], nitems - 1u) : item;   // (as below)
             int64_t lo_t = 0, hi_t = a.ntrees;  // goff[lo_t] <= item < goff[hi_t]
             while (hi_t - lo_t > 1) {
                 const int64_t mid = (lo_t + hi_t) >> 1;
@@ -722,7 +722,8 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             ti = lo_t;
             g = (int64_t)(it - a.goff[ti]);
         } else {
-            g = a.tree0.gorder ? (int64_t)a.tree0.gorder[item] : (int64_t)item;
+            // (the limit holds after a sort whose wait ran out: ST_TIMEOUT is set)
+            g = a.tree0.gorder ? (int64_t)min(a.tree0.gorder[item], (uint32_t)a.tree0.nall - 1u) : (int64_t)item;
         }
         const TreeView &T = kMulti ? a.trees[ti] : a.tree0;
         const uint32_t seg = kOneSeg ? 0u : T.gseg[g];

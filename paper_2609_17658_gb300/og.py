@@ -121,6 +121,8 @@ def lib():
         L.og_debug_fail_allocations.restype = C.c_int
         L.og_debug_scan_wait_timeout.argtypes = [P, i64]
         L.og_debug_scan_wait_timeout.restype = C.c_int
+        L.og_debug_sort_wait_timeout.argtypes = [P, i64, C.c_int32]
+        L.og_debug_sort_wait_timeout.restype = C.c_int
         L.og_serve_cancel.argtypes = [P, C.c_uint64]
         L.og_serve_cancel.restype = C.c_int
         L.og_sort_keys_noalloc.argtypes = [P, P, P, i64, P]
@@ -186,6 +188,13 @@ def og_debug_scan_wait_timeout(ctx, n: int) -> None:
     bounded wait runs out (tests of error handling; see include/og.h); raises
     OGError with OG_ERR_TIMEOUT."""
     _check(lib().og_debug_scan_wait_timeout(ctx, int(n)))
+
+
+def og_debug_sort_wait_timeout(ctx, n: int, keys_held: bool = False) -> None:
+    """Run the library's one-launch sort of n pairs with one block keeping back
+    its counts (or its keys); raises OGError(OG_ERR_TIMEOUT) once the bounded
+    waits of the others have run out and every pair left is one that came in."""
+    _check(lib().og_debug_sort_wait_timeout(ctx, int(n), int(bool(keys_held))))
 
 
 def og_serve_cancel(ctx, ticket: int) -> None:

@@ -172,3 +172,20 @@ def test_bounded_device_wait_runs_out_and_the_context_stays_usable():
             with pytest.raises(og.OGError) as e:
                 og.og_debug_scan_wait_timeout(ctx.h, n)
             assert e.value.status == og.OG_ERR_ARG
+
+
+@pytest.mark.parametrize("n", [16, 5000, 40000, 65536])
+@pytest.mark.parametrize("keys_held", [False, True])
+def test_a_wait_of_the_one_launch_sort_runs_out(n, keys_held):
+    """A block of the one-launch sort keeps back its digit counts, or its keys: the
+    other blocks' bounded waits run out, what is left in the arrays are pairs that
+    came in (the call checks every one), the status is OG_ERR_TIMEOUT, and the
+    same context then builds and walks bitwise as before."""
+    pos, mass, prm = _system(n=3000)
+    with og.Context(0) as ctx:
+        ref, rpp, rpn = og.Tree(ctx, pos, mass, prm).force()
+        with pytest.raises(og.OGError) as e:
+            og.og_debug_sort_wait_timeout(ctx.h, n, keys_held)
+        assert e.value.status == og.OG_ERR_TIMEOUT
+        acc, npp, npn = og.Tree(ctx, pos, mass, prm).force()
+    assert np.array_equal(acc, ref) and np.array_equal(npp, rpp) and np.array_equal(npn, rpn)
