@@ -916,10 +916,21 @@ og_status og_batch_force(og_ctx *c, int64_t nbox, const og_box *boxes, og_batch_
     t->h_seg_off[nbox] = off;
     // inputs.  Device pointers: a table of the boxes' arrays, read and written by
     // the kernels in place (512 boxes of 3 to 6 arrays each are as many copies of
-    // 2 to 4 us otherwise).  Host pointers: one buffer that holds them all.
+    // 2 to 4 us otherwise).  Host pointers, or device arrays that do not lie on their
+    // element's boundary (a copy takes those, a kernel's load does not): one buffer
+    // that holds them all.
+    auto aligned = [](const void *q, uintptr_t a) { return ((uintptr_t)q & (a - 1)) == 0; };
+    bool in_place = dev;
+    for (int64_t b = 0; b < nbox && in_place; ++b) {
+        const og_box &x = boxes[b];
+        in_place = aligned(x.pos, 8) && aligned(x.mass, 8) && aligned(x.a_old, 4) && aligned(x.acc, 4) &&
+                   aligned(x.n_pp, 4) && aligned(x.n_pn, 4);
+    }
+    const cudaMemcpyKind in_kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    const cudaMemcpyKind out_kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     const bool have_aold = p0.opening == OG_OPEN_REL && boxes[0].a_old != nullptr;
     const size_t table = ((size_t)nbox * sizeof(BoxIO) + 255) & ~(size_t)255;
-    size_t in_bytes = dev ? table
+    size_t in_bytes = in_place ? table
                           : (size_t)total * 4 * sizeof(double) + (have_aold ? (size_t)total * 3 * sizeof(float) : 0) + 512;
     void *in = nullptr;
     cudaError_t e;
@@ -927,7 +938,7 @@ og_status og_batch_force(og_ctx *c, int64_t nbox, const og_box *boxes, og_batch_
     double *d_pos = nullptr, *d_mass = nullptr;
     float *d_aold = nullptr;
     std::vector<BoxIO> io;
-    if (dev) {
+    if (in_place) {
         io.resize((size_t)nbox);
         for (int64_t b = 0; b < nbox; ++b)
             io[(size_t)b] = {boxes[b].pos, boxes[b].mass, boxes[b].a_old, boxes[b].acc, boxes[b].n_pp, boxes[b].n_pn};
@@ -945,9 +956,9 @@ og_status og_batch_force(og_ctx *c, int64_t nbox, const og_box *boxes, og_batch_
         d_aold = have_aold ? reinterpret_cast<float *>(d_mass + total) : nullptr;
         for (int64_t b = 0; b < nbox; ++b) {
             const int64_t o = t->h_seg_off[b], nb = boxes[b].n;
-            cudaMemcpyAsync(d_pos + 3 * o, boxes[b].pos, (size_t)nb * 3 * sizeof(double), cudaMemcpyHostToDevice, s);
-            cudaMemcpyAsync(d_mass + o, boxes[b].mass, (size_t)nb * sizeof(double), cudaMemcpyHostToDevice, s);
-            if (have_aold) cudaMemcpyAsync(d_aold + 3 * o, boxes[b].a_old, (size_t)nb * 3 * sizeof(float), cudaMemcpyHostToDevice, s);
+            cudaMemcpyAsync(d_pos + 3 * o, boxes[b].pos, (size_t)nb * 3 * sizeof(double), in_kind, s);
+            cudaMemcpyAsync(d_mass + o, boxes[b].mass, (size_t)nb * sizeof(double), in_kind, s);
+            if (have_aold) cudaMemcpyAsync(d_aold + 3 * o, boxes[b].a_old, (size_t)nb * 3 * sizeof(float), in_kind, s);
         }
     }
     og_status st = build_tree(t, d_pos, d_mass);
@@ -960,7 +971,7 @@ og_status og_batch_force(og_ctx *c, int64_t nbox, const og_box *boxes, og_batch_
         return st;
     }
     // results back to every box in its own order
-    if (dev) {
+    if (in_place) {
         k_unpermute_boxes<<<nblk(total), kT, 0, s>>>(total, t->inv, t->sseg, t->seg_off, t->io, t->a_sorted,
                                                      t->npp_sorted, t->npn_sorted); note_launch();
         cudaFreeAsync(in, s);
@@ -976,9 +987,9 @@ og_status og_batch_force(og_ctx *c, int64_t nbox, const og_box *boxes, og_batch_
                                                o_acc, o_pp, o_pn, ForceReport{}); note_launch();
         for (int64_t b = 0; b < nbox; ++b) {
             const int64_t o = t->h_seg_off[b], nb = boxes[b].n;
-            cudaMemcpyAsync(boxes[b].acc, o_acc + 3 * o, (size_t)nb * 3 * sizeof(float), cudaMemcpyDeviceToHost, s);
-            if (boxes[b].n_pp) cudaMemcpyAsync(boxes[b].n_pp, o_pp + o, (size_t)nb * sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-            if (boxes[b].n_pn) cudaMemcpyAsync(boxes[b].n_pn, o_pn + o, (size_t)nb * sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+            cudaMemcpyAsync(boxes[b].acc, o_acc + 3 * o, (size_t)nb * 3 * sizeof(float), out_kind, s);
+            if (boxes[b].n_pp) cudaMemcpyAsync(boxes[b].n_pp, o_pp + o, (size_t)nb * sizeof(uint32_t), out_kind, s);
+            if (boxes[b].n_pn) cudaMemcpyAsync(boxes[b].n_pn, o_pn + o, (size_t)nb * sizeof(uint32_t), out_kind, s);
         }
         cudaFreeAsync(out, s);
     }
