@@ -379,12 +379,11 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
                     float *acc_sorted, float *ms_out, bool use_order,
                     const uint32_t *subset = nullptr, int64_t nsubset = 0,
                     float *pot_sorted = nullptr, bool defer = false);
-// One walk launch over the groups of several trees (the serving loop), in
+// One Barnes-Hut walk launch over the groups of several trees (the serving loop), in
 // decreasing order of their previous list lengths.  Every tree's per-box
 // parameters must agree on split on/off.  tree_interactions (or null): the
 // interactions evaluated for each tree.
-og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int opening,
-                     const float *const *a_old_sorted, float *const *acc_sorted, float *ms_out,
+og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, float *const *acc_sorted, float *ms_out,
                      int64_t *interactions, int64_t *tree_interactions = nullptr);
 // cell extents for a built tree (so that it can join a walk of refitted trees)
 og_status cell_extents(og_tree *t);

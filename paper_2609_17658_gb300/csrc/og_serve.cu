@@ -288,8 +288,7 @@ void engine_step(Server *S) {
         float ms1 = 0;
         int64_t in1 = 0;
         std::vector<int64_t> ti(tv.size(), 0);
-        st = walk_multi(c, tv.data(), (int64_t)tv.size(), OG_OPEN_BH, nullptr, av.data(), &ms1, &in1,
-                        ti.data());
+        st = walk_multi(c, tv.data(), (int64_t)tv.size(), av.data(), &ms1, &in1, ti.data());
         ms += ms1;
         inter += in1;
         for (size_t q = 0; q < idx.size(); ++q) tinter[idx[q]] = ti[q];

@@ -158,7 +158,7 @@ struct WalkArgs {
     int64_t list_cap;
     unsigned long long *work;     // item counter
     int warps, chunk;             // launch shape: warps per block, far-chunk entries
-    uint2 *sitems;                // further parts of groups: (group, tree << 8 | part)
+    uint2 *sitems;                // further parts of groups: (group, part)
     unsigned long long *nsplit;   // their number
     int second;                   // the launch that walks them
     int one_seg;                  // a single tree of one box: its parameters are p0
@@ -676,6 +676,8 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a);
 
 template <int kOpen, bool kSplit, bool kDump, bool kRefit, bool kMulti, bool kPot, bool kOneSeg>
 __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
+    // walks in parts: the relative criterion, one tree
+    constexpr bool kParted = kOpen == OG_OPEN_REL && !kMulti;
     extern __shared__ __align__(16) unsigned char smem[];
     // layout: per warp, its stack, near chunk and far chunk (warp_smem bytes);
     // blockDim.x = 32 * a.warps and the launch sizes smem to match
@@ -693,13 +695,13 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
     // item is its own number (neighbours on different SMs), the rest come from a
     // counter: the first ones taken there too would queue every warp of the launch
     // on one address.
-    const uint32_t nitems = a.second ? (uint32_t)*a.nsplit : (uint32_t)(kMulti ? a.nitems : a.tree0.ngroups);
+    const uint32_t nitems = kParted && a.second ? (uint32_t)*a.nsplit : (uint32_t)(kMulti ? a.nitems : a.tree0.ngroups);
     uint32_t item = gridDim.x * (uint32_t)warp + blockIdx.x;
     auto advance = [&] {
         const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
         if (nitems <= nwarps) return false;
         uint32_t k = 0;
-        if (lane == 0) k = (uint32_t)atomicAdd(a.work + (a.second ? 4 : 0), 1ull);
+        if (lane == 0) k = (uint32_t)atomicAdd(a.work + (kParted && a.second ? 4 : 0), 1ull);
         item = nwarps + __shfl_sync(FULL, k, 0);
         return true;
     };
@@ -707,11 +709,10 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         int64_t g;
         int64_t ti = 0;
         uint32_t part = 0;
-        if (a.second) {
+        if (kParted && a.second) {
             const uint2 it = a.sitems[item];
             g = it.x;
-            part = it.y & 0xffu;
-            if (kMulti) ti = it.y >> 8;
+            part = it.y;
         } else if (kMulti) {
             const uint64_t it = a.items ? min(a.items[item], nitems - 1u) : item;   // (as below)
             int64_t lo_t = 0, hi_t = a.ntrees;  // goff[lo_t] <= item < goff[hi_t]
@@ -774,7 +775,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
 
         // the root's children, or this part's share of what the first part left
         int sp = 1, cf = 0, cn = 0;
-        if (part > 0u) {
+        if (kParted && part > 0u) {
             const uint32_t left = T.nspill[g];
             sp = left >= part ? (int)((left - part) / (kParts - 1u)) + 1 : 0;
             for (int k = lane; k < sp; k += 32)
@@ -783,7 +784,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             stk[0] = make_uint2(T.ncbeg[seg], T.nccnt[seg]);
         }
         __syncwarp();
-        uint32_t quota = part > 0u || !p.split_long ? 0xffffffffu : kQuota;
+        const uint32_t quota = !kParted || part > 0u || !p.split_long ? 0xffffffffu : kQuota;
         bool leave = false;
         uint32_t rounds = 0;
         const uint32_t nchild = (uint32_t)T.nchild, max_rounds = (uint32_t)T.max_rounds;
@@ -896,7 +897,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             __syncwarp();
             // a chunk above its limit, or the walk's end, is evaluated; flushes are
             // rare, so they are hinted off the round's path
-            leave = rounds >= quota && sp > 0 && sp <= kSpill;
+            leave = kParted && rounds >= quota && sp > 0 && sp <= kSpill;
             const bool done = sp == 0 || leave;
             if (__builtin_expect(done || cn > kNearFlush, 0)) {
                 const int q = pad_chunk(chn, cn, R, 1u, lane, box.hi);
@@ -946,7 +947,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         }
         // A group in parts: every part leaves its sums and counts, and the one that
         // finishes last adds them up in the order of the parts.
-        if (leave || part > 0u) {
+        if (kParted && (leave || part > 0u)) {
             const uint64_t m = (uint64_t)T.n, ax = kPot ? 4u : 3u;
             if (rep == 0u) {
                 float *w = T.psum + part * ax * m;
@@ -966,7 +967,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                     T.pdone[g] = 0u;
                     const unsigned long long at = atomicAdd(a.nsplit, (unsigned long long)(kParts - 1u));
                     for (uint32_t q = 1; q < kParts; ++q)
-                        a.sitems[at + q - 1u] = make_uint2((uint32_t)g, ((uint32_t)ti << 8) | q);
+                        a.sitems[at + q - 1u] = make_uint2((uint32_t)g, q);
                 }
                 __syncwarp();
                 continue;
@@ -1048,7 +1049,7 @@ void launch_walk_t(const WalkArgs &a, int64_t nitems, cudaStream_t s, int sms) {
     if (want < grid) grid = want;
     if (grid < 1) grid = 1;
     launch_pdl(kern, (unsigned)grid, (unsigned)a.warps * 32u, smem, s, a);
-    if (a.nsplit) {
+    if (kOpen == OG_OPEN_REL && a.nsplit) {
         // the further parts: their number is known on the device only
         WalkArgs b = a;
         b.second = 1;
@@ -1066,8 +1067,11 @@ void launch_walk(const WalkArgs &a, bool dump, bool refit, bool multi, bool pot,
         if (refit) launch_walk_t<kOpen, kSplit, false, true, false, true, true>(a, nitems, s, sms);
         else launch_walk_t<kOpen, kSplit, false, false, false, true, true>(a, nitems, s, sms);
     } else if (multi) {
-        if (refit) launch_walk_t<kOpen, kSplit, false, true, true>(a, nitems, s, sms);
-        else launch_walk_t<kOpen, kSplit, false, false, true>(a, nitems, s, sms);
+        // several trees: the serving loop's walks, Barnes-Hut
+        if constexpr (kOpen == OG_OPEN_BH) {
+            if (refit) launch_walk_t<kOpen, kSplit, false, true, true>(a, nitems, s, sms);
+            else launch_walk_t<kOpen, kSplit, false, false, true>(a, nitems, s, sms);
+        }
     } else if (dump) {
         if (refit) launch_walk_t<kOpen, kSplit, true, true, false>(a, nitems, s, sms);
         else launch_walk_t<kOpen, kSplit, true, false, false>(a, nitems, s, sms);
@@ -1437,20 +1441,19 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
     return OG_OK;
 }
 
-og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int opening,
-                     const float *const *a_old_sorted, float *const *acc_sorted, float *ms_out,
+og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, float *const *acc_sorted, float *ms_out,
                      int64_t *interactions, int64_t *tree_interactions) {
     cudaStream_t s = c->stream;
     if (ntrees < 1) return OG_OK;
     std::vector<TreeView> hv((size_t)ntrees);
     std::vector<uint64_t> hoff((size_t)ntrees + 1);
-    std::vector<PassScratch> sc((size_t)ntrees);
     bool split = false, refit = false;
     uint64_t total = 0;
     for (int64_t k = 0; k < ntrees; ++k) {
         WalkParams wp;
-        og_status st = prepare_view(trees[k], opening, false, a_old_sorted ? a_old_sorted[k] : nullptr,
-                                    acc_sorted[k], false, true, &hv[k], &wp, &sc[k]);
+        PassScratch none;
+        og_status st = prepare_view(trees[k], OG_OPEN_BH, false, nullptr, acc_sorted[k], false, true, &hv[k], &wp,
+                                    &none);
         if (st) return st;
         if (k == 0) split = wp.split;
         else if (wp.split != split) {
@@ -1475,24 +1478,9 @@ og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int openi
     const int64_t nitems = (int64_t)total;
     size_t bytes = (size_t)ntrees * sizeof(TreeView) + (size_t)(ntrees + 1) * 8 + (size_t)nitems * 24 +
                    radix_sort_scratch_bytes(nitems) + (size_t)ntrees * 8 + 4096;
-    // the parts of long walks: their items, then every tree's scratch
-    const size_t parts_at = (bytes + 255) & ~(size_t)255;
-    size_t item_bytes = 0, pass_bytes = 0;
-    for (const PassScratch &x : sc) {
-        item_bytes += (size_t)x.item_bytes();
-        pass_bytes += (size_t)x.bytes();
-    }
-    bytes = parts_at + item_bytes + pass_bytes;
     void *tmp = nullptr;
     cudaError_t err;
     if ((err = dev_malloc_async(&tmp, bytes, s)) != cudaSuccess) return cuda_fail(err, "cudaMallocAsync (walk items)");
-    {
-        char *at = static_cast<char *>(tmp) + parts_at + item_bytes;
-        for (int64_t k = 0; k < ntrees; ++k) {
-            sc[k].place(at, hv[k]);
-            at += sc[k].bytes();
-        }
-    }
     char *q = static_cast<char *>(tmp);
     TreeView *dv = reinterpret_cast<TreeView *>(q);
     q += ((size_t)ntrees * sizeof(TreeView) + 255) & ~(size_t)255;
@@ -1517,10 +1505,6 @@ og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int openi
     a.items = alt ? v1 : v0;
     a.ntrees = ntrees;
     a.nitems = nitems;
-    if (item_bytes) {
-        a.sitems = reinterpret_cast<uint2 *>(static_cast<char *>(tmp) + parts_at);
-        a.nsplit = c->d_counters + 3;
-    }
     a.tree_inter = tint;
     cudaMemsetAsync(tint, 0, (size_t)ntrees * sizeof(unsigned long long), s);
     clear_counters(c);
@@ -1528,7 +1512,7 @@ og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, int openi
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     cudaEventRecord(e0, s);
-    launch(a, opening, split, false, refit, true, nitems, s);
+    launch(a, OG_OPEN_BH, split, false, refit, true, nitems, s);
     cudaEventRecord(e1, s);
     std::vector<unsigned long long> hti(tree_interactions ? (size_t)ntrees : 0);
     if (tree_interactions)
