@@ -158,7 +158,11 @@ og_status og_tree_refit(og_tree *t, const double *pos);
  * a_old: float[N][3] previous accelerations for OG_OPEN_REL, or NULL (then a
  *        first Barnes-Hut pass with theta_first_pass supplies them);
  * acc:   float[N][3] out;  n_pp, n_pn: uint32[N] out or NULL.
- * n_pp(i) = PP entries of i's group list minus itself, n_pn(i) = PN entries. */
+ * n_pp(i) = PP entries of i's group list minus itself, n_pn(i) = PN entries.
+ * Device memory beside the tree, for the duration of the call: 24 B per group
+ * for their order, and with OG_OPEN_REL and a box of 2049 to 196608 particles
+ * some 20 B per particle and 8 MB for walks in parts; the host arrays' copies
+ * come on top.  The same holds for the other force calls. */
 og_status og_tree_force(og_tree *t, const float *a_old, float *acc, uint32_t *n_pp,
                         uint32_t *n_pn);
 

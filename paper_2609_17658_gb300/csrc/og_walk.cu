@@ -45,6 +45,7 @@
 // atomic counter, in decreasing order of the previous pass's list length
 // when that is known (longest first shortens the tail of the launch), and in
 // parts where a list is much longer than the others (kQuota).
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <type_traits>
@@ -90,8 +91,18 @@ constexpr int kMaxChunk = 1024;
 // parts: 262-302 us at 100k.  The Barnes-Hut lists are even enough that splitting
 // them gained nothing at any size (131k 258 -> 265-280 us).
 constexpr uint32_t kQuota = 48, kParts = 8;
-constexpr int kSpill = kStackCap;      // ranges a walk can leave
+constexpr int kSpill = 192;            // ranges a walk can leave (with more it goes on until they are fewer)
+static_assert(kSpill > kStackDeep && kSpill <= kStackCap, "above kStackDeep a walk soon comes back below it");
 constexpr int64_t kSplitMin = 2048, kSplitMax = 196608;
+// Few groups leave anything: 1 to 2 in 100 of a clustered system of 10k to 190k, 1812 of
+// 370k in a batch of 8M particles.  What they leave goes to slots that the groups take
+// as they come, one for every 320 particles (6 in 100 groups) up to kSlotMax.  A
+// group that finds no slot left walks its parts one after another in its own warp,
+// and adds them up in the same order, so its sums are the same; a launch with that
+// many of them is a full one anyhow.  At most 18 B a particle and 8 MB for the warps' own
+// places, where a place per group and partial sums per particle took 250 B a particle.
+constexpr int64_t kSlotParticles = 320, kSlotMin = 32, kSlotMax = 2048;
+constexpr int kWarpsPerSm = 21;        // resident ones at most (96 registers a thread)
 
 // shared memory of one warp: its stack, near chunk and far chunk
 __host__ __device__ constexpr size_t warp_smem(int chunk) {
@@ -139,12 +150,21 @@ struct TreeView {
     float *pot;                   // [n] sorted, out (potential launches only)
     uint32_t *npp, *npn;          // [n] sorted, out
     int has_cost;                 // gcost holds the list lengths of a previous pass
-    // groups walked in parts (null: never); in scratch of the pass
-    uint2 *spill;                 // kSpill child ranges per group
-    uint32_t *nspill, *pdone;     // their number, and the further parts finished, per group
-    uint2 *pcnt;                  // [part][group] PP and PN entries
-    float *psum;                  // partial sums: [part][axis][particle]
     int64_t nall;                 // groups of the tree (ngroups: those to walk)
+};
+
+// Places of groups walked in parts, in scratch of the pass: slots that the groups
+// take, then one place per warp for the groups that find none.
+struct Parts {
+    uint32_t slots, own;          // their numbers
+    unsigned long long *taken;    // groups that asked for a slot (null: no walks in parts)
+    uint2 *head;                  // [slot, then warp] group, ranges left
+    uint32_t *done;               // [slot, then warp] further parts finished
+    uint2 *spill;                 // [slot, then warp][kSpill] child ranges
+    uint2 *cnt;                   // [slot][part] PP and PN entries
+    float *sums;                  // [slot][part][axis][target]
+    uint2 *own_cnt;               // [warp], summed over the parts so far
+    float *own_sums;              // [warp][axis][target], the same
 };
 
 struct WalkArgs {
@@ -158,9 +178,8 @@ struct WalkArgs {
     int64_t list_cap;
     unsigned long long *work;     // item counter
     int warps, chunk;             // launch shape: warps per block, far-chunk entries
-    uint2 *sitems;                // further parts of groups: (group, part)
-    unsigned long long *nsplit;   // their number
-    int second;                   // the launch that walks them
+    Parts parts;
+    int second;                   // the launch that walks the further parts
     int one_seg;                  // a single tree of one box: its parameters are p0
     WalkParams p0;                // the box's parameters, in the launch's own argument space
     unsigned long long *inter;    // interactions evaluated
@@ -695,7 +714,9 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
     // item is its own number (neighbours on different SMs), the rest come from a
     // counter: the first ones taken there too would queue every warp of the launch
     // on one address.
-    const uint32_t nitems = kParted && a.second ? (uint32_t)*a.nsplit : (uint32_t)(kMulti ? a.nitems : a.tree0.ngroups);
+    const uint32_t nitems =
+        kParted && a.second ? (uint32_t)min(*a.parts.taken, (unsigned long long)a.parts.slots) * (kParts - 1u)
+                            : (uint32_t)(kMulti ? a.nitems : a.tree0.ngroups);
     uint32_t item = gridDim.x * (uint32_t)warp + blockIdx.x;
     auto advance = [&] {
         const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
@@ -705,14 +726,14 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         item = nwarps + __shfl_sync(FULL, k, 0);
         return true;
     };
-    for (bool more = true; more && item < nitems; more = advance()) {
+    uint32_t job = 0;              // a further part of a group (kParted): its place << 3 | part
+    static_assert(kParts == 8, "a job's low three bits");
+    for (bool more = true; more && item < nitems; more = (kParted && !a.second && job) || advance()) {
         int64_t g;
         int64_t ti = 0;
-        uint32_t part = 0;
-        if (kParted && a.second) {
-            const uint2 it = a.sitems[item];
-            g = it.x;
-            part = it.y;
+        if (kParted && a.second) job = item / (kParts - 1u) << 3 | (1u + item % (kParts - 1u));
+        if (kParted && job) {
+            g = a.parts.head[job >> 3].x;
         } else if (kMulti) {
             const uint64_t it = a.items ? min(a.items[item], nitems - 1u) : item;   // (as below)
             int64_t lo_t = 0, hi_t = a.ntrees;  // goff[lo_t] <= item < goff[hi_t]
@@ -775,11 +796,12 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
 
         // the root's children, or this part's share of what the first part left
         int sp = 1, cf = 0, cn = 0;
+        const uint32_t part = job & 7u;
         if (kParted && part > 0u) {
-            const uint32_t left = T.nspill[g];
+            const uint32_t left = a.parts.head[job >> 3].y;
             sp = left >= part ? (int)((left - part) / (kParts - 1u)) + 1 : 0;
             for (int k = lane; k < sp; k += 32)
-                stk[k] = T.spill[(uint64_t)g * kSpill + part - 1u + (uint32_t)k * (kParts - 1u)];
+                stk[k] = a.parts.spill[(uint64_t)(job >> 3) * kSpill + part - 1u + (uint32_t)k * (kParts - 1u)];
         } else if (lane == 0) {
             stk[0] = make_uint2(T.ncbeg[seg], T.nccnt[seg]);
         }
@@ -927,6 +949,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         }
         if (overflow) {
             if (lane == 0) atomicOr(a.status, ST_STACK_OVF);
+            job = 0u;
             __syncwarp();
             continue;
         }
@@ -948,53 +971,87 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         // A group in parts: every part leaves its sums and counts, and the one that
         // finishes last adds them up in the order of the parts.
         if (kParted && (leave || part > 0u)) {
-            const uint64_t m = (uint64_t)T.n, ax = kPot ? 4u : 3u;
-            if (rep == 0u) {
-                float *w = T.psum + part * ax * m;
-                w[i0] = vx.x; w[m + i0] = vy.x; w[2 * m + i0] = vz.x;
-                if (kPot) w[3 * m + i0] = vp.x;
-                if (two) {
-                    w[i1] = vx.y; w[m + i1] = vy.y; w[2 * m + i1] = vz.y;
-                    if (kPot) w[3 * m + i1] = vp.y;
+            constexpr uint32_t ax = kPot ? 4u : 3u;
+            const uint32_t t0 = 2u * tl, t1 = t0 + 1u;   // this lane's targets (t1 if `two`)
+            const uint32_t slots = a.parts.slots;
+            uint32_t slot = job >> 3;
+            if (part == 0u) {
+                unsigned long long k = 0;
+                if (lane == 0) k = atomicAdd(a.parts.taken, 1ull);
+                slot = __shfl_sync(FULL, (uint32_t)min(k, (unsigned long long)slots), 0);
+                if (slot == slots) slot += blockIdx.x * (blockDim.x >> 5) + (uint32_t)warp;
+                for (int q = lane; q < sp; q += 32) a.parts.spill[(uint64_t)slot * kSpill + q] = stk[q];
+                if (lane == 0) {
+                    a.parts.head[slot] = make_uint2((uint32_t)g, (uint32_t)sp);
+                    a.parts.done[slot] = 0u;
                 }
             }
-            if (lane == 0) T.pcnt[(uint64_t)part * (uint64_t)T.nall + (uint64_t)g] = make_uint2(cnt_pp, cnt_pn);
-            if (part == 0u) {
-                // the further parts and the ranges they share (read by the second launch)
-                for (int k = lane; k < sp; k += 32) T.spill[(uint64_t)g * kSpill + k] = stk[k];
-                if (lane == 0) {
-                    T.nspill[g] = (uint32_t)sp;
-                    T.pdone[g] = 0u;
-                    const unsigned long long at = atomicAdd(a.nsplit, (unsigned long long)(kParts - 1u));
-                    for (uint32_t q = 1; q < kParts; ++q)
-                        a.sitems[at + q - 1u] = make_uint2((uint32_t)g, q);
+            if (slot >= slots) {
+                // no slot: the parts follow in this warp, as its next items
+                float *w = a.parts.own_sums + (uint64_t)(slot - slots) * (ax * 32u);
+                auto run = [&](uint32_t at, float &v) {
+                    if (part > 0u) v = __fadd_rn(w[at], v);
+                    w[at] = v;
+                };
+                if (rep == 0u) {
+                    run(t0, vx.x); run(32u + t0, vy.x); run(64u + t0, vz.x);
+                    if (kPot) run(96u + t0, vp.x);
+                    if (two) {
+                        run(t1, vx.y); run(32u + t1, vy.y); run(64u + t1, vz.y);
+                        if (kPot) run(96u + t1, vp.y);
+                    }
+                }
+                uint2 &c = a.parts.own_cnt[slot - slots];
+                if (part > 0u) {
+                    cnt_pp += c.x;
+                    cnt_pn += c.y;
                 }
                 __syncwarp();
-                continue;
-            }
-            __threadfence();
-            __syncwarp();
-            uint32_t before = 0;
-            if (lane == 0) before = atomicAdd(&T.pdone[g], 1u);
-            before = __shfl_sync(FULL, before, 0);
-            if (before + 2u != kParts) continue;
-            __threadfence();
-            auto total = [&](uint64_t at) {
-                float v = __ldcg(T.psum + at);
-                for (uint32_t q = 1; q < kParts; ++q) v = __fadd_rn(v, __ldcg(T.psum + q * ax * m + at));
-                return v;
-            };
-            if (rep == 0u) {
-                vx = make_float2(total(i0), total(i1));
-                vy = make_float2(total(m + i0), total(m + i1));
-                vz = make_float2(total(2 * m + i0), total(2 * m + i1));
-                if (kPot) vp = make_float2(total(3 * m + i0), total(3 * m + i1));
-            }
-            cnt_pp = cnt_pn = 0u;
-            for (uint32_t q = 0; q < kParts; ++q) {
-                const uint2 c = __ldcg(&T.pcnt[(uint64_t)q * (uint64_t)T.nall + (uint64_t)g]);
-                cnt_pp += c.x;
-                cnt_pn += c.y;
+                if (lane == 0) c = make_uint2(cnt_pp, cnt_pn);
+                job = part + 1u < kParts ? slot << 3 | (part + 1u) : 0u;
+                __syncwarp();
+                if (job) continue;
+            } else {
+                float *w = a.parts.sums + ((uint64_t)slot * kParts + part) * (ax * 32u);
+                if (rep == 0u) {
+                    w[t0] = vx.x; w[32u + t0] = vy.x; w[64u + t0] = vz.x;
+                    if (kPot) w[96u + t0] = vp.x;
+                    if (two) {
+                        w[t1] = vx.y; w[32u + t1] = vy.y; w[64u + t1] = vz.y;
+                        if (kPot) w[96u + t1] = vp.y;
+                    }
+                }
+                if (lane == 0) a.parts.cnt[(uint64_t)slot * kParts + part] = make_uint2(cnt_pp, cnt_pn);
+                if (part == 0u) {          // the second launch walks the further parts
+                    __syncwarp();
+                    continue;
+                }
+                __threadfence();
+                __syncwarp();
+                uint32_t before = 0;
+                if (lane == 0) before = atomicAdd(&a.parts.done[slot], 1u);
+                before = __shfl_sync(FULL, before, 0);
+                if (before + 2u != kParts) continue;
+                __threadfence();
+                w = a.parts.sums + (uint64_t)slot * kParts * (ax * 32u);
+                auto total = [&](uint32_t at) {
+                    float v = __ldcg(w + at);
+                    for (uint32_t q = 1; q < kParts; ++q) v = __fadd_rn(v, __ldcg(w + q * (ax * 32u) + at));
+                    return v;
+                };
+                if (rep == 0u) {
+                    const uint32_t u1 = two ? t1 : t0;
+                    vx = make_float2(total(t0), total(u1));
+                    vy = make_float2(total(32u + t0), total(32u + u1));
+                    vz = make_float2(total(64u + t0), total(64u + u1));
+                    if (kPot) vp = make_float2(total(96u + t0), total(96u + u1));
+                }
+                cnt_pp = cnt_pn = 0u;
+                for (uint32_t q = 0; q < kParts; ++q) {
+                    const uint2 c = __ldcg(&a.parts.cnt[(uint64_t)slot * kParts + q]);
+                    cnt_pp += c.x;
+                    cnt_pn += c.y;
+                }
             }
         }
         if (rep == 0u) {
@@ -1047,13 +1104,15 @@ void launch_walk_t(const WalkArgs &a, int64_t nitems, cudaStream_t s, int sms) {
     int64_t want = (nitems + a.warps - 1) / a.warps;
     int64_t grid = (int64_t)sms * per_sm;
     if (want < grid) grid = want;
+    // every warp has a place of its own, where a group may find no slot
+    if (a.parts.own && grid > a.parts.own / a.warps) grid = a.parts.own / a.warps;
     if (grid < 1) grid = 1;
     launch_pdl(kern, (unsigned)grid, (unsigned)a.warps * 32u, smem, s, a);
-    if (kOpen == OG_OPEN_REL && a.nsplit) {
+    if (kOpen == OG_OPEN_REL && a.parts.taken) {
         // the further parts: their number is known on the device only
         WalkArgs b = a;
         b.second = 1;
-        const int64_t most = nitems * (int64_t)(kParts - 1u), all = (int64_t)sms * per_sm;
+        const int64_t most = a.parts.slots * (int64_t)(kParts - 1u), all = (int64_t)sms * per_sm;
         grid = (most + a.warps - 1) / a.warps;
         launch_pdl(kern, (unsigned)(grid < all ? grid : all), (unsigned)a.warps * 32u, smem, s, b);
     }
@@ -1119,6 +1178,13 @@ __global__ void k_item_keys(int64_t nitems, int64_t ntrees, const uint64_t *__re
     vals[q] = (uint32_t)q;
 }
 
+int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
 template <int kOpen>
 void dispatch(const WalkArgs &a, bool split, bool dump, bool refit, bool multi, bool pot,
               int64_t nitems, cudaStream_t s, int sms) {
@@ -1128,39 +1194,43 @@ void dispatch(const WalkArgs &a, bool split, bool dump, bool refit, bool multi, 
 
 void launch(const WalkArgs &a, int opening, bool split, bool dump, bool refit, bool multi,
             int64_t nitems, cudaStream_t s, bool pot = false) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     if (opening == OG_OPEN_BH) dispatch<OG_OPEN_BH>(a, split, dump, refit, multi, pot, nitems, s, sms);
     else dispatch<OG_OPEN_REL>(a, split, dump, refit, multi, pot, nitems, s, sms);
 }
 
-// Scratch of one tree's pass: the partial results of groups walked in parts.
-struct PassScratch {
-    uint64_t n = 0, groups = 0, axes = 3;
-    bool used = false;
-    static uint64_t up(uint64_t b) { return (b + 255u) & ~(uint64_t)255u; }
-    uint64_t item_bytes() const { return used ? up(groups * (kParts - 1u) * sizeof(uint2)) : 0; }
-    uint64_t bytes() const {
-        if (!used) return 0;
-        return up(groups * kSpill * sizeof(uint2)) + 2 * up(groups * 4u) + up(groups * kParts * sizeof(uint2)) +
-               up(n * kParts * axes * 4u);
+// The places of a pass of `groups` walks over n particles: one allocation, laid out by place().
+struct PartsScratch {
+    uint64_t slots, own, axes;
+    PartsScratch(int64_t n, int64_t groups, bool pot) : axes(pot ? 4u : 3u) {
+        const int64_t want = std::min(std::max(n / kSlotParticles, kSlotMin), kSlotMax);
+        slots = (uint64_t)std::min(want, groups);
+        own = want >= groups ? 0u : (uint64_t)std::min<int64_t>(groups + kMaxWarps, (int64_t)sm_count() * kWarpsPerSm);
     }
-    // hand out the arrays from q (bytes() long)
-    void place(char *q, TreeView &v) const {
-        if (!used) return;
-        v.spill = reinterpret_cast<uint2 *>(q); q += up(groups * kSpill * sizeof(uint2));
-        v.nspill = reinterpret_cast<uint32_t *>(q); q += up(groups * 4u);
-        v.pdone = reinterpret_cast<uint32_t *>(q); q += up(groups * 4u);
-        v.pcnt = reinterpret_cast<uint2 *>(q); q += up(groups * kParts * sizeof(uint2));
-        v.psum = reinterpret_cast<float *>(q);
+    uint64_t place(char *base, Parts *p) const {
+        uint64_t at = 0;
+        auto take = [&](auto *&q, uint64_t count) {
+            using T = std::remove_reference_t<decltype(*q)>;
+            q = reinterpret_cast<T *>(base + at);
+            at += (count * sizeof(T) + 255u) & ~(uint64_t)255u;
+        };
+        take(p->head, slots + own);
+        take(p->done, slots + own);
+        take(p->spill, (slots + own) * kSpill);
+        take(p->cnt, slots * kParts);
+        take(p->sums, slots * kParts * axes * 32u);
+        take(p->own_cnt, own);
+        take(p->own_sums, own * axes * 32u);
+        p->slots = (uint32_t)slots;
+        p->own = (uint32_t)own;
+        return at;
     }
 };
 
 // Per-box parameters of a pass (uploaded if the launch reads them as a table) and the tree's view.  The first
 // pass of the relative criterion is Barnes-Hut with theta_first_pass.
 og_status prepare_view(og_tree *t, int opening, bool first_pass, const float *a_old_sorted,
-                       float *acc_sorted, bool pot, bool table, TreeView *v, WalkParams *wp0, PassScratch *sc) {
+                       float *acc_sorted, bool table, TreeView *v, WalkParams *wp0, bool *split_long) {
     cudaStream_t s = t->ctx->stream;
     const int64_t B = t->nseg;
     t->h_wp.resize((size_t)B);
@@ -1172,11 +1242,8 @@ og_status prepare_view(og_tree *t, int opening, bool first_pass, const float *a_
         if (!first_pass && t->unscaled_out) t->h_wp[b].out_scale = 1.0f;
         const int64_t nb = (int64_t)t->h_seg_off[b + 1] - (int64_t)t->h_seg_off[b];
         t->h_wp[b].split_long = opening == OG_OPEN_REL && nb > kSplitMin && nb <= kSplitMax;
-        if (t->h_wp[b].split_long) sc->used = true;
+        if (t->h_wp[b].split_long) *split_long = true;
     }
-    sc->n = (uint64_t)t->n;
-    sc->groups = (uint64_t)t->ngroups;
-    sc->axes = pot ? 4u : 3u;
     *wp0 = t->h_wp[0];
     WalkParams *dp = t->segp + (first_pass ? 0 : B);
     if (table) {
@@ -1343,23 +1410,23 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
     cudaStream_t s = t->ctx->stream;
     WalkArgs a{};
     WalkParams wp;
-    PassScratch sc;
+    bool split_long = false;
     // one box without list dumps: the parameters come with the launch
     const bool dump = (t->seg_prm[0].flags & OG_DEBUG_DUMP_LISTS) != 0 && !pot_sorted;
-    og_status st = prepare_view(t, opening, first_pass, a_old_sorted, acc_sorted, pot_sorted != nullptr,
-                                t->nseg > 1 || dump, &a.tree0, &wp, &sc);
+    og_status st = prepare_view(t, opening, first_pass, a_old_sorted, acc_sorted, t->nseg > 1 || dump, &a.tree0,
+                                &wp, &split_long);
     if (st) return st;
     fill_common(a, t->ctx, t);
     a.one_seg = t->nseg == 1 ? 1 : 0;
     a.p0 = t->h_wp[0];
     cudaError_t err;
     void *sort_tmp = nullptr, *pass_tmp = nullptr;
-    if (sc.used) {
-        if ((err = dev_malloc_async(&pass_tmp, sc.item_bytes() + sc.bytes(), s)) != cudaSuccess)
+    if (split_long) {
+        const PartsScratch sc(t->n, subset ? nsubset : t->ngroups, pot_sorted != nullptr);
+        if ((err = dev_malloc_async(&pass_tmp, sc.place(nullptr, &a.parts), s)) != cudaSuccess)
             return cuda_fail(err, "cudaMallocAsync (walk parts)");
-        a.sitems = static_cast<uint2 *>(pass_tmp);
-        a.nsplit = t->ctx->d_counters + 3;
-        sc.place(static_cast<char *>(pass_tmp) + sc.item_bytes(), a.tree0);
+        sc.place(static_cast<char *>(pass_tmp), &a.parts);
+        a.parts.taken = t->ctx->d_counters + 3;
     }
     auto release = [&] {
         if (pass_tmp) cudaFreeAsync(pass_tmp, s);
@@ -1451,9 +1518,9 @@ og_status walk_multi(og_ctx *c, og_tree *const *trees, int64_t ntrees, float *co
     uint64_t total = 0;
     for (int64_t k = 0; k < ntrees; ++k) {
         WalkParams wp;
-        PassScratch none;
-        og_status st = prepare_view(trees[k], OG_OPEN_BH, false, nullptr, acc_sorted[k], false, true, &hv[k], &wp,
-                                    &none);
+        bool split_long = false;             // never with Barnes-Hut
+        og_status st = prepare_view(trees[k], OG_OPEN_BH, false, nullptr, acc_sorted[k], true, &hv[k], &wp,
+                                    &split_long);
         if (st) return st;
         if (k == 0) split = wp.split;
         else if (wp.split != split) {
