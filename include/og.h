@@ -161,7 +161,7 @@ og_status og_tree_refit(og_tree *t, const double *pos);
  * n_pp(i) = PP entries of i's group list minus itself, n_pn(i) = PN entries.
  * Device memory beside the tree, for the duration of the call: 24 B per group
  * for their order, and with OG_OPEN_REL and a box of 2049 to 196608 particles
- * some 20 B per particle and 8 MB for walks in parts; the host arrays' copies
+ * some 31 B per particle and 12 MB for walks in parts; the host arrays' copies
  * come on top.  The same holds for the other force calls. */
 og_status og_tree_force(og_tree *t, const float *a_old, float *acc, uint32_t *n_pp,
                         uint32_t *n_pn);

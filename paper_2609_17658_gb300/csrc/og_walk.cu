@@ -99,7 +99,7 @@ constexpr int64_t kSplitMin = 2048, kSplitMax = 196608;
 // as they come, one for every 320 particles (6 in 100 groups) up to kSlotMax.  A
 // group that finds no slot left walks its parts one after another in its own warp,
 // and adds them up in the same order, so its sums are the same; a launch with that
-// many of them is a full one anyhow.  At most 18 B a particle and 8 MB for the warps' own
+// many of them is a full one anyhow.  At most 31 B a particle and 12 MB for the warps' own
 // places, where a place per group and partial sums per particle took 250 B a particle.
 constexpr int64_t kSlotParticles = 320, kSlotMin = 32, kSlotMax = 2048;
 constexpr int kWarpsPerSm = 21;        // resident ones at most (96 registers a thread)
@@ -162,9 +162,9 @@ struct Parts {
     uint32_t *done;               // [slot, then warp] further parts finished
     uint2 *spill;                 // [slot, then warp][kSpill] child ranges
     uint2 *cnt;                   // [slot][part] PP and PN entries
-    float *sums;                  // [slot][part][axis][target]
+    float2 *sums;                 // [slot][part][axis][target] and their compensations
     uint2 *own_cnt;               // [warp], summed over the parts so far
-    float *own_sums;              // [warp][axis][target], the same
+    float2 *own_sums;             // [warp][axis][target], the same
 };
 
 struct WalkArgs {
@@ -396,7 +396,16 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float v) {
     sum = t;
 }
 
-// compensated totals of a lane's two targets
+// (s - k) + (os - ok) into s and k, exact but for the rounding of k
+__device__ __forceinline__ void pair_add(float &s, float &k, float os, float ok) {
+    const float t = __fadd_rn(s, os);
+    const float b = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(os, b));   // s + os - t, exactly
+    k = __fsub_rn(__fadd_rn(k, ok), e);
+    s = t;
+}
+
+// compensated totals of a lane's two targets: s - k
 struct Acc {
     float2 sx{0.f, 0.f}, sy{0.f, 0.f}, sz{0.f, 0.f}, kx{0.f, 0.f}, ky{0.f, 0.f}, kz{0.f, 0.f};
     __device__ __forceinline__ void add(const Sums &t) {
@@ -954,19 +963,18 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             continue;
         }
         uint32_t cnt_pn = __reduce_add_sync(FULL, my_pn), cnt_pp = cnt_all - cnt_pn;
-        float2 vx = make_float2(__fsub_rn(acc.sx.x, acc.kx.x), __fsub_rn(acc.sx.y, acc.kx.y));
-        float2 vy = make_float2(__fsub_rn(acc.sy.x, acc.ky.x), __fsub_rn(acc.sy.y, acc.ky.y));
-        float2 vz = make_float2(__fsub_rn(acc.sz.x, acc.kz.x), __fsub_rn(acc.sz.y, acc.kz.y));
-        float2 vp = kPot ? make_float2(__fsub_rn(psum.x, pcomp.x), __fsub_rn(psum.y, pcomp.y)) : make_float2(0.f, 0.f);
-        // replicas of a target: fixed-order pairwise sums, replica r with r + o
+        // replicas of a target: fixed-order pairwise sums, replica r with r + o, their
+        // compensations carried along
         for (uint32_t o = 1; o < R; o <<= 1) {
             const bool in = rep + o < R;
-            auto fold = [&](float &v) {
-                const float w = __shfl_down_sync(FULL, v, o * P);
-                if (in) v = __fadd_rn(v, w);
+            auto fold = [&](float &v, float &k) {
+                const float ov = __shfl_down_sync(FULL, v, o * P), ok = __shfl_down_sync(FULL, k, o * P);
+                if (in) pair_add(v, k, ov, ok);
             };
-            fold(vx.x); fold(vx.y); fold(vy.x); fold(vy.y); fold(vz.x); fold(vz.y);
-            if (kPot) { fold(vp.x); fold(vp.y); }
+            fold(acc.sx.x, acc.kx.x); fold(acc.sx.y, acc.kx.y);
+            fold(acc.sy.x, acc.ky.x); fold(acc.sy.y, acc.ky.y);
+            fold(acc.sz.x, acc.kz.x); fold(acc.sz.y, acc.kz.y);
+            if (kPot) { fold(psum.x, pcomp.x); fold(psum.y, pcomp.y); }
         }
         // A group in parts: every part leaves its sums and counts, and the one that
         // finishes last adds them up in the order of the parts.
@@ -988,17 +996,26 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             }
             if (slot >= slots) {
                 // no slot: the parts follow in this warp, as its next items
-                float *w = a.parts.own_sums + (uint64_t)(slot - slots) * (ax * 32u);
-                auto run = [&](uint32_t at, float &v) {
-                    if (part > 0u) v = __fadd_rn(w[at], v);
-                    w[at] = v;
+                float2 *w = a.parts.own_sums + (uint64_t)(slot - slots) * (ax * 32u);
+                auto run = [&](uint32_t at, float &v, float &k) {
+                    if (part > 0u) {
+                        float2 o = w[at];
+                        pair_add(o.x, o.y, v, k);
+                        v = o.x;
+                        k = o.y;
+                    }
+                    w[at] = make_float2(v, k);
                 };
                 if (rep == 0u) {
-                    run(t0, vx.x); run(32u + t0, vy.x); run(64u + t0, vz.x);
-                    if (kPot) run(96u + t0, vp.x);
+                    run(t0, acc.sx.x, acc.kx.x);
+                    run(32u + t0, acc.sy.x, acc.ky.x);
+                    run(64u + t0, acc.sz.x, acc.kz.x);
+                    if (kPot) run(96u + t0, psum.x, pcomp.x);
                     if (two) {
-                        run(t1, vx.y); run(32u + t1, vy.y); run(64u + t1, vz.y);
-                        if (kPot) run(96u + t1, vp.y);
+                        run(t1, acc.sx.y, acc.kx.y);
+                        run(32u + t1, acc.sy.y, acc.ky.y);
+                        run(64u + t1, acc.sz.y, acc.kz.y);
+                        if (kPot) run(96u + t1, psum.y, pcomp.y);
                     }
                 }
                 uint2 &c = a.parts.own_cnt[slot - slots];
@@ -1012,13 +1029,17 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 __syncwarp();
                 if (job) continue;
             } else {
-                float *w = a.parts.sums + ((uint64_t)slot * kParts + part) * (ax * 32u);
+                float2 *w = a.parts.sums + ((uint64_t)slot * kParts + part) * (ax * 32u);
                 if (rep == 0u) {
-                    w[t0] = vx.x; w[32u + t0] = vy.x; w[64u + t0] = vz.x;
-                    if (kPot) w[96u + t0] = vp.x;
+                    w[t0] = make_float2(acc.sx.x, acc.kx.x);
+                    w[32u + t0] = make_float2(acc.sy.x, acc.ky.x);
+                    w[64u + t0] = make_float2(acc.sz.x, acc.kz.x);
+                    if (kPot) w[96u + t0] = make_float2(psum.x, pcomp.x);
                     if (two) {
-                        w[t1] = vx.y; w[32u + t1] = vy.y; w[64u + t1] = vz.y;
-                        if (kPot) w[96u + t1] = vp.y;
+                        w[t1] = make_float2(acc.sx.y, acc.kx.y);
+                        w[32u + t1] = make_float2(acc.sy.y, acc.ky.y);
+                        w[64u + t1] = make_float2(acc.sz.y, acc.kz.y);
+                        if (kPot) w[96u + t1] = make_float2(psum.y, pcomp.y);
                     }
                 }
                 if (lane == 0) a.parts.cnt[(uint64_t)slot * kParts + part] = make_uint2(cnt_pp, cnt_pn);
@@ -1034,17 +1055,26 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 if (before + 2u != kParts) continue;
                 __threadfence();
                 w = a.parts.sums + (uint64_t)slot * kParts * (ax * 32u);
-                auto total = [&](uint32_t at) {
-                    float v = __ldcg(w + at);
-                    for (uint32_t q = 1; q < kParts; ++q) v = __fadd_rn(v, __ldcg(w + q * (ax * 32u) + at));
-                    return v;
+                auto total = [&](uint32_t at, float &v, float &k) {
+                    const float2 o = __ldcg(w + at);
+                    v = o.x;
+                    k = o.y;
+                    for (uint32_t q = 1; q < kParts; ++q) {
+                        const float2 x = __ldcg(w + q * (ax * 32u) + at);
+                        pair_add(v, k, x.x, x.y);
+                    }
                 };
                 if (rep == 0u) {
-                    const uint32_t u1 = two ? t1 : t0;
-                    vx = make_float2(total(t0), total(u1));
-                    vy = make_float2(total(32u + t0), total(32u + u1));
-                    vz = make_float2(total(64u + t0), total(64u + u1));
-                    if (kPot) vp = make_float2(total(96u + t0), total(96u + u1));
+                    total(t0, acc.sx.x, acc.kx.x);
+                    total(32u + t0, acc.sy.x, acc.ky.x);
+                    total(64u + t0, acc.sz.x, acc.kz.x);
+                    if (kPot) total(96u + t0, psum.x, pcomp.x);
+                    if (two) {
+                        total(t1, acc.sx.y, acc.kx.y);
+                        total(32u + t1, acc.sy.y, acc.ky.y);
+                        total(64u + t1, acc.sz.y, acc.kz.y);
+                        if (kPot) total(96u + t1, psum.y, pcomp.y);
+                    }
                 }
                 cnt_pp = cnt_pn = 0u;
                 for (uint32_t q = 0; q < kParts; ++q) {
@@ -1055,19 +1085,19 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             }
         }
         if (rep == 0u) {
-            T.acc[i0] = vx.x * p.out_scale;
-            T.acc[T.n + i0] = vy.x * p.out_scale;
-            T.acc[2 * T.n + i0] = vz.x * p.out_scale;
+            T.acc[i0] = __fsub_rn(acc.sx.x, acc.kx.x) * p.out_scale;
+            T.acc[T.n + i0] = __fsub_rn(acc.sy.x, acc.ky.x) * p.out_scale;
+            T.acc[2 * T.n + i0] = __fsub_rn(acc.sz.x, acc.kz.x) * p.out_scale;
             T.npp[i0] = cnt_pp - 1u;
             T.npn[i0] = cnt_pn;
-            if (kPot) T.pot[i0] = -vp.x * p.pot_scale;
+            if (kPot) T.pot[i0] = -__fsub_rn(psum.x, pcomp.x) * p.pot_scale;
             if (two) {
-                T.acc[i1] = vx.y * p.out_scale;
-                T.acc[T.n + i1] = vy.y * p.out_scale;
-                T.acc[2 * T.n + i1] = vz.y * p.out_scale;
+                T.acc[i1] = __fsub_rn(acc.sx.y, acc.kx.y) * p.out_scale;
+                T.acc[T.n + i1] = __fsub_rn(acc.sy.y, acc.ky.y) * p.out_scale;
+                T.acc[2 * T.n + i1] = __fsub_rn(acc.sz.y, acc.kz.y) * p.out_scale;
                 T.npp[i1] = cnt_pp - 1u;
                 T.npn[i1] = cnt_pn;
-                if (kPot) T.pot[i1] = -vp.y * p.pot_scale;
+                if (kPot) T.pot[i1] = -__fsub_rn(psum.y, pcomp.y) * p.pot_scale;
             }
         }
         if (lane == 0) {
