@@ -94,14 +94,15 @@ constexpr uint32_t kQuota = 48, kParts = 8;
 constexpr int kSpill = 192;            // ranges a walk can leave (with more it goes on until they are fewer)
 static_assert(kSpill > kStackDeep && kSpill <= kStackCap, "above kStackDeep a walk soon comes back below it");
 constexpr int64_t kSplitMin = 2048, kSplitMax = 196608;
-// Few groups leave anything: 1 to 2 in 100 of a clustered system of 10k to 190k, 1812 of
-// 370k in a batch of 8M particles.  What they leave goes to slots that the groups take
-// as they come, one for every 320 particles (6 in 100 groups) up to kSlotMax.  A
-// group that finds no slot left walks its parts one after another in its own warp,
-// and adds them up in the same order, so its sums are the same; a launch with that
-// many of them is a full one anyhow.  At most 31 B a particle and 12 MB for the warps' own
-// places, where a place per group and partial sums per particle took 250 B a particle.
-constexpr int64_t kSlotParticles = 320, kSlotMin = 32, kSlotMax = 2048;
+// What a group leaves goes to a slot; the groups take slots as they come.  Mostly few do (1 to 2 in
+// 100 groups of a clustered system of 10k to 190k, 1812 of 370k in a batch of 8M particles),
+// without the force split nearly all.  A group that finds no slot left walks its parts one
+// after another in its own warp and adds them up in the same order, so its sums are the
+// same; a launch with that many of them is a full one anyhow.  65k uniform particles without
+// the split: 485 us with a slot for every group, 788 with 204 slots, 851 without parts.
+// At most 76 MB of slots (groups of 32) and 13 MB of the warps' own places, where a place per
+// group and partial sums per particle took 250 B a particle of the whole forest.
+constexpr int64_t kSlotMax = 8192;
 constexpr int kWarpsPerSm = 21;        // resident ones at most (96 registers a thread)
 
 // shared memory of one warp: its stack, near chunk and far chunk
@@ -157,6 +158,7 @@ struct TreeView {
 // take, then one place per warp for the groups that find none.
 struct Parts {
     uint32_t slots, own;          // their numbers
+    uint32_t targets;             // of a group at most
     unsigned long long *taken;    // groups that asked for a slot (null: no walks in parts)
     uint2 *head;                  // [slot, then warp] group, ranges left
     uint32_t *done;               // [slot, then warp] further parts finished
@@ -979,7 +981,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         // A group in parts: every part leaves its sums and counts, and the one that
         // finishes last adds them up in the order of the parts.
         if (kParted && (leave || part > 0u)) {
-            constexpr uint32_t ax = kPot ? 4u : 3u;
+            const uint32_t tg1 = a.parts.targets, ax = (kPot ? 4u : 3u) * tg1;   // of one part
             const uint32_t t0 = 2u * tl, t1 = t0 + 1u;   // this lane's targets (t1 if `two`)
             const uint32_t slots = a.parts.slots;
             uint32_t slot = job >> 3;
@@ -996,7 +998,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             }
             if (slot >= slots) {
                 // no slot: the parts follow in this warp, as its next items
-                float2 *w = a.parts.own_sums + (uint64_t)(slot - slots) * (ax * 32u);
+                float2 *w = a.parts.own_sums + (uint64_t)(slot - slots) * ax;
                 auto run = [&](uint32_t at, float &v, float &k) {
                     if (part > 0u) {
                         float2 o = w[at];
@@ -1008,14 +1010,14 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 };
                 if (rep == 0u) {
                     run(t0, acc.sx.x, acc.kx.x);
-                    run(32u + t0, acc.sy.x, acc.ky.x);
-                    run(64u + t0, acc.sz.x, acc.kz.x);
-                    if (kPot) run(96u + t0, psum.x, pcomp.x);
+                    run(tg1 + t0, acc.sy.x, acc.ky.x);
+                    run(2u * tg1 + t0, acc.sz.x, acc.kz.x);
+                    if (kPot) run(3u * tg1 + t0, psum.x, pcomp.x);
                     if (two) {
                         run(t1, acc.sx.y, acc.kx.y);
-                        run(32u + t1, acc.sy.y, acc.ky.y);
-                        run(64u + t1, acc.sz.y, acc.kz.y);
-                        if (kPot) run(96u + t1, psum.y, pcomp.y);
+                        run(tg1 + t1, acc.sy.y, acc.ky.y);
+                        run(2u * tg1 + t1, acc.sz.y, acc.kz.y);
+                        if (kPot) run(3u * tg1 + t1, psum.y, pcomp.y);
                     }
                 }
                 uint2 &c = a.parts.own_cnt[slot - slots];
@@ -1029,17 +1031,17 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 __syncwarp();
                 if (job) continue;
             } else {
-                float2 *w = a.parts.sums + ((uint64_t)slot * kParts + part) * (ax * 32u);
+                float2 *w = a.parts.sums + ((uint64_t)slot * kParts + part) * ax;
                 if (rep == 0u) {
                     w[t0] = make_float2(acc.sx.x, acc.kx.x);
-                    w[32u + t0] = make_float2(acc.sy.x, acc.ky.x);
-                    w[64u + t0] = make_float2(acc.sz.x, acc.kz.x);
-                    if (kPot) w[96u + t0] = make_float2(psum.x, pcomp.x);
+                    w[tg1 + t0] = make_float2(acc.sy.x, acc.ky.x);
+                    w[2u * tg1 + t0] = make_float2(acc.sz.x, acc.kz.x);
+                    if (kPot) w[3u * tg1 + t0] = make_float2(psum.x, pcomp.x);
                     if (two) {
                         w[t1] = make_float2(acc.sx.y, acc.kx.y);
-                        w[32u + t1] = make_float2(acc.sy.y, acc.ky.y);
-                        w[64u + t1] = make_float2(acc.sz.y, acc.kz.y);
-                        if (kPot) w[96u + t1] = make_float2(psum.y, pcomp.y);
+                        w[tg1 + t1] = make_float2(acc.sy.y, acc.ky.y);
+                        w[2u * tg1 + t1] = make_float2(acc.sz.y, acc.kz.y);
+                        if (kPot) w[3u * tg1 + t1] = make_float2(psum.y, pcomp.y);
                     }
                 }
                 if (lane == 0) a.parts.cnt[(uint64_t)slot * kParts + part] = make_uint2(cnt_pp, cnt_pn);
@@ -1054,26 +1056,26 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 before = __shfl_sync(FULL, before, 0);
                 if (before + 2u != kParts) continue;
                 __threadfence();
-                w = a.parts.sums + (uint64_t)slot * kParts * (ax * 32u);
+                w = a.parts.sums + (uint64_t)slot * kParts * ax;
                 auto total = [&](uint32_t at, float &v, float &k) {
                     const float2 o = __ldcg(w + at);
                     v = o.x;
                     k = o.y;
                     for (uint32_t q = 1; q < kParts; ++q) {
-                        const float2 x = __ldcg(w + q * (ax * 32u) + at);
+                        const float2 x = __ldcg(w + q * ax + at);
                         pair_add(v, k, x.x, x.y);
                     }
                 };
                 if (rep == 0u) {
                     total(t0, acc.sx.x, acc.kx.x);
-                    total(32u + t0, acc.sy.x, acc.ky.x);
-                    total(64u + t0, acc.sz.x, acc.kz.x);
-                    if (kPot) total(96u + t0, psum.x, pcomp.x);
+                    total(tg1 + t0, acc.sy.x, acc.ky.x);
+                    total(2u * tg1 + t0, acc.sz.x, acc.kz.x);
+                    if (kPot) total(3u * tg1 + t0, psum.x, pcomp.x);
                     if (two) {
                         total(t1, acc.sx.y, acc.kx.y);
-                        total(32u + t1, acc.sy.y, acc.ky.y);
-                        total(64u + t1, acc.sz.y, acc.kz.y);
-                        if (kPot) total(96u + t1, psum.y, pcomp.y);
+                        total(tg1 + t1, acc.sy.y, acc.ky.y);
+                        total(2u * tg1 + t1, acc.sz.y, acc.kz.y);
+                        if (kPot) total(3u * tg1 + t1, psum.y, pcomp.y);
                     }
                 }
                 cnt_pp = cnt_pn = 0u;
@@ -1229,13 +1231,12 @@ void launch(const WalkArgs &a, int opening, bool split, bool dump, bool refit, b
     else dispatch<OG_OPEN_REL>(a, split, dump, refit, multi, pot, nitems, s, sms);
 }
 
-// The places of a pass of `groups` walks over n particles: one allocation, laid out by place().
+// The places of a pass of `groups` walks: one allocation, laid out by place().
 struct PartsScratch {
-    uint64_t slots, own, axes;
-    PartsScratch(int64_t n, int64_t groups, bool pot) : axes(pot ? 4u : 3u) {
-        const int64_t want = std::min(std::max(n / kSlotParticles, kSlotMin), kSlotMax);
-        slots = (uint64_t)std::min(want, groups);
-        own = want >= groups ? 0u : (uint64_t)std::min<int64_t>(groups + kMaxWarps, (int64_t)sm_count() * kWarpsPerSm);
+    uint64_t slots, own, targets, axes;
+    PartsScratch(int64_t groups, int group_max, bool pot) : targets((uint64_t)group_max), axes(pot ? 4u : 3u) {
+        slots = (uint64_t)std::min(kSlotMax, groups);
+        own = kSlotMax >= groups ? 0u : (uint64_t)std::min<int64_t>(groups + kMaxWarps, (int64_t)sm_count() * kWarpsPerSm);
     }
     uint64_t place(char *base, Parts *p) const {
         uint64_t at = 0;
@@ -1248,11 +1249,12 @@ struct PartsScratch {
         take(p->done, slots + own);
         take(p->spill, (slots + own) * kSpill);
         take(p->cnt, slots * kParts);
-        take(p->sums, slots * kParts * axes * 32u);
+        take(p->sums, slots * kParts * axes * targets);
         take(p->own_cnt, own);
-        take(p->own_sums, own * axes * 32u);
+        take(p->own_sums, own * axes * targets);
         p->slots = (uint32_t)slots;
         p->own = (uint32_t)own;
+        p->targets = (uint32_t)targets;
         return at;
     }
 };
@@ -1452,7 +1454,7 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
     cudaError_t err;
     void *sort_tmp = nullptr, *pass_tmp = nullptr;
     if (split_long) {
-        const PartsScratch sc(t->n, subset ? nsubset : t->ngroups, pot_sorted != nullptr);
+        const PartsScratch sc(subset ? nsubset : t->ngroups, t->prm.group_max, pot_sorted != nullptr);
         if ((err = dev_malloc_async(&pass_tmp, sc.place(nullptr, &a.parts), s)) != cudaSuccess)
             return cuda_fail(err, "cudaMallocAsync (walk parts)");
         sc.place(static_cast<char *>(pass_tmp), &a.parts);

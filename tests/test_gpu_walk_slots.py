@@ -27,10 +27,10 @@ def ctx():
     c.close()
 
 
-@pytest.mark.parametrize("n,group_max", [(9001, 32), (9001, 5), (6001, 1)])
+@pytest.mark.parametrize("n,group_max", [(9001, 32), (9001, 5), (8192, 1), (8193, 1), (16001, 1)])
 def test_with_and_without_a_slot(ctx, n, group_max):
-    """Every group's list spans a third of the box, so nearly all leave parts: hundreds
-    of groups to 32 slots."""
+    """Every group's list spans a third of the box, so nearly all leave parts: up to 8192
+    groups find slots, a half of 16,001 groups do not."""
     pos, mass = gi.uniform(n, 17)
     prm = gi.default_params(eps=0.002, r_s=0.1, opening=gi.OPEN_REL, alpha=1e-9, group_max=group_max)
     a_old = np.random.default_rng(2).normal(size=(n, 3)).astype(np.float32)
@@ -52,7 +52,7 @@ def test_with_and_without_a_slot(ctx, n, group_max):
         og.og_tree_force_active(t.h, on, out, a_old, cnt)
         assert np.array_equal(out[on > 0], acc[on > 0]) and np.array_equal(cnt[on > 0], npp[on > 0])
     ot = oracle.Tree(pos, mass, prm)
-    ref, rpp, rpn = ot.force(a_old=a_old, groups=np.arange(0, t.info()["groups"], 16))
+    ref, rpp, rpn = ot.force(a_old=a_old, groups=np.arange(0, t.info()["groups"], 32))
     on = np.isfinite(ref[:, 0])
     assert np.array_equal(npp[on], rpp[on]) and np.array_equal(npn[on], rpn[on])
     parity.check_accel(acc[on], ref[on])
@@ -61,8 +61,8 @@ def test_with_and_without_a_slot(ctx, n, group_max):
 
 def test_scratch_of_a_pass_is_bounded(ctx):
     """Groups of one particle: 60,000 groups.  A place of 3 KB for each would take 190 MB;
-    the slots, the warps' own places, the staged arrays and the order of the groups
-    take 18 B a particle, 8 MB, 32 B a particle and some 2 MB: 13 MB."""
+    8192 slots, the warps' own places, the staged arrays and the order of the groups
+    take 15, 5, 2 and some 2 MB."""
     n = 60000
     pos, mass = gi.halo_mix(n, 5, n_halo=60)
     side = n ** (1.0 / 3.0)
@@ -89,5 +89,5 @@ def test_scratch_of_a_pass_is_bounded(ctx):
         assert cudart.cudaMemPoolSetAttribute(pool, used_high, C.byref(v)) == 0
         t.force(a_old=a_old)
         assert cudart.cudaMemPoolGetAttribute(pool, used_high, C.byref(v)) == 0
-        assert v.value - before < 24 << 20, (v.value, before)
+        assert v.value - before < 48 << 20, (v.value, before)
     t.free()
