@@ -67,7 +67,8 @@ constexpr int kStackCap = 384;
 constexpr int kStackDeep = kStackCap - 64 - 7 * kLevels - 1;
 // A round appends at most 64 entries to either chunk, and a chunk is evaluated
 // after the round that takes it above a limit: kNearFlush entries, or `chunk`
-// far ones (WalkArgs::chunk, chosen at launch).  Both have room for that round and
+// far ones (WalkArgs::chunk, chosen at launch; 64 fewer with two replicas, far_limit in
+// k_walk).  Both have room for that round and
 // for the padding of an evaluation: fewer than kMaxRep entries in the near
 // chunk, kMaxRep x kFarStep in the far one.
 constexpr int kMaxRep = 16;        // replicas of a group's targets at most
@@ -158,15 +159,15 @@ struct TreeView {
 // take, then one place per warp for the groups that find none.
 struct Parts {
     uint32_t slots, own;          // their numbers
-    uint32_t targets;             // of a group at most
+    uint32_t pairs;               // of targets in a group at most
     unsigned long long *taken;    // groups that asked for a slot (null: no walks in parts)
     uint2 *head;                  // [slot, then warp] group, ranges left
     uint32_t *done;               // [slot, then warp] further parts finished
     uint2 *spill;                 // [slot, then warp][kSpill] child ranges
     uint2 *cnt;                   // [slot][part] PP and PN entries
-    float2 *sums;                 // [slot][part][axis][target] and their compensations
+    float4 *sums;                 // [slot][part][axis][pair]: two targets' totals, two compensations
     uint2 *own_cnt;               // [warp], summed over the parts so far
-    float2 *own_sums;             // [warp][axis][target], the same
+    float4 *own_sums;             // [warp][axis][pair], summed over the parts so far
 };
 
 struct WalkArgs {
@@ -391,19 +392,23 @@ __device__ __forceinline__ int pad_chunk(uint4 *ch, int cnt, uint32_t R, uint32_
     return (int)q;
 }
 
-__device__ __forceinline__ void kahan_add(float &sum, float &comp, float v) {
-    const float y = __fsub_rn(v, comp);
-    const float t = __fadd_rn(sum, y);
-    comp = __fsub_rn(__fsub_rn(t, sum), y);
+// a - b, each half rounded once
+__device__ __forceinline__ float2 sub2(const float2 &a, const float2 &b) { return __ffma2_rn(b, dup(-1.0f), a); }
+
+// v into the compensated totals sum - comp of a lane's two targets
+__device__ __forceinline__ void kahan_add(float2 &sum, float2 &comp, const float2 &v) {
+    const float2 y = sub2(v, comp);
+    const float2 t = __fadd2_rn(sum, y);
+    comp = sub2(sub2(t, sum), y);
     sum = t;
 }
 
 // (s - k) + (os - ok) into s and k, exact but for the rounding of k
-__device__ __forceinline__ void pair_add(float &s, float &k, float os, float ok) {
-    const float t = __fadd_rn(s, os);
-    const float b = __fsub_rn(t, s);
-    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(os, b));   // s + os - t, exactly
-    k = __fsub_rn(__fadd_rn(k, ok), e);
+__device__ __forceinline__ void pair_add(float2 &s, float2 &k, const float2 &os, const float2 &ok) {
+    const float2 t = __fadd2_rn(s, os);
+    const float2 b = sub2(t, s);
+    const float2 e = __fadd2_rn(sub2(s, sub2(t, b)), sub2(os, b));   // s + os - t, exactly
+    k = sub2(__fadd2_rn(k, ok), e);
     s = t;
 }
 
@@ -411,12 +416,9 @@ __device__ __forceinline__ void pair_add(float &s, float &k, float os, float ok)
 struct Acc {
     float2 sx{0.f, 0.f}, sy{0.f, 0.f}, sz{0.f, 0.f}, kx{0.f, 0.f}, ky{0.f, 0.f}, kz{0.f, 0.f};
     __device__ __forceinline__ void add(const Sums &t) {
-        kahan_add(sx.x, kx.x, t.x.x);
-        kahan_add(sx.y, kx.y, t.x.y);
-        kahan_add(sy.x, ky.x, t.y.x);
-        kahan_add(sy.y, ky.y, t.y.y);
-        kahan_add(sz.x, kz.x, t.z.x);
-        kahan_add(sz.y, kz.y, t.z.y);
+        kahan_add(sx, kx, t.x);
+        kahan_add(sy, ky, t.y);
+        kahan_add(sz, kz, t.z);
     }
 };
 
@@ -783,6 +785,12 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         const uint32_t tl = (uint32_t)lane - rep * P;
         const uint32_t R = min(32u / P, (uint32_t)kMaxRep);
         const uint32_t share = min(rep, R - 1u);    // the lanes left over repeat the last share, unused
+        // far entries after which the chunk is evaluated: a lane's plain sum of one
+        // evaluation takes at most chunk / 2 terms (two replicas: 64 entries short of the
+        // chunk, as a round may add 64; more replicas: the chunk).  Sums of 2000 terms of
+        // one sign in groups of 32 err by 1.9 roundings this way and 2.1 with the whole chunk
+        // for all; the time is within 1 %.
+        const int far_limit = min(chunk, (chunk >> 1) * (int)R - 64);
         const uint32_t i0 = gb + 2u * tl;
         const bool two = 2u * tl + 1u < gsize;
         const uint32_t i1 = two ? i0 + 1u : i0;
@@ -937,22 +945,16 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 __syncwarp();
                 const Sums t = eval_near<kSplit, kPot>(chn + share * (uint32_t)q, q, tg, p);
                 acc.add(t);
-                if (kPot) {
-                    kahan_add(psum.x, pcomp.x, t.p.x);
-                    kahan_add(psum.y, pcomp.y, t.p.y);
-                }
+                if (kPot) kahan_add(psum, pcomp, t.p);
                 cn = 0;
                 __syncwarp();
             }
-            if (__builtin_expect(done || cf > chunk, 0)) {
+            if (__builtin_expect(done || cf > far_limit, 0)) {
                 const int q = pad_chunk(chf, cf, R, (uint32_t)kFarStep, lane, box.hi);
                 __syncwarp();
                 const Sums t = eval_far<kSplit, kPot>(chf + share * (uint32_t)q, q, tg, p);
                 acc.add(t);
-                if (kPot) {
-                    kahan_add(psum.x, pcomp.x, t.p.x);
-                    kahan_add(psum.y, pcomp.y, t.p.y);
-                }
+                if (kPot) kahan_add(psum, pcomp, t.p);
                 cf = 0;
                 __syncwarp();
             }
@@ -969,20 +971,21 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         // compensations carried along
         for (uint32_t o = 1; o < R; o <<= 1) {
             const bool in = rep + o < R;
-            auto fold = [&](float &v, float &k) {
-                const float ov = __shfl_down_sync(FULL, v, o * P), ok = __shfl_down_sync(FULL, k, o * P);
-                if (in) pair_add(v, k, ov, ok);
+            auto fold = [&](float2 &v, float2 &k) {
+                float2 ov, ok, nv = v, nk = k;
+                ov.x = __shfl_down_sync(FULL, v.x, o * P); ov.y = __shfl_down_sync(FULL, v.y, o * P);
+                ok.x = __shfl_down_sync(FULL, k.x, o * P); ok.y = __shfl_down_sync(FULL, k.y, o * P);
+                pair_add(nv, nk, ov, ok);
+                if (in) { v = nv; k = nk; }
             };
-            fold(acc.sx.x, acc.kx.x); fold(acc.sx.y, acc.kx.y);
-            fold(acc.sy.x, acc.ky.x); fold(acc.sy.y, acc.ky.y);
-            fold(acc.sz.x, acc.kz.x); fold(acc.sz.y, acc.kz.y);
-            if (kPot) { fold(psum.x, pcomp.x); fold(psum.y, pcomp.y); }
+            fold(acc.sx, acc.kx); fold(acc.sy, acc.ky); fold(acc.sz, acc.kz);
+            if (kPot) fold(psum, pcomp);
         }
         // A group in parts: every part leaves its sums and counts, and the one that
         // finishes last adds them up in the order of the parts.
         if (kParted && (leave || part > 0u)) {
-            const uint32_t tg1 = a.parts.targets, ax = (kPot ? 4u : 3u) * tg1;   // of one part
-            const uint32_t t0 = 2u * tl, t1 = t0 + 1u;   // this lane's targets (t1 if `two`)
+            // per axis and lane one record of the two targets' totals
+            const uint32_t pairs = a.parts.pairs, ax = (kPot ? 4u : 3u) * pairs;   // of one part
             const uint32_t slots = a.parts.slots;
             uint32_t slot = job >> 3;
             if (part == 0u) {
@@ -998,27 +1001,15 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             }
             if (slot >= slots) {
                 // no slot: the parts follow in this warp, as its next items
-                float2 *w = a.parts.own_sums + (uint64_t)(slot - slots) * ax;
-                auto run = [&](uint32_t at, float &v, float &k) {
-                    if (part > 0u) {
-                        float2 o = w[at];
-                        pair_add(o.x, o.y, v, k);
-                        v = o.x;
-                        k = o.y;
-                    }
-                    w[at] = make_float2(v, k);
+                float4 *w = a.parts.own_sums + (uint64_t)(slot - slots) * ax;
+                auto run = [&](uint32_t axis, float2 &v, float2 &k) {
+                    float4 &q = w[axis * pairs + tl];
+                    if (part > 0u) pair_add(v, k, make_float2(q.x, q.y), make_float2(q.z, q.w));
+                    q = make_float4(v.x, v.y, k.x, k.y);
                 };
                 if (rep == 0u) {
-                    run(t0, acc.sx.x, acc.kx.x);
-                    run(tg1 + t0, acc.sy.x, acc.ky.x);
-                    run(2u * tg1 + t0, acc.sz.x, acc.kz.x);
-                    if (kPot) run(3u * tg1 + t0, psum.x, pcomp.x);
-                    if (two) {
-                        run(t1, acc.sx.y, acc.kx.y);
-                        run(tg1 + t1, acc.sy.y, acc.ky.y);
-                        run(2u * tg1 + t1, acc.sz.y, acc.kz.y);
-                        if (kPot) run(3u * tg1 + t1, psum.y, pcomp.y);
-                    }
+                    run(0u, acc.sx, acc.kx); run(1u, acc.sy, acc.ky); run(2u, acc.sz, acc.kz);
+                    if (kPot) run(3u, psum, pcomp);
                 }
                 uint2 &c = a.parts.own_cnt[slot - slots];
                 if (part > 0u) {
@@ -1031,18 +1022,12 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 __syncwarp();
                 if (job) continue;
             } else {
-                float2 *w = a.parts.sums + ((uint64_t)slot * kParts + part) * ax;
+                float4 *w = a.parts.sums + ((uint64_t)slot * kParts + part) * ax;
                 if (rep == 0u) {
-                    w[t0] = make_float2(acc.sx.x, acc.kx.x);
-                    w[tg1 + t0] = make_float2(acc.sy.x, acc.ky.x);
-                    w[2u * tg1 + t0] = make_float2(acc.sz.x, acc.kz.x);
-                    if (kPot) w[3u * tg1 + t0] = make_float2(psum.x, pcomp.x);
-                    if (two) {
-                        w[t1] = make_float2(acc.sx.y, acc.kx.y);
-                        w[tg1 + t1] = make_float2(acc.sy.y, acc.ky.y);
-                        w[2u * tg1 + t1] = make_float2(acc.sz.y, acc.kz.y);
-                        if (kPot) w[3u * tg1 + t1] = make_float2(psum.y, pcomp.y);
-                    }
+                    w[tl] = make_float4(acc.sx.x, acc.sx.y, acc.kx.x, acc.kx.y);
+                    w[pairs + tl] = make_float4(acc.sy.x, acc.sy.y, acc.ky.x, acc.ky.y);
+                    w[2u * pairs + tl] = make_float4(acc.sz.x, acc.sz.y, acc.kz.x, acc.kz.y);
+                    if (kPot) w[3u * pairs + tl] = make_float4(psum.x, psum.y, pcomp.x, pcomp.y);
                 }
                 if (lane == 0) a.parts.cnt[(uint64_t)slot * kParts + part] = make_uint2(cnt_pp, cnt_pn);
                 if (part == 0u) {          // the second launch walks the further parts
@@ -1057,26 +1042,16 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 if (before + 2u != kParts) continue;
                 __threadfence();
                 w = a.parts.sums + (uint64_t)slot * kParts * ax;
-                auto total = [&](uint32_t at, float &v, float &k) {
-                    const float2 o = __ldcg(w + at);
-                    v = o.x;
-                    k = o.y;
-                    for (uint32_t q = 1; q < kParts; ++q) {
-                        const float2 x = __ldcg(w + q * ax + at);
-                        pair_add(v, k, x.x, x.y);
+                auto total = [&](uint32_t axis, float2 &v, float2 &k) {
+                    v = k = make_float2(0.f, 0.f);
+                    for (uint32_t q = 0; q < kParts; ++q) {
+                        const float4 x = __ldcg(w + q * ax + axis * pairs + tl);
+                        pair_add(v, k, make_float2(x.x, x.y), make_float2(x.z, x.w));
                     }
                 };
                 if (rep == 0u) {
-                    total(t0, acc.sx.x, acc.kx.x);
-                    total(tg1 + t0, acc.sy.x, acc.ky.x);
-                    total(2u * tg1 + t0, acc.sz.x, acc.kz.x);
-                    if (kPot) total(3u * tg1 + t0, psum.x, pcomp.x);
-                    if (two) {
-                        total(t1, acc.sx.y, acc.kx.y);
-                        total(tg1 + t1, acc.sy.y, acc.ky.y);
-                        total(2u * tg1 + t1, acc.sz.y, acc.kz.y);
-                        if (kPot) total(3u * tg1 + t1, psum.y, pcomp.y);
-                    }
+                    total(0u, acc.sx, acc.kx); total(1u, acc.sy, acc.ky); total(2u, acc.sz, acc.kz);
+                    if (kPot) total(3u, psum, pcomp);
                 }
                 cnt_pp = cnt_pn = 0u;
                 for (uint32_t q = 0; q < kParts; ++q) {
@@ -1087,19 +1062,23 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             }
         }
         if (rep == 0u) {
-            T.acc[i0] = __fsub_rn(acc.sx.x, acc.kx.x) * p.out_scale;
-            T.acc[T.n + i0] = __fsub_rn(acc.sy.x, acc.ky.x) * p.out_scale;
-            T.acc[2 * T.n + i0] = __fsub_rn(acc.sz.x, acc.kz.x) * p.out_scale;
+            const float2 vx = __fmul2_rn(sub2(acc.sx, acc.kx), dup(p.out_scale));
+            const float2 vy = __fmul2_rn(sub2(acc.sy, acc.ky), dup(p.out_scale));
+            const float2 vz = __fmul2_rn(sub2(acc.sz, acc.kz), dup(p.out_scale));
+            const float2 vp = kPot ? __fmul2_rn(sub2(psum, pcomp), dup(-p.pot_scale)) : vx;
+            T.acc[i0] = vx.x;
+            T.acc[T.n + i0] = vy.x;
+            T.acc[2 * T.n + i0] = vz.x;
             T.npp[i0] = cnt_pp - 1u;
             T.npn[i0] = cnt_pn;
-            if (kPot) T.pot[i0] = -__fsub_rn(psum.x, pcomp.x) * p.pot_scale;
+            if (kPot) T.pot[i0] = vp.x;
             if (two) {
-                T.acc[i1] = __fsub_rn(acc.sx.y, acc.kx.y) * p.out_scale;
-                T.acc[T.n + i1] = __fsub_rn(acc.sy.y, acc.ky.y) * p.out_scale;
-                T.acc[2 * T.n + i1] = __fsub_rn(acc.sz.y, acc.kz.y) * p.out_scale;
+                T.acc[i1] = vx.y;
+                T.acc[T.n + i1] = vy.y;
+                T.acc[2 * T.n + i1] = vz.y;
                 T.npp[i1] = cnt_pp - 1u;
                 T.npn[i1] = cnt_pn;
-                if (kPot) T.pot[i1] = -__fsub_rn(psum.y, pcomp.y) * p.pot_scale;
+                if (kPot) T.pot[i1] = vp.y;
             }
         }
         if (lane == 0) {
@@ -1233,8 +1212,8 @@ void launch(const WalkArgs &a, int opening, bool split, bool dump, bool refit, b
 
 // The places of a pass of `groups` walks: one allocation, laid out by place().
 struct PartsScratch {
-    uint64_t slots, own, targets, axes;
-    PartsScratch(int64_t groups, int group_max, bool pot) : targets((uint64_t)group_max), axes(pot ? 4u : 3u) {
+    uint64_t slots, own, pairs, axes;
+    PartsScratch(int64_t groups, int group_max, bool pot) : pairs((uint64_t)(group_max + 1) / 2), axes(pot ? 4u : 3u) {
         slots = (uint64_t)std::min(kSlotMax, groups);
         own = kSlotMax >= groups ? 0u : (uint64_t)std::min<int64_t>(groups + kMaxWarps, (int64_t)sm_count() * kWarpsPerSm);
     }
@@ -1249,12 +1228,12 @@ struct PartsScratch {
         take(p->done, slots + own);
         take(p->spill, (slots + own) * kSpill);
         take(p->cnt, slots * kParts);
-        take(p->sums, slots * kParts * axes * targets);
+        take(p->sums, slots * kParts * axes * pairs);
         take(p->own_cnt, own);
-        take(p->own_sums, own * axes * targets);
+        take(p->own_sums, own * axes * pairs);
         p->slots = (uint32_t)slots;
         p->own = (uint32_t)own;
-        p->targets = (uint32_t)targets;
+        p->pairs = (uint32_t)pairs;
         return at;
     }
 };

@@ -69,3 +69,21 @@ def test_parts_add_no_rounding(ctx):
             t.free()
     whole, parts = (_rms(np.concatenate(e[o])) for o in (gi.OPEN_BH, gi.OPEN_REL))
     assert parts <= 1.1 * whole, (parts / ONE, whole / ONE)
+
+
+def test_plain_sums_stay_within_half_a_chunk(ctx):
+    """Groups of 31 and 32 targets (two replicas) at the default chunk of 256 entries: the
+    error of plain sums over at most 128 terms."""
+    n, e = 2000, []
+    for seed in range(6):
+        pos, mass = gi.uniform(n, 40 + seed)
+        t = og.Tree(ctx, pos, mass, _params(opening=gi.OPEN_BH, theta=0.0, walk_chunk=256))
+        _, npp, _, pot = t.force_pot()
+        assert (npp == n - 1).all()
+        beg, end, perm = t.export(og.OG_F_GBEG), t.export(og.OG_F_GEND), t.export(og.OG_F_PERM)
+        full = np.concatenate([perm[b:f] for b, f in zip(beg, end) if f - b >= 31])
+        assert len(full) > n // 4
+        e.append(_error(pot, _exact(pos, mass))[full])
+        t.free()
+    limit = ONE * np.sqrt(1.0 + 128 ** 2 / (3.0 * n))
+    assert _rms(np.concatenate(e)) <= limit, (_rms(np.concatenate(e)) / ONE, limit / ONE)
