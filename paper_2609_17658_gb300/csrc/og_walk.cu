@@ -68,15 +68,17 @@ constexpr int kStackDeep = kStackCap - 64 - 7 * kLevels - 1;
 // A round appends at most 64 entries to either chunk, and a chunk is evaluated
 // after the round that takes it above a limit: kNearFlush entries, or `chunk`
 // far ones (WalkArgs::chunk, chosen at launch; 64 fewer with two replicas, far_limit in
-// k_walk).  Both have room for that round and
-// for the padding of an evaluation: fewer than kMaxRep entries in the near
-// chunk, kMaxRep x kFarStep in the far one.
-constexpr int kMaxRep = 16;        // replicas of a group's targets at most
+// k_walk).  Both have room for that round and for the padding of an evaluation:
+// fewer than kMaxRep entries in the near chunk, kMaxRep x kFarStep in the far one.  The
+// 32 replicas of one pair of targets pad the near chunk to 128 at most, and the far one,
+// evaluated 64 entries sooner, to chunk + 127.
+constexpr int kMaxRep = 16;        // replicas of a group's targets at most (one or two targets: 32)
 constexpr int kFarStep = 4;        // far entries in flight per lane
 constexpr int kNearChunk = 128;
 constexpr int kNearFlush = kNearChunk - 64 - kMaxRep;
 constexpr int kFarPad = 64 + kMaxRep * kFarStep;
 constexpr int kMaxChunk = 1024;
+static_assert((kNearFlush + 64 + 31) / 32 * 32 <= kNearChunk && 32 * kFarStep - 1 <= kFarPad, "32 replicas' padding");
 
 // Long walks in parts.  The relative criterion gives a few groups (large boxes,
 // small accelerations) lists 15 times the mean, and one warp needs 0.3-0.5 ms for
@@ -783,14 +785,16 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         const uint32_t P = (gsize + 1u) >> 1;
         const uint32_t rep = ((uint32_t)lane * (65536u / P + 1u)) >> 16;   // lane / P
         const uint32_t tl = (uint32_t)lane - rep * P;
-        const uint32_t R = min(32u / P, (uint32_t)kMaxRep);
+        const uint32_t R = P == 1u ? 32u : min(32u / P, (uint32_t)kMaxRep);
         const uint32_t share = min(rep, R - 1u);    // the lanes left over repeat the last share, unused
         // far entries after which the chunk is evaluated: a lane's plain sum of one
         // evaluation takes at most chunk / 2 terms (two replicas: 64 entries short of the
         // chunk, as a round may add 64; more replicas: the chunk).  Sums of 2000 terms of
         // one sign in groups of 32 err by 1.9 roundings this way and 2.1 with the whole chunk
         // for all; the time is within 1 %.
-        const int far_limit = min(chunk, (chunk >> 1) * (int)R - 64);
+        // Groups of one or two targets take every lane (262k particles in groups of 1: 2.72 ms
+        // with 16 replicas, 2.58 with 32, 2.69 with one target a lane).
+        const int far_limit = P == 1u ? chunk - 64 : min(chunk, (chunk >> 1) * (int)R - 64);
         const uint32_t i0 = gb + 2u * tl;
         const bool two = 2u * tl + 1u < gsize;
         const uint32_t i1 = two ? i0 + 1u : i0;
@@ -1215,7 +1219,8 @@ struct PartsScratch {
     uint64_t slots, own, pairs, axes;
     PartsScratch(int64_t groups, int group_max, bool pot) : pairs((uint64_t)(group_max + 1) / 2), axes(pot ? 4u : 3u) {
         slots = (uint64_t)std::min(kSlotMax, groups);
-        own = kSlotMax >= groups ? 0u : (uint64_t)std::min<int64_t>(groups + kMaxWarps, (int64_t)sm_count() * kWarpsPerSm);
+        const int64_t warps = std::min<int64_t>(groups + kMaxWarps, (int64_t)sm_count() * kWarpsPerSm);
+        own = kSlotMax >= groups ? 0u : (uint64_t)warps;
     }
     uint64_t place(char *base, Parts *p) const {
         uint64_t at = 0;

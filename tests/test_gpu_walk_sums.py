@@ -14,8 +14,10 @@ import numpy as np
 import pytest
 
 import og_inputs as gi
+import oracle
 from paper_2609_17658_gb300 import build as B
 from paper_2609_17658_gb300 import og
+from tests import parity
 
 pytestmark = pytest.mark.gpu
 ONE = 0.42 * 2.0 ** -24
@@ -24,6 +26,7 @@ ONE = 0.42 * 2.0 ** -24
 @pytest.fixture(scope="module")
 def ctx():
     B.build()
+    oracle.build()
     c = og.Context(0)
     yield c
     c.close()
@@ -87,3 +90,20 @@ def test_plain_sums_stay_within_half_a_chunk(ctx):
         t.free()
     limit = ONE * np.sqrt(1.0 + 128 ** 2 / (3.0 * n))
     assert _rms(np.concatenate(e)) <= limit, (_rms(np.concatenate(e)) / ONE, limit / ONE)
+
+
+@pytest.mark.parametrize("walk_chunk", [64, 65, 191, 192, 321, 1024])
+@pytest.mark.parametrize("group_max", [1, 2, 3])
+def test_small_groups_at_the_edges_of_a_chunk(ctx, group_max, walk_chunk):
+    """One pair of targets takes 32 replicas, whose padding ends at the chunk's last
+    entries; a softening wide enough that near entries fill their chunk too."""
+    n = 3000
+    pos, mass = gi.halo_mix(n, 9, n_halo=4)
+    prm = gi.default_params(eps=0.02, r_s=0.08, opening=gi.OPEN_BH, theta=0.2, group_max=group_max,
+                            walk_chunk=walk_chunk)
+    t, ot = og.Tree(ctx, pos, mass, prm), oracle.Tree(pos, mass, prm)
+    acc, npp, npn = t.force()
+    ref, rpp, rpn = ot.force()
+    assert np.array_equal(npp, rpp) and np.array_equal(npn, rpn)
+    parity.check_accel(acc, ref)
+    t.free()
