@@ -24,8 +24,8 @@
 //          Threading        nextnode / sibling threading (unified index space)
 //   a5     exact node moments and centres of mass (og_moments.h): prefix
 //                           sums over the sorted particles, one pass over the nodes
-//          k_level_hist .. k_level_scatter   node ids bucketed by tree level (a
-//                           refit's extents only, made on the first refit)
+//          k_level_hist .. k_level_scatter   node ids bucketed by tree level (made on
+//                           the first refit that moves a particle by a quarter of the box)
 //          ExtentRanges    a refit's node extents from ranges of the sorted particles
 //          k_extents_level  the same level by level, for drifts above a quarter of the
 //          k_extents_run    box: a launch per large level, runs of small ones in a block
@@ -1067,7 +1067,9 @@ struct ExtRecords {
     const uint32_t *__restrict__ ext_s;
     const uint32_t *__restrict__ ext_l;
     CExt *cext;
+    const uint32_t *__restrict__ skip;       // null, or: nonzero, nothing to do
     __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        if (skip && *skip) return;
         int64_t c = (int64_t)bid * blockDim.x + threadIdx.x;
         if (c >= nchild) return;
         const uint32_t item = child[c];
@@ -1113,7 +1115,8 @@ __device__ __forceinline__ uint32_t gather21(uint64_t x) {
 // (16 us each at 200k particles, 210 us in all; this way 25).
 // A position counts from the key's cell the particle had in the build, X = origin
 // + signed drift, so it does not wrap where it leaves the box; a drift of a
-// quarter of the box or more is left to the level-by-level form.
+// quarter of the box or more is left to the level-by-level form, whose launches follow
+// while the rest of the refit still runs (these stages then return at once).
 struct Tile {
     long long lo[3], hi[3];
 };
@@ -1140,7 +1143,7 @@ constexpr long long kNoMin = 1ll << 62, kNoMax = -(1ll << 62);
 // the tiles of 32
 __global__ void k_repos(int64_t n, const uint32_t *__restrict__ perm, const uint4 *__restrict__ q4,
                         const uint64_t *__restrict__ skey, uint32_t *px, uint32_t *py, uint32_t *pz,
-                        Tile *__restrict__ t32, uint32_t *far) {
+                        Tile *__restrict__ t32, uint32_t *far, uint32_t *h_far) {
     pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     long long lo[3] = {kNoMin, kNoMin, kNoMin}, hi[3] = {kNoMax, kNoMax, kNoMax};
@@ -1159,7 +1162,10 @@ __global__ void k_repos(int64_t n, const uint32_t *__restrict__ perm, const uint
             wide = wide || d >= (1 << 30) || d <= -(1 << 30);
             lo[a] = hi[a] = (long long)o + d;
         }
-        if (wide) atomicOr(far, 1u);
+        if (wide) {
+            *far = 1u;                             // whichever of several writes
+            *h_far = 1u;                           // page-locked: the host reads it beside the next kernels
+        }
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -1182,7 +1188,9 @@ struct Tiles1024 {
     int64_t n32;
     const Tile *__restrict__ t32;
     Tile *__restrict__ t1024;
+    const uint32_t *__restrict__ far;
     __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        if (*far) return;
         const int64_t w = ((int64_t)bid * blockDim.x + threadIdx.x) >> 5;
         const int lane = threadIdx.x & 31;
         if (32 * w >= n32) return;
@@ -1227,7 +1235,9 @@ struct ExtentRanges {
     const Tile *__restrict__ t1024;
     uint32_t *ext_s;
     uint32_t *ext_l;
+    const uint32_t *__restrict__ far;
     __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        if (*far) return;
         const int64_t j = (int64_t)bid * blockDim.x + threadIdx.x;
         const int lane = threadIdx.x & 31;
         const int lev = j < m ? nlev[j] : 0;
@@ -1303,7 +1313,9 @@ struct ExtentTop {
     const uint32_t *__restrict__ norg;
     uint32_t *ext_s;
     uint32_t *ext_l;
+    const uint32_t *__restrict__ far;
     __device__ __forceinline__ void operator()(uint32_t bid, uint32_t nb) const {
+        if (*far) return;
         const uint32_t root = bid;
         const uint32_t slot = ncbeg[root] + threadIdx.x;
         if (threadIdx.x < nccnt[root] && slot < (uint64_t)nchild && child[slot] >= n) {
@@ -1534,7 +1546,7 @@ og_status cell_extents(og_tree *t) {
     ensure_origins(t);
     cudaStream_t s = t->ctx->stream;
     launch_pdl(k_cell_ext, nblk(t->nnodes), kT, 0, s, t->nnodes, t->nlev, t->norg, t->next_s, t->next_l);
-    run_stage<kT>(s, nblk(t->nchild), ExtRecords{t->n, t->nchild, t->child, t->next_s, t->next_l, t->cext});
+    run_stage<kT>(s, nblk(t->nchild), ExtRecords{t->n, t->nchild, t->child, t->next_s, t->next_l, t->cext, nullptr});
     return OG_OK;
 }
 
@@ -1573,20 +1585,25 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
     cudaEventRecord(e0, s);
     FirstClear fc{};
     fc.far = far;
+    // cleared by the host: no kernel of an earlier call still writes these words
+    uint32_t *h_far = pinned_counts(t->ctx);
+    *h_far = 0u;
     launch_pdl(k_quantize_keys, nblk(n), kT, 0, s, d_pos, n, B, t->seg_off, B > 1 ? pseg : nullptr,
                (const BoxIO *)nullptr, t->geom, t->h_geom[0], q4, (uint64_t *)nullptr, (uint64_t *)nullptr,
                (uint32_t *)nullptr, fc, t->ctx->d_status);
-    launch_pdl(k_repos, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, t->skey, t->px, t->py, t->pz, t32, far);
+    launch_pdl(k_repos, nblk(n), kT, 0, s, n, t->perm, (const uint4 *)q4, t->skey, t->px, t->py, t->pz, t32, far,
+               h_far);
+    cudaEventRecord(t->ctx->ev_to_side, s);
     const Moments mom(t, mom_scratch);
-    const Tiles1024 tiles1024{n32, t32, t1024};
+    const Tiles1024 tiles1024{n32, t32, t1024, far};
     const ExtentRanges ranges{t->nnodes, t->nlev, t->nbeg, t->nend, t->norg, t->px, t->py, t->pz, t32, t1024,
-                              t->next_s, t->next_l};
+                              t->next_s, t->next_l, far};
     const ExtentTop top{n, t->nlev, t->nbeg, t->nend, t->ncbeg, t->nccnt, t->nocc, t->child, t->px, t->py, t->pz,
-                        t->nchild, t->norg, t->next_s, t->next_l};
+                        t->nchild, t->norg, t->next_s, t->next_l, far};
     const GroupFin group_fin{n, nullptr, t->ngroups, t->gbeg, t->gend, t->px, t->py, t->pz, t->sseg, t->gbox, t->gseg};
     const Records records{n, nullptr, t->nchild, t->nchild, t->child, t->px, t->py, t->pz, t->pm32, t->pm64, t->nlev,
                           t->ncbeg, t->nccnt, t->nmom, t->ncom, t->crec, t->ctx->d_status};
-    const ExtRecords ext_records{n, t->nchild, t->child, t->next_s, t->next_l, t->cext};
+    const ExtRecords ext_records{n, t->nchild, t->child, t->next_s, t->next_l, t->cext, far};
     if (n <= kShareMax) {
         run_stages<kT>(s, (unsigned)mom.ntiles, mom.tiles(), nblk(32 * n1024), tiles1024, stride_grid(t->ngroups),
                        group_fin);
@@ -1608,29 +1625,24 @@ og_status refit_tree(og_tree *t, const double *d_pos) {
         run_stage<kT>(s, stride_grid(t->nchild), records);
         run_stage<kT>(s, nblk(t->nchild), ext_records);
     }
-    uint32_t *h_far = pinned_counts(t->ctx);
-    cudaMemcpyAsync(h_far, far, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-    cudaEventRecord(e1, s);
-    err = cudaStreamSynchronize(s);
-    if (err == cudaSuccess && *h_far) {
-        // a drift of a quarter of the box or more: the extents level by level
-        og_status st = level_lists(t, lcount);
-        if (st) {
-            cudaFreeAsync(scratch, s);
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            return st;
+    // the flag is there once k_repos has run
+    err = cudaEventSynchronize(t->ctx->ev_to_side);
+    og_status st = OG_OK;
+    if (err == cudaSuccess && *static_cast<volatile uint32_t *>(h_far)) {
+        st = level_lists(t, lcount);
+        if (st == OG_OK) {
+            extents_bottom_up(t, t->next_s, t->next_l);
+            run_stage<kT>(s, nblk(t->nchild), ExtRecords{n, t->nchild, t->child, t->next_s, t->next_l, t->cext,
+                                                         nullptr});
         }
-        extents_bottom_up(t, t->next_s, t->next_l);
-        run_stage<kT>(s, nblk(t->nchild), ExtRecords{n, t->nchild, t->child, t->next_s, t->next_l, t->cext});
-        cudaEventRecord(e1, s);
-        err = cudaStreamSynchronize(s);
     }
+    cudaEventRecord(e1, s);
+    if (err == cudaSuccess) err = cudaStreamSynchronize(s);
     cudaFreeAsync(scratch, s);
-    if (err != cudaSuccess) {
+    if (err != cudaSuccess || st != OG_OK) {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
-        return cuda_fail(err, "refit");
+        return st != OG_OK ? st : cuda_fail(err, "refit");
     }
     float ms = 0;
     cudaEventElapsedTime(&ms, e0, e1);
