@@ -161,8 +161,8 @@ og_status og_tree_refit(og_tree *t, const double *pos);
  * n_pp(i) = PP entries of i's group list minus itself, n_pn(i) = PN entries.
  * Device memory beside the tree, for the duration of the call: 24 B per group
  * for their order, and with OG_OPEN_REL and a box of 2049 to 196608 particles
- * up to 7.8 KB (9.8 KB with the potential) a group for walks in parts, 90 MB at
- * most; the host arrays' copies come on top.  The same holds for the other force calls. */
+ * up to 8.2 KB (10.2 KB with the potential) a group for walks in parts, 96 MB
+ * at most; the host arrays' copies come on top.  The same holds for the other force calls. */
 og_status og_tree_force(og_tree *t, const float *a_old, float *acc, uint32_t *n_pp,
                         uint32_t *n_pn);
 

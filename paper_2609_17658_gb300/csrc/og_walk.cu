@@ -58,13 +58,16 @@ namespace og {
 namespace {
 
 constexpr int kMaxWarps = 8;       // warps per block: 1..kMaxWarps, chosen at launch
-// Stack of child ranges per warp.  A round pushes at most 64 ranges, so below
-// kStackDeep it ends at most 63 above; from kStackDeep on a round takes a
-// single range (one node, at most 8 child nodes): a plain depth-first walk that
-// adds at most 7 ranges per tree level, 7 x 21 on the deepest path, so the
-// stack never holds more than kStackDeep + 63 + 147 ranges.
-constexpr int kStackCap = 384;
-constexpr int kStackDeep = kStackCap - 64 - 7 * kLevels - 1;
+// Stack of child ranges per warp.  A round that takes several ranges may leave at most
+// kStackSafe on it: from there a plain depth-first walk, one range (one node, at most 8
+// child nodes) a round, ends within the stack, as it adds at most 7 ranges per tree
+// level, 7 x 21 on the deepest path.  A round that would leave more is undone and taken
+// again with half as many ranges; the next ones take twice as many again.  (One range a round from 172
+// on, without trying: walks that open much of a large tree, on trees refitted after
+// drifts of a tenth of the box, 48 ms where 768 entries and no such rule took 30.)
+// One entry more keeps the range that a round takes in part.
+constexpr int kStackCap = 383;
+constexpr int kStackSafe = kStackCap - 7 * kLevels;
 // A round appends at most 64 entries to either chunk, and a chunk is evaluated
 // after the round that takes it above a limit: kNearFlush entries, or `chunk`
 // far ones (WalkArgs::chunk, chosen at launch; 64 fewer with two replicas, far_limit in
@@ -94,8 +97,8 @@ static_assert((kNearFlush + 64 + 31) / 32 * 32 <= kNearChunk && 32 * kFarStep - 
 // parts: 262-302 us at 100k.  The Barnes-Hut lists are even enough that splitting
 // them gained nothing at any size (131k 258 -> 265-280 us).
 constexpr uint32_t kQuota = 48, kParts = 8;
-constexpr int kSpill = 192;            // ranges a walk can leave (with more it goes on until they are fewer)
-static_assert(kSpill > kStackDeep && kSpill <= kStackCap, "above kStackDeep a walk soon comes back below it");
+constexpr int kSpill = 240;            // ranges a walk can leave (with more it goes on until they are fewer)
+static_assert(kSpill >= kStackSafe && kSpill <= kStackCap, "above kStackSafe a walk soon comes back below it");
 constexpr int64_t kSplitMin = 2048, kSplitMax = 196608;
 // What a group leaves goes to a slot; the groups take slots as they come.  Mostly few do (1 to 2 in
 // 100 groups of a clustered system of 10k to 190k, 1812 of 370k in a batch of 8M particles),
@@ -103,14 +106,14 @@ constexpr int64_t kSplitMin = 2048, kSplitMax = 196608;
 // after another in its own warp and adds them up in the same order, so its sums are the
 // same; a launch with that many of them is a full one anyhow.  65k uniform particles without
 // the split: 485 us with a slot for every group, 788 with 204 slots, 851 without parts.
-// At most 76 MB of slots (groups of 32) and 13 MB of the warps' own places, where a place per
+// At most 83 MB of slots (groups of 32) and 13 MB of the warps' own places, where a place per
 // group and partial sums per particle took 250 B a particle of the whole forest.
 constexpr int64_t kSlotMax = 8192;
 constexpr int kWarpsPerSm = 21;        // resident ones at most (96 registers a thread)
 
 // shared memory of one warp: its stack, near chunk and far chunk
 __host__ __device__ constexpr size_t warp_smem(int chunk) {
-    return kStackCap * sizeof(uint2) + ((size_t)chunk + kNearChunk + kFarPad) * sizeof(uint4);
+    return (kStackCap + 1) * sizeof(uint2) + ((size_t)chunk + kNearChunk + kFarPad) * sizeof(uint4);
 }
 constexpr size_t kMaxBlockSmem = kMaxWarps * warp_smem(kMaxChunk);
 static_assert(kMaxBlockSmem <= 227 * 1024, "walk block exceeds the shared memory of an SM");
@@ -719,7 +722,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
     const int chunk = a.chunk;
     unsigned char *wbase = smem + (size_t)warp * warp_smem(chunk);
     uint2 *stk = reinterpret_cast<uint2 *>(wbase);
-    uint4 *chn = reinterpret_cast<uint4 *>(wbase + kStackCap * sizeof(uint2));
+    uint4 *chn = reinterpret_cast<uint4 *>(wbase + (kStackCap + 1) * sizeof(uint2));
     uint4 *chf = chn + kNearChunk;
     const unsigned FULL = 0xffffffffu;
     const unsigned lt = (1u << lane) - 1u;
@@ -832,6 +835,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         const uint32_t quota = !kParted || part > 0u || !p.split_long ? 0xffffffffu : kQuota;
         bool leave = false;
         uint32_t rounds = 0;
+        int most = 32;                        // ranges the next round takes at most
         const uint32_t nchild = (uint32_t)T.nchild, max_rounds = (uint32_t)T.max_rounds;
         uint32_t cnt_all = 0, my_pn = 0;      // entries (warp), node entries (this lane)
         Acc acc;
@@ -839,8 +843,8 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         bool overflow = false;
 
         while (true) {
-            // every round consumes at least one child record and a record is
-            // visited at most once per walk: more rounds than records is a bug
+            // every round that is not undone consumes at least one child record and a
+            // record is visited at most once per walk: more rounds than that is a bug
             if (++rounds > max_rounds) {
                 overflow = true;
                 if (lane == 0) atomicOr(a.status, ST_INTERNAL);
@@ -848,7 +852,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             }
             // a round takes up to 64 child records from the top ranges of the
             // stack: slot l and slot l + 32 go to lane l
-            const int nr = sp > kStackDeep ? 1 : (sp < 32 ? sp : 32);
+            const int nr = min(sp, most);
             uint2 Rg = make_uint2(0u, 0u);
             if (lane < nr) Rg = stk[sp - 1 - lane];
             const uint32_t cnt = Rg.y;
@@ -869,9 +873,12 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             const unsigned shi = __reduce_or_sync(FULL, mine && excl >= 32u && excl < 64u ? 1u << (excl - 32u) : 0u);
             __syncwarp();
             sp -= nfull;
-            if (lane == nfull && mine && excl < 64u) {
-                const uint32_t used = 64u - excl;
-                stk[sp - 1] = make_uint2(Rg.x + used, Rg.y - used);
+            if (lane == nfull && mine) {
+                stk[kStackCap] = Rg;               // in case the round is undone
+                if (excl < 64u) {
+                    const uint32_t used = 64u - excl;
+                    stk[sp - 1] = make_uint2(Rg.x + used, Rg.y - used);
+                }
             }
             // this lane's two child slots: the range of a slot is the last one
             // starting at or before it
@@ -894,7 +901,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 // children, inside the child array)
                 const unsigned bo0 = __ballot_sync(FULL, c0.open), bo1 = __ballot_sync(FULL, c1.open);
                 const int np0 = __popc(bo0), npush = np0 + __popc(bo1);
-                if (sp + npush > kStackCap) return false;
+                if (sp + npush > (most > 1 ? kStackSafe : kStackCap)) return false;
                 if (c0.open) stk[sp + __popc(bo0 & lt)] = make_uint2(c0.push_ref, c0.push_cnt);
                 if (c1.open) stk[sp + np0 + __popc(bo1 & lt)] = make_uint2(c1.push_ref, c1.push_cnt);
                 sp += npush;
@@ -935,10 +942,21 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
             bool ok;
             if (kSplit && __builtin_expect(compact, 1)) ok = take(std::integral_constant<bool, true>{});
             else ok = take(std::integral_constant<bool, false>{});
-            if (!ok) {
-                overflow = true;
-                break;
+            if (__builtin_expect(!ok, 0)) {
+                if (most == 1) {
+                    overflow = true;
+                    break;
+                }
+                // undo: the ranges taken whole still lie above sp
+                const int taken = min(sp + nfull, most);
+                __syncwarp();
+                if (nfull < taken && lane == 0) stk[sp - 1] = stk[kStackCap];
+                __syncwarp();
+                sp += nfull;
+                most = taken >> 1;
+                continue;
             }
+            most = sp > kStackSafe ? 1 : min(2 * most, 32);
             __syncwarp();
             // a chunk above its limit, or the walk's end, is evaluated; flushes are
             // rare, so they are hinted off the round's path
@@ -1279,7 +1297,7 @@ og_status prepare_view(og_tree *t, int opening, bool first_pass, const float *a_
     w.crec = t->crec;
     w.cext = t->cext;
     w.nchild = t->nchild;
-    w.max_rounds = t->nchild + 2;
+    w.max_rounds = 6 * (t->nchild + 2);      // a round is undone five times at most (32 ranges, 16, .. 2)
     w.gseg = t->gseg;
     w.ncbeg = t->ncbeg;
     w.nccnt = t->nccnt;
