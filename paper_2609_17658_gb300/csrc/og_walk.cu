@@ -189,6 +189,11 @@ struct WalkArgs {
     Parts parts;
     int second;                   // the launch that walks the further parts
     int one_seg;                  // a single tree of one box: its parameters are p0
+    // The pass that only supplies the relative criterion's previous accelerations: plain
+    // sums of whole chunks and of replicas.  Its error of some 2e-7 moves no more than a few
+    // decisions of the second pass either way, and the list of a group does not change with
+    // how the second pass rounds its sums.
+    int plain;
     WalkParams p0;                // the box's parameters, in the launch's own argument space
     unsigned long long *inter;    // interactions evaluated
     unsigned long long *tree_inter;  // several trees: interactions per tree, or null
@@ -715,6 +720,8 @@ template <int kOpen, bool kSplit, bool kDump, bool kRefit, bool kMulti, bool kPo
 __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
     // walks in parts: the relative criterion, one tree
     constexpr bool kParted = kOpen == OG_OPEN_REL && !kMulti;
+    // (read from the arguments where it is used: held over the walk it costs a spill)
+    auto plain = [&] { return kOpen == OG_OPEN_BH && !kMulti && a.plain != 0; };
     extern __shared__ __align__(16) unsigned char smem[];
     // layout: per warp, its stack, near chunk and far chunk (warp_smem bytes);
     // blockDim.x = 32 * a.warps and the launch sizes smem to match
@@ -788,7 +795,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         const uint32_t P = (gsize + 1u) >> 1;
         const uint32_t rep = ((uint32_t)lane * (65536u / P + 1u)) >> 16;   // lane / P
         const uint32_t tl = (uint32_t)lane - rep * P;
-        const uint32_t R = P == 1u ? 32u : min(32u / P, (uint32_t)kMaxRep);
+        const uint32_t R = P == 1u && !plain() ? 32u : min(32u / P, (uint32_t)kMaxRep);
         const uint32_t share = min(rep, R - 1u);    // the lanes left over repeat the last share, unused
         // far entries after which the chunk is evaluated: a lane's plain sum of one
         // evaluation takes at most chunk / 2 terms (two replicas: 64 entries short of the
@@ -797,7 +804,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         // for all; the time is within 1 %.
         // Groups of one or two targets take every lane (262k particles in groups of 1: 2.72 ms
         // with 16 replicas, 2.58 with 32, 2.69 with one target a lane).
-        const int far_limit = P == 1u ? chunk - 64 : min(chunk, (chunk >> 1) * (int)R - 64);
+        const int far_limit = plain() ? chunk : P == 1u ? chunk - 64 : min(chunk, (chunk >> 1) * (int)R - 64);
         const uint32_t i0 = gb + 2u * tl;
         const bool two = 2u * tl + 1u < gsize;
         const uint32_t i1 = two ? i0 + 1u : i0;
@@ -990,7 +997,14 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
         }
         uint32_t cnt_pn = __reduce_add_sync(FULL, my_pn), cnt_pp = cnt_all - cnt_pn;
         // replicas of a target: fixed-order pairwise sums, replica r with r + o, their
-        // compensations carried along
+        // compensations carried along (plain sums: rounded away)
+        auto settle = [&](float2 &v, float2 &k) {
+            if (plain()) {
+                v = sub2(v, k);
+                k = dup(0.0f);
+            }
+        };
+        settle(acc.sx, acc.kx); settle(acc.sy, acc.ky); settle(acc.sz, acc.kz);
         for (uint32_t o = 1; o < R; o <<= 1) {
             const bool in = rep + o < R;
             auto fold = [&](float2 &v, float2 &k) {
@@ -998,7 +1012,7 @@ __global__ void __maxnreg__(kPot ? 128 : 96) k_walk(WalkArgs a) {
                 ov.x = __shfl_down_sync(FULL, v.x, o * P); ov.y = __shfl_down_sync(FULL, v.y, o * P);
                 ok.x = __shfl_down_sync(FULL, k.x, o * P); ok.y = __shfl_down_sync(FULL, k.y, o * P);
                 pair_add(nv, nk, ov, ok);
-                if (in) { v = nv; k = nk; }
+                if (in) { v = nv; k = plain() ? dup(0.0f) : nk; }
             };
             fold(acc.sx, acc.kx); fold(acc.sy, acc.ky); fold(acc.sz, acc.kz);
             if (kPot) fold(psum, pcomp);
@@ -1453,6 +1467,7 @@ og_status walk_pass(og_tree *t, int opening, bool first_pass, const float *a_old
     fill_common(a, t->ctx, t);
     a.one_seg = t->nseg == 1 ? 1 : 0;
     a.p0 = t->h_wp[0];
+    a.plain = first_pass ? 1 : 0;
     cudaError_t err;
     void *sort_tmp = nullptr, *pass_tmp = nullptr;
     if (split_long) {
