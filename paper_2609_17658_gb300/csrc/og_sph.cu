@@ -31,6 +31,8 @@
 // The round count is bounded by the number of nodes plus the buckets' extra
 // rounds.  Groups with very many candidates go to a block each (k_sph_long).
 #include <cmath>
+#include <map>
+#include <mutex>
 
 #include "og_internal.h"
 
@@ -484,6 +486,23 @@ constexpr int64_t kExpectMin = 16384;
 // scratch of a search: the long groups' number and list, the expected number
 inline size_t long_bytes(int64_t ng) { return (size_t)(ng + 2) * 4; }
 
+// blocks of k_sph_long that the device holds at once, asked once per device
+int64_t resident_long() {
+    static std::mutex mu;
+    static std::map<int, int64_t> blocks;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = blocks.find(dev);
+    if (it == blocks.end()) {
+        int sms = 1, per = 1;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sph_long, kLongThreads, 0);
+        it = blocks.emplace(dev, (int64_t)sms * (per < 1 ? 1 : per)).first;
+    }
+    return it->second;
+}
+
 // the density of every group of the tree, at a.hg
 void search(SphArgs &a, char *scratch, cudaStream_t s) {
     if (a.ngroups < 1) return;
@@ -498,8 +517,8 @@ void search(SphArgs &a, char *scratch, cudaStream_t s) {
         a.many = many;
     }
     k_sph_density<<<nblk(a.ngroups, kSphWarps), 32 * kSphWarps, kSphSmem, s>>>(a); note_launch();
-    const unsigned most = (unsigned)(a.ngroups < 456 ? a.ngroups : 456);   // 152 SMs x 3 blocks
-    k_sph_long<<<most, kLongThreads, 0, s>>>(a); note_launch();
+    const int64_t most = a.ngroups < resident_long() ? a.ngroups : resident_long();
+    k_sph_long<<<(unsigned)most, kLongThreads, 0, s>>>(a); note_launch();
 }
 
 }  // namespace
