@@ -256,6 +256,18 @@ og_status status_from(og_ctx *c, uint32_t st) {
     return OG_ERR_STATE;
 }
 
+// Whether the host itself may touch a caller's array (null: nothing to touch).  A call
+// without OG_DEVICE_PTRS that is given device memory keeps the copies' answer to it.
+static bool host_reads(const void *q) {
+    cudaPointerAttributes at;
+    if (!q) return true;
+    if (cudaPointerGetAttributes(&at, q) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type != cudaMemoryTypeDevice;
+}
+
 og_status validate(const og_params *p, int64_t n) {
     if (!p) { set_error("params is NULL"); return OG_ERR_ARG; }
     if (n < 1 || n > kMaxN) { set_error("N = %lld out of range [1, %lld]", (long long)n, (long long)kMaxN); return OG_ERR_ARG; }
@@ -472,7 +484,7 @@ og_status og_tree_build(og_ctx *c, const double *pos, const double *mass, int64_
             return cuda_fail(e, "cudaMallocAsync (inputs)");
         }
         double *dp = static_cast<double *>(staging);
-        if (bytes <= kStageBytes) {
+        if (bytes <= kStageBytes && host_reads(pos) && host_reads(mass)) {
             // small: through the context's page-locked memory in one copy (the build
             // synchronises, so no copy of an earlier call still reads it)
             char *h = pinned_stage(c);
@@ -621,7 +633,8 @@ og_status og_tree_force(og_tree *t, const float *a_old, float *acc, uint32_t *n_
     void *out_tmp = nullptr;
     // small host outputs: the last kernel writes them to the context's page-locked
     // memory, and the host copies them on after the call's synchronisation
-    const bool staged = !dev && (size_t)n * 20 <= kStageBytes;
+    const bool staged = !dev && (size_t)n * 20 <= kStageBytes && host_reads(acc) && host_reads(n_pp) &&
+                        host_reads(n_pn);
     if (staged) {
         d_acc = reinterpret_cast<float *>(pinned_stage(c));
         d_npp = n_pp ? reinterpret_cast<uint32_t *>(d_acc + 3 * n) : nullptr;

@@ -610,7 +610,7 @@ __device__ __forceinline__ Cls classify(const TreeView &T, uint32_t ci, bool has
 // whose prune distance is below 2^29: signed differences to the near and far
 // sides, no wrap to tell apart, and one straight line for particles and nodes,
 // so that the two records of a lane overlap.  About 60 instructions a record,
-// where the interval form below takes about 100 in two divergent branches.
+// where the interval form above takes about 100 in two divergent branches.
 //
 // With a = lo - c and b = c - hi (signed), the gap of c is max(a, b, 0).  It
 // differs from the gap on the circle only where both a and b are positive,

@@ -49,3 +49,41 @@ def test_host_arrays_equal_device_arrays(n, rel):
     t2.free()
     one.close()
     two.close()
+
+
+def _status_of_device_arrays(ctx, n, outputs):
+    """Status of a build (or of a force call's outputs) that is given device memory in a
+    host-pointer call, and the forces if it took it."""
+    import ctypes as C
+
+    import torch
+    pos, mass = gi.uniform(n, 7)
+    prm = og.params_from_dict(gi.default_params(eps=1e-3, r_s=0.02, opening=gi.OPEN_BH))
+    dpos, dmass = torch.from_numpy(pos).cuda(), torch.from_numpy(mass).cuda()
+    dacc = torch.zeros((n, 3), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    h, acc = C.c_void_p(), np.zeros((n, 3), np.float32)
+    src = (pos.ctypes.data, mass.ctypes.data) if outputs else (dpos.data_ptr(), dmass.data_ptr())
+    st = og.lib().og_tree_build(ctx.h, C.c_void_p(src[0]), C.c_void_p(src[1]), n, C.byref(prm), C.byref(h))
+    if st != og.OG_OK:
+        return st, None
+    dst = dacc.data_ptr() if outputs else acc.ctypes.data
+    st = og.lib().og_tree_force(h, None, C.c_void_p(dst), None, None)
+    og.og_tree_free(h)
+    torch.cuda.synchronize()
+    return st, dacc.cpu().numpy() if outputs else acc
+
+
+@pytest.mark.parametrize("outputs", [False, True])
+def test_device_arrays_in_a_host_call(outputs):
+    """The host's own copies of small arrays must not touch device memory: a call that
+    is given it answers as it does for large arrays, which are copied by CUDA."""
+    B.build()
+    with og.Context(0) as ctx:
+        large, _ = _status_of_device_arrays(ctx, 40000, outputs)
+        small, got = _status_of_device_arrays(ctx, 4096, outputs)
+        assert small == large
+        pos, mass = gi.uniform(4096, 7)
+        want, _, _ = og.Tree(ctx, pos, mass, gi.default_params(eps=1e-3, r_s=0.02, opening=gi.OPEN_BH)).force()
+        if small == og.OG_OK:
+            assert np.array_equal(got, want)
