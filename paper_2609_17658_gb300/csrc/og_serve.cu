@@ -44,11 +44,12 @@ constexpr int kT = 256;
 inline unsigned nblk(int64_t n) { return (unsigned)((n + kT - 1) / kT); }
 constexpr int kMaxActive = 256;
 constexpr int kMaxRefits = 64;   // refits between builds at most
-// costs in walk interactions (about 2e-12 s each on the multi-tree walk): a
-// build about 0.18 ms of launch-bound work plus 0.3 ns per particle, a refit
-// about 0.17 ms plus 0.18 ns per particle; a refitted tree's walk costs 13 %
-// more per interaction (it reads node extents); measured on GB300 at
-// 2e4, 2e5 and 2e6 particles
+// costs in walk interactions, at 2e-12 s each: a build 0.18 ms plus 0.3 ns per
+// particle, a refit 0.17 ms plus 0.18 ns per particle, a refitted tree's walk 13 %
+// more per interaction (it reads node extents).  Measured on an earlier build of this
+// library, at 2e4, 2e5 and 2e6 particles; now 20k, 200k and 1M particles take 0.08, 0.10
+// and 0.25 ms to refit and 0.09, 0.18 and 0.42 to build, an interaction 1.4e-12 s.  Kept as
+// they are: they decide which tree a request is walked with, and so its lists and bits.
 constexpr double kBuildFixedInter = 9.0e7, kBuildPerParticleInter = 150.0;
 constexpr double kRefitFixedInter = 8.5e7, kRefitPerParticleInter = 90.0;
 constexpr double kRefitWalkFactor = 1.13;

@@ -29,9 +29,10 @@
 //                   accumulation over the chunk, then a compensated (Kahan) add
 //                   into the totals.  A group of g targets takes P = ceil(g / 2)
 //                   lanes; 32 / P replicas of them split the chunk's entries,
-//                   and the replicas' totals are added in a fixed order at the end.
+//                   and the replicas' totals are added in a fixed order at the end,
+//                   with their compensations.
 //
-// What bounds it (2.1M clustered, Barnes-Hut pass, 2.75 ms): instruction issue
+// What bounds it (2.1M clustered, Barnes-Hut pass, 2.7 ms): instruction issue
 // (74 % of cycles) and the pipes behind it.  2.4 G warp instructions, 1.3 G of
 // them the far loop: 42 a pair of interactions, beside which the pair keeps the
 // multi-function pipe 40 cycles and the FMA pipe 36 busy, so no one unit can be
@@ -39,7 +40,7 @@
 // for 6 or 8 blocks per SM, or 2 to 8 entries in flight all measured within 2 %.
 // The list building is the other 1 G, about 390 a round of 64 slots.  Two targets
 // a lane, the straight-line classification and the erfc from 1 / r took the pass
-// from 3.40 to 2.75 ms and the two-pass walk from 7.10 to 5.73 ms.
+// from 3.40 to 2.75 ms and the two-pass walk from 7.10 to 5.73 ms (5.69 now).
 //
 // Work distribution: persistent blocks; warps take groups from a global
 // atomic counter, in decreasing order of the previous pass's list length
@@ -90,7 +91,10 @@ static_assert((kNearFlush + 64 + 31) / 32 * 32 <= kNearChunk && 32 * kFarStep - 
 // which a second launch walks.  This depends on nothing but the group's own
 // walk, so a group's sums are the same whatever else is in the launch.
 // Only for boxes of 2049 to 196608 particles: below, no walk gets that far; above,
-// the other groups fill the time and the parts cost more than they save.
+// the other groups fill the time and the parts cost more than they save.  The rule looks
+// at the box and not at the launch, for the same reason; boxes of that size in a batch that
+// fills the GPU pay for it: 64 boxes of 4k to 65k 2.80 ms with parts, 2.69 without, both
+// passes 4.32 and 4.07; 128 boxes of 4k to 262k 11.96 and 11.92.
 // Clustered, accelerations given: 32k 197 -> 154 us, 100k 356 -> 262, 131k 433 ->
 // 309, 262k 499 -> 522 (not split); both passes: 65k 901 -> 554, 131k 785 -> 658,
 // 2.1M 5.71 -> 6.08 ms (not split).  A quota of 32, 40 or 64 rounds, or 16 and 32
